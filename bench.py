@@ -38,8 +38,9 @@ WORKLOAD = "single vector d=2^26 FP32 N(0,1) + 10% exact duplicates, lambda cycl
 # Algorithmic HBM bytes per element for each kernel kind of the device-wide
 # path (FP32 storage): what a launch must read and write at the least.
 ALGO_BYTES_PER_ELEM_F32 = {
-    "onesweep": 8,    # read key (pass 0: the value) + write key
-    "hist": 4,        # read the value
+    "partition": 8,   # read key (first pass: the value) + write key
+    "bin_sort": 8,    # read key + write key
+    "sort_plan": 4,   # read the value
     "tile_hull": 4,   # read the sorted key (hull vertices are data dependent, not counted)
     "lookup": 12,     # read w, write out and cluster id (I/O floor)
 }
@@ -58,9 +59,9 @@ MODEL_B = {"key_only_52B": 52, "index_payload_80B": 80}
 # ncu capture of the bench's own workload, and the hash of the source files the
 # kernel is built from when the counters were taken; reported as null once any
 # of them changes (see profiles/).
-NCU_SOURCES = {"onesweep": ["ws_sort.cu", "ws_kernels.cuh", "ws_block.cuh", "ws_common.cuh"]}
-NCU_TRAFFIC = {"onesweep": 511.8e6}   # d = 2^26, mean of the 4 passes (1 ncu pass each)
-NCU_SOURCE_HASH = {"onesweep": "bb6a5940a12a3213"}
+NCU_SOURCES = {}
+NCU_TRAFFIC = {}
+NCU_SOURCE_HASH = {}
 
 
 def source_hash(files=None) -> str:

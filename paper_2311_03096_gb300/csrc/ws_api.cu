@@ -63,9 +63,22 @@ struct ws_plan {
     void* keys_a = nullptr;
     void* keys_b = nullptr;
     uint32_t* hist = nullptr;
-    uint64_t* lookback = nullptr;
-    uint32_t* tile_counter = nullptr;
-    uint32_t* epoch = nullptr;
+    SortCtl* ctl = nullptr;       // start of the words cleared before every sort
+    size_t sort_zero_bytes = 0;
+    unsigned long long* seg_hi = nullptr;
+    unsigned long long* seg_lo = nullptr;
+    uint32_t* seg_en = nullptr;
+    uint32_t* cells = nullptr;
+    uint32_t* bin_cnt = nullptr;
+    int n_bins = 0, max_bins = 0, two_level = 0;
+    WsSortShape sort_shape;
+    void* bins = nullptr;
+    uint32_t* bin_start = nullptr;
+    uint32_t* cur1 = nullptr;
+    uint32_t* cur2 = nullptr;
+    int32_t* bin_seg = nullptr;
+    OverBin* over = nullptr;
+    uint32_t* over_cnt = nullptr;
     int32_t* seg_emin = nullptr;
     uint16_t* vp = nullptr;
     i128* vx = nullptr;
@@ -116,9 +129,23 @@ LargeWork<T> make_work(const ws_plan* p) {
     W.keys_a = (K*)p->keys_a;
     W.keys_b = (K*)p->keys_b;
     W.hist = p->hist;
-    W.lookback = p->lookback;
-    W.tile_counter = p->tile_counter;
-    W.epoch = p->epoch;
+    W.ctl = p->ctl;
+    W.sort_zero_bytes = p->sort_zero_bytes;
+    W.seg_hi = p->seg_hi;
+    W.seg_lo = p->seg_lo;
+    W.seg_en = p->seg_en;
+    W.cells = p->cells;
+    W.bin_cnt = p->bin_cnt;
+    W.n_bins = p->n_bins;
+    W.sort_shape = p->sort_shape;
+    W.two_level = p->two_level;
+    W.bins = p->bins;
+    W.bin_start = p->bin_start;
+    W.cur1 = p->cur1;
+    W.cur2 = p->cur2;
+    W.bin_seg = p->bin_seg;
+    W.over = p->over;
+    W.over_cnt = p->over_cnt;
     W.seg_emin = p->seg_emin;
     W.vp = p->vp;
     W.vx = p->vx;
@@ -178,6 +205,12 @@ int ceil_log2(int64_t v) {
     return k;
 }
 
+ws_status map_cuda(cudaError_t e) {
+    if (e == cudaSuccess) return WS_OK;
+    cudaGetLastError();
+    return e == cudaErrorMemoryAllocation ? WS_ERR_NOMEM : WS_ERR_CUDA;
+}
+
 ws_status build_plan(ws_plan* p) {
     const bool f64 = p->dtype == WS_F64;
     const int64_t small_cap = f64 ? SmallCfg<double>::CAP : SmallCfg<float>::CAP;
@@ -190,6 +223,9 @@ ws_status build_plan(ws_plan* p) {
     std::vector<LargeSeg> lsegs;
     std::vector<TileDesc> stiles, htiles;
     int64_t kpos = 0, dir_pos = 0;
+    int64_t bin_pos = 0, coarse_pos = 0, cell_pos = 0;
+    std::vector<int32_t> bin_seg;
+    int samp_max = 0;
     for (int64_t s = 0; s < p->n_seg; ++s) {
         int64_t a = p->h_offsets[s], len = p->h_offsets[s + 1] - a;
         if (len <= p->small_max || len <= 1) { small.push_back((int32_t)s); continue; }
@@ -216,6 +252,29 @@ ws_status build_plan(ws_plan* p) {
         ls.dir_cap_log2 = std::min(ceil_log2(len), WS_DIR_MAX_LOG2);
         ls.dir_pos = dir_pos;
         dir_pos += ((int64_t)1 << ls.dir_cap_log2) + 1;
+        // distribution sort: bins, buckets of the first pass, map
+        ls.nbins = len <= WS_BIN_CAP ? 1 : (int32_t)std::min<int64_t>((len + WS_BIN_MEAN - 1) / WS_BIN_MEAN, WS_BINS_MAX);
+        ls.fine_log2 = 0;
+        if (ls.nbins > WS_ONE_LEVEL) {
+            ls.fine_log2 = 7;
+            while (((ls.nbins - 1) >> ls.fine_log2) + 1 > WS_ONE_LEVEL) ++ls.fine_log2;
+            p->two_level = 1;
+        }
+        ls.n_coarse = ((ls.nbins - 1) >> ls.fine_log2) + 1;
+        ls.ncell = ls.fine_log2 ? WS_CELLS : WS_CELLS / 2;
+        // samples per tile: 100 per bin for one-pass segments, 50 for longer ones (about 2^20 at most)
+        ls.samp_log2 = ls.fine_log2 ? 7 : 8;
+        while (ls.samp_log2 > 5 && ((int64_t)ls.sort_count << ls.samp_log2) > ((int64_t)1 << 20)) --ls.samp_log2;
+        samp_max = std::max(samp_max, (int)ls.samp_log2);
+        ls.bin_pos = (int32_t)bin_pos;
+        ls.coarse_pos = (int32_t)coarse_pos;
+        ls.cell_pos = (int32_t)cell_pos;
+        bin_pos += ls.nbins;
+        coarse_pos += ls.n_coarse;
+        cell_pos += 3 * ls.ncell;   // counts of the cells, then of their parts (at most two per cell on average)
+        if (cell_pos > INT32_MAX || bin_pos > INT32_MAX) return WS_ERR_NOMEM;
+        p->max_bins = std::max(p->max_bins, (int)ls.nbins);
+        bin_seg.insert(bin_seg.end(), (size_t)ls.nbins, (int32_t)lseg);
         kpos += (len + 3) & ~(int64_t)3;   // keep every segment's keys 16-byte aligned
         lsegs.push_back(ls);
     }
@@ -246,19 +305,43 @@ ws_status build_plan(ws_plan* p) {
     if ((st = plan_upload(p, &p->d_lsegs, lsegs))) return st;
     if ((st = plan_upload(p, &p->d_sort_tiles, stiles))) return st;
     if ((st = plan_upload(p, &p->d_hull_tiles, htiles))) return st;
-    const int P = f64 ? 8 : 4;
     const size_t nk = (size_t)p->n_keys, nh = (size_t)p->n_hull_tiles, slots = nk + (size_t)p->n_lseg;
     if ((st = plan_alloc(p, &p->keys_a, ksize * nk))) return st;
     if ((st = plan_alloc(p, &p->keys_b, ksize * nk))) return st;
-    if ((st = plan_alloc(p, (void**)&p->hist, sizeof(uint32_t) * p->n_lseg * P * 256))) return st;
-    if ((st = plan_alloc(p, (void**)&p->lookback, sizeof(uint64_t) * (size_t)P * p->n_sort_tiles * 256))) return st;
-    if ((st = plan_alloc(p, (void**)&p->tile_counter, sizeof(uint32_t) * P))) return st;
-    if ((st = plan_alloc(p, (void**)&p->epoch, sizeof(uint32_t)))) return st;
+    if ((st = plan_alloc(p, (void**)&p->hist, sizeof(uint64_t) * (3 * 256 + 2)))) return st;
+    {
+        // one block, cleared before every sort: control words, sampled ranges, cells, bin counts
+        const size_t nl = (size_t)p->n_lseg;
+        const size_t o_hi = sizeof(SortCtl), o_lo = o_hi + 8 * nl, o_en = o_lo + 8 * nl, o_cells = o_en + 4 * nl,
+                     o_cnt = o_cells + 4 * (size_t)cell_pos;
+        p->sort_zero_bytes = o_cnt + 4 * (size_t)bin_pos;
+        unsigned char* z = nullptr;
+        if ((st = plan_alloc(p, (void**)&z, p->sort_zero_bytes))) return st;
+        p->ctl = (SortCtl*)z;
+        p->seg_hi = (unsigned long long*)(z + o_hi);
+        p->seg_lo = (unsigned long long*)(z + o_lo);
+        p->seg_en = (uint32_t*)(z + o_en);
+        p->cells = (uint32_t*)(z + o_cells);
+        p->bin_cnt = (uint32_t*)(z + o_cnt);
+        p->n_bins = (int)bin_pos;
+    }
+    {
+        const cudaError_t e = f64 ? ws_sort_prepare<double>(p->max_bins, p->n_sort_tiles, samp_max, &p->sort_shape)
+                                  : ws_sort_prepare<float>(p->max_bins, p->n_sort_tiles, samp_max, &p->sort_shape);
+        if (e) return map_cuda(e);
+    }
+    if ((st = plan_upload(p, &p->bin_seg, bin_seg))) return st;
+    if ((st = plan_alloc(p, &p->bins, 2 * (p->sort_shape.wide ? 4 : 2) * nk))) return st;
+    if ((st = plan_alloc(p, (void**)&p->bin_start, sizeof(uint32_t) * (size_t)bin_pos))) return st;
+    if ((st = plan_alloc(p, (void**)&p->cur1, sizeof(uint32_t) * (size_t)coarse_pos))) return st;
+    if ((st = plan_alloc(p, (void**)&p->cur2, sizeof(uint32_t) * (size_t)bin_pos))) return st;
+    if ((st = plan_alloc(p, (void**)&p->over, sizeof(OverBin) * (size_t)bin_pos))) return st;
+    // (a bin of n > WS_BIN_CAP keys has at most n / (WS_SORT_TILE / 2) + 1 tiles, all of them at most this many)
+    static_assert(WS_BIN_CAP >= WS_SORT_TILE / 2, "oversize bins average at least half a tile's keys per tile");
+    if ((st = plan_alloc(p, (void**)&p->over_cnt,
+                         sizeof(uint32_t) * 256 * ((size_t)p->n_keys / (WS_SORT_TILE / 2) + 1)))) return st;
     if ((st = plan_alloc(p, (void**)&p->seg_emin, sizeof(int32_t) * p->n_lseg))) return st;
     if ((st = plan_alloc(p, &p->stat_partial, ws_R_partial_bytes(p->n_sort_tiles)))) return st;
-    if (cudaMemset(p->epoch, 0, sizeof(uint32_t)) != cudaSuccess) return WS_ERR_CUDA;
-    if (cudaMemset(p->lookback, 0, sizeof(uint64_t) * (size_t)P * p->n_sort_tiles * 256) != cudaSuccess)
-        return WS_ERR_CUDA;
     if ((st = plan_alloc(p, (void**)&p->vp, sizeof(uint16_t) * nh * (WS_HULL_TILE + 1)))) return st;
     if ((st = plan_alloc(p, (void**)&p->vx, sizeof(i128) * nh * (WS_HULL_TILE + 1)))) return st;
     if ((st = plan_alloc(p, (void**)&p->nvert, sizeof(int32_t) * nh))) return st;
@@ -291,12 +374,6 @@ ws_status build_plan(ws_plan* p) {
 }
 
 __global__ void k_set_lambda(double* dst, double v) { *dst = v; }
-
-ws_status map_cuda(cudaError_t e) {
-    if (e == cudaSuccess) return WS_OK;
-    cudaGetLastError();
-    return e == cudaErrorMemoryAllocation ? WS_ERR_NOMEM : WS_ERR_CUDA;
-}
 
 // The one-CTA segments and the device-wide chain touch disjoint elements, so
 // with both present the one-CTA kernel runs on the plan's side stream, after
@@ -331,15 +408,18 @@ ws_status run_forward(ws_plan* p, const void* values, const double* lambdas, voi
     const int fp64 = prec == WS_PREC_FP64 ? 1 : 0;
     cudaStream_t ss;
     if (!fork(p, st, &ss)) return WS_ERR_CUDA;
-    cudaError_t e = ws_launch_small<T>((const T*)values, p->d_offsets, p->d_small, p->n_small, lambdas, (T*)out, ids,
-                                       n_clusters, fp64, ep, p->ctx->status, ss, &p->ctx->prof, p->small_gen,
-                                       p->small_gen_count, p->ic_cap >= 0 ? p->ic_cap : p->ctx->ic_cap, ids_prev);
-    if (e) { join(p, st); return map_cuda(e); }
+    cudaError_t e = cudaSuccess;
+    // (the device-wide chain first: its cooperative first kernel would
+    // otherwise wait for the one-CTA kernel to drain)
     if (p->n_lseg > 0) {
         LargeWork<T> W = make_work<T>(p);
         e = ws_large_prox<T>(W, (const T*)values, lambdas, (T*)out, ids, n_clusters, fp64, ep, p->ctx->status,
                              p->ctx->spin_limit, p->n_levels, st);
     }
+    if (e) { join(p, st); return map_cuda(e); }
+    e = ws_launch_small<T>((const T*)values, p->d_offsets, p->d_small, p->n_small, lambdas, (T*)out, ids, n_clusters,
+                           fp64, ep, p->ctx->status, ss, &p->ctx->prof, p->small_gen, p->small_gen_count,
+                           p->ic_cap >= 0 ? p->ic_cap : p->ctx->ic_cap, ids_prev);
     if (!join(p, st)) return WS_ERR_CUDA;
     return e ? map_cuda(e) : WS_OK;
 }
@@ -783,7 +863,7 @@ ws_status ws_debug_sort(ws_plan* plan, const void* values, void* sorted_out, voi
     return map_cuda(e);
 }
 
-static const char* const kKernelNames[WSK_COUNT] = {"small", "hist", "hist_scan", "onesweep", "tile_hull",
+static const char* const kKernelNames[WSK_COUNT] = {"small", "sort_plan", "partition", "bin_sort", "oversize", "tile_hull",
                                                      "root", "table", "big_gaps", "lookup", "backward", "misc",
                                                      "tile_general", "junction", "climb"};
 
@@ -812,10 +892,10 @@ ws_status ws_debug_profile_read(ws_ctx* ctx, int kind, double* total_ms, int64_t
     if (!ctx || kind < 0 || kind >= WSK_COUNT) return WS_ERR_INVALID;
     WsProf& P = ctx->prof;
     if (P.n > 0) {   // fold the recorded event pairs into the per-kind totals
-        if (cudaEventSynchronize(P.ev[2 * P.n - 1]) != cudaSuccess) return WS_ERR_CUDA;
-        for (int i = 0; i < P.n; ++i) {
+        for (int i = 0; i < P.n; ++i) {   // (two streams: the last recorded pair need not be the last to complete)
             float ms = 0.0f;
-            if (cudaEventElapsedTime(&ms, P.ev[2 * i], P.ev[2 * i + 1]) != cudaSuccess) return WS_ERR_CUDA;
+            if (cudaEventSynchronize(P.ev[2 * i + 1]) != cudaSuccess ||
+                cudaEventElapsedTime(&ms, P.ev[2 * i], P.ev[2 * i + 1]) != cudaSuccess) return WS_ERR_CUDA;
             ctx->prof_ms[P.kind[i]] += ms;
             ctx->prof_cnt[P.kind[i]] += 1;
         }

@@ -496,15 +496,11 @@ cudaError_t ws_large_backward(const LargeWork<T>& W, const T* g, const int32_t* 
     if (e) return e;
     const int nt = W.n_sort_tiles;
     // slot buckets of 2^s slots (2^21 slots of 20 bytes: about 40 MB, well
-    // inside L2); their counters live in the sort histogram buffer, which
-    // holds at least 3 nb + 2 words for the nb allowed here
+    // inside L2); their counters: 3 nb + 2 words
     typedef typename KeyOf<T>::K K;
-    constexpr int P = KeyOf<T>::BITS / 8;
     const int64_t total_slots = W.n_keys + W.n_lseg;
-    const int64_t words = (int64_t)sizeof(uint32_t) * W.n_lseg * P * 256 / sizeof(unsigned long long);
-    const int nb_max = (int)std::min<int64_t>(BK_MAX, (words - 2) / 3);
     int s = 21;
-    while (((total_slots + ((int64_t)1 << s) - 1) >> s) > nb_max) ++s;
+    while (((total_slots + ((int64_t)1 << s) - 1) >> s) > BK_MAX) ++s;
     const int nb = (int)((total_slots + ((int64_t)1 << s) - 1) >> s);
     unsigned long long* bk_cnt = reinterpret_cast<unsigned long long*>(W.hist);
     unsigned long long* bk_off = bk_cnt + nb;

@@ -48,10 +48,8 @@ template <> struct KeyOf<float> {
     static constexpr int EXPMASK = 0xff;
     static constexpr int FIX_OFS = 34;   // 58 - (MANT + 1)
     static constexpr int L_BASE = 184;   // L = L_BASE - emax  (150 + FIX_OFS)
-    __device__ __forceinline__ static K to_key(float v) {
-        uint32_t b = __float_as_uint(v);
-        return b ^ ((b >> 31) ? 0xffffffffu : 0x80000000u);
-    }
+    __device__ __forceinline__ static K key_of_bits(K b) { return b ^ ((b >> 31) ? 0xffffffffu : 0x80000000u); }
+    __device__ __forceinline__ static K to_key(float v) { return key_of_bits(__float_as_uint(v)); }
     __device__ __forceinline__ static float from_key(K k) {
         return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xffffffffu));
     }
@@ -64,10 +62,10 @@ template <> struct KeyOf<double> {
     static constexpr int EXPMASK = 0x7ff;
     static constexpr int FIX_OFS = 5;     // 58 - (MANT + 1)
     static constexpr int L_BASE = 1080;   // 1075 + FIX_OFS
-    __device__ __forceinline__ static K to_key(double v) {
-        uint64_t b = (uint64_t)__double_as_longlong(v);
+    __device__ __forceinline__ static K key_of_bits(K b) {
         return b ^ ((b >> 63) ? 0xffffffffffffffffull : 0x8000000000000000ull);
     }
+    __device__ __forceinline__ static K to_key(double v) { return key_of_bits((uint64_t)__double_as_longlong(v)); }
     __device__ __forceinline__ static double from_key(K k) {
         return __longlong_as_double((long long)(k ^ ((k >> 63) ? 0x8000000000000000ull : 0xffffffffffffffffull)));
     }

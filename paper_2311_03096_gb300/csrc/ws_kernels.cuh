@@ -10,7 +10,7 @@ template <> struct SmallCfg<double> { static constexpr int M = 16; static conste
 // Opt-in per-launch timing (CUDA events recorded on the launching stream
 // around every kernel) and a launch counter.  Host-side only.
 enum WsKernelKind {
-    WSK_SMALL = 0, WSK_HIST, WSK_HIST_SCAN, WSK_ONESWEEP, WSK_TILE_HULL, WSK_ROOT,
+    WSK_SMALL = 0, WSK_SORT_PLAN, WSK_PARTITION, WSK_BIN_SORT, WSK_OVERSIZE, WSK_TILE_HULL, WSK_ROOT,
     WSK_TABLE, WSK_BIG_GAPS, WSK_LOOKUP, WSK_BWD, WSK_MISC, WSK_TILE_GENERAL, WSK_JUNCTION, WSK_CLIMB, WSK_COUNT
 };
 struct WsProf {
@@ -35,10 +35,19 @@ struct WsProf {
     do { (PROF)->begin((ST), (KIND)); __VA_ARGS__; (PROF)->end((ST)); } while (0)
 
 // Large-path tile geometry.
-constexpr int WS_SORT_NT = 512;              // threads per onesweep CTA
-constexpr int WS_SORT_ITEMS = 12;            // keys per thread (a multiple of 4: 16-byte loads in k_hist)
-constexpr int WS_SORT_CHAINS = 1;            // independent ranking chains per warp
+constexpr int WS_SORT_NT = 512;              // threads per partition CTA
+constexpr int WS_SORT_ITEMS = 12;            // keys per thread
 constexpr int WS_SORT_TILE = WS_SORT_NT * WS_SORT_ITEMS;   // 6144 keys per sort tile
+// Distribution sort (ws_sort.cu): bins of about WS_BIN_MEAN keys, sorted by
+// one CTA up to WS_BIN_CAP keys.  The ratio 1.6 leaves room for the error of
+// the sampled map (5 to 8 % standard deviation on N(0, 1), largest bin 1.2 to
+// 1.55 times the mean; 2816 let a few bins of the tails overflow).
+constexpr int WS_BIN_CAP = 4096;
+constexpr int WS_BIN_MEAN = 2560;
+constexpr int WS_BINS_MAX = 1 << 19;         // per segment (a partition's rank word holds 19 bits of bin)
+constexpr int WS_FAN = 512;                  // buckets a partition tile counts at a time
+constexpr int WS_ONE_LEVEL = 512;            // segments of at most this many bins take one partition pass
+constexpr int WS_CELLS = 2048;               // cells of the map (two-level segments; half as many otherwise)
 constexpr int WS_HULL_NT = 256;              // threads per hull-tile CTA
 constexpr int WS_HULL_M = 16;                // points per thread chunk
 constexpr int WS_HULL_TILE = WS_HULL_NT * WS_HULL_M;       // 4096 elements per hull tile
@@ -64,7 +73,37 @@ struct LargeSeg {
     int32_t hull_first, hull_count;   // hull tiles
     int64_t dir_pos;   // directory slice start
     int32_t dir_cap_log2;             // directory slice holds 2^dir_cap_log2 + 1 entries
-    int32_t pad;
+    // distribution sort
+    int32_t nbins;             // bins of the segment
+    int32_t fine_log2;         // first pass: bucket = bin >> fine_log2 (0: one pass only)
+    int32_t n_coarse;          // buckets of the first pass
+    int32_t ncell;             // cells of the segment's map (a power of two)
+    int32_t samp_log2;         // sampled elements per sort tile
+    int32_t bin_pos, coarse_pos, cell_pos;   // slices of the per-bin / bucket / cell arrays
+};
+
+// Sort control words, cleared before every sort.
+struct SortCtl {
+    uint32_t bar;          // grid barrier of the plan kernel
+    uint32_t abort;        // a barrier gave up: the keys are not moved
+    uint32_t over_count;   // bins above WS_BIN_CAP
+    uint32_t over_bar;     // grid barrier of the oversize kernel
+    unsigned long long over_diff;   // key bits that vary inside any oversize bin
+    unsigned long long pad;
+};
+
+// Map header of a segment: cell = (key - kmin) >> shift.
+struct SortHdr {
+    uint64_t kmin;
+    int32_t shift;
+};
+
+// A bin above WS_BIN_CAP.
+struct OverBin {
+    int64_t start;          // first key
+    int32_t n;
+    int32_t first_tile;     // of the oversize kernel's tiles
+    unsigned long long diff;   // key bits that vary inside the bin
 };
 
 // A piece of a node hull: vertices [lo, hi) of hull tile `tile`; cum = rank of
@@ -125,6 +164,16 @@ template <typename T>
 cudaError_t ws_launch_small_backward(const T* g, const int32_t* ids, const int64_t* offsets, const int32_t* seg_list,
                                      int n_list, T* gin, uint32_t* status, cudaStream_t st, WsProf* prof);
 
+// Launch shapes of a plan's sort (host).
+struct WsSortShape {
+    bool wide = false;                                 // 32-bit bin numbers
+    int hist_cap = 0;                                  // shared words of the plan kernel (bins counted, samples kept)
+    int max_bins = 0;                                  // of the longest segment
+    int samp_max = 0;                                  // log2 of the most samples per tile
+    int plan_grid = 1, part_grid = 1, over_grid = 1;   // CTAs resident at once
+};
+template <typename T> cudaError_t ws_sort_prepare(int max_bins, int n_tiles, int samp_max, WsSortShape* sh);
+
 // Large path workspace pointers (all device).
 template <typename T>
 struct LargeWork {
@@ -136,11 +185,26 @@ struct LargeWork {
     const TileDesc* hull_tiles;
     K* keys_a;
     K* keys_b;
-    uint32_t* hist;          // [n_lseg][passes][256]
-    uint64_t* lookback;      // [passes][n_sort_tiles][256]
-    uint32_t* tile_counter;  // [passes]
-    uint32_t* epoch;         // [1] look-back epoch, advanced by every sort
+    // sort: the first sort_zero_bytes from ctl on are cleared before every sort
+    SortCtl* ctl;
+    size_t sort_zero_bytes;
+    unsigned long long* seg_hi;   // [n_lseg] largest sampled key
+    unsigned long long* seg_lo;   // [n_lseg] complement of the smallest sampled key
+    uint32_t* seg_en;        // [n_lseg] INT_MAX - smallest effective exponent of a nonzero value
+    uint32_t* cells;         // [3 cells] sampled keys per cell, then per part of a cell
+    uint32_t* bin_cnt;       // [n_bins]
+    // (not cleared)
+    int n_bins, two_level;
+    WsSortShape sort_shape;
+    void* bins;              // [2][n_keys] bin of every key (16 bits, or 32 in plans with longer segments)
+    uint32_t* bin_start;     // [n_bins] first key of every bin, relative to its segment
+    uint32_t* cur1;          // [coarse buckets] write cursors of the first pass
+    uint32_t* cur2;          // [n_bins] write cursors of the second pass
+    const int32_t* bin_seg;  // [n_bins] segment of every bin
+    OverBin* over;           // [n_bins] oversize bins
+    uint32_t* over_cnt;      // [n_keys / (WS_SORT_TILE / 2) + 1][256] digit counts of their tiles
     int32_t* seg_emin;       // [n_lseg] smallest effective exponent of a nonzero value
+    uint32_t* hist;          // counters of the backward's slot buckets: >= 3 * 256 + 2 64-bit words
     // hull
     uint16_t* vp;            // [n_hull_tiles][WS_HULL_TILE + 1] vertex points (tile-local)
     i128* vx;                // [n_hull_tiles][WS_HULL_TILE + 1] X at vertices (tile-local)

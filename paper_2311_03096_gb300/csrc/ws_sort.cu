@@ -1,335 +1,1143 @@
-// ws_sort.cu -- segmented LSD radix sort of the keys of the large segments
-// (the pre-processing every prox algorithm of Sec. 4 assumes).
+// ws_sort.cu -- sort of the keys of the large segments (the pre-processing
+// every prox algorithm of Sec. 4 assumes), as a distribution sort.
 //
 // Only keys move: because equal weights always share a cluster, the result of
-// the prox never depends on the order of ties, so no index payload is sorted
-// and no unpermute scatter is needed later (the values are recovered by a
-// key -> cluster lookup in the caller's order).
+// the prox never depends on the order of ties, so no index payload is sorted,
+// no pass has to be stable, and a pass needs no look-back over earlier tiles:
+//   k_sort_plan   samples every segment, fits a monotone map key -> bin (a
+//                 piecewise linear image of the sampled distribution, so that
+//                 bins come out about equal whatever the distribution), counts
+//                 every key's bin, and turns the counts into bin starts;
+//   k_part        moves the keys into their bins: one pass for segments of at
+//                 most WS_ONE_LEVEL bins, otherwise a pass into buckets of
+//                 2^fine_log2 bins and a second one inside the buckets.  A
+//                 tile ranks its keys with one shared-memory atomic each and
+//                 reserves its runs with one global atomic per bucket;
+//   k_bin_sort    sorts every bin in one CTA;
+//   k_oversize    an LSD radix sort of the bins that do not fit one CTA (heavy
+//                 ties, or a distribution that the map does not resolve),
+//                 returns at once when there are none.
+// The map only decides how even the bins are: it is monotone in the key by
+// construction, so the result is the sorted sequence for any input.
 //
-// One histogram pass computes every digit histogram of every large segment;
-// then each 8-bit digit pass is a single "onesweep" kernel: a CTA ranks its
-// 6144 keys by digit in shared memory, publishes its per-digit counts, gets
-// the counts of the earlier tiles of the same segment through a decoupled
-// look-back (bounded waits), and writes its keys as per-digit contiguous runs.
+// Measured against 8-bit LSD passes with decoupled look-back (a histogram and
+// four passes of 0.322 ms at 2^26 FP32 keys, eight passes for FP64; 0.245 of
+// HBM, bound by the stable in-warp ranking), us:
+//   FP32 2^26    1394 -> 882 (plan 150, partition 2 x 217, bins 293, oversize 6)
+//   FP32 2^24     398 -> 271 (68, 2 x 58, 82, 6)
+//   FP64 2^22     319 -> 147 (53, 2 x 23, 41, 6)
+//   1024 FP32 segments of 16 .. 2^20 elements (9.7e7 keys)   2085 -> 1310
+// The partition is bound by shared-memory wavefronts (17 per 32 keys: the
+// counters, the staging and the copy out; 0.7 of the pipe), the bin sort by
+// issue (0.64) and the same pipe, the plan by the read of the values (0.104 of
+// its 0.150 ms) and five barriers.
 #include <algorithm>
 
 #include "ws_kernels.cuh"
 
 namespace {
 
-// Look-back word: [63:62] status (1 = tile aggregate, 2 = inclusive prefix),
-// [61:40] epoch of the call that wrote it, [39:0] count.  Every call uses a
-// new epoch (incremented on the device, so CUDA-graph replays also advance
-// it), which makes the words of the previous call read as "not ready"
-// without clearing the array.
-constexpr uint64_t LB_AGG = 1ull << 62;
-constexpr uint64_t LB_INC = 2ull << 62;
-constexpr uint64_t LB_STATUS = 3ull << 62;
-constexpr int LB_EPOCH_SHIFT = 40;
-constexpr uint64_t LB_EPOCH_MASK = ((1ull << 22) - 1ull) << LB_EPOCH_SHIFT;
-constexpr uint64_t LB_CNT = (1ull << LB_EPOCH_SHIFT) - 1ull;
+constexpr int PLAN_NT = 1024;
+constexpr int OVER_NT = WS_SORT_NT;
 
-__device__ __forceinline__ void st_relaxed_u64(uint64_t* p, uint64_t v) {
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ uint64_t ld_relaxed_u64(const uint64_t* p) {
-    uint64_t v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+__device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
 
-// Also the smallest effective exponent of a nonzero value of each segment
-// (seg_emin, reduced with atomicMin; cleared to INT_MAX before the launch),
-// which fixes the segment's fixed-point scale.  A persistent grid: each CTA
-// walks the tiles blockIdx.x, blockIdx.x + gridDim.x, ... (increasing, so it
-// meets each segment in one run) and adds its shared-memory counts to the
-// segment's global histogram once per segment, not once per tile.
-template <typename T>
-__global__ void __launch_bounds__(WS_SORT_NT) k_hist(const T* __restrict__ values, const TileDesc* __restrict__ tiles,
-                                                     int n_tiles, uint32_t* hist, int32_t* seg_emin,
-                                                     uint32_t* status) {
-    typedef KeyOf<T> KO;
-    constexpr int P = KO::BITS / 8;
-    __shared__ uint32_t h[P * 256];
-    __shared__ int s_emin;
-    for (int i = threadIdx.x; i < P * 256; i += WS_SORT_NT) h[i] = 0;
-    if (threadIdx.x == 0) s_emin = 0x7fffffff;
-    __syncthreads();
-    bool bad = false;
-    int emin = 0x7fffffff;
-    auto count = [&](T v) {
-        bad |= !ws_isfinite(v);
-        if (v != (T)0) emin = min(emin, ws_eff_exp(v));
-        const typename KO::K k = KO::to_key(v);
-#pragma unroll
-        for (int p = 0; p < P; ++p) atomicAdd(&h[p * 256 + (int)((k >> (8 * p)) & 0xff)], 1u);
-    };
-    auto flush = [&](int lseg) {   // (all threads; ends with zero counts)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) emin = min(emin, __shfl_xor_sync(0xffffffffu, emin, o));
-        if ((threadIdx.x & 31) == 0 && emin != 0x7fffffff) atomicMin(&s_emin, emin);
-        emin = 0x7fffffff;
+// Barrier over a cooperative grid: arrivals are counted in *ctr (cleared
+// before the launch).  A wait that gives up sets the timeout status and the
+// abort word; the CTA then goes on without waiting (every access of the
+// kernels below is in bounds whatever the other CTAs have written).
+struct GridBarrier {
+    uint32_t* ctr;
+    uint32_t* abort;
+    uint32_t* status;
+    uint64_t limit;
+    uint32_t target;
+    bool dead;   // (thread 0)
+    __device__ __forceinline__ void sync() {
         __syncthreads();
-        if (threadIdx.x == 0 && s_emin != 0x7fffffff) atomicMin(&seg_emin[lseg], s_emin);
-        uint32_t* gh = hist + (size_t)lseg * P * 256;
-        for (int i = threadIdx.x; i < P * 256; i += WS_SORT_NT) {
-            if (h[i]) atomicAdd(&gh[i], h[i]);
-            h[i] = 0;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) s_emin = 0x7fffffff;
-        __syncthreads();
-    };
-    constexpr int VEC = 16 / (int)sizeof(T);                  // values per 16-byte load
-    constexpr int NV = WS_SORT_TILE / (WS_SORT_NT * VEC);     // 16-byte loads per thread
-    int cur = -1;
-    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-        const TileDesc td = tiles[tile];
-        if (td.lseg != cur) {
-            if (cur >= 0) flush(cur);
-            cur = td.lseg;
-        }
-        const T* src = values + td.vpos;
-        if (td.len == WS_SORT_TILE && (((uintptr_t)src) & 15) == 0) {
-            // whole, aligned tile: every load issued before the first count
-            uint4 buf[NV];
-#pragma unroll
-            for (int j = 0; j < NV; ++j) buf[j] = __ldcs(reinterpret_cast<const uint4*>(src) + j * WS_SORT_NT + threadIdx.x);
-#pragma unroll
-            for (int j = 0; j < NV; ++j) {
-                const T* e = reinterpret_cast<const T*>(&buf[j]);
-#pragma unroll
-                for (int u = 0; u < VEC; ++u) count(e[u]);
+        if (threadIdx.x == 0) {
+            target += gridDim.x;
+            __threadfence();
+            atomicAdd(ctr, 1u);
+            uint64_t it = 0;
+            while (!dead && (int32_t)(ld_acquire_u32(ctr) - target) < 0) {
+                if (++it > limit) {
+                    dead = true;
+                    atomicExch(abort, 1u);
+                    ws_flag(status, WS_STATUS_TIMEOUT);
+                    break;
+                }
+                ws_backoff((int)min(it, (uint64_t)1 << 20));
             }
-        } else {
-            for (int i = threadIdx.x; i < td.len; i += WS_SORT_NT) count(src[i]);
+            __threadfence();
         }
+        __syncthreads();
     }
-    if (cur >= 0) flush(cur);
-    if (bad) ws_flag(status, WS_STATUS_NONFINITE);
+};
+
+// ---------------------------------------------------------------------------
+// The map of a segment.  The sampled key range is cut into ncell cells of
+// equal width, a cell with many samples into 2^bits equal parts (so that a
+// part holds about the same number of samples wherever there are enough of
+// them, and the density changes little inside one).  Knot i is the expected
+// number of bins filled by the keys below part i; inside a part the map is
+// linear in the key, with a slope rounded down by 2^-20.  Every step rounds
+// monotonically, so the image of a part never passes the next knot and the map
+// is monotone over the whole key range.  Keys above the sampled range go to
+// the last bin, keys below it to the first.
+// ---------------------------------------------------------------------------
+struct MapTab {
+    uint32_t split[WS_CELLS + 1];       // first part | width of a part << 16 (log2; the last entry: above the range)
+    float2 knots[2 * WS_CELLS + 1];     // map value at the start of the part, its slope
+};
+
+template <typename T>
+struct KeyMap {
+    typedef typename KeyOf<T>::K K;
+    K kmin;
+    int shift;
+    uint32_t ncell, last;
+    __device__ __forceinline__ void init(const SortHdr& h, int ncell_, int nbins) {
+        kmin = (K)h.kmin;
+        shift = h.shift;
+        ncell = (uint32_t)ncell_;
+        last = (uint32_t)(nbins - 1);
+    }
+    // position inside a part of width 2^s2, at most 24 bits of it
+    __device__ __forceinline__ static uint32_t low(K d, int s2) {
+        const K x = d & (((K)1 << s2) - 1);
+        return (uint32_t)(sizeof(K) == 4 ? x : x >> max(s2 - 24, 0));
+    }
+    // slope of a part of width 2^s2 that covers db bins
+    __device__ __forceinline__ static float slope(float db, int s2) {
+        return ldexpf(db * (1.0f - 1.0f / 1048576.0f), -(sizeof(K) == 4 ? s2 : min(s2, 24)));
+    }
+    __device__ __forceinline__ uint32_t bin(K k, const MapTab& m) const {
+        const K d = max(k, kmin) - kmin;
+        const uint32_t e = m.split[(uint32_t)min(d >> shift, (K)ncell)];
+        const int s2 = (int)(e >> 16);
+        const K in = d & (((K)1 << shift) - 1);
+        const uint32_t i = min((e & 0xffffu) + (uint32_t)(in >> s2), 2u * WS_CELLS);
+        const float2 kn = m.knots[i];
+        return min((uint32_t)(int)fmaf((float)low(d, s2), kn.y, kn.x), last);
+    }
+};
+
+// Sampled element j of m = 2^mlog of a tile: a pair of neighbours (one sector)
+// at a pseudo-random place of every (m / 2)-th of the tile; all elements of a
+// tile of at most m.
+__device__ __forceinline__ int sample_pos(int tile, int j, int len, int mlog) {
+    if (len <= (1 << mlog)) return j;
+    const uint32_t q = (uint32_t)j >> 1;
+    uint32_t h = (uint32_t)tile * 0x9E3779B9u + q * 0x85EBCA6Bu;
+    h ^= h >> 15; h *= 0x2C1B3C6Du; h ^= h >> 13;
+    return min((int)((q * (uint32_t)len + __umulhi(h, (uint32_t)len)) >> (mlog - 1)) + (j & 1), len - 1);
 }
 
-// exclusive scan of every (segment, pass) histogram, in place
-__global__ void __launch_bounds__(256) k_hist_scan(uint32_t* hist, uint32_t* epoch) {
-    __shared__ uint32_t ws[8];
-    if (blockIdx.x == 0 && threadIdx.x == 0) *epoch = (*epoch + 1u) & ((1u << 22) - 1u);
-    uint32_t* h = hist + (size_t)blockIdx.x * 256;
-    uint32_t v = h[threadIdx.x];
-    uint32_t tot;
-    uint32_t ex = ws_block_excl_scan<256, int>((int)v, (int*)ws, (int*)&tot);
-    h[threadIdx.x] = ex;
-}
+// ---------------------------------------------------------------------------
+// Plan: sample, map, bin counts, bin starts.  A cooperative grid with one
+// barrier between the phases.  Bound by the read of the values (the count)
+// and, for short segments, by the barriers (about 2 us each).
+// ---------------------------------------------------------------------------
+struct PlanSmem {
+    unsigned long long hi, lo;
+    int emin, parts;
+    int wsum[PLAN_NT / 32];
+};
 
-template <typename T, bool FIRST>
-__global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_onesweep(const T* __restrict__ values,
-                                                            const typename KeyOf<T>::K* __restrict__ keys_in,
-                                                            typename KeyOf<T>::K* __restrict__ keys_out,
-                                                            const TileDesc* __restrict__ tiles,
-                                                            const LargeSeg* __restrict__ lsegs,
-                                                            const uint32_t* __restrict__ hist, uint64_t* lookback,
-                                                            uint32_t* counter, const uint32_t* __restrict__ epoch_p,
-                                                            int pass, uint32_t* status, uint64_t spin_limit) {
+template <typename T, typename B>
+__global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ values,
+                                                          const TileDesc* __restrict__ tiles, int n_tiles,
+                                                          const LargeSeg* __restrict__ lsegs, int n_lseg,
+                                                          SortCtl* ctl, unsigned long long* seg_hi,
+                                                          unsigned long long* seg_lo, uint32_t* seg_en,
+                                                          uint32_t* cells, uint32_t* bin_cnt, B* bins,
+                                                          uint32_t* bin_start, uint32_t* cur1, uint32_t* cur2,
+                                                          int32_t* seg_emin, int max_bins, int hist_cap, int samp_max,
+                                                          uint64_t spin_limit, uint32_t* status) {
     typedef KeyOf<T> KO;
     typedef typename KO::K K;
-    constexpr int P = KO::BITS / 8;
-    constexpr int NT = WS_SORT_NT, ITEMS = WS_SORT_ITEMS, TILE = WS_SORT_TILE, NW = NT / 32;
+    __shared__ PlanSmem S;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    K* skeys = reinterpret_cast<K*>(smem_raw);
-    uint32_t* whist = reinterpret_cast<uint32_t*>(smem_raw + sizeof(K) * TILE);   // [NW][256] per-warp counts
-    uint32_t* mbins = whist + NW * 256;                                             // [NW][256] peer masks
-    uint32_t* dstart = mbins + NW * 256;
-    int64_t* gbase = reinterpret_cast<int64_t*>(dstart + 256);
-    __shared__ int s_tile;
-    __shared__ int s_timeout;
+    MapTab& tab = *reinterpret_cast<MapTab*>(smem_raw);
+    uint32_t* hist = reinterpret_cast<uint32_t*>(smem_raw + sizeof(MapTab));      // [hist_cap]
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    uint32_t* my = whist + w * 256;
-    uint32_t* mb = mbins + w * 256;
-    for (int i = lane; i < 256; i += 32) { my[i] = 0; mb[i] = 0; }
-    if (t == 0) { s_tile = (int)atomicAdd(counter, 1u); s_timeout = 0; }
-    __syncthreads();
-    const int tile = s_tile;
-    const TileDesc td = tiles[tile];
-    const int64_t seg_k = lsegs[td.lseg].kpos;
-    const uint32_t* dbase = hist + ((size_t)td.lseg * P + pass) * 256;
-    const uint64_t ep = (uint64_t)(*epoch_p) << LB_EPOCH_SHIFT;
-    const int shift = 8 * pass;
-    uint64_t* my_lb = lookback + (size_t)tile * 256;
+    GridBarrier bar{&ctl->bar, &ctl->abort, status, spin_limit, 0u, false};
+    // this CTA's tiles, contiguous
+    const int t0 = (int)((int64_t)n_tiles * blockIdx.x / gridDim.x);
+    const int t1 = (int)((int64_t)n_tiles * (blockIdx.x + 1) / gridDim.x);
+    const int seg0 = t0 < t1 ? tiles[t0].lseg : -1;
+    // the CTA's sampled keys stay in the (later) histogram's shared memory if they fit
+    K* cache = reinterpret_cast<K*>(hist);
+    const bool cached = ((size_t)(t1 - t0) << samp_max) * sizeof(K) <= (size_t)hist_cap * sizeof(uint32_t);
 
-    // Warp w holds keys [w*32*ITEMS, (w+1)*32*ITEMS) of the tile, item k of
-    // lane l being key w*32*ITEMS + 32k + l, so ranking items in order k and
-    // lanes in order l is stable.
-    K key[ITEMS];
-    static_assert(ITEMS % 2 == 0 && TILE <= 65536, "ranks are packed two per word");
-    uint32_t pos2[ITEMS / 2];   // warp-local rank of item k in half k % 2 of word k / 2 (fewer registers)
-    const int base = w * 32 * ITEMS + lane;
-#pragma unroll
-    for (int k = 0; k < ITEMS; ++k) {
-        const int p = base + k * 32;
-        const bool v = p < td.len;
-        if (FIRST) key[k] = v ? KO::to_key(values[td.vpos + p]) : (K)0;
-        else key[k] = v ? keys_in[td.kpos + p] : (K)0;
-    }
-    // Rank within the warp: the lanes holding the same digit find each other
-    // by OR-ing their lane bits into the digit's shared-memory word; the
-    // lowest of them advances the warp's count of that digit.
-    const unsigned lt = (1u << lane) - 1u;
-#pragma unroll
-    for (int k = 0; k < ITEMS; ++k) {
-        const bool v = base + k * 32 < td.len;
-        const uint32_t dg = (uint32_t)(key[k] >> shift) & 0xffu;
-        if (v) atomicOr(&mb[dg], 1u << lane);
-        __syncwarp();
-        const unsigned peers = v ? mb[dg] : 0u;
-        const int before = v ? (int)my[dg] : 0;
-        __syncwarp();
-        const int r = __popc(peers & lt);
-        const uint32_t rk = (uint32_t)(before + r);
-        if (k % 2 == 0) pos2[k / 2] = rk; else pos2[k / 2] |= rk << 16;
-        if (v && r == 0) { my[dg] = (uint32_t)(before + __popc(peers)); mb[dg] = 0u; }
-        __syncwarp();
-    }
+    // 1. range of the sampled keys (one warp per tile; the CTA's first segment
+    // is combined in shared memory)
+    if (t == 0) { S.hi = 0; S.lo = 0; }
     __syncthreads();
-    // Per digit: exclusive scan over the warps, and the tile's count, which is
-    // published at once so that later tiles' look-backs can pass this one.
-    uint32_t cnt = 0;
-    if (t < 256) {
-#pragma unroll
-        for (int ww = 0; ww < NW; ++ww) {
-            const uint32_t c = whist[ww * 256 + t];
-            whist[ww * 256 + t] = cnt;
-            cnt += c;
-        }
-        st_relaxed_u64(&my_lb[t], (td.tin == 0 ? LB_INC : LB_AGG) | ep | (uint64_t)cnt);
-    }
-    // exclusive scan of the counts over the 256 digits
-    {
-        uint32_t tot;
-        const uint32_t ex = ws_block_excl_scan<NT, int>((int)cnt, (int*)mbins, (int*)&tot);
-        if (t < 256) dstart[t] = ex;
-    }
-    __syncthreads();
-    // stage the tile in digit order (frees the key registers before the
-    // look-back)
-#pragma unroll
-    for (int k = 0; k < ITEMS; ++k) {
-        if (base + k * 32 < td.len) {
-            const uint32_t dg = (uint32_t)(key[k] >> shift) & 0xffu;
-            const int rk = (int)((pos2[k / 2] >> (16 * (k % 2))) & 0xffffu);
-            skeys[rk + (int)(dstart[dg] + my[dg])] = key[k];
-        }
-    }
-
-    // look back over earlier tiles of the segment (windows of 4 predecessors
-    // per round trip)
-    if (t < 256) {
-        int64_t gb;   // global position of this digit's first key of the tile, minus its local start
-        if (td.tin == 0) {
-            gb = 0;
-        } else {
-            uint64_t run = 0;
-            int j = tile - 1;
-            uint64_t it = 0;
-            bool done = false;
-            while (!done) {
-                constexpr int WIN = 4;
-                uint64_t v[WIN];
-                const int nwin = min(WIN, j - td.first + 1);
-#pragma unroll
-                for (int u = 0; u < WIN; ++u)
-                    if (u < nwin) v[u] = ld_relaxed_u64(&lookback[(size_t)(j - u) * 256 + t]);
-                int u = 0;
-                for (; u < nwin; ++u) {
-                    uint64_t x = v[u];
-                    while ((x & LB_STATUS) == 0 || (x & LB_EPOCH_MASK) != ep) {
-                        if (++it > spin_limit) { s_timeout = 1; break; }
-                        ws_backoff((int)min(it, (uint64_t)1 << 20));
-                        x = ld_relaxed_u64(&lookback[(size_t)(j - u) * 256 + t]);
-                    }
-                    if ((x & LB_STATUS) == 0 || (x & LB_EPOCH_MASK) != ep) { done = true; break; }   // gave up
-                    run += x & LB_CNT;
-                    if ((x & LB_STATUS) == LB_INC || j - u <= td.first) { done = true; break; }
-                }
-                if (!done) j -= nwin;
-            }
-            st_relaxed_u64(&my_lb[t], LB_INC | ep | (run + cnt));
-            gb = (int64_t)run;
-        }
-        gbase[t] = seg_k + (int64_t)dbase[t] + gb - (int64_t)dstart[t];
-    }
-    __syncthreads();
-    if (t == 0 && s_timeout) ws_flag(status, WS_STATUS_TIMEOUT);
+    for (int tile = t0 + w; tile < t1; tile += PLAN_NT / 32) {
+        const TileDesc td = tiles[tile];
+        const int ml = lsegs[td.lseg].samp_log2;
+        const int m = min(td.len, 1 << ml);
+        K hi = 0, lo = 0;   // (lo: complement, so that 0 is neutral)
+        K* keep = cache + ((size_t)(tile - t0) << samp_max);
 #pragma unroll 4
-    for (int k = 0; k < ITEMS; ++k) {
-        const int j = t + k * NT;
-        if (j < td.len) {
-            const K kk = skeys[j];
-            const uint32_t dg = (uint32_t)(kk >> shift) & 0xffu;
-            keys_out[gbase[dg] + j] = kk;
+        for (int j = lane; j < m; j += 32) {
+            const K k = KO::to_key(__ldg(values + td.vpos + sample_pos(tile, j, td.len, ml)));
+            if (cached) keep[j] = k;
+            hi = max(hi, k);
+            lo = max(lo, (K)~k);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            hi = max(hi, ws_shfl_xor_k(hi, o));
+            lo = max(lo, ws_shfl_xor_k(lo, o));
+        }
+        if (lane == 0) {
+            if (td.lseg == seg0) {
+                atomicMax(&S.hi, (unsigned long long)hi);
+                atomicMax(&S.lo, (unsigned long long)lo);
+            } else {
+                atomicMax(seg_hi + td.lseg, (unsigned long long)hi);
+                atomicMax(seg_lo + td.lseg, (unsigned long long)lo);
+            }
+        }
+    }
+    __syncthreads();
+    if (t == 0 && seg0 >= 0) {
+        atomicMax(seg_hi + seg0, S.hi);
+        atomicMax(seg_lo + seg0, S.lo);
+    }
+    bar.sync();
+
+    // header of a segment from its sampled range
+    auto header = [&](int lseg, const LargeSeg& sg) {
+        SortHdr h;
+        const K hi = (K)__ldcg(seg_hi + lseg), lo = (K)~(K)__ldcg(seg_lo + lseg);
+        // cells aligned in the key space, so that no cell (or part of one)
+        // straddles a binade, where the density per key jumps by two
+        const K range = hi > lo ? hi - lo : (K)0;
+        const int cl = 31 - __clz(sg.ncell);
+        const int bl = range ? 64 - __clzll((long long)(uint64_t)range) : 0;
+        h.shift = max(bl - cl, 0);
+        if (hi > lo && (hi >> h.shift) - (lo >> h.shift) >= (K)sg.ncell) ++h.shift;
+        h.kmin = (uint64_t)((lo >> h.shift) << h.shift);
+        return h;
+    };
+    // f(offset above kmin) for every sample of tiles [ta, tb) of one segment
+    auto samples = [&](const LargeSeg& sg, const SortHdr& h, int ta, int tb, auto f) {
+        const int m = 1 << sg.samp_log2;
+#pragma unroll 4
+        for (int i = t; i < (tb - ta) << sg.samp_log2; i += PLAN_NT) {
+            const int tile = ta + (i >> sg.samp_log2), j = i & (m - 1);
+            const int64_t o = (int64_t)(tile - sg.sort_first) * WS_SORT_TILE;
+            const int len = (int)min((int64_t)WS_SORT_TILE, sg.len - o);
+            if (j < len) {
+                const K k = cached ? cache[((size_t)(tile - t0) << samp_max) + j]
+                                   : KO::to_key(__ldg(values + sg.vpos + o + sample_pos(tile, j, len, sg.samp_log2)));
+                f(k > (K)h.kmin ? k - (K)h.kmin : (K)0);
+            }
+        }
+    };
+
+    // 2. sampled keys per cell (counted in shared memory, added to the
+    // segment's cells once per CTA)
+    for (int ta = t0; ta < t1;) {
+        const int lseg = tiles[ta].lseg;
+        const LargeSeg sg = lsegs[lseg];
+        const int tb = min(t1, sg.sort_first + sg.sort_count);
+        const SortHdr h = header(lseg, sg);
+        uint32_t* sc = tab.split;   // [ncell]
+        for (int i = t; i < sg.ncell; i += PLAN_NT) sc[i] = 0;
+        __syncthreads();
+        samples(sg, h, ta, tb, [&](K d) { atomicAdd(&sc[(uint32_t)min(d >> h.shift, (K)(sg.ncell - 1))], 1u); });
+        __syncthreads();
+        for (int i = t; i < sg.ncell; i += PLAN_NT)
+            if (sc[i]) atomicAdd(cells + sg.cell_pos + i, sc[i]);
+        __syncthreads();
+        ta = tb;
+    }
+    bar.sync();
+
+    // Parts of every cell, from the cell counts (every CTA for the segments
+    // it needs; into tab.split): a cell of c samples gets 2^floor(log2(c / thr))
+    // parts, thr = the larger of 96 samples (10 % noise) and 1 / ncell of all
+    // (so at most ncell parts beside one per cell).  Cells with less than 8 thr
+    // are cut down to 48 samples a part if that fits: in the tails the density
+    // varies more inside a cell than the noise costs.  Returns the number.
+    auto parts_of = [&](const LargeSeg& sg, const SortHdr& h) -> int {
+        constexpr int PER = WS_CELLS / PLAN_NT;
+        int v[PER], bits[PER], sum = 0;
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int c = t * PER + i;
+            v[i] = c < sg.ncell ? (int)__ldcg(cells + sg.cell_pos + c) : 0;
+            sum += v[i];
+        }
+        int tot;
+        ws_block_excl_scan<PLAN_NT, int>(sum, S.wsum, &tot);
+        const int thr = max(96, tot / sg.ncell + 1);
+        const int bmax = min(h.shift, 12);
+        auto log2_of = [](int q) { return q > 0 ? 31 - __clz(q) : 0; };
+        int ex = 0;
+        for (int fine = 1; fine >= 0; --fine) {
+            sum = 0;
+#pragma unroll
+            for (int i = 0; i < PER; ++i) {
+                bits[i] = log2_of(v[i] / thr);
+                if (fine && bits[i] < 3) bits[i] = min(log2_of(v[i] / 48), 3);
+                bits[i] = min(bits[i], bmax);
+                if (t * PER + i < sg.ncell) sum += 1 << bits[i];
+            }
+            ex = ws_block_excl_scan<PLAN_NT, int>(sum, S.wsum, &tot);
+            if (tot <= 2 * sg.ncell) break;   // (uniform; always without the fine cut)
+        }
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int c = t * PER + i;
+            if (c < sg.ncell) {
+                tab.split[c] = (uint32_t)min(ex, 2 * sg.ncell) | ((uint32_t)(h.shift - bits[i]) << 16);
+                ex += 1 << bits[i];
+            }
+        }
+        if (t == 0) tab.split[sg.ncell] = (uint32_t)min(tot, 2 * sg.ncell) | ((uint32_t)h.shift << 16);
+        __syncthreads();
+        return min(tot, 2 * sg.ncell);
+    };
+
+    // 3. sampled keys per part
+    for (int ta = t0; ta < t1;) {
+        const int lseg = tiles[ta].lseg;
+        const LargeSeg sg = lsegs[lseg];
+        const int tb = min(t1, sg.sort_first + sg.sort_count);
+        const SortHdr h = header(lseg, sg);
+        const int parts = parts_of(sg, h);
+        uint32_t* sc = reinterpret_cast<uint32_t*>(tab.knots);   // [parts]
+        for (int i = t; i < parts; i += PLAN_NT) sc[i] = 0;
+        __syncthreads();
+        const K mask = (K)(((K)1 << h.shift) - 1);
+        samples(sg, h, ta, tb, [&](K d) {
+            const uint32_t c = (uint32_t)min(d >> h.shift, (K)(sg.ncell - 1));
+            const uint32_t e = tab.split[c];
+            const uint32_t i = (e & 0xffffu) + (uint32_t)((d & mask) >> (int)(e >> 16));
+            if (i < (uint32_t)parts) atomicAdd(&sc[i], 1u);
+        });
+        __syncthreads();
+        uint32_t* gp = cells + sg.cell_pos + sg.ncell;
+        for (int i = t; i < parts; i += PLAN_NT)
+            if (sc[i]) atomicAdd(gp + i, sc[i]);
+        __syncthreads();
+        ta = tb;
+    }
+    bar.sync();
+
+    // 4. knots of every segment (every CTA for the segments it needs), the bin
+    // of every key, finiteness, smallest exponent
+    bool bad = false;
+    for (int ta = t0; ta < t1;) {
+        const int lseg = tiles[ta].lseg;
+        const LargeSeg sg = lsegs[lseg];
+        const int tb = min(t1, sg.sort_first + sg.sort_count);
+        const bool local = sg.nbins <= hist_cap;
+        const SortHdr h = header(lseg, sg);
+        const int parts = parts_of(sg, h);
+        {
+            constexpr int PER = 2 * WS_CELLS / PLAN_NT;
+            int v[PER], sum = 0;
+#pragma unroll
+            for (int i = 0; i < PER; ++i) {
+                const int c = t * PER + i;
+                v[i] = c < parts ? (int)__ldcg(cells + sg.cell_pos + sg.ncell + c) : 0;
+                sum += v[i];
+            }
+            int tot;
+            int ex = ws_block_excl_scan<PLAN_NT, int>(sum, S.wsum, &tot);
+            const float scale = (float)sg.nbins / (float)max(tot, 1);
+#pragma unroll
+            for (int i = 0; i < PER; ++i) {
+                const int c = t * PER + i;
+                if (c < parts) tab.knots[c].x = fminf((float)ex * scale, (float)sg.nbins);
+                ex += v[i];
+            }
+            if (t == 0) tab.knots[parts] = make_float2((float)sg.nbins, 0.0f);
+            __syncthreads();
+            for (int c = t; c < sg.ncell; c += PLAN_NT) {
+                const uint32_t e = tab.split[c];
+                const int s2 = (int)(e >> 16);
+                const int q1 = min((int)(e & 0xffffu) + (1 << (h.shift - s2)), parts);
+                for (int q = (int)(e & 0xffffu); q < q1; ++q)
+                    tab.knots[q].y = KeyMap<T>::slope(tab.knots[q + 1].x - tab.knots[q].x, s2);
+            }
+        }
+        KeyMap<T> map;
+        map.init(h, sg.ncell, sg.nbins);
+        if (local)
+            for (int i = t; i < sg.nbins; i += PLAN_NT) hist[i] = 0;
+        if (t == 0) S.emin = 0x7fffffff;
+        __syncthreads();
+        const int64_t o0 = (int64_t)(ta - sg.sort_first) * WS_SORT_TILE;
+        const int64_t n = min((int64_t)(tb - sg.sort_first) * WS_SORT_TILE, sg.len) - o0;
+        const T* src = values + sg.vpos + o0;
+        B* bo = bins + sg.kpos + o0;   // (16-byte aligned keys: 8-byte aligned at least for two-byte bins)
+        uint32_t* gcnt = bin_cnt + sg.bin_pos;
+        K amax = 0, amin = ~(K)0;   // largest magnitude bits; smallest ones minus 1 (zero wraps to the largest)
+        auto bin_of = [&](T v) -> uint32_t {
+            const K mag = (K)KO::bits(v) & (~(K)0 >> 1);
+            amax = max(amax, mag);
+            amin = min(amin, mag - 1);
+            const uint32_t b = map.bin(KO::to_key(v), tab);
+            if (local) atomicAdd(&hist[b], 1u);
+            else atomicAdd(gcnt + b, 1u);
+            return b;
+        };
+        if (((uintptr_t)src & 15) == 0) {
+            // 16-byte loads, four in flight per thread
+            constexpr int VEC = 16 / (int)sizeof(T), U = 4;
+            const int64_t nv = n / VEC;
+            const uint4* vs = reinterpret_cast<const uint4*>(src);
+            auto one = [&](const uint4& q, int64_t i) {
+                const T* e = reinterpret_cast<const T*>(&q);
+                __align__(16) B r[VEC];
+#pragma unroll
+                for (int k = 0; k < VEC; ++k) r[k] = (B)bin_of(e[k]);
+                if (sizeof(r) == 16) *reinterpret_cast<uint4*>(bo + i * VEC) = *reinterpret_cast<const uint4*>(r);
+                else if (sizeof(r) == 8) *reinterpret_cast<uint2*>(bo + i * VEC) = *reinterpret_cast<const uint2*>(r);
+                else *reinterpret_cast<uint32_t*>(bo + i * VEC) = *reinterpret_cast<const uint32_t*>(r);
+            };
+            int64_t i = t;
+            for (; i + (U - 1) * PLAN_NT < nv; i += U * PLAN_NT) {
+                uint4 buf[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) buf[u] = __ldg(vs + i + u * PLAN_NT);
+#pragma unroll
+                for (int u = 0; u < U; ++u) one(buf[u], i + u * PLAN_NT);
+            }
+            for (; i < nv; i += PLAN_NT) one(__ldg(vs + i), i);
+            for (int64_t k = nv * VEC + t; k < n; k += PLAN_NT) bo[k] = (B)bin_of(src[k]);
+        } else {
+            constexpr int U = 8;
+            int64_t i = t;
+            for (; i + (U - 1) * PLAN_NT < n; i += U * PLAN_NT) {
+                T v[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) v[u] = __ldg(src + i + u * PLAN_NT);
+#pragma unroll
+                for (int u = 0; u < U; ++u) bo[i + u * PLAN_NT] = (B)bin_of(v[u]);
+            }
+            for (; i < n; i += PLAN_NT) bo[i] = (B)bin_of(src[i]);
+        }
+        bad |= (amax >> KO::MANT) >= (K)KO::EXPMASK;
+        int emin = amin != ~(K)0 ? max((int)((amin + 1) >> KO::MANT), 1) : 0x7fffffff;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) emin = min(emin, __shfl_xor_sync(WS_FULL_MASK, emin, o));
+        if (lane == 0 && emin != 0x7fffffff) atomicMin(&S.emin, emin);
+        __syncthreads();
+        if (t == 0 && S.emin != 0x7fffffff) atomicMax(seg_en + lseg, (uint32_t)(0x7fffffff - S.emin));
+        if (local)
+            for (int q = t; q < sg.nbins; q += PLAN_NT)
+                if (hist[q]) atomicAdd(gcnt + q, hist[q]);
+        __syncthreads();
+        ta = tb;
+    }
+    if (bad) ws_flag(status, WS_STATUS_NONFINITE);
+    bar.sync();
+
+    // 5. bin starts and the passes' cursors: a CTA per segment and run of
+    // PLAN_NT bins, which adds up the counts before its run itself
+    for (int c0 = 0; c0 < max_bins; c0 += PLAN_NT) {
+        const int first = (int)(((int64_t)blockIdx.x + (int64_t)gridDim.x * (c0 / PLAN_NT) - c0 / PLAN_NT) % gridDim.x);
+        for (int lseg = first; lseg < n_lseg; lseg += gridDim.x) {
+            const LargeSeg sg = lsegs[lseg];
+            if (c0 >= sg.nbins) continue;   // (uniform)
+            const uint32_t* c = bin_cnt + sg.bin_pos;
+            int before = 0;
+#pragma unroll 8
+            for (int b = t; b < c0; b += PLAN_NT) before += (int)__ldcg(c + b);
+            int base;
+            ws_block_excl_scan<PLAN_NT, int>(before, S.wsum, &base);
+            const int b = c0 + t;
+            const int own = b < sg.nbins ? (int)__ldcg(c + b) : 0;
+            const uint32_t start = (uint32_t)(base + ws_block_excl_scan<PLAN_NT, int>(own, S.wsum, nullptr));
+            if (b < sg.nbins) {
+                bin_start[sg.bin_pos + b] = start;
+                if (sg.fine_log2 == 0) cur1[sg.coarse_pos + b] = start;
+                else {
+                    cur2[sg.bin_pos + b] = start;
+                    if ((b & ((1 << sg.fine_log2) - 1)) == 0) cur1[sg.coarse_pos + (b >> sg.fine_log2)] = start;
+                }
+            }
+            if (c0 == 0 && t == 0) seg_emin[lseg] = (int32_t)(0x7fffffffu - __ldcg(seg_en + lseg));
         }
     }
 }
+
+// ---------------------------------------------------------------------------
+// Partition passes.  FIRST: the values into buckets of 2^fine_log2 bins (to
+// keys_a) or straight into bins (one-level segments, to keys_b).  Otherwise:
+// the buckets of two-level segments into bins (keys_a to keys_b); a tile lies
+// in one bucket or two as a rule, and takes further rounds of WS_FAN bins
+// where its buckets are sparse.
+// ---------------------------------------------------------------------------
+template <typename T, typename B>
+struct PartSmem {
+    typename KeyOf<T>::K key[WS_SORT_TILE];
+    B bin[WS_SORT_TILE];
+    uint32_t cnt[WS_FAN];     // counts, then starts inside the tile
+    int32_t delta[WS_FAN];    // destination of the bucket's run minus its start inside the tile
+    int wsum[WS_SORT_NT / 32];
+};
+
+template <typename T, typename B, bool FIRST>
+__global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
+    const T* __restrict__ values, const typename KeyOf<T>::K* __restrict__ keys_in, const B* __restrict__ bins_in,
+    typename KeyOf<T>::K* __restrict__ out_a, typename KeyOf<T>::K* __restrict__ out_b, B* __restrict__ bins_out,
+    const TileDesc* __restrict__ tiles, int n_tiles, const LargeSeg* __restrict__ lsegs, uint32_t* cursor,
+    const SortCtl* ctl, uint32_t* status) {
+    typedef KeyOf<T> KO;
+    typedef typename KO::K K;
+    constexpr int NT = WS_SORT_NT, ITEMS = WS_SORT_ITEMS;
+    static_assert(WS_FAN == NT, "one bucket per thread");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    PartSmem<T, B>& s = *reinterpret_cast<PartSmem<T, B>*>(smem_raw);
+    if (ctl->abort) return;
+    const int t = threadIdx.x;
+    // the next tile of this CTA from `tile` on that this pass moves
+    auto next_tile = [&](int tile) {
+        if (!FIRST)
+            while (tile < n_tiles && lsegs[tiles[tile].lseg].fine_log2 == 0) tile += gridDim.x;
+        return tile;
+    };
+    K key[ITEMS];         // (loaded raw; made keys when the tile's turn comes, so that the loads stay in flight)
+    uint32_t br[ITEMS];   // bin << 13 | rank
+    auto load = [&](const TileDesc& td) {
+        const K* src = FIRST ? reinterpret_cast<const K*>(values) + td.vpos : keys_in + td.kpos;
+        const B* bsrc = bins_in + td.kpos;
+#pragma unroll
+        for (int k = 0; k < ITEMS; ++k) {
+            const int p = t + k * NT;
+            if (p < td.len) {
+                key[k] = __ldg(src + p);
+                br[k] = __ldg(bsrc + p);
+            }
+        }
+    };
+    int tile = next_tile(blockIdx.x);
+    if (tile >= n_tiles) return;
+    load(tiles[tile]);
+    while (tile < n_tiles) {
+        const int nxt = next_tile(tile + gridDim.x);
+        const int len = tiles[tile].len;
+        const LargeSeg& sg = lsegs[tiles[tile].lseg];
+        const int fl = sg.fine_log2;
+        // the tile's buckets: all of the segment's (first pass), the bins of
+        // its first to last bucket (second)
+        int base = 0, nbk = sg.n_coarse;
+        if (!FIRST) {
+            const int64_t kp = tiles[tile].kpos;
+            base = ((int)__ldg(bins_in + kp) >> fl) << fl;
+            nbk = max(min(sg.nbins, (((int)__ldg(bins_in + kp + len - 1) >> fl) + 1) << fl) - base, 1);
+        }
+        const int bsh = FIRST ? 13 + fl : 13;
+#pragma unroll
+        for (int k = 0; k < ITEMS; ++k) {
+            if (FIRST) key[k] = KO::key_of_bits(key[k]);
+            br[k] <<= 13;
+        }
+        for (int r0 = 0; r0 < nbk; r0 += WS_FAN) {
+            const uint32_t off = (uint32_t)(base + r0);
+            __syncthreads();   // (the previous use of the shared memory is over)
+            s.cnt[t] = 0;
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < ITEMS; ++k) {
+                const uint32_t b = (br[k] >> bsh) - off;
+                if (t + k * NT < len && b < WS_FAN) br[k] = (br[k] & ~0x1fffu) | atomicAdd(&s.cnt[b], 1u);
+            }
+            __syncthreads();
+            // start inside the tile, and the run's destination
+            const uint32_t c = s.cnt[t];
+            const uint32_t g =
+                c ? atomicAdd(cursor + (FIRST ? sg.coarse_pos : sg.bin_pos + base) + r0 + t, c) : 0u;
+            int total;
+            const int ex = ws_block_excl_scan<NT, int>((int)c, s.wsum, &total);
+            s.cnt[t] = (uint32_t)ex;
+            s.delta[t] = (int32_t)g - ex;
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < ITEMS; ++k) {
+                const uint32_t b = (br[k] >> bsh) - off;
+                if (t + k * NT < len && b < WS_FAN) {
+                    const uint32_t j = s.cnt[b] + (br[k] & 0x1fffu);
+                    s.key[j] = key[k];
+                    s.bin[j] = (B)(br[k] >> 13);
+                }
+            }
+            __syncthreads();
+            // (the key registers are free: the next tile's loads overlap the copy)
+            if (r0 + WS_FAN >= nbk && nxt < n_tiles) load(tiles[nxt]);
+            // bucket runs, copied out by consecutive threads
+            K* dst = (FIRST && fl != 0 ? out_a : out_b) + sg.kpos;
+            B* bdst = bins_out + sg.kpos;
+            const uint32_t slen = (uint32_t)sg.len;
+#pragma unroll 4
+            for (int j = t; j < total; j += NT) {
+                const B bn = s.bin[j];
+                const uint32_t p = (uint32_t)(s.delta[((uint32_t)bn >> (bsh - 13)) - off] + j);
+                if (p < slen) {   // (always)
+                    dst[p] = s.key[j];
+                    if (FIRST && fl != 0) bdst[p] = bn;
+                }
+            }
+        }
+        tile = nxt;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Sort of one bin per CTA: the keys into 1024 groups by a monotone linear map
+// of the bin's range (2.5 keys each on average), every group of at most 8 keys
+// in one thread's registers by a sorting network, larger ones (one in a
+// thousand, more in the tails, where the density varies inside a bin) by a
+// warp that counts ranks.  A bin with a group of more than BIN_WARP_MAX keys
+// (ties, a very uneven density) takes LSD radix passes over the bits that vary
+// in it.
+// ---------------------------------------------------------------------------
+constexpr int BIN_NT = 256;
+constexpr int BIN_GPT = 4;                       // groups per thread
+constexpr int BIN_GROUPS = BIN_GPT * BIN_NT;
+constexpr int BIN_WARP_MAX = 256;
+constexpr int BIN_ITEMS = WS_BIN_CAP / BIN_NT;
+
+template <typename T>
+struct BinSmem {
+    typedef typename KeyOf<T>::K K;
+    K key[WS_BIN_CAP];
+    union {
+        uint32_t cnt[BIN_GROUPS];
+        struct {
+            uint32_t whist[(BIN_NT / 32) * 256];
+            uint32_t dcount[256], dstart[256];
+        } radix;
+    } u;
+    K lo, hi;
+    int wsum[BIN_NT / 32];
+    int n_list;
+    uint32_t list[WS_BIN_CAP / 9 + 1];   // start << 16 | keys of the groups for the warps
+};
+
+// Batcher's odd-even merge sorting network.
+template <int N, typename K>
+__device__ __forceinline__ void sort_network(K (&v)[N]) {
+#pragma unroll
+    for (int p = 1; p < N; p *= 2)
+#pragma unroll
+        for (int k = p; k >= 1; k /= 2)
+#pragma unroll
+            for (int j = k % p; j + k < N; j += 2 * k)
+#pragma unroll
+                for (int i = 0; i < k; ++i)
+                    if (j + i + k < N && (j + i) / (2 * p) == (j + i + k) / (2 * p)) {
+                        const K a = v[j + i], c = v[j + i + k];
+                        v[j + i] = min(a, c);
+                        v[j + i + k] = max(a, c);
+                    }
+}
+
+template <int N, typename K>
+__device__ __forceinline__ void sort_group(K* key, int n) {
+    K v[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = i < n ? key[i] : ~(K)0;
+    sort_network<N, K>(v);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+        if (i < n) key[i] = v[i];
+}
+
+// Sort of n <= BIN_WARP_MAX keys by one warp: every key's rank by counting
+// (ties by place).
+template <typename K>
+__device__ __noinline__ void sort_warp(K* key, int n) {
+    const int lane = threadIdx.x & 31;
+    constexpr int PER = BIN_WARP_MAX / 32;
+    K v[PER];
+    int r[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        v[k] = lane + 32 * k < n ? key[lane + 32 * k] : ~(K)0;
+        r[k] = 0;
+    }
+    for (int j = 0; j < n; ++j) {
+        const K x = key[j];
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            if (32 * k >= n) break;   // (uniform)
+            r[k] += (x < v[k] || (x == v[k] && j < lane + 32 * k)) ? 1 : 0;
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < PER; ++k)
+        if (lane + 32 * k < n) key[r[k]] = v[k];
+    __syncwarp();
+}
+
+__device__ __forceinline__ uint32_t warp_min_k(uint32_t v) { return __reduce_min_sync(WS_FULL_MASK, v); }
+__device__ __forceinline__ uint32_t warp_max_k(uint32_t v) { return __reduce_max_sync(WS_FULL_MASK, v); }
+__device__ __forceinline__ uint64_t warp_min_k(uint64_t v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = min(v, ws_shfl_xor_k(v, o));
+    return v;
+}
+__device__ __forceinline__ uint64_t warp_max_k(uint64_t v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = max(v, ws_shfl_xor_k(v, o));
+    return v;
+}
+
+template <typename T>
+__device__ __noinline__ void bin_radix(BinSmem<T>& s, int n, typename KeyOf<T>::K diff) {
+    typedef typename KeyOf<T>::K K;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    for (int pass = 0; pass < KeyOf<T>::BITS / 8; ++pass) {
+        if (((diff >> (8 * pass)) & 0xff) == 0) continue;
+        K key[BIN_ITEMS];
+        uint32_t dg[BIN_ITEMS];
+        bool valid[BIN_ITEMS];
+        int pos[BIN_ITEMS];
+#pragma unroll
+        for (int k = 0; k < BIN_ITEMS; ++k) {
+            const int p = w * 32 * BIN_ITEMS + k * 32 + lane;
+            valid[k] = p < n;
+            key[k] = valid[k] ? s.key[p] : (K)0;
+            dg[k] = (uint32_t)((key[k] >> (8 * pass)) & 0xff);
+        }
+        __syncthreads();
+        ws_rank_digits<BIN_NT, BIN_ITEMS, 1>(dg, valid, pos, s.u.radix.whist, s.u.radix.dcount, s.u.radix.dstart);
+#pragma unroll
+        for (int k = 0; k < BIN_ITEMS; ++k)
+            if (valid[k]) s.key[pos[k]] = key[k];
+        __syncthreads();
+    }
+}
+
+// Monotone image of a double in FP32 by truncation (no FP64 conversion).
+__device__ __forceinline__ float ws_trunc_f32(float v) { return v; }
+__device__ __forceinline__ float ws_trunc_f32(double v) {
+    const uint64_t b = (uint64_t)__double_as_longlong(v);
+    const int e = (int)((b >> 52) & 0x7ff) - 896;
+    const uint32_t sign = (uint32_t)(b >> 32) & 0x80000000u;
+    uint32_t m = (uint32_t)(b >> 29) & 0x7fffffu;
+    if (e <= 0) return __uint_as_float(sign);
+    if (e >= 255) return __uint_as_float(sign | 0x7f7fffffu);
+    return __uint_as_float(sign | ((uint32_t)e << 23) | m);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>::K* __restrict__ keys,
+                                                        typename KeyOf<T>::K* __restrict__ sorted,
+                                                        const int32_t* __restrict__ bin_seg,
+                                                        const LargeSeg* __restrict__ lsegs,
+                                                        const uint32_t* __restrict__ bin_start,
+                                                        const uint32_t* __restrict__ bin_cnt, SortCtl* ctl,
+                                                        OverBin* over, int64_t n_keys) {
+    typedef KeyOf<T> KO;
+    typedef typename KO::K K;
+    __shared__ BinSmem<T> s;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    if (ctl->abort) {   // the keys were not moved: a sequence that is sorted, so that later steps see a valid one
+        for (int64_t i = (int64_t)blockIdx.x * BIN_NT + t; i < n_keys; i += (int64_t)gridDim.x * BIN_NT)
+            sorted[i] = KO::to_key((T)0);
+        return;
+    }
+    const int bin = blockIdx.x;
+    const LargeSeg& sg = lsegs[bin_seg[bin]];
+    const int64_t start = sg.kpos + (int64_t)bin_start[bin];
+    const int n = (int)bin_cnt[bin];
+    if (n <= 0) return;
+    if (n > WS_BIN_CAP) {
+        if (t == 0) {
+            const uint32_t i = atomicAdd(&ctl->over_count, 1u);
+            over[i].start = start;
+            over[i].n = n;
+            over[i].diff = 0;
+        }
+        return;
+    }
+    const K* src = keys + start;
+    K* dst = sorted + start;
+    reinterpret_cast<uint4*>(s.u.cnt)[t] = make_uint4(0, 0, 0, 0);
+    if (t == 0) { s.lo = ~(K)0; s.hi = 0; s.n_list = 0; }
+    K key[BIN_ITEMS];
+#pragma unroll
+    for (int k = 0; k < BIN_ITEMS; ++k) {
+        const int p = t + k * BIN_NT;
+        key[k] = p < n ? __ldg(src + p) : (K)0;
+    }
+    K lo = ~(K)0, hi = 0;
+#pragma unroll
+    for (int k = 0; k < BIN_ITEMS; ++k) {
+        if (k * BIN_NT >= n) break;   // (uniform)
+        if (t + k * BIN_NT < n) { lo = min(lo, key[k]); hi = max(hi, key[k]); }
+    }
+    lo = warp_min_k(lo);
+    hi = warp_max_k(hi);
+    __syncthreads();
+    if (lane == 0) { ws_atomic_min_k(&s.lo, lo); ws_atomic_max_k(&s.hi, hi); }
+    __syncthreads();
+    lo = s.lo;
+    hi = s.hi;
+    // group: linear in the key where sign and exponent are shared (the value is
+    // linear in the key there), else linear in the value
+    const bool same = ((lo ^ hi) >> KO::MANT) == 0;
+    const int dsh = max(0, 64 - __clzll((long long)((uint64_t)(hi - lo) | 1ull)) - 24);
+    const float x0 = ws_trunc_f32(KO::from_key(lo));
+    const float span = same ? (float)(uint32_t)((hi - lo) >> dsh) + 1.0f : ws_trunc_f32(KO::from_key(hi)) - x0;
+    const float scale = (span > 0.0f && span <= 3.0e38f) ? (float)BIN_GROUPS / span : 0.0f;
+    uint32_t br[BIN_ITEMS];   // group << 16 | rank
+#pragma unroll
+    for (int k = 0; k < BIN_ITEMS; ++k) {
+        if (k * BIN_NT >= n) break;   // (uniform)
+        if (t + k * BIN_NT < n) {
+            const float f = same ? (float)(uint32_t)((key[k] - lo) >> dsh) : ws_trunc_f32(KO::from_key(key[k])) - x0;
+            const uint32_t b = min((uint32_t)(int)(f * scale), (uint32_t)BIN_GROUPS - 1u);
+            br[k] = (b << 16) | atomicAdd(&s.u.cnt[b], 1u);
+        }
+    }
+    __syncthreads();
+    // this thread's four groups
+    static_assert(BIN_GPT == 4 && BIN_NT == 256, "a thread's group counts are one 16-byte word; eight warps");
+    const uint4 c4 = reinterpret_cast<const uint4*>(s.u.cnt)[t];
+    const int sum = (int)(c4.x + c4.y + c4.z + c4.w);
+    const int inc = ws_warp_incl_scan<int>(sum);
+    if (lane == 31) s.wsum[w] = inc;
+    if (__syncthreads_or(max(max(c4.x, c4.y), max(c4.z, c4.w)) > BIN_WARP_MAX)) {   // radix passes (uniform)
+#pragma unroll
+        for (int k = 0; k < BIN_ITEMS; ++k)
+            if (t + k * BIN_NT < n) s.key[t + k * BIN_NT] = key[k];
+        __syncthreads();
+        // (every bit below the highest one in which the extremes differ may vary)
+        const int top = 64 - __clzll((long long)(uint64_t)(lo ^ hi));
+        bin_radix<T>(s, n, top ? (K)(~(uint64_t)0 >> (64 - top)) : (K)0);
+        for (int i = t; i < n; i += BIN_NT) dst[i] = s.key[i];
+        return;
+    }
+    const int wt = s.wsum[lane & 7];
+    const int g0 = inc - sum + __reduce_add_sync(WS_FULL_MASK, lane < w ? wt : 0);
+    reinterpret_cast<uint4*>(s.u.cnt)[t] = make_uint4((uint32_t)g0, g0 + c4.x, g0 + c4.x + c4.y, g0 + c4.x + c4.y + c4.z);
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < BIN_ITEMS; ++k) {
+        if (k * BIN_NT >= n) break;   // (uniform)
+        if (t + k * BIN_NT < n) s.key[s.u.cnt[br[k] >> 16] + (br[k] & 0xffffu)] = key[k];
+    }
+    __syncthreads();
+    {
+        const int c[BIN_GPT] = {(int)c4.x, (int)c4.y, (int)c4.z, (int)c4.w};
+        int g = g0;
+#pragma unroll
+        for (int i = 0; i < BIN_GPT; ++i) {
+            if (c[i] <= 8) sort_group<8, K>(s.key + g, c[i]);
+            else s.list[atomicAdd(&s.n_list, 1)] = ((uint32_t)g << 16) | (uint32_t)c[i];
+            g += c[i];
+        }
+    }
+    __syncthreads();
+    const int nl = s.n_list;
+    if (nl > 0) {   // (uniform)
+        for (int i = w; i < nl; i += BIN_NT / 32) sort_warp<K>(s.key + (s.list[i] >> 16), (int)(s.list[i] & 0xffffu));
+        __syncthreads();
+    }
+#pragma unroll
+    for (int k = 0; k < BIN_ITEMS; ++k) {
+        if (k * BIN_NT >= n) break;   // (uniform)
+        const int p = t + k * BIN_NT;
+        if (p < n) dst[p] = s.key[p];
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Oversize bins: LSD radix passes over the digits that vary, all bins side by
+// side, as a cooperative grid with a barrier between the steps.  A bin's keys
+// start in keys_b and swap buffers with every pass that its digits need; they
+// end in keys_a (copied there if the number of passes is even).
+// ---------------------------------------------------------------------------
+struct OverSmem {
+    uint32_t whist[(OVER_NT / 32) * 256];
+    uint32_t dcount[256], dstart[256], base[256];
+    int wsum[OVER_NT / 32];
+    int carry;
+    int ent;
+    unsigned long long diff;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* ka, typename KeyOf<T>::K* kb,
+                                                         SortCtl* ctl, OverBin* over, uint32_t* over_cnt,
+                                                         uint64_t spin_limit, uint32_t* status) {
+    typedef KeyOf<T> KO;
+    typedef typename KO::K K;
+    constexpr int NT = OVER_NT, ITEMS = WS_SORT_ITEMS, TILE = WS_SORT_TILE, P = KO::BITS / 8;
+    __shared__ OverSmem s;
+    const int cnt = (int)ctl->over_count;
+    if (cnt == 0 || ctl->abort) return;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    GridBarrier bar{&ctl->over_bar, &ctl->abort, status, spin_limit, 0u, false};
+    // tiles of the bins, in list order
+    if (blockIdx.x == 0) {
+        if (t == 0) s.carry = 0;
+        __syncthreads();
+        for (int e0 = 0; e0 < cnt; e0 += NT) {
+            const int e = e0 + t;
+            const int nt = e < cnt ? (over[e].n + TILE - 1) / TILE : 0;
+            int tot;
+            const int ex = ws_block_excl_scan<NT, int>(nt, s.wsum, &tot);
+            if (e < cnt) __stcg(&over[e].first_tile, s.carry + ex);
+            __syncthreads();
+            if (t == 0) s.carry += tot;
+            __syncthreads();
+        }
+    }
+    bar.sync();
+    const int n_tiles = __ldcg(&over[cnt - 1].first_tile) + (over[cnt - 1].n + TILE - 1) / TILE;
+    // entry of a tile (all threads; ends synchronised)
+    auto entry = [&](int tile) -> int {
+        __syncthreads();
+        if (t == 0) {
+            int lo = 0, hi = cnt - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (__ldcg(&over[mid].first_tile) <= tile) lo = mid; else hi = mid - 1;
+            }
+            s.ent = lo;
+            s.diff = 0;
+        }
+        __syncthreads();
+        return s.ent;
+    };
+    auto passes_before = [&](unsigned long long diff, int p) {   // passes that the digits below p need
+        int c = 0;
+        for (int q = 0; q < p; ++q) c += ((diff >> (8 * q)) & 0xffull) != 0;
+        return c;
+    };
+    // bits that vary
+    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        const int e = entry(tile);
+        const int64_t st = over[e].start;
+        const int o0 = (tile - __ldcg(&over[e].first_tile)) * TILE, n = min(TILE, over[e].n - o0);
+        const K k0 = kb[st];
+        K d = 0;
+        for (int i = t; i < n; i += NT) d |= kb[st + o0 + i] ^ k0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) d |= ws_shfl_xor_k(d, o);
+        if (lane == 0 && d) atomicOr(&s.diff, (unsigned long long)d);
+        __syncthreads();
+        if (t == 0 && s.diff) {
+            atomicOr(&over[e].diff, s.diff);
+            atomicOr(&ctl->over_diff, s.diff);
+        }
+    }
+    bar.sync();
+    const unsigned long long all = __ldcg(&ctl->over_diff);
+    for (int p = 0; p < P; ++p) {
+        if (((all >> (8 * p)) & 0xffull) == 0) continue;   // (uniform over the grid)
+        // digit counts of every tile
+        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+            const int e = entry(tile);
+            const unsigned long long diff = __ldcg(&over[e].diff);
+            if (((diff >> (8 * p)) & 0xffull) == 0) continue;
+            const K* src = ((passes_before(diff, p) & 1) ? ka : kb) + over[e].start;
+            const int o0 = (tile - __ldcg(&over[e].first_tile)) * TILE, n = min(TILE, over[e].n - o0);
+            if (t < 256) s.dcount[t] = 0;
+            __syncthreads();
+            for (int i = t; i < n; i += NT) atomicAdd(&s.dcount[(int)((__ldcg(src + o0 + i) >> (8 * p)) & 0xff)], 1u);
+            __syncthreads();
+            if (t < 256) __stcg(over_cnt + (size_t)tile * 256 + t, s.dcount[t]);
+        }
+        bar.sync();
+        // counts -> first position of every (tile, digit), one CTA per bin
+        for (int e = blockIdx.x; e < cnt; e += gridDim.x) {
+            const unsigned long long diff = __ldcg(&over[e].diff);
+            if (((diff >> (8 * p)) & 0xffull) == 0) continue;
+            uint32_t* c = over_cnt + (size_t)__ldcg(&over[e].first_tile) * 256;
+            const int nt = (over[e].n + TILE - 1) / TILE;
+            __syncthreads();
+            uint32_t run = 0;
+            if (t < 256) {
+                int i = 0;
+                for (; i + 8 <= nt; i += 8) {
+                    uint32_t v[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) v[u] = __ldcg(c + (size_t)(i + u) * 256 + t);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) { __stcg(c + (size_t)(i + u) * 256 + t, run); run += v[u]; }
+                }
+                for (; i < nt; ++i) {
+                    const uint32_t v = __ldcg(c + (size_t)i * 256 + t);
+                    __stcg(c + (size_t)i * 256 + t, run);
+                    run += v;
+                }
+            }
+            const int ex = ws_block_excl_scan<NT, int>((int)run, s.wsum, nullptr);
+            if (t < 256)
+                for (int i = 0; i < nt; ++i) __stcg(c + (size_t)i * 256 + t, __ldcg(c + (size_t)i * 256 + t) + (uint32_t)ex);
+        }
+        bar.sync();
+        // stable scatter
+        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+            const int e = entry(tile);
+            const unsigned long long diff = __ldcg(&over[e].diff);
+            if (((diff >> (8 * p)) & 0xffull) == 0) continue;
+            const bool odd = passes_before(diff, p) & 1;
+            const K* src = (odd ? ka : kb) + over[e].start;
+            K* dst = (odd ? kb : ka) + over[e].start;
+            const int ne = over[e].n;
+            const int o0 = (tile - __ldcg(&over[e].first_tile)) * TILE, n = min(TILE, ne - o0);
+            K key[ITEMS];
+            uint32_t dg[ITEMS];
+            bool valid[ITEMS];
+            int pos[ITEMS];
+#pragma unroll
+            for (int k = 0; k < ITEMS; ++k) {
+                const int i = w * 32 * ITEMS + k * 32 + lane;
+                valid[k] = i < n;
+                key[k] = valid[k] ? __ldcg(src + o0 + i) : (K)0;
+                dg[k] = (uint32_t)((key[k] >> (8 * p)) & 0xff);
+            }
+            if (t < 256) s.base[t] = __ldcg(over_cnt + (size_t)tile * 256 + t);
+            ws_rank_digits<NT, ITEMS, 1>(dg, valid, pos, s.whist, s.dcount, s.dstart);
+#pragma unroll
+            for (int k = 0; k < ITEMS; ++k)
+                if (valid[k]) {
+                    const uint32_t q = s.base[dg[k]] + (uint32_t)pos[k] - s.dstart[dg[k]];
+                    if (q < (uint32_t)ne) dst[q] = key[k];
+                }
+        }
+        bar.sync();
+    }
+    // bins whose keys are still in keys_b
+    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        const int e = entry(tile);
+        if (passes_before(__ldcg(&over[e].diff), P) & 1) continue;
+        const int64_t st = over[e].start;
+        const int o0 = (tile - __ldcg(&over[e].first_tile)) * TILE, n = min(TILE, over[e].n - o0);
+        for (int i = t; i < n; i += NT) ka[st + o0 + i] = __ldcg(kb + st + o0 + i);
+    }
+}
+
+// Shared memory of the plan kernel for hist_cap bins counted locally.
+size_t plan_smem(int hist_cap) { return sizeof(MapTab) + 4 * (size_t)hist_cap; }
 
 }  // namespace
 
+// Launch shapes of a plan's sort (and the kernels' shared-memory limits on
+// the plan's device).  max_bins: of its longest segment; samp_max: log2 of the
+// largest number of samples per tile.
+template <typename T, typename B>
+static cudaError_t sort_prepare(int max_bins, int n_tiles, WsSortShape* sh) {
+    constexpr int HIST_MAX = 45056;
+    auto* kp = k_sort_plan<T, B>;
+    auto* k1 = k_part<T, B, true>;
+    auto* k2 = k_part<T, B, false>;
+    auto* ko = k_oversize<T>;
+    const size_t ksm = sizeof(PartSmem<T, B>);
+    cudaError_t e = cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan_smem(HIST_MAX));
+    if (!e) e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ksm);
+    if (!e) e = cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ksm);
+    if (e) return e;
+    int dev = 0, sms = 0, np = 0, n1 = 0, no = 0;
+    if ((e = cudaGetDevice(&dev))) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return e;
+    // shared words of the plan kernel (one CTA per SM): the bins of the longest
+    // segment and the CTA's samples, as far as they fit
+    sh->plan_grid = std::min(sms, n_tiles);
+    const int64_t keep = ((int64_t)((n_tiles + sh->plan_grid - 1) / sh->plan_grid) << sh->samp_max) *
+                         (int64_t)(sizeof(typename KeyOf<T>::K) / 4);
+    sh->hist_cap = (int)std::min<int64_t>(std::max<int64_t>(std::max<int64_t>(max_bins, 1024), keep), HIST_MAX);
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&np, kp, PLAN_NT, plan_smem(sh->hist_cap)))) return e;
+    if (np < 1) return cudaErrorInvalidConfiguration;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, k1, WS_SORT_NT, ksm))) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&no, ko, OVER_NT, 0))) return e;
+    sh->part_grid = std::max(1, sms * n1);
+    sh->over_grid = std::max(1, sms * no);
+    return cudaSuccess;
+}
+
 template <typename T>
-size_t ws_onesweep_smem() {
+cudaError_t ws_sort_prepare(int max_bins, int n_tiles, int samp_max, WsSortShape* sh) {
+    sh->wide = max_bins > 65536;
+    sh->samp_max = samp_max;
+    sh->max_bins = max_bins;
+    return sh->wide ? sort_prepare<T, uint32_t>(max_bins, n_tiles, sh) : sort_prepare<T, uint16_t>(max_bins, n_tiles, sh);
+}
+
+template <typename T, typename B>
+static cudaError_t sort_run(const LargeWork<T>& W, const T* values, uint32_t* status, uint64_t spin_limit,
+                            cudaStream_t st) {
     typedef typename KeyOf<T>::K K;
-    return sizeof(K) * WS_SORT_TILE + sizeof(uint32_t) * (2 * (WS_SORT_NT / 32) * 256 + 256) +
-           sizeof(int64_t) * 256;
+    cudaError_t e = cudaMemsetAsync(W.ctl, 0, W.sort_zero_bytes, st);
+    if (e) return e;
+    const WsSortShape& sh = W.sort_shape;
+    // bins of the keys: in the caller's order, then in the first pass's
+    B* bins = (B*)W.bins;
+    B* bins2 = bins + W.n_keys;
+    {
+        int n_tiles = W.n_sort_tiles, n_lseg = W.n_lseg, hc = sh.hist_cap, sm = sh.samp_max, mb = sh.max_bins;
+        const TileDesc* tiles = W.sort_tiles;
+        const LargeSeg* lsegs = W.lsegs;
+        void* args[] = {(void*)&values, &tiles, &n_tiles, &lsegs, &n_lseg, (void*)&W.ctl, (void*)&W.seg_hi,
+                        (void*)&W.seg_lo, (void*)&W.seg_en, (void*)&W.cells, (void*)&W.bin_cnt, &bins,
+                        (void*)&W.bin_start, (void*)&W.cur1, (void*)&W.cur2, (void*)&W.seg_emin, &mb, &hc, &sm, &spin_limit,
+                        &status};
+        WS_LAUNCH(W.prof, WSK_SORT_PLAN, st,
+                  e = cudaLaunchCooperativeKernel((const void*)k_sort_plan<T, B>,
+                                                  dim3(sh.plan_grid), dim3(PLAN_NT), args,
+                                                  plan_smem(sh.hist_cap), st));
+        if (e) return e;
+    }
+    const size_t ksm = sizeof(PartSmem<T, B>);
+    const int grid = std::min(sh.part_grid, W.n_sort_tiles);
+    WS_LAUNCH(W.prof, WSK_PARTITION, st,
+              (k_part<T, B, true><<<grid, WS_SORT_NT, ksm, st>>>(values, nullptr, bins, W.keys_a, W.keys_b, bins2,
+                                                                 W.sort_tiles, W.n_sort_tiles, W.lsegs, W.cur1, W.ctl,
+                                                                 status)));
+    if (W.two_level)
+        WS_LAUNCH(W.prof, WSK_PARTITION, st,
+                  (k_part<T, B, false><<<grid, WS_SORT_NT, ksm, st>>>(nullptr, W.keys_a, bins2, nullptr, W.keys_b,
+                                                                      nullptr, W.sort_tiles, W.n_sort_tiles, W.lsegs,
+                                                                      W.cur2, W.ctl, status)));
+    WS_LAUNCH(W.prof, WSK_BIN_SORT, st,
+              (k_bin_sort<T><<<W.n_bins, BIN_NT, 0, st>>>(W.keys_b, W.keys_a, W.bin_seg, W.lsegs, W.bin_start,
+                                                          W.bin_cnt, W.ctl, W.over, W.n_keys)));
+    {
+        K* ka = W.keys_a;
+        K* kb = W.keys_b;
+        void* args[] = {&ka, &kb, (void*)&W.ctl, (void*)&W.over, (void*)&W.over_cnt, &spin_limit, &status};
+        WS_LAUNCH(W.prof, WSK_OVERSIZE, st,
+                  e = cudaLaunchCooperativeKernel((const void*)k_oversize<T>,
+                                                  dim3(std::min(sh.over_grid, W.n_sort_tiles)), dim3(OVER_NT), args, 0,
+                                                  st));
+        if (e) return e;
+    }
+    return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t ws_large_sort(const LargeWork<T>& W, const T* values, uint32_t* status, uint64_t spin_limit,
                           cudaStream_t st, typename KeyOf<T>::K** sorted) {
-    typedef typename KeyOf<T>::K K;
-    constexpr int P = KeyOf<T>::BITS / 8;
-    cudaError_t e;
     *sorted = nullptr;
     if (W.n_sort_tiles == 0) return cudaSuccess;
-    e = cudaMemsetAsync(W.hist, 0, sizeof(uint32_t) * (size_t)W.n_lseg * P * 256, st);
-    if (e) return e;
-    e = cudaMemsetAsync(W.tile_counter, 0, sizeof(uint32_t) * P, st);
-    if (e) return e;
-    e = cudaMemsetAsync(W.seg_emin, 0x7f, sizeof(int32_t) * (size_t)W.n_lseg, st);
-    if (e) return e;
-    // the histogram's persistent grid: every CTA resident at once
-    static const int hist_grid = [] {
-        int dev = 0, sms = 0, per_sm = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hist<T>, WS_SORT_NT, 0) != cudaSuccess) {
-            cudaGetLastError();
-            return 2 * 152;
-        }
-        return std::max(1, sms * std::max(per_sm, 1));
-    }();
-    WS_LAUNCH(W.prof, WSK_HIST, st,
-              (k_hist<T><<<W.n_sort_tiles < hist_grid ? W.n_sort_tiles : hist_grid, WS_SORT_NT, 0, st>>>(
-                  values, W.sort_tiles, W.n_sort_tiles, W.hist, W.seg_emin, status)));
-    WS_LAUNCH(W.prof, WSK_HIST_SCAN, st, (k_hist_scan<<<W.n_lseg * P, 256, 0, st>>>(W.hist, W.epoch)));
-    size_t smem = ws_onesweep_smem<T>();
-    e = cudaFuncSetAttribute(k_onesweep<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e) return e;
-    e = cudaFuncSetAttribute(k_onesweep<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e) return e;
-    K* src = W.keys_b;
-    K* dst = W.keys_a;
-    for (int p = 0; p < P; ++p) {
-        uint64_t* lb = W.lookback + (size_t)p * W.n_sort_tiles * 256;
-        if (p == 0)
-            WS_LAUNCH(W.prof, WSK_ONESWEEP, st, (k_onesweep<T, true><<<W.n_sort_tiles, WS_SORT_NT, smem, st>>>(
-                values, nullptr, dst, W.sort_tiles, W.lsegs, W.hist, lb, W.tile_counter + p, W.epoch, p, status,
-                spin_limit)));
-        else
-            WS_LAUNCH(W.prof, WSK_ONESWEEP, st, (k_onesweep<T, false><<<W.n_sort_tiles, WS_SORT_NT, smem, st>>>(
-                values, src, dst, W.sort_tiles, W.lsegs, W.hist, lb, W.tile_counter + p, W.epoch, p, status,
-                spin_limit)));
-        K* tmp = src; src = dst; dst = tmp;
-    }
-    *sorted = src;   // the buffer written last
-    return cudaGetLastError();
+    *sorted = W.keys_a;
+    return W.sort_shape.wide ? sort_run<T, uint32_t>(W, values, status, spin_limit, st)
+                             : sort_run<T, uint16_t>(W, values, status, spin_limit, st);
 }
 
+template cudaError_t ws_sort_prepare<float>(int, int, int, WsSortShape*);
+template cudaError_t ws_sort_prepare<double>(int, int, int, WsSortShape*);
 template cudaError_t ws_large_sort<float>(const LargeWork<float>&, const float*, uint32_t*, uint64_t, cudaStream_t,
                                           uint32_t**);
 template cudaError_t ws_large_sort<double>(const LargeWork<double>&, const double*, uint32_t*, uint64_t,

@@ -1,0 +1,99 @@
+"""The distribution sort of the device-wide path, bit for bit against numpy:
+bins at their edges, one and two partition passes, distributions that the
+sampled map resolves well or not at all, and ties beyond one bin's capacity."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2311_03096_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+UINT = {np.float32: np.uint32, np.float64: np.uint64}
+TT = {np.float32: torch.float32, np.float64: torch.float64}
+
+
+@pytest.fixture(scope="module")
+def ws():
+    from paper_2311_03096_gb300 import ws as m
+
+    return m
+
+
+@pytest.fixture
+def ctx(ws):
+    c = ws.Context.get()
+    c.set_small_max(0)
+    yield c
+    c.set_small_max(-1)
+
+
+def draw(kind, d, dt, seed=5):
+    rng = np.random.default_rng(seed)
+    x = rng.standard_normal(d)
+    if kind == "duplicates":
+        return inputs.with_duplicates(x.astype(dt), 0.1, seed)
+    if kind == "narrow":            # one binade, a sliver of it, and one far outlier
+        x = 1.0 + 1e-4 * x
+        x[d // 3] = -3e30
+    elif kind == "sparse":          # half zeros of both signs (one heavy tie), the rest spread
+        x[rng.random(d) < 0.5] = 0.0
+        x[rng.random(d) < 0.1] *= -0.0
+    elif kind == "few":             # a handful of values, neighbours in the map
+        x = np.array([-0.5, 0.25, 0.2500001, 0.2500002, 3.0])[rng.integers(0, 5, d)]
+    elif kind == "binades":         # sixty binades, both signs
+        x = np.ldexp(x, rng.integers(-30, 30, d))
+    elif kind == "clusters":        # spikes that the cells of the map do not resolve
+        x = rng.integers(-20, 20, d) + 1e-5 * x
+    elif kind == "sorted":
+        x = np.sort(x)
+    elif kind == "constant":
+        x = np.full(d, 0.37)
+    return x.astype(dt)
+
+
+def check(ws, ctx, w):
+    dt = w.dtype.type
+    plan = ws.Plan([0, w.shape[0]], TT[dt])
+    s = torch.zeros(w.shape[0], dtype=TT[dt], device="cuda")
+    plan.debug_sort(torch.from_numpy(w).cuda(), s)
+    ctx.check(what="debug_sort")
+    # the IEEE total order (-0 before +0) as signed integers
+    b = w.view(UINT[dt])
+    top = UINT[dt](1) << UINT[dt](8 * w.itemsize - 1)
+    keys = np.sort(np.where(b & top, ~b, b | top))
+    want = np.where(keys & top, keys ^ top, ~keys)
+    assert np.array_equal(s.cpu().numpy().view(UINT[dt]), want)
+
+
+@pytest.mark.parametrize("dt", [np.float32, np.float64])
+@pytest.mark.parametrize("d", [2, 31, 2560, 4095, 4096, 4097, 5633, 6144, 6145, 40961])
+def test_bin_edges(ws, ctx, d, dt):
+    check(ws, ctx, draw("duplicates", d, dt))
+
+
+@pytest.mark.parametrize("dt", [np.float32, np.float64])
+@pytest.mark.parametrize("kind", ["narrow", "sparse", "few", "binades", "clusters", "sorted", "constant"])
+def test_distributions(ws, ctx, kind, dt):
+    check(ws, ctx, draw(kind, 300007, dt))
+
+
+@pytest.mark.parametrize("dt", [np.float32, np.float64])
+@pytest.mark.parametrize("kind", ["duplicates", "sparse", "clusters", "sorted"])
+def test_two_passes(ws, ctx, kind, dt):
+    check(ws, ctx, draw(kind, 512 * 2560 + 1 + 70001, dt))
+
+
+def test_segments(ws, ctx):
+    """One- and two-pass segments, ties and tiny ones side by side."""
+    kinds = ["duplicates", "constant", "sparse", "few", "narrow", "clusters"]
+    lens = [1600000, 5000, 70000, 2, 40000, 9001, 4097, 1500001]
+    parts = [draw(kinds[i % len(kinds)], n, np.float32, seed=i) for i, n in enumerate(lens)]
+    w = np.concatenate(parts)
+    plan = ws.Plan(np.concatenate([[0], np.cumsum(lens)]), torch.float32)
+    s = torch.zeros(w.shape[0], device="cuda")
+    for _ in range(2):   # (a second call finds the first one's cursors and cells)
+        plan.debug_sort(torch.from_numpy(w).cuda(), s)
+        ctx.check(what="debug_sort")
+        got = np.split(s.cpu().numpy(), np.cumsum(lens)[:-1])
+        for g, p in zip(got, parts):
+            assert np.array_equal(np.sort(g), g) and np.array_equal(np.sort(p), g)
