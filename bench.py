@@ -42,7 +42,9 @@ ALGO_BYTES_PER_ELEM_F32 = {
     "bin_sort": 8,    # read key + write key
     "sort_plan": 4,   # read the value
     "tile_hull": 4,   # read the sorted key (hull vertices are data dependent, not counted)
-    "lookup": 12,     # read w, write out and cluster id (I/O floor)
+    "bin_out": 10,    # read the rank in the bin, write value and cluster id
+    "regroup": 20,    # read a place, read and write value and cluster id
+    "output": 20,     # read a place, value and cluster id, write out and cluster id
 }
 
 # Whole-step byte models per element (FP32 storage), fixed before tuning:

@@ -100,8 +100,13 @@ struct ws_plan {
     i128* seg_total = nullptr;
     int32_t* seg_below = nullptr;
     SegRuntime* rt = nullptr;
-    void* table = nullptr;
-    DirEntry* dir = nullptr;
+    void* cval = nullptr;
+    uint2* rank_words = nullptr;
+    uint32_t* dest1 = nullptr;
+    uint32_t* dest2 = nullptr;
+    uint16_t* bin_idx = nullptr;
+    void* pairs_a = nullptr;
+    void* pairs_b = nullptr;
     void* stat_partial = nullptr;
     void* bsum = nullptr;
     int32_t* bcnt = nullptr;
@@ -168,8 +173,13 @@ LargeWork<T> make_work(const ws_plan* p) {
     W.seg_total = p->seg_total;
     W.seg_below = p->seg_below;
     W.rt = p->rt;
-    W.table = (CEntry<T>*)p->table;
-    W.dir = p->dir;
+    W.cval = (T*)p->cval;
+    W.rank_words = p->rank_words;
+    W.dest1 = p->dest1;
+    W.dest2 = p->dest2;
+    W.bin_idx = p->bin_idx;
+    W.pairs_a = (OutPair<T>*)p->pairs_a;
+    W.pairs_b = (OutPair<T>*)p->pairs_b;
     W.bsum = (T*)p->bsum;
     W.bcnt = p->bcnt;
     W.bacc = p->bacc;
@@ -222,7 +232,7 @@ ws_status build_plan(ws_plan* p) {
     std::vector<int32_t> small;
     std::vector<LargeSeg> lsegs;
     std::vector<TileDesc> stiles, htiles;
-    int64_t kpos = 0, dir_pos = 0;
+    int64_t kpos = 0;
     int64_t bin_pos = 0, coarse_pos = 0, cell_pos = 0;
     std::vector<int32_t> bin_seg;
     int samp_max = 0;
@@ -249,9 +259,6 @@ ws_status build_plan(ws_plan* p) {
             htiles.push_back(td);
         }
         ls.hull_count = (int32_t)htiles.size() - ls.hull_first;
-        ls.dir_cap_log2 = std::min(ceil_log2(len), WS_DIR_MAX_LOG2);
-        ls.dir_pos = dir_pos;
-        dir_pos += ((int64_t)1 << ls.dir_cap_log2) + 1;
         // distribution sort: bins, buckets of the first pass, map
         ls.nbins = len <= WS_BIN_CAP ? 1 : (int32_t)std::min<int64_t>((len + WS_BIN_MEAN - 1) / WS_BIN_MEAN, WS_BINS_MAX);
         ls.fine_log2 = 0;
@@ -362,12 +369,22 @@ ws_status build_plan(ws_plan* p) {
     if ((st = plan_alloc(p, (void**)&p->seg_total, sizeof(i128) * p->n_lseg))) return st;
     if ((st = plan_alloc(p, (void**)&p->seg_below, sizeof(int32_t) * p->n_lseg))) return st;
     if ((st = plan_alloc(p, (void**)&p->rt, sizeof(SegRuntime) * p->n_lseg))) return st;
-    // (+4 entries: the lookup reads whole 32-byte sectors of the table)
-    if ((st = plan_alloc(p, &p->table, (f64 ? sizeof(CEntry<double>) : sizeof(CEntry<float>)) * (slots + 4)))) return st;
-    if ((st = plan_alloc(p, (void**)&p->dir, sizeof(DirEntry) * (size_t)dir_pos))) return st;
+    if ((st = plan_alloc(p, &p->cval, vsize * slots))) return st;
+    if ((st = plan_alloc(p, (void**)&p->rank_words, sizeof(uint2) * nh * (WS_HULL_TILE / 32)))) return st;
+    if ((st = plan_alloc(p, (void**)&p->dest1, sizeof(uint32_t) * nk))) return st;
+    if (p->two_level && (st = plan_alloc(p, (void**)&p->dest2, sizeof(uint32_t) * nk))) return st;
+    if ((st = plan_alloc(p, (void**)&p->bin_idx, sizeof(uint16_t) * nk))) return st;
     if ((st = plan_alloc(p, &p->bsum, vsize * slots))) return st;
     if ((st = plan_alloc(p, (void**)&p->bcnt, sizeof(int32_t) * slots))) return st;
-    if ((st = plan_alloc(p, (void**)&p->bacc, 2 * sizeof(unsigned long long) * slots))) return st;
+    {
+        // the backward's cluster sums and the forward's output pairs share one
+        // block (neither is kept from one call to the next)
+        const size_t pair = f64 ? sizeof(OutPair<double>) : sizeof(OutPair<float>);
+        const size_t sums = 2 * sizeof(unsigned long long) * slots, pairs = (p->two_level ? 2 : 1) * pair * nk;
+        if ((st = plan_alloc(p, (void**)&p->bacc, std::max(sums, pairs)))) return st;
+        p->pairs_b = p->bacc;
+        p->pairs_a = (unsigned char*)p->pairs_b + pair * nk;   // (two-level plans only)
+    }
     if ((st = plan_alloc(p, (void**)&p->bwd_seg, 2 * sizeof(int32_t) * p->n_lseg))) return st;
     if (cudaMemset(p->rt, 0, sizeof(SegRuntime) * p->n_lseg) != cudaSuccess) return WS_ERR_CUDA;
     return WS_OK;
@@ -852,19 +869,19 @@ ws_status ws_debug_sort(ws_plan* plan, const void* values, void* sorted_out, voi
     if (plan->dtype == WS_F64) {
         LargeWork<double> W = make_work<double>(plan);
         uint64_t* sorted = nullptr;
-        e = ws_large_sort<double>(W, (const double*)values, plan->ctx->status, plan->ctx->spin_limit, st, &sorted);
+        e = ws_large_sort<double>(W, (const double*)values, false, plan->ctx->status, plan->ctx->spin_limit, st, &sorted);
         if (!e) e = ws_large_copy_sorted<double>(W, sorted, (double*)sorted_out, st);
     } else {
         LargeWork<float> W = make_work<float>(plan);
         uint32_t* sorted = nullptr;
-        e = ws_large_sort<float>(W, (const float*)values, plan->ctx->status, plan->ctx->spin_limit, st, &sorted);
+        e = ws_large_sort<float>(W, (const float*)values, false, plan->ctx->status, plan->ctx->spin_limit, st, &sorted);
         if (!e) e = ws_large_copy_sorted<float>(W, sorted, (float*)sorted_out, st);
     }
     return map_cuda(e);
 }
 
 static const char* const kKernelNames[WSK_COUNT] = {"small", "sort_plan", "partition", "bin_sort", "oversize", "tile_hull",
-                                                     "root", "table", "big_gaps", "lookup", "backward", "misc",
+                                                     "root", "values", "bin_out", "regroup", "output", "backward", "misc",
                                                      "tile_general", "junction", "climb"};
 
 const char* ws_debug_kernel_name(int kind) {

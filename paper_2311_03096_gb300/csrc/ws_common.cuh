@@ -311,7 +311,7 @@ __device__ __forceinline__ double ws_i128_to_double(i128 v) {
 // truncated to an integer Q; the remainder R = S - Q n is exact in 128 bits
 // and |R / n| <= 2^-21 |S/n| + 1, so S/n = Q + R/n with R/n taken in FP32 has
 // an error below 2^-42 |S/n| + 2^-21 (in the units of S).
-__device__ __forceinline__ double ws_div_i128_n(i128 S, int64_t n) {
+__device__ __forceinline__ double ws_div_i128_n(i128 S, int n) {
     const float q = ws_i128_to_float_scaled(S, 0) / (float)n;
     const uint32_t bits = __float_as_uint(q);
     const int e = (int)((bits >> 23) & 0xffu) - 150;   // q = m 2^e, m the 24-bit significand
@@ -351,8 +351,9 @@ template <typename T> struct ValueOut;
 template <> struct ValueOut<float> {
     __device__ __forceinline__ static float value(i128 SX, int64_t a, int64_t b, float xsingle, const SegConst& sc,
                                                   bool fp64, const WsEpi& ep) {
-        int64_t n = b - a;
-        int64_t t = sc.d - a - b;
+        // (int, not int64: segments are shorter than 2^31, and 64-bit integers
+        // convert at the FP64 rate)
+        const int n = (int)(b - a), t = (int)(sc.d - a - b);
         if (fp64) {
             double mean = (n == 1) ? (double)xsingle : ldexp(ws_div_i128_n(SX, n), -sc.L);
             return (float)ws_epilogue<double>(mean, sc.mu_d * (double)t, ep.beta, ep.gamma, ep.on != 0);
@@ -360,12 +361,19 @@ template <> struct ValueOut<float> {
         float mean = (n == 1) ? xsingle : ldexpf(ws_i128_to_float_scaled(SX, 0) / (float)n, -sc.L);
         return ws_epilogue<float>(mean, sc.mu_f * (float)t, ep.beta_f, ep.gamma_f, ep.on != 0);
     }
+    // The same for a sum of less than 2^62 in magnitude (the 128-bit
+    // conversion shifts nothing out of it), in FP32 arithmetic.
+    __device__ __forceinline__ static float value64(int64_t SX, int n, int t, float xsingle, const SegConst& sc,
+                                                    const WsEpi& ep) {
+        const float f = ws_u64_to_float((uint64_t)(SX < 0 ? -SX : SX));
+        const float mean = (n == 1) ? xsingle : ldexpf((SX < 0 ? -f : f) / (float)n, -sc.L);
+        return ws_epilogue<float>(mean, sc.mu_f * (float)t, ep.beta_f, ep.gamma_f, ep.on != 0);
+    }
 };
 template <> struct ValueOut<double> {
     __device__ __forceinline__ static double value(i128 SX, int64_t a, int64_t b, double xsingle,
                                                    const SegConst& sc, bool fp64, const WsEpi& ep) {
-        int64_t n = b - a;
-        int64_t t = sc.d - a - b;
+        const int n = (int)(b - a), t = (int)(sc.d - a - b);
         if (!fp64) {
             // FP32 arithmetic on the exact sum, widened to the output type
             float mean = (n == 1) ? (float)xsingle : ldexpf(ws_i128_to_float_scaled(SX, 0) / (float)n, -sc.L);
@@ -379,26 +387,6 @@ template <> struct ValueOut<double> {
 // ---------------------------------------------------------------------------
 // Bounded spin-wait helper: every device-side wait has an iteration limit.
 // ---------------------------------------------------------------------------
-// L2 eviction priorities.  The lookup directory is re-read at random by every
-// weight while the weights and outputs stream through L2 once, so the
-// directory is loaded and stored with evict_last and the streams with
-// evict_first (.cs).
-__device__ __forceinline__ uint64_t ws_policy_evict_last() {
-    uint64_t p;
-    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-    return p;
-}
-__device__ __forceinline__ uint2 ws_ld_u2_last(const void* ptr, uint64_t pol) {
-    uint2 v;
-    asm volatile("ld.global.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;"
-                 : "=r"(v.x), "=r"(v.y) : "l"(ptr), "l"(pol));
-    return v;
-}
-__device__ __forceinline__ void ws_st_u2_last(void* ptr, uint2 v, uint64_t pol) {
-    asm volatile("st.global.L2::cache_hint.v2.u32 [%0], {%1, %2}, %3;" ::"l"(ptr), "r"(v.x), "r"(v.y), "l"(pol)
-                 : "memory");
-}
-
 __device__ __forceinline__ void ws_backoff(int it) {
     if (it > 64) __nanosleep(it > 4096 ? 256 : 32);
 }

@@ -11,7 +11,7 @@ template <> struct SmallCfg<double> { static constexpr int M = 16; static conste
 // around every kernel) and a launch counter.  Host-side only.
 enum WsKernelKind {
     WSK_SMALL = 0, WSK_SORT_PLAN, WSK_PARTITION, WSK_BIN_SORT, WSK_OVERSIZE, WSK_TILE_HULL, WSK_ROOT,
-    WSK_TABLE, WSK_BIG_GAPS, WSK_LOOKUP, WSK_BWD, WSK_MISC, WSK_TILE_GENERAL, WSK_JUNCTION, WSK_CLIMB, WSK_COUNT
+    WSK_VALUES, WSK_BIN_OUT, WSK_REGROUP, WSK_OUTPUT, WSK_BWD, WSK_MISC, WSK_TILE_GENERAL, WSK_JUNCTION, WSK_CLIMB, WSK_COUNT
 };
 struct WsProf {
     bool enabled = false;
@@ -40,8 +40,8 @@ constexpr int WS_SORT_ITEMS = 12;            // keys per thread
 constexpr int WS_SORT_TILE = WS_SORT_NT * WS_SORT_ITEMS;   // 6144 keys per sort tile
 // Distribution sort (ws_sort.cu): bins of about WS_BIN_MEAN keys, sorted by
 // one CTA up to WS_BIN_CAP keys.  The ratio 1.6 leaves room for the error of
-// the sampled map (5 to 8 % standard deviation on N(0, 1), largest bin 1.2 to
-// 1.55 times the mean; 2816 let a few bins of the tails overflow).
+// the sampled map (5 to 14 % standard deviation on N(0, 1), the largest bin 1.2
+// to 1.55 times the mean; a mean of 2816 let a few bins of the tails overflow).
 constexpr int WS_BIN_CAP = 4096;
 constexpr int WS_BIN_MEAN = 2560;
 constexpr int WS_BINS_MAX = 1 << 19;         // per segment (a partition's rank word holds 19 bits of bin)
@@ -71,8 +71,6 @@ struct LargeSeg {
     int32_t seg;       // index in the caller's segment list
     int32_t sort_first, sort_count;   // sort tiles
     int32_t hull_first, hull_count;   // hull tiles
-    int64_t dir_pos;   // directory slice start
-    int32_t dir_cap_log2;             // directory slice holds 2^dir_cap_log2 + 1 entries
     // distribution sort
     int32_t nbins;             // bins of the segment
     int32_t fine_log2;         // first pass: bucket = bin >> fine_log2 (0: one pass only)
@@ -104,6 +102,7 @@ struct OverBin {
     int32_t n;
     int32_t first_tile;     // of the oversize kernel's tiles
     unsigned long long diff;   // key bits that vary inside the bin
+    int32_t lseg, pad;
 };
 
 // A piece of a node hull: vertices [lo, hi) of hull tile `tile`; cum = rank of
@@ -117,18 +116,10 @@ struct __align__(16) Piece {
     i128 off;
 };
 
-// Cluster table entry (sorted by key within a segment).
-template <typename T> struct CEntry;
-template <> struct CEntry<float> { uint32_t key; float val; };
-template <> struct CEntry<double> { uint64_t key; double val; };
-
-// Directory entry: first cluster whose start falls in the bucket (or in a
-// later one) and the top 32 bits of that cluster's start key.
-struct DirEntry {
-    int32_t idx;
-    uint32_t key32;
-};
-constexpr int WS_DIR_MAX_LOG2 = 22;   // <= 2^22 buckets per segment (32 MiB: stays in L2)
+// Value and cluster id of one element, on its way back to the caller's order.
+template <typename T> struct OutPair;
+template <> struct __align__(8) OutPair<float> { float val; int32_t id; };
+template <> struct __align__(16) OutPair<double> { double val; int32_t id, pad; };
 
 // Constants of the exact hull test at one fixed-point unit scale of a
 // segment: the units of a one-binade hull tile (ulps of its binade) or the
@@ -149,10 +140,9 @@ constexpr int WS_NSCALE = 64;   // per segment: binade shifts 0 .. FIX_OFS, then
 // Per-segment run-time values computed on the device.
 struct SegRuntime {
     int64_t n_clusters;
-    int64_t table_pos;  // first cluster-table entry of the segment
+    int64_t table_pos;  // first cluster value of the segment
     int32_t emax;
-    int32_t dir_log2;   // directory holds 2^dir_log2 buckets (+1 sentinel)
-    float lo, scale;    // bucket map: floor((x - lo) * scale)
+    int32_t pad;
 };
 
 template <typename T>
@@ -227,8 +217,14 @@ struct LargeWork {
     i128* seg_total;         // [n_lseg] X of the whole segment
     int32_t* seg_below;      // [n_lseg] a tile-hull vertex lies below the segment's chord
     SegRuntime* rt;          // [n_lseg]
-    CEntry<T>* table;        // [n_keys + n_lseg]
-    DirEntry* dir;           // directory slices
+    T* cval;                 // [n_keys + n_lseg] cluster values
+    uint2* rank_words;       // [n_hull_tiles][WS_HULL_TILE / 32] cluster starts among 32 sorted positions, starts before
+    // way back to the caller's order
+    uint32_t* dest1;         // [n_keys] where the first pass put every key (relative to its segment)
+    uint32_t* dest2;         // [n_keys] the same of the second pass (two-level plans)
+    uint16_t* bin_idx;       // [n_keys] for every sorted position, its key's place in the unsorted bin
+    OutPair<T>* pairs_a;     // [n_keys] in the first pass's order (two-level segments)
+    OutPair<T>* pairs_b;     // [n_keys] in bin order; before that, scratch of the oversize bins' sort
     // backward
     T* bsum;                 // [n_keys + n_lseg] cluster means
     int32_t* bcnt;           // [n_keys + n_lseg] cluster sizes
@@ -237,9 +233,10 @@ struct LargeWork {
     WsProf* prof;            // host-side launch accounting
 };
 
+// way_back: also record where every key goes (dest1, dest2, bin_idx).
 template <typename T>
-cudaError_t ws_large_sort(const LargeWork<T>& W, const T* values, uint32_t* status, uint64_t spin_limit,
-                          cudaStream_t st, typename KeyOf<T>::K** sorted);
+cudaError_t ws_large_sort(const LargeWork<T>& W, const T* values, bool way_back, uint32_t* status,
+                          uint64_t spin_limit, cudaStream_t st, typename KeyOf<T>::K** sorted);
 // Lean tile hulls and the junction resolution (ws_tile.cu).
 template <typename T>
 cudaError_t ws_large_hull_fast(const LargeWork<T>& W, const typename KeyOf<T>::K* sorted, const double* lambdas,

@@ -1,6 +1,6 @@
 // ws_large.cu -- the device-wide path for segments longer than one CTA:
 //   sorted keys -> per-tile exact hulls -> tree of bridge merges across tiles
-//   -> cluster table -> key -> cluster lookup in the caller's order.
+//   -> cluster values and starts -> the sort's passes undone, to the caller's order.
 //
 // The hull of the points P_p = (p, S_p) (see ws_common.cuh) is built tile by
 // tile (4096 elements per CTA); adjacent tile hulls are then merged up a
@@ -654,14 +654,11 @@ __global__ void __launch_bounds__(HNT) k_climb(const TileDesc* __restrict__ htil
 }
 
 // ---------------------------------------------------------------------------
-// 4. root of each segment: cluster count, piece index per tile, bucket map
+// 4. root of each segment: cluster count, piece index per tile
 // ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(256) k_root(const LargeSeg* __restrict__ lsegs,
-                                              const typename KeyOf<T>::K* __restrict__ sorted, const Piece* pieces,
+__global__ void __launch_bounds__(256) k_root(const LargeSeg* __restrict__ lsegs, const Piece* pieces,
                                               const int32_t* npieces, int32_t* tile_piece, SegRuntime* rt,
                                               int64_t* n_clusters_out) {
-    typedef KeyOf<T> KO;
     const int lseg = blockIdx.x;
     const LargeSeg ls = lsegs[lseg];
     const Piece* P = pieces + ls.hull_first;
@@ -669,285 +666,332 @@ __global__ void __launch_bounds__(256) k_root(const LargeSeg* __restrict__ lsegs
     for (int i = threadIdx.x; i < np; i += 256) tile_piece[P[i].tile] = i;
     if (threadIdx.x == 0) {
         const Piece last = P[np - 1];
-        int64_t nvtx = (int64_t)last.cum + (last.hi - last.lo);
-        int64_t c = nvtx - 1;
-        SegRuntime r = rt[lseg];
-        r.n_clusters = c;
-        r.table_pos = ls.kpos + lseg;
-        int D = 0;
-        while (D < ls.dir_cap_log2 && ((int64_t)1 << D) < c) ++D;
-        r.dir_log2 = D;
-        float lo = (float)KO::from_key(sorted[ls.kpos]);
-        float hi = (float)KO::from_key(sorted[ls.kpos + ls.len - 1]);
-        float range = hi - lo;
-        float scale = (range > 0.0f && range <= 3.0e38f) ? (float)((int64_t)1 << D) / range : 0.0f;
-        if (!(scale <= 3.0e38f)) scale = 0.0f;
-        r.lo = lo; r.scale = scale;
-        rt[lseg] = r;
+        const int64_t c = (int64_t)last.cum + (last.hi - last.lo) - 1;
+        rt[lseg].n_clusters = c;
+        rt[lseg].table_pos = ls.kpos + lseg;
         if (n_clusters_out) n_clusters_out[ls.seg] = c;
     }
 }
 
-__device__ __forceinline__ int ws_bucket(float x, float lo, float scale, int nb) {
-    float f = (x - lo) * scale;
-    int b = (f >= (float)nb) ? nb - 1 : (f > 0.0f ? (int)f : 0);
-    return b > nb - 1 ? nb - 1 : b;
-}
-
 // ---------------------------------------------------------------------------
-// 5. cluster table + directory fill (one CTA per hull tile; eight CTAs per
-//    SM at 32 registers: its reads are latency bound, so warps beat registers)
+// 5. cluster values, and for every 32 sorted positions the bitmap of cluster
+// starts among them with the number of starts before them (one CTA per hull
+// tile).  The cluster of a sorted position is then one word away; no search by
+// value is needed.  A cluster of at most SUM_MAX elements takes its exact sum
+// from the tile's keys (4 bytes per element, in shared memory) instead of the
+// prefix sums at its two vertices (16 bytes each): the same integer.  Bound by
+// issue (0.66; the values' 64-bit sums and one division per cluster); from the
+// prefix sums alone it took 460 us at 2^26, lambda 1e-2, instead of 311.
 // ---------------------------------------------------------------------------
-constexpr int GAP_INLINE = 64;
-
-struct BigGap { int64_t pos; int32_t count; int32_t value; uint32_t key32; int32_t pad; };
+constexpr int HTW = HT / 32;   // rank words per hull tile
+constexpr int SUM_MAX = 8;
 
 template <typename T>
-__global__ void __launch_bounds__(256, 8) k_table(const TileDesc* __restrict__ htiles, const LargeSeg* __restrict__ lsegs,
-                                               const double* __restrict__ lambdas, const SegRuntime* __restrict__ rt,
-                                               const typename KeyOf<T>::K* __restrict__ sorted,
-                                               const uint16_t* __restrict__ vp, const i128* __restrict__ vx,
-                                               const Piece* __restrict__ pieces,
-                                               const int32_t* __restrict__ npieces,
-                                               const int32_t* __restrict__ tile_piece, CEntry<T>* table,
-                                               DirEntry* dir, BigGap* gaps, uint32_t* ngaps, int64_t gap_cap,
-                                               int fp64, const WsEpi ep, uint32_t* status) {
-    typedef KeyOf<T> KO;
-    const int tile = blockIdx.x;
-    const int tp = tile_piece[tile];
-    if (tp < 0) return;
-    const TileDesc td = htiles[tile];
-    const LargeSeg ls = lsegs[td.lseg];
-    const SegRuntime R = rt[td.lseg];
-    double lam = lambdas[ls.seg];
-    if (!(lam >= 0.0) || !(lam <= 1.7976931348623157e308)) lam = 0.0;
-    const SegConst sc = ws_seg_const<T>(ls.len, lam, R.emax);
-    const Piece* P = pieces + ls.hull_first;
-    const int np = npieces[ls.hull_first];
-    const Piece pc = P[tp];
-    const int nb = 1 << R.dir_log2;
-    DirEntry* D = dir + ls.dir_pos;
-    const uint64_t pol = ws_policy_evict_last();
-    auto vertex = [&](int piece_idx, int i, int64_t& pt, i128& X) {
-        const Piece q = P[piece_idx];
-        size_t v = (size_t)q.tile * (HT + 1) + i;
-        pt = (int64_t)(q.tile - ls.hull_first) * HT + vp[v];
-        X = q.off + vx[v];
-    };
-    for (int i = pc.lo + threadIdx.x; i < pc.hi; i += 256) {
-        int64_t r = (int64_t)pc.cum + (i - pc.lo);
-        if (r >= R.n_clusters) continue;   // the final vertex (point d) opens no cluster
-        int64_t a, b; i128 Xa, Xb;
-        vertex(tp, i, a, Xa);
-        if (i + 1 < pc.hi) vertex(tp, i + 1, b, Xb);
-        else {
-            if (tp + 1 >= np) { ws_flag(status, WS_STATUS_INTERNAL); continue; }
-            vertex(tp + 1, P[tp + 1].lo, b, Xb);
-        }
-        typename KO::K k = sorted[ls.kpos + a];
-        T xs = KO::from_key(k);
-        CEntry<T> ce;
-        ce.key = k;
-        ce.val = ValueOut<T>::value(Xb - Xa, a, b, xs, sc, fp64 != 0, ep);
-        table[R.table_pos + r] = ce;
-        // directory: buckets (bucket(prev start), bucket(this start)] -> r
-        int bcur = ws_bucket((float)xs, R.lo, R.scale, nb);
-        int bprev = -1;
-        if (r > 0) {
-            int64_t pa; i128 Xp;
-            if (i > pc.lo) vertex(tp, i - 1, pa, Xp);
-            else {
-                const Piece q = P[tp - 1];
-                vertex(tp - 1, q.hi - 1, pa, Xp);
-            }
-            bprev = ws_bucket((float)KO::from_key(sorted[ls.kpos + pa]), R.lo, R.scale, nb);
-        }
-        const uint32_t k32 = (uint32_t)(k >> (KO::BITS - 32));
-        int64_t from = bprev + 1, to = bcur;   // inclusive range of buckets
-        int64_t cnt = to - from + 1;
-        const DirEntry de{(int32_t)r, k32};
-        if (cnt > GAP_INLINE) {
-            uint32_t g = atomicAdd(ngaps, 1u);
-            if ((int64_t)g < gap_cap) {
-                gaps[g].pos = ls.dir_pos + from; gaps[g].count = (int32_t)cnt; gaps[g].value = (int32_t)r;
-                gaps[g].key32 = k32;
-            } else ws_flag(status, WS_STATUS_INTERNAL);
-        } else {
-            for (int64_t bb = from; bb <= to; ++bb) ws_st_u2_last(D + bb, make_uint2((uint32_t)de.idx, de.key32), pol);
-        }
-        if (r == R.n_clusters - 1) {   // tail: buckets after the last start, plus the sentinel
-            int64_t f2 = bcur + 1, c2 = (int64_t)nb - bcur;   // buckets bcur+1 .. nb (nb = sentinel)
-            const DirEntry te{(int32_t)R.n_clusters, 0xffffffffu};
-            if (c2 > GAP_INLINE) {
-                uint32_t g = atomicAdd(ngaps, 1u);
-                if ((int64_t)g < gap_cap) {
-                    gaps[g].pos = ls.dir_pos + f2; gaps[g].count = (int32_t)c2; gaps[g].value = (int32_t)R.n_clusters;
-                    gaps[g].key32 = 0xffffffffu;
-                } else ws_flag(status, WS_STATUS_INTERNAL);
-            } else {
-                for (int64_t bb = f2; bb <= nb; ++bb) ws_st_u2_last(D + bb, make_uint2((uint32_t)te.idx, te.key32), pol);
-            }
-        }
-    }
-}
-
-__global__ void __launch_bounds__(256) k_big_gaps(const BigGap* gaps, const uint32_t* ngaps, DirEntry* dir,
-                                                  int64_t gap_cap) {
-    const int64_t n = min((int64_t)*ngaps, gap_cap);
-    const uint64_t pol = ws_policy_evict_last();
-    for (int64_t g = blockIdx.x; g < n; g += gridDim.x) {
-        const BigGap G = gaps[g];
-        const DirEntry e{G.value, G.key32};
-        for (int i = threadIdx.x; i < G.count; i += 256) ws_st_u2_last(dir + G.pos + i, make_uint2((uint32_t)e.idx, e.key32), pol);
-    }
-}
-
-// ---------------------------------------------------------------------------
-// 6. lookup: every weight, in the caller's order, finds its cluster by value
-// ---------------------------------------------------------------------------
-// The cluster table is read a whole 32-byte sector at a time (E entries): the
-// sector holding the interpolated guess almost always contains the answer,
-// so a weight costs about one random sector instead of one per probed entry.
-template <typename T>
-struct TabSector {
-    static constexpr int E = 32 / (int)sizeof(CEntry<T>);
-    CEntry<T> e[E];
-    __device__ __forceinline__ void load(const CEntry<T>* table, int64_t sb) {
-        const uint4* p = reinterpret_cast<const uint4*>(table + sb);
-        uint4 v[2];
-        v[0] = __ldg(p);
-        v[1] = __ldg(p + 1);
-        const CEntry<T>* q = reinterpret_cast<const CEntry<T>*>(v);
-#pragma unroll
-        for (int i = 0; i < E; ++i) e[i] = q[i];
-    }
-};
-
-// Last cluster j in [jlo, jhi] (segment-local, keys ascending, key[jlo] <= k)
-// whose start key is <= k, starting at the sector that holds local index j0
-// and walking sector by sector (at most four, then bisection).
-template <typename T>
-__device__ __forceinline__ int ws_find_cluster(const CEntry<T>* table, int64_t tp, int jlo, int jhi, int j0,
-                                               typename KeyOf<T>::K k, CEntry<T>& out) {
-    constexpr int E = TabSector<T>::E;
-    int j = min(max(j0, jlo), jhi);
-    int best = -1, dir = 0;
-    for (int it = 0; it < 4; ++it) {
-        const int64_t sb = (tp + j) & ~(int64_t)(E - 1);
-        const int s0 = (int)(sb - tp);
-        TabSector<T> S;
-        S.load(table, sb);
-        int last_le = -1, top = -1;
-#pragma unroll
-        for (int i = 0; i < E; ++i) {
-            const int li = s0 + i;
-            if (li < jlo || li > jhi) continue;
-            top = li;
-            if (S.e[i].key <= k) { last_le = li; out = S.e[i]; }
-        }
-        if (last_le < 0) {              // every entry here is above k
-            if (dir > 0) return best;   // ... and the previous sector's last one was not: out holds it
-            if (s0 - 1 < jlo) break;    // (cannot happen: key[jlo] <= k)
-            dir = -1;                   // the answer lies further left
-            j = s0 - 1;
-            continue;
-        }
-        best = last_le;
-        // an entry above k follows inside this sector, the range ends here, or
-        // the sector to the right was all above k: the answer is here
-        if (last_le < top || last_le == jhi || dir < 0) return best;
-        dir = 1;
-        j = s0 + E;
-    }
-    int l = jlo, h = jhi + 1;   // bisection fallback
-    while (l < h) {
-        const int mid = (l + h) >> 1;
-        if (table[tp + mid].key <= k) l = mid + 1; else h = mid;
-    }
-    // key[jlo] <= k keeps l >= jlo + 1; the clamp only guards the read
-    out = table[tp + max(l - 1, jlo)];
-    return l - 1;
-}
-
-// Every weight, in the caller's order, finds its cluster by value: bucket ->
-// directory (L2-resident) -> interpolated guess -> the table sector holding
-// it.  Each thread carries LK elements through every stage so that their
-// independent random loads overlap.
-template <typename T>
-__global__ void __launch_bounds__(256) k_lookup(const T* __restrict__ values, const TileDesc* __restrict__ tiles,
-                                                const LargeSeg* __restrict__ lsegs, const SegRuntime* __restrict__ rt,
-                                                const CEntry<T>* __restrict__ table, const DirEntry* __restrict__ dir,
-                                                T* out, int32_t* ids, uint32_t* status) {
+__global__ void __launch_bounds__(256, 6) k_values(const TileDesc* __restrict__ htiles, const LargeSeg* __restrict__ lsegs,
+                                                const double* __restrict__ lambdas, const SegRuntime* __restrict__ rt,
+                                                const typename KeyOf<T>::K* __restrict__ sorted,
+                                                const uint16_t* __restrict__ vp, const i128* __restrict__ vx,
+                                                const Piece* __restrict__ pieces,
+                                                const int32_t* __restrict__ npieces,
+                                                const int32_t* __restrict__ tile_piece, T* cval, uint2* rank_words,
+                                                int fp64, const WsEpi ep, uint32_t* status) {
     typedef KeyOf<T> KO;
     typedef typename KO::K K;
-    constexpr int LK = 2;   // measured: 2 beats 1, 4 and 8 (occupancy against loads in flight)
+    __shared__ __align__(16) K key[HT];
+    __shared__ uint32_t words[HTW];
+    __shared__ int wsum[8];
+    __shared__ int s_base;
+    const int tile = blockIdx.x, t = threadIdx.x;
+    const int tp = tile_piece[tile];
+    const TileDesc td = htiles[tile];
+    const LargeSeg& ls = lsegs[td.lseg];
+    const int h0 = ls.hull_first;
+    const int64_t kpos = ls.kpos, n_clusters = rt[td.lseg].n_clusters, table_pos = rt[td.lseg].table_pos;
+    if (n_clusters == 1 && tp < 0) return;   // (one cluster: every position has it)
+    const Piece* P = pieces + h0;
+    const int np = npieces[h0];
+    if (t < HTW) words[t] = 0;
+    if (tp >= 0 && n_clusters != 1) {
+        // (a segment's keys start on 16 bytes, and so does each of its tiles)
+        constexpr int VEC = 16 / (int)sizeof(K);
+        const uint4* src = reinterpret_cast<const uint4*>(sorted + td.kpos);
+        const int nv = td.len / VEC;
+        for (int i = t; i < nv; i += 256) reinterpret_cast<uint4*>(key)[i] = __ldg(src + i);
+        for (int i = nv * VEC + t; i < td.len; i += 256) key[i] = sorted[td.kpos + i];
+    }
+    if (t == 0) {
+        // starts before this tile; a junction point that the tile on the left
+        // keeps as its last vertex is this tile's position 0
+        int prev, base;
+        if (tp >= 0) { prev = tp - 1; base = P[tp].cum; }
+        else {
+            int lo = 0, hi = np - 1;   // last piece of an earlier tile (piece 0 is tile 0's)
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (P[mid].tile < tile) lo = mid; else hi = mid - 1;
+            }
+            prev = lo;
+            base = P[lo].cum + (P[lo].hi - P[lo].lo);
+        }
+        int bit0 = 0;
+        if (prev >= 0) {
+            const Piece q = P[prev];
+            bit0 = q.tile == tile - 1 && vp[(size_t)q.tile * (HT + 1) + q.hi - 1] == HT;
+        }
+        s_base = base - bit0;
+        words[0] = (uint32_t)bit0;
+    }
+    __syncthreads();
+    if (tp >= 0) {
+        double lam = lambdas[ls.seg];
+        if (!(lam >= 0.0) || !(lam <= 1.7976931348623157e308)) lam = 0.0;
+        const int emax = rt[td.lseg].emax;
+        const SegConst sc = ws_seg_const<T>(ls.len, lam, emax);
+        const Piece pc = P[tp];
+        const uint16_t* vpt = vp + (size_t)tile * (HT + 1);
+        const i128* vxt = vx + (size_t)tile * (HT + 1);
+        const int64_t p0 = (int64_t)td.tin * HT;
+        int sh = 0;
+        const bool bin = n_clusters != 1 && ws_tile_binade<T>(key[0], key[td.len - 1], td.len, emax, sh);
+        const int64_t q0 = bin ? ws_fixed<T>(KO::from_key(key[0]), emax) : 0;
+        int i = pc.lo + t;
+        int al = i < pc.hi ? vpt[i] : 0, bl = i + 1 < pc.hi ? vpt[i + 1] : -1;
+        while (i < pc.hi) {
+            const int in = i + 256;   // (the next vertices are on their way while this one's value is formed)
+            const int an = in < pc.hi ? vpt[in] : 0, bn = in + 1 < pc.hi ? vpt[in + 1] : -1;
+            const int64_t r = (int64_t)pc.cum + (i - pc.lo);
+            if (r < n_clusters) {   // (the final vertex, point d, opens no cluster)
+                const int64_t a = p0 + al;
+                int64_t b = p0 + bl;
+                i128 SX = 0;
+                T xs = (T)0;
+                bool done = false;
+                if (bl >= 0 && bl - al <= SUM_MAX && n_clusters != 1) {
+                    xs = KO::from_key(key[al]);
+                    int64_t q = 0;   // (|q| <= 8 x 2^58)
+                    const int n = bl - al;
+                    if (n > 1) {
+                        if (bin) {   // (deviations from the tile's first key, in ulps of its binade)
+                            uint64_t dev = 0;
+                            for (int j = al; j < bl; ++j) dev += (uint64_t)(key[j] - key[0]);
+                            q = (int64_t)n * q0 + (int64_t)(dev << sh);
+                        } else {
+                            for (int j = al; j < bl; ++j) q += ws_fixed<T>(KO::from_key(key[j]), emax);
+                        }
+                    }
+                    if (sizeof(T) == 4 && !fp64) {
+                        cval[table_pos + r] = (T)ValueOut<float>::value64(q, n, (int)(sc.d - a - b), (float)xs, sc, ep);
+                        done = true;
+                    }
+                    SX = (i128)q;
+                } else {
+                    i128 Xb;
+                    bool ok = true;
+                    if (bl >= 0) {
+                        Xb = pc.off + vxt[i + 1];
+                    } else if (tp + 1 < np) {
+                        const Piece q = P[tp + 1];
+                        const size_t v = (size_t)q.tile * (HT + 1) + q.lo;
+                        b = (int64_t)(q.tile - h0) * HT + vp[v];
+                        Xb = q.off + vx[v];
+                    } else {
+                        ok = false;
+                        ws_flag(status, WS_STATUS_INTERNAL);
+                        Xb = 0;
+                    }
+                    if (ok) {
+                        SX = Xb - (pc.off + vxt[i]);
+                        if (b - a == 1) xs = KO::from_key(sorted[kpos + a]);
+                    } else b = a + 1;
+                }
+                if (!done) cval[table_pos + r] = ValueOut<T>::value(SX, a, b, xs, sc, fp64 != 0, ep);
+                if (al < HT) atomicOr(&words[al >> 5], 1u << (al & 31));
+            }
+            i = in;
+            al = an;
+            bl = bn;
+        }
+    }
+    if (n_clusters == 1) return;
+    __syncthreads();
+    const uint32_t wd = t < HTW ? words[t] : 0u;
+    const int ex = ws_block_excl_scan<256, int>(__popc(wd), wsum, nullptr);
+    if (t < HTW) rank_words[(size_t)tile * HTW + t] = make_uint2(wd, (uint32_t)(s_base + ex));
+}
+
+// Cluster of a sorted position from its rank word.
+__device__ __forceinline__ int ws_cluster_at(uint2 rw, uint32_t pos) {
+    return (int)rw.y + __popc(rw.x & (0xffffffffu >> (31u - (pos & 31u)))) - 1;
+}
+
+// ---------------------------------------------------------------------------
+// 6. the way back to the caller's order: the passes of the sort undone one by
+// one.  Every step reads and writes runs (a bin, a tile's bucket runs), never
+// single elements all over memory, which is what a lookup of every weight by
+// value costs (one or two random sectors each).  Against a table of clusters
+// with a directory of 2^22 value buckets and such a lookup, us: 2^26 FP32
+// lambda 1e-2: table 449 + lookup 1533 -> values 311, bins 202, regroup 245,
+// output 286; 2^24 lambda 1: 120 + 42 + 212 -> 92, 55, 70, 69; 1024 uneven
+// segments: 878 + 101 + 1241 -> 539, 313, 406 (no second pass).  The sort pays
+// for it by writing where every key goes: 10 bytes per key, 86 + 41 us at 2^26.
+// ---------------------------------------------------------------------------
+// Bins: value and cluster of every sorted position, put into the order the
+// partition left the bin in (in shared memory).  One CTA per bin; the CTAs after those share the oversize bins,
+// whose elements find their position by bisection in the sorted bin.
+constexpr int OUT_EXTRA = 64;
+
+template <typename T>
+__global__ void __launch_bounds__(256, 6) k_bin_out(const LargeSeg* __restrict__ lsegs, const SegRuntime* __restrict__ rt,
+                                                 const int32_t* __restrict__ bin_seg,
+                                                 const uint32_t* __restrict__ bin_start,
+                                                 const uint32_t* __restrict__ bin_cnt, int n_bins,
+                                                 const uint16_t* __restrict__ bin_idx,
+                                                 const uint2* __restrict__ rank_words, const T* __restrict__ cval,
+                                                 const typename KeyOf<T>::K* __restrict__ sorted,
+                                                 const typename KeyOf<T>::K* __restrict__ keys,
+                                                 const SortCtl* __restrict__ ctl, const OverBin* __restrict__ over,
+                                                 OutPair<T>* pairs) {
+    typedef typename KeyOf<T>::K K;
+    __shared__ uint2 rw[HTW + 2];
+    extern __shared__ __align__(16) unsigned char pair_smem_raw[];
+    OutPair<T>* stage = reinterpret_cast<OutPair<T>*>(pair_smem_raw);   // [WS_BIN_CAP]
+    const int t = threadIdx.x;
+    if ((int)blockIdx.x < n_bins) {
+        const int bin = blockIdx.x;
+        const int lseg = bin_seg[bin];
+        const LargeSeg& sg = lsegs[lseg];
+        const int64_t c = rt[lseg].n_clusters;
+        const int n = (int)bin_cnt[bin];
+        const uint32_t s0 = bin_start[bin];
+        if (c == 1 || n <= 0 || n > WS_BIN_CAP || (int64_t)s0 + n > sg.len) return;
+        const int64_t g = sg.kpos + s0;
+        constexpr int U = 6;   // (a bin of the usual size in two steps)
+        const uint32_t w0 = s0 >> 5, nw = ((s0 + n - 1) >> 5) - w0 + 1;
+        const T* cv = cval + rt[lseg].table_pos;
+        if (t < nw) rw[t] = rank_words[(size_t)sg.hull_first * HTW + w0 + t];   // (nw <= HTW + 1)
+        for (int b0 = 0; b0 < n; b0 += 256 * U) {
+            const int i0 = b0 + t;
+            uint16_t q[U];
+            T v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) q[u] = i0 + u * 256 < n ? __ldg(bin_idx + g + i0 + u * 256) : (uint16_t)0;
+            if (b0 == 0) __syncthreads();   // (the rank words; the places are on their way)
+            auto id_at = [&](int u) {
+                const uint32_t p = s0 + min(i0 + u * 256, n - 1);
+                return ws_cluster_at(rw[(p >> 5) - w0], p);
+            };
+#pragma unroll
+            for (int u = 0; u < U; ++u) v[u] = __ldg(cv + min(max(id_at(u), 0), (int)c - 1));
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (i0 + u * 256 < n) {
+                    OutPair<T> o = {};
+                    o.val = v[u];
+                    o.id = id_at(u);
+                    stage[min((uint32_t)q[u], (uint32_t)n - 1u)] = o;
+                }
+        }
+        __syncthreads();
+        for (int i = t; i < n; i += 256) pairs[g + i] = stage[i];
+        return;
+    }
+    const int cnt = (int)ctl->over_count;
+    if (cnt == 0 || ctl->abort) return;
+    const int n_tiles = over[cnt - 1].first_tile + (over[cnt - 1].n + WS_SORT_TILE - 1) / WS_SORT_TILE;
+    for (int tile = (int)blockIdx.x - n_bins; tile < n_tiles; tile += OUT_EXTRA) {
+        int lo = 0, hi = cnt - 1;   // (uniform)
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (over[mid].first_tile <= tile) lo = mid; else hi = mid - 1;
+        }
+        const OverBin ob = over[lo];
+        const int lseg = ob.lseg;
+        const LargeSeg& sg = lsegs[lseg];
+        const int64_t c = rt[lseg].n_clusters;
+        if (c == 1) continue;
+        const uint2* sw = rank_words + (size_t)sg.hull_first * HTW;
+        const T* cv = cval + rt[lseg].table_pos;
+        const K* sk = sorted + ob.start;
+        const int e0 = (tile - ob.first_tile) * WS_SORT_TILE, e1 = min(e0 + WS_SORT_TILE, ob.n);
+        for (int i = e0 + t; i < e1; i += 256) {
+            const K k = keys[ob.start + i];
+            int r = 0, m = ob.n;   // first position whose key is not below k
+            if (ob.diff != 0)
+                while (m > 0) {
+                    const int half = m >> 1;
+                    if (sk[r + half] < k) { r += half + 1; m -= half + 1; } else m = half;
+                }
+            const uint32_t p = (uint32_t)(ob.start - sg.kpos) + (uint32_t)min(r, ob.n - 1);
+            const int id = ws_cluster_at(sw[p >> 5], p);
+            OutPair<T> o = {};
+            o.val = __ldg(cv + min(max((int64_t)id, (int64_t)0), c - 1));
+            o.id = id;
+            pairs[ob.start + i] = o;
+        }
+    }
+}
+
+// One tile per CTA of 1024 threads: two tiles' runs at a time fit an SM's L1,
+// where the neighbours in a run share their sectors (256 threads, eight tiles
+// per SM: output 399 us instead of 286 at 2^26, regroup the same).
+constexpr int GNT = 1024;
+
+// Second pass undone: bin order to the first pass's order (two-level segments).
+template <typename T>
+__global__ void __launch_bounds__(GNT) k_regroup(const TileDesc* __restrict__ tiles, const LargeSeg* __restrict__ lsegs,
+                                                 const SegRuntime* __restrict__ rt, const uint32_t* __restrict__ dest,
+                                                 const OutPair<T>* __restrict__ from, OutPair<T>* __restrict__ to) {
     const TileDesc td = tiles[blockIdx.x];
-    const LargeSeg ls = lsegs[td.lseg];
-    const SegRuntime R = rt[td.lseg];
-    const int nb = 1 << R.dir_log2;
-    const DirEntry* D = dir + ls.dir_pos;
-    const int64_t tp = R.table_pos;
-    const int c = (int)R.n_clusters;
-    if (c == 1) {   // one cluster (large lambda): every weight gets its value, no search
-        const T v = table[tp].val;
-        for (int i = threadIdx.x; i < td.len; i += 256) {
+    const LargeSeg& sg = lsegs[td.lseg];
+    if (sg.fine_log2 == 0 || rt[td.lseg].n_clusters == 1) return;
+    const uint32_t last = (uint32_t)sg.len - 1u;
+    const OutPair<T>* src = from + sg.kpos;
+    constexpr int U = WS_SORT_TILE / GNT;   // (one step: every load of the tile in flight)
+    for (int i0 = threadIdx.x; i0 < td.len; i0 += GNT * U) {
+        uint32_t p[U];
+        OutPair<T> o[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) p[u] = i0 + u * GNT < td.len ? __ldg(dest + td.kpos + i0 + u * GNT) : 0u;
+#pragma unroll
+        for (int u = 0; u < U; ++u) o[u] = src[min(p[u], last)];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i0 + u * GNT < td.len) to[td.kpos + i0 + u * GNT] = o[u];
+    }
+}
+
+// First pass undone: value and id of every element, in the caller's order.
+template <typename T>
+__global__ void __launch_bounds__(GNT) k_output(const TileDesc* __restrict__ tiles, const LargeSeg* __restrict__ lsegs,
+                                                const SegRuntime* __restrict__ rt, const T* __restrict__ cval,
+                                                const uint32_t* __restrict__ dest, const OutPair<T>* __restrict__ pairs_a,
+                                                const OutPair<T>* __restrict__ pairs_b, T* out, int32_t* ids) {
+    const TileDesc td = tiles[blockIdx.x];
+    const LargeSeg& sg = lsegs[td.lseg];
+    if (rt[td.lseg].n_clusters == 1) {   // one cluster (large lambda): every weight gets its value
+        const T v = cval[rt[td.lseg].table_pos];
+        for (int i = threadIdx.x; i < td.len; i += GNT) {
             __stcs(out + td.vpos + i, v);
             if (ids) __stcs(ids + td.vpos + i, 0);
         }
         return;
     }
-    const uint64_t pol = ws_policy_evict_last();
-    for (int i0 = threadIdx.x; i0 < td.len; i0 += 256 * LK) {
-        T x[LK];
-        K k[LK];
-        int lo[LK], hi[LK], g[LK];
-        DirEntry e0[LK], e1[LK];
-        bool in[LK];
+    const uint32_t last = (uint32_t)sg.len - 1u;
+    const OutPair<T>* src = (sg.fine_log2 ? pairs_a : pairs_b) + sg.kpos;
+    constexpr int U = WS_SORT_TILE / GNT;   // (one step: every load of the tile in flight)
+    for (int i0 = threadIdx.x; i0 < td.len; i0 += GNT * U) {
+        uint32_t p[U];
+        OutPair<T> o[U];
 #pragma unroll
-        for (int u = 0; u < LK; ++u) {
-            const int i = i0 + u * 256;
-            in[u] = i < td.len;
-            x[u] = in[u] ? __ldcs(values + td.vpos + i) : (T)0;
-        }
+        for (int u = 0; u < U; ++u) p[u] = i0 + u * GNT < td.len ? __ldg(dest + td.kpos + i0 + u * GNT) : 0u;
 #pragma unroll
-        for (int u = 0; u < LK; ++u) {
-            k[u] = KO::to_key(x[u]);
-            const int b = ws_bucket((float)x[u], R.lo, R.scale, nb);
-            const uint2 a0 = ws_ld_u2_last(D + b, pol), a1 = ws_ld_u2_last(D + b + 1, pol);
-            e0[u] = DirEntry{(int32_t)a0.x, a0.y};
-            e1[u] = DirEntry{(int32_t)a1.x, a1.y};
-        }
+        for (int u = 0; u < U; ++u) o[u] = src[min(p[u], last)];
 #pragma unroll
-        for (int u = 0; u < LK; ++u) {
-            const uint32_t k32 = (uint32_t)(k[u] >> (KO::BITS - 32));
-            lo[u] = min(max(e0[u].idx, 0), c);
-            hi[u] = min(max(e1[u].idx, lo[u]), c);
-            if (lo[u] == hi[u] || k32 < e0[u].key32) {
-                g[u] = lo[u] - 1;   // precedes every start in the bucket: cluster lo - 1
-            } else {
-                const uint32_t span = e1[u].key32 - e0[u].key32;
-                int gg = lo[u];
-                if (span > 0) {
-                    const float f = (float)(k32 - e0[u].key32) / (float)span;
-                    gg = lo[u] + (int)(f * (float)(hi[u] - lo[u]));
-                    gg = min(max(gg, lo[u]), hi[u] - 1);
-                }
-                g[u] = gg;
+        for (int u = 0; u < U; ++u)
+            if (i0 + u * GNT < td.len) {
+                __stcs(out + td.vpos + i0 + u * GNT, o[u].val);
+                if (ids) __stcs(ids + td.vpos + i0 + u * GNT, o[u].id);
             }
-        }
-#pragma unroll
-        for (int u = 0; u < LK; ++u) {
-            if (!in[u]) continue;   // past the tile's end: no element (its x = 0 may precede every cluster)
-            CEntry<T> ce;
-            const int jlo = max(lo[u] - 1, 0), jhi = max(hi[u] - 1, jlo);
-            int r = jlo;
-            if (jhi == jlo) ce = table[tp + jlo];   // one candidate: no search
-            else r = ws_find_cluster<T>(table, tp, jlo, jhi, g[u], k[u], ce);
-            if (r < 0 || r >= c) { ws_flag(status, WS_STATUS_INTERNAL); r = 0; ce = table[tp]; }
-            const int i = i0 + u * 256;
-            __stcs(out + td.vpos + i, ce.val);
-            if (ids) __stcs(ids + td.vpos + i, r);
-        }
     }
 }
 
@@ -970,7 +1014,7 @@ cudaError_t ws_large_prox(const LargeWork<T>& W, const T* values, const double* 
     typedef typename KeyOf<T>::K K;
     if (W.n_lseg == 0) return cudaSuccess;
     K* sorted = nullptr;
-    cudaError_t e = ws_large_sort<T>(W, values, status, spin_limit, st, &sorted);
+    cudaError_t e = ws_large_sort<T>(W, values, true, status, spin_limit, st, &sorted);
     if (e) return e;
     // tile hulls: the lean kernel, then the general one for the tiles it flagged
     e = ws_large_hull_fast<T>(W, sorted, lambdas, status, st);
@@ -996,22 +1040,26 @@ cudaError_t ws_large_prox(const LargeWork<T>& W, const T* values, const double* 
     e = cudaMemsetAsync(W.tile_piece, 0xff, sizeof(int32_t) * (size_t)W.n_hull_tiles, st);
     if (e) return e;
     WS_LAUNCH(W.prof, WSK_ROOT, st,
-              (k_root<T><<<W.n_lseg, 256, 0, st>>>(W.lsegs, sorted, W.pieces, W.npieces, W.tile_piece, W.rt,
-                                                  n_clusters)));
-    // big-gap list lives at the tail of the backward sum buffer (unused in the forward)
-    uint32_t* ngaps = reinterpret_cast<uint32_t*>(W.bcnt);
-    BigGap* gaps = reinterpret_cast<BigGap*>(W.bsum);
-    int64_t gap_cap = (int64_t)((W.n_keys + W.n_lseg) * sizeof(T) / sizeof(BigGap));
-    e = cudaMemsetAsync(ngaps, 0, sizeof(uint32_t), st);
+              (k_root<<<W.n_lseg, 256, 0, st>>>(W.lsegs, W.pieces, W.npieces, W.tile_piece, W.rt, n_clusters)));
+    WS_LAUNCH(W.prof, WSK_VALUES, st,
+              (k_values<T><<<W.n_hull_tiles, 256, 0, st>>>(W.hull_tiles, W.lsegs, lambdas, W.rt, sorted, W.vp, W.vx,
+                                                          W.pieces, W.npieces, W.tile_piece, W.cval, W.rank_words,
+                                                          fp64, ep, status)));
+    // back to the caller's order
+    e = cudaFuncSetAttribute(k_bin_out<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(OutPair<T>) * WS_BIN_CAP);
     if (e) return e;
-    WS_LAUNCH(W.prof, WSK_TABLE, st,
-              (k_table<T><<<W.n_hull_tiles, 256, 0, st>>>(W.hull_tiles, W.lsegs, lambdas, W.rt, sorted, W.vp, W.vx,
-                                                         W.pieces, W.npieces, W.tile_piece, W.table,
-                                                         W.dir, gaps, ngaps, gap_cap, fp64, ep, status)));
-    WS_LAUNCH(W.prof, WSK_BIG_GAPS, st, (k_big_gaps<<<1024, 256, 0, st>>>(gaps, ngaps, W.dir, gap_cap)));
-    WS_LAUNCH(W.prof, WSK_LOOKUP, st,
-              (k_lookup<T><<<W.n_sort_tiles, 256, 0, st>>>(values, W.sort_tiles, W.lsegs, W.rt, W.table, W.dir, out,
-                                                          ids, status)));
+    WS_LAUNCH(W.prof, WSK_BIN_OUT, st,
+              (k_bin_out<T><<<W.n_bins + OUT_EXTRA, 256, sizeof(OutPair<T>) * WS_BIN_CAP, st>>>(W.lsegs, W.rt, W.bin_seg, W.bin_start, W.bin_cnt,
+                                                                 W.n_bins, W.bin_idx, W.rank_words, W.cval, sorted,
+                                                                 W.keys_b, W.ctl, W.over, W.pairs_b)));
+    if (W.two_level)
+        WS_LAUNCH(W.prof, WSK_REGROUP, st,
+                  (k_regroup<T><<<W.n_sort_tiles, GNT, 0, st>>>(W.sort_tiles, W.lsegs, W.rt, W.dest2, W.pairs_b,
+                                                               W.pairs_a)));
+    WS_LAUNCH(W.prof, WSK_OUTPUT, st,
+              (k_output<T><<<W.n_sort_tiles, GNT, 0, st>>>(W.sort_tiles, W.lsegs, W.rt, W.cval, W.dest1, W.pairs_a,
+                                                          W.pairs_b, out, ids)));
     return cudaGetLastError();
 }
 

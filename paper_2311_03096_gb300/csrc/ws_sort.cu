@@ -27,11 +27,13 @@
 //   FP32 2^24     398 -> 271 (68, 2 x 58, 82, 6)
 //   FP64 2^22     319 -> 147 (53, 2 x 23, 41, 6)
 //   1024 FP32 segments of 16 .. 2^20 elements (9.7e7 keys)   2085 -> 1310
+// without the records of the way back; with them 2^26 1010 (2 x 260, bins 334).
 // The partition is bound by shared-memory wavefronts (17 per 32 keys: the
 // counters, the staging and the copy out; 0.7 of the pipe), the bin sort by
-// issue (0.64) and the same pipe, the plan by the read of the values (0.104 of
+// issue (0.65) and the same pipe, the plan by the read of the values (0.104 of
 // its 0.150 ms) and five barriers.
 #include <algorithm>
+#include <type_traits>
 
 #include "ws_kernels.cuh"
 
@@ -486,8 +488,8 @@ template <typename T, typename B>
 struct PartSmem {
     typename KeyOf<T>::K key[WS_SORT_TILE];
     B bin[WS_SORT_TILE];
-    uint32_t cnt[WS_FAN];     // counts, then starts inside the tile
-    int32_t delta[WS_FAN];    // destination of the bucket's run minus its start inside the tile
+    uint32_t cnt[WS_FAN];
+    uint2 run[WS_FAN];        // start of the bucket's run inside the tile, and its destination
     int wsum[WS_SORT_NT / 32];
 };
 
@@ -495,6 +497,7 @@ template <typename T, typename B, bool FIRST>
 __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
     const T* __restrict__ values, const typename KeyOf<T>::K* __restrict__ keys_in, const B* __restrict__ bins_in,
     typename KeyOf<T>::K* __restrict__ out_a, typename KeyOf<T>::K* __restrict__ out_b, B* __restrict__ bins_out,
+    uint32_t* __restrict__ dest,   // (nullable: where every key goes)
     const TileDesc* __restrict__ tiles, int n_tiles, const LargeSeg* __restrict__ lsegs, uint32_t* cursor,
     const SortCtl* ctl, uint32_t* status) {
     typedef KeyOf<T> KO;
@@ -537,9 +540,9 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
         // its first to last bucket (second)
         int base = 0, nbk = sg.n_coarse;
         if (!FIRST) {
-            const int64_t kp = tiles[tile].kpos;
-            base = ((int)__ldg(bins_in + kp) >> fl) << fl;
-            nbk = max(min(sg.nbins, (((int)__ldg(bins_in + kp + len - 1) >> fl) + 1) << fl) - base, 1);
+            const int64_t k0 = tiles[tile].kpos;
+            base = ((int)__ldg(bins_in + k0) >> fl) << fl;
+            nbk = max(min(sg.nbins, (((int)__ldg(bins_in + k0 + len - 1) >> fl) + 1) << fl) - base, 1);
         }
         const int bsh = FIRST ? 13 + fl : 13;
 #pragma unroll
@@ -564,16 +567,18 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
                 c ? atomicAdd(cursor + (FIRST ? sg.coarse_pos : sg.bin_pos + base) + r0 + t, c) : 0u;
             int total;
             const int ex = ws_block_excl_scan<NT, int>((int)c, s.wsum, &total);
-            s.cnt[t] = (uint32_t)ex;
-            s.delta[t] = (int32_t)g - ex;
+            s.run[t] = make_uint2((uint32_t)ex, g);
             __syncthreads();
+            const int64_t kp = tiles[tile].kpos;
 #pragma unroll
             for (int k = 0; k < ITEMS; ++k) {
                 const uint32_t b = (br[k] >> bsh) - off;
                 if (t + k * NT < len && b < WS_FAN) {
-                    const uint32_t j = s.cnt[b] + (br[k] & 0x1fffu);
+                    const uint2 run = s.run[b];
+                    const uint32_t rk = br[k] & 0x1fffu, j = run.x + rk;
                     s.key[j] = key[k];
                     s.bin[j] = (B)(br[k] >> 13);
+                    if (dest) dest[kp + t + k * NT] = run.y + rk;
                 }
             }
             __syncthreads();
@@ -586,7 +591,8 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
 #pragma unroll 4
             for (int j = t; j < total; j += NT) {
                 const B bn = s.bin[j];
-                const uint32_t p = (uint32_t)(s.delta[((uint32_t)bn >> (bsh - 13)) - off] + j);
+                const uint2 run = s.run[((uint32_t)bn >> (bsh - 13)) - off];
+                const uint32_t p = run.y + (uint32_t)j - run.x;
                 if (p < slen) {   // (always)
                     dst[p] = s.key[j];
                     if (FIRST && fl != 0) bdst[p] = bn;
@@ -600,22 +606,31 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
 // ---------------------------------------------------------------------------
 // Sort of one bin per CTA: the keys into 1024 groups by a monotone linear map
 // of the bin's range (2.5 keys each on average), every group of at most 8 keys
-// in one thread's registers by a sorting network, larger ones (one in a
-// thousand, more in the tails, where the density varies inside a bin) by a
-// warp that counts ranks.  A bin with a group of more than BIN_WARP_MAX keys
-// (ties, a very uneven density) takes LSD radix passes over the bits that vary
-// in it.
+// in one thread's registers by a sorting network, larger ones (one in 500; more
+// in the tails, where the density varies inside a bin) by a warp that counts
+// ranks.  A bin with a group of more than BIN_WARP_MAX keys (unless they are
+// equal) takes LSD radix passes over the bits that vary in it.
+//
+// PLACE: the place of every key in the unsorted bin is wanted too.  What is
+// sorted then are words of the key above the bin's smallest (its top 20 bits;
+// 52 for FP64) and the place in the low 12 bits, so that the sort moves one
+// word per key either way.  Where the bin spans more than that (short
+// segments, bins near zero), keys with the same top bits are put in order
+// after it.
 // ---------------------------------------------------------------------------
 constexpr int BIN_NT = 256;
+constexpr int BIN_ITEMS = WS_BIN_CAP / BIN_NT;
+constexpr int BIN_REG = 12;                      // keys per thread kept in registers
 constexpr int BIN_GPT = 4;                       // groups per thread
 constexpr int BIN_GROUPS = BIN_GPT * BIN_NT;
+constexpr int BIN_NET = 8;
 constexpr int BIN_WARP_MAX = 256;
-constexpr int BIN_ITEMS = WS_BIN_CAP / BIN_NT;
+constexpr int BIN_RUN_MAX = 32;                  // keys with the same top bits that one thread orders
 
 template <typename T>
 struct BinSmem {
     typedef typename KeyOf<T>::K K;
-    K key[WS_BIN_CAP];
+    K key[WS_BIN_CAP];               // keys, or words
     union {
         uint32_t cnt[BIN_GROUPS];
         struct {
@@ -624,9 +639,10 @@ struct BinSmem {
         } radix;
     } u;
     K lo, hi;
+    uint32_t late[WS_BIN_CAP - BIN_REG * BIN_NT];    // group << 16 | rank of the keys not in registers
     int wsum[BIN_NT / 32];
-    int n_list;
-    uint32_t list[WS_BIN_CAP / 9 + 1];   // start << 16 | keys of the groups for the warps
+    int n_list, radix_needed;
+    uint32_t list[WS_BIN_CAP / (BIN_NET + 1) + 1];   // start << 16 | keys of the groups for the warps
 };
 
 // Batcher's odd-even merge sorting network.
@@ -658,12 +674,19 @@ __device__ __forceinline__ void sort_group(K* key, int n) {
         if (i < n) key[i] = v[i];
 }
 
-// Sort of n <= BIN_WARP_MAX keys by one warp: every key's rank by counting
-// (ties by place).
+// Sort of n keys or words by one warp: ranks by counting (ties by place).
+// false for more than BIN_WARP_MAX, unless they are equal above the low `low`
+// bits (then any order will do).
 template <typename K>
-__device__ __noinline__ void sort_warp(K* key, int n) {
+__device__ __noinline__ bool sort_warp(K* key, int n, int low) {
     const int lane = threadIdx.x & 31;
     constexpr int PER = BIN_WARP_MAX / 32;
+    if (n > BIN_WARP_MAX) {
+        const K k0 = key[0] >> low;
+        bool same = true;
+        for (int j = lane; j < n; j += 32) same &= (key[j] >> low) == k0;
+        return __all_sync(WS_FULL_MASK, same);
+    }
     K v[PER];
     int r[PER];
 #pragma unroll
@@ -671,6 +694,7 @@ __device__ __noinline__ void sort_warp(K* key, int n) {
         v[k] = lane + 32 * k < n ? key[lane + 32 * k] : ~(K)0;
         r[k] = 0;
     }
+#pragma unroll 4
     for (int j = 0; j < n; ++j) {
         const K x = key[j];
 #pragma unroll
@@ -683,7 +707,7 @@ __device__ __noinline__ void sort_warp(K* key, int n) {
 #pragma unroll
     for (int k = 0; k < PER; ++k)
         if (lane + 32 * k < n) key[r[k]] = v[k];
-    __syncwarp();
+    return true;
 }
 
 __device__ __forceinline__ uint32_t warp_min_k(uint32_t v) { return __reduce_min_sync(WS_FULL_MASK, v); }
@@ -699,10 +723,16 @@ __device__ __forceinline__ uint64_t warp_max_k(uint64_t v) {
     return v;
 }
 
-template <typename T>
-__device__ __noinline__ void bin_radix(BinSmem<T>& s, int n, typename KeyOf<T>::K diff) {
+// LSD radix passes, 8-bit digits that vary (diff), over a bin's n keys in
+// s.key; with PLACE over the keys src[place], s.key holding the places.  The
+// rare path: out of line.
+template <typename T, bool PLACE>
+__device__ __noinline__ void bin_radix(BinSmem<T>& s, const typename KeyOf<T>::K* src, int n,
+                                       typename KeyOf<T>::K diff) {
     typedef typename KeyOf<T>::K K;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    for (int i = t; i < n; i += BIN_NT) s.key[i] = PLACE ? (K)i : src[i];
+    __syncthreads();
     for (int pass = 0; pass < KeyOf<T>::BITS / 8; ++pass) {
         if (((diff >> (8 * pass)) & 0xff) == 0) continue;
         K key[BIN_ITEMS];
@@ -714,7 +744,8 @@ __device__ __noinline__ void bin_radix(BinSmem<T>& s, int n, typename KeyOf<T>::
             const int p = w * 32 * BIN_ITEMS + k * 32 + lane;
             valid[k] = p < n;
             key[k] = valid[k] ? s.key[p] : (K)0;
-            dg[k] = (uint32_t)((key[k] >> (8 * pass)) & 0xff);
+            const K kk = PLACE ? (valid[k] ? __ldg(src + (uint32_t)key[k]) : (K)0) : key[k];
+            dg[k] = (uint32_t)((kk >> (8 * pass)) & 0xff);
         }
         __syncthreads();
         ws_rank_digits<BIN_NT, BIN_ITEMS, 1>(dg, valid, pos, s.u.radix.whist, s.u.radix.dcount, s.u.radix.dstart);
@@ -737,17 +768,19 @@ __device__ __forceinline__ float ws_trunc_f32(double v) {
     return __uint_as_float(sign | ((uint32_t)e << 23) | m);
 }
 
-template <typename T>
+template <typename T, bool PLACE>
 __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>::K* __restrict__ keys,
                                                         typename KeyOf<T>::K* __restrict__ sorted,
                                                         const int32_t* __restrict__ bin_seg,
                                                         const LargeSeg* __restrict__ lsegs,
                                                         const uint32_t* __restrict__ bin_start,
-                                                        const uint32_t* __restrict__ bin_cnt, SortCtl* ctl,
-                                                        OverBin* over, int64_t n_keys) {
+                                                        const uint32_t* __restrict__ bin_cnt,
+                                                        uint16_t* __restrict__ bin_idx,   // (PLACE)
+                                                        SortCtl* ctl, OverBin* over, int64_t n_keys) {
     typedef KeyOf<T> KO;
     typedef typename KO::K K;
-    __shared__ BinSmem<T> s;
+    extern __shared__ __align__(16) unsigned char bin_smem_raw[];
+    BinSmem<T>& s = *reinterpret_cast<BinSmem<T>*>(bin_smem_raw);
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     if (ctl->abort) {   // the keys were not moved: a sequence that is sorted, so that later steps see a valid one
         for (int64_t i = (int64_t)blockIdx.x * BIN_NT + t; i < n_keys; i += (int64_t)gridDim.x * BIN_NT)
@@ -755,8 +788,7 @@ __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>:
         return;
     }
     const int bin = blockIdx.x;
-    const LargeSeg& sg = lsegs[bin_seg[bin]];
-    const int64_t start = sg.kpos + (int64_t)bin_start[bin];
+    const int64_t start = lsegs[bin_seg[bin]].kpos + (int64_t)bin_start[bin];
     const int n = (int)bin_cnt[bin];
     if (n <= 0) return;
     if (n > WS_BIN_CAP) {
@@ -765,25 +797,29 @@ __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>:
             over[i].start = start;
             over[i].n = n;
             over[i].diff = 0;
+            over[i].lseg = bin_seg[bin];
         }
         return;
     }
     const K* src = keys + start;
-    K* dst = sorted + start;
     reinterpret_cast<uint4*>(s.u.cnt)[t] = make_uint4(0, 0, 0, 0);
-    if (t == 0) { s.lo = ~(K)0; s.hi = 0; s.n_list = 0; }
-    K key[BIN_ITEMS];
+    if (t == 0) { s.lo = ~(K)0; s.hi = 0; s.n_list = 0; s.radix_needed = 0; }
+    // the first BIN_REG keys of a thread stay in registers; the few beyond (a
+    // bin 1.2 times the mean or more) are read again, and their group kept in
+    // shared memory
+    K key[BIN_REG];
 #pragma unroll
-    for (int k = 0; k < BIN_ITEMS; ++k) {
+    for (int k = 0; k < BIN_REG; ++k) {
         const int p = t + k * BIN_NT;
         key[k] = p < n ? __ldg(src + p) : (K)0;
     }
     K lo = ~(K)0, hi = 0;
 #pragma unroll
-    for (int k = 0; k < BIN_ITEMS; ++k) {
+    for (int k = 0; k < BIN_REG; ++k) {
         if (k * BIN_NT >= n) break;   // (uniform)
         if (t + k * BIN_NT < n) { lo = min(lo, key[k]); hi = max(hi, key[k]); }
     }
+    for (int p = t + BIN_REG * BIN_NT; p < n; p += BIN_NT) { const K k = __ldg(src + p); lo = min(lo, k); hi = max(hi, k); }
     lo = warp_min_k(lo);
     hi = warp_max_k(hi);
     __syncthreads();
@@ -794,20 +830,29 @@ __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>:
     // group: linear in the key where sign and exponent are shared (the value is
     // linear in the key there), else linear in the value
     const bool same = ((lo ^ hi) >> KO::MANT) == 0;
-    const int dsh = max(0, 64 - __clzll((long long)((uint64_t)(hi - lo) | 1ull)) - 24);
+    const int range_bits = 64 - __clzll((long long)((uint64_t)(hi - lo) | 1ull));
+    const int dsh = max(0, range_bits - 24);
+    const int cut = PLACE ? max(0, range_bits - (KO::BITS - 12)) : 0;   // key bits that the words leave out
     const float x0 = ws_trunc_f32(KO::from_key(lo));
     const float span = same ? (float)(uint32_t)((hi - lo) >> dsh) + 1.0f : ws_trunc_f32(KO::from_key(hi)) - x0;
     const float scale = (span > 0.0f && span <= 3.0e38f) ? (float)BIN_GROUPS / span : 0.0f;
-    uint32_t br[BIN_ITEMS];   // group << 16 | rank
+    auto group_of = [&](K k) -> uint32_t {   // group << 16 | rank
+        const float f = same ? (float)(uint32_t)((k - lo) >> dsh) : ws_trunc_f32(KO::from_key(k)) - x0;
+        const uint32_t b = min((uint32_t)(int)(f * scale), (uint32_t)BIN_GROUPS - 1u);
+        return (b << 16) | atomicAdd(&s.u.cnt[b], 1u);
+    };
+    auto word_of = [&](K k, int p) -> K { return PLACE ? (K)((((k - lo) >> cut) << 12) | (K)p) : k; };
+    uint32_t br[BIN_REG];
 #pragma unroll
-    for (int k = 0; k < BIN_ITEMS; ++k) {
+    for (int k = 0; k < BIN_REG; ++k) {
         if (k * BIN_NT >= n) break;   // (uniform)
-        if (t + k * BIN_NT < n) {
-            const float f = same ? (float)(uint32_t)((key[k] - lo) >> dsh) : ws_trunc_f32(KO::from_key(key[k])) - x0;
-            const uint32_t b = min((uint32_t)(int)(f * scale), (uint32_t)BIN_GROUPS - 1u);
-            br[k] = (b << 16) | atomicAdd(&s.u.cnt[b], 1u);
+        const int p = t + k * BIN_NT;
+        if (p < n) {
+            br[k] = group_of(key[k]);
+            key[k] = word_of(key[k], p);
         }
     }
+    for (int p = t + BIN_REG * BIN_NT; p < n; p += BIN_NT) s.late[p - BIN_REG * BIN_NT] = group_of(__ldg(src + p));
     __syncthreads();
     // this thread's four groups
     static_assert(BIN_GPT == 4 && BIN_NT == 256, "a thread's group counts are one 16-byte word; eight warps");
@@ -815,25 +860,20 @@ __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>:
     const int sum = (int)(c4.x + c4.y + c4.z + c4.w);
     const int inc = ws_warp_incl_scan<int>(sum);
     if (lane == 31) s.wsum[w] = inc;
-    if (__syncthreads_or(max(max(c4.x, c4.y), max(c4.z, c4.w)) > BIN_WARP_MAX)) {   // radix passes (uniform)
-#pragma unroll
-        for (int k = 0; k < BIN_ITEMS; ++k)
-            if (t + k * BIN_NT < n) s.key[t + k * BIN_NT] = key[k];
-        __syncthreads();
-        // (every bit below the highest one in which the extremes differ may vary)
-        const int top = 64 - __clzll((long long)(uint64_t)(lo ^ hi));
-        bin_radix<T>(s, n, top ? (K)(~(uint64_t)0 >> (64 - top)) : (K)0);
-        for (int i = t; i < n; i += BIN_NT) dst[i] = s.key[i];
-        return;
-    }
+    __syncthreads();
     const int wt = s.wsum[lane & 7];
     const int g0 = inc - sum + __reduce_add_sync(WS_FULL_MASK, lane < w ? wt : 0);
-    reinterpret_cast<uint4*>(s.u.cnt)[t] = make_uint4((uint32_t)g0, g0 + c4.x, g0 + c4.x + c4.y, g0 + c4.x + c4.y + c4.z);
+    reinterpret_cast<uint4*>(s.u.cnt)[t] =
+        make_uint4((uint32_t)g0, g0 + c4.x, g0 + c4.x + c4.y, g0 + c4.x + c4.y + c4.z);
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < BIN_ITEMS; ++k) {
+    for (int k = 0; k < BIN_REG; ++k) {
         if (k * BIN_NT >= n) break;   // (uniform)
         if (t + k * BIN_NT < n) s.key[s.u.cnt[br[k] >> 16] + (br[k] & 0xffffu)] = key[k];
+    }
+    for (int p = t + BIN_REG * BIN_NT; p < n; p += BIN_NT) {
+        const uint32_t b = s.late[p - BIN_REG * BIN_NT];
+        s.key[s.u.cnt[b >> 16] + (b & 0xffffu)] = word_of(__ldg(src + p), p);
     }
     __syncthreads();
     {
@@ -841,7 +881,7 @@ __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>:
         int g = g0;
 #pragma unroll
         for (int i = 0; i < BIN_GPT; ++i) {
-            if (c[i] <= 8) sort_group<8, K>(s.key + g, c[i]);
+            if (c[i] <= BIN_NET) sort_group<BIN_NET, K>(s.key + g, c[i]);
             else s.list[atomicAdd(&s.n_list, 1)] = ((uint32_t)g << 16) | (uint32_t)c[i];
             g += c[i];
         }
@@ -849,22 +889,53 @@ __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>:
     __syncthreads();
     const int nl = s.n_list;
     if (nl > 0) {   // (uniform)
-        for (int i = w; i < nl; i += BIN_NT / 32) sort_warp<K>(s.key + (s.list[i] >> 16), (int)(s.list[i] & 0xffffu));
+        for (int i = w; i < nl; i += BIN_NT / 32)
+            if (!sort_warp<K>(s.key + (s.list[i] >> 16), (int)(s.list[i] & 0xffffu), PLACE ? 12 : 0) && lane == 0)
+                s.radix_needed = 1;
         __syncthreads();
     }
-#pragma unroll
-    for (int k = 0; k < BIN_ITEMS; ++k) {
-        if (k * BIN_NT >= n) break;   // (uniform)
-        const int p = t + k * BIN_NT;
-        if (p < n) dst[p] = s.key[p];
+    if (PLACE && cut > 0 && !s.radix_needed) {   // (uniform)
+        // runs with the same top bits: the thread of a run's first word orders it by the whole keys
+        for (int i = t; i < n; i += BIN_NT) {
+            const K top = s.key[i] >> 12;
+            if (i > 0 && (s.key[i - 1] >> 12) == top) continue;
+            int e = i + 1;
+            while (e < n && e - i <= BIN_RUN_MAX && (s.key[e] >> 12) == top) ++e;
+            if (e - i > BIN_RUN_MAX) { s.radix_needed = 1; continue; }
+            for (int a = i + 1; a < e; ++a) {
+                const K wa = s.key[a], ka = __ldg(src + ((uint32_t)wa & 0xfffu));
+                int j = a - 1;
+                while (j >= i && __ldg(src + ((uint32_t)s.key[j] & 0xfffu)) > ka) { s.key[j + 1] = s.key[j]; --j; }
+                s.key[j + 1] = wa;
+            }
+        }
+        __syncthreads();
+    }
+    const bool radix = s.radix_needed != 0;   // (uniform)
+    if (radix) {
+        __syncthreads();
+        bin_radix<T, PLACE>(s, src, n, (K)(~(uint64_t)0 >> (64 - range_bits)) | (lo ^ hi));
+    }
+    K* dst = sorted + start;
+#pragma unroll 4
+    for (int p = t; p < n; p += BIN_NT) {
+        const K c = s.key[p];
+        if (PLACE) {
+            const uint32_t q = (uint32_t)c & 0xfffu;
+            dst[p] = cut > 0 || radix ? __ldg(src + q) : lo + (c >> 12);
+            bin_idx[start + p] = (uint16_t)q;
+        } else {
+            dst[p] = c;
+        }
     }
 }
 
 // ---------------------------------------------------------------------------
 // Oversize bins: LSD radix passes over the digits that vary, all bins side by
 // side, as a cooperative grid with a barrier between the steps.  A bin's keys
-// start in keys_b and swap buffers with every pass that its digits need; they
-// end in keys_a (copied there if the number of passes is even).
+// stay in keys_b (the way back needs them); its passes alternate between
+// keys_a and a scratch buffer so that the last one writes keys_a (a bin of
+// equal keys is copied there).
 // ---------------------------------------------------------------------------
 struct OverSmem {
     uint32_t whist[(OVER_NT / 32) * 256];
@@ -876,8 +947,9 @@ struct OverSmem {
 };
 
 template <typename T>
-__global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* ka, typename KeyOf<T>::K* kb,
-                                                         SortCtl* ctl, OverBin* over, uint32_t* over_cnt,
+__global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* ka,
+                                                         const typename KeyOf<T>::K* __restrict__ kb,
+                                                         typename KeyOf<T>::K* kt, SortCtl* ctl, OverBin* over, uint32_t* over_cnt,
                                                          uint64_t spin_limit, uint32_t* status) {
     typedef KeyOf<T> KO;
     typedef typename KO::K K;
@@ -924,6 +996,9 @@ __global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* k
         for (int q = 0; q < p; ++q) c += ((diff >> (8 * q)) & 0xffull) != 0;
         return c;
     };
+    // where pass i of m writes, and where it reads
+    auto out_of = [&](int i, int m) -> K* { return ((m - 1 - i) & 1) ? kt : ka; };
+    auto in_of = [&](int i, int m) -> const K* { return i == 0 ? kb : out_of(i - 1, m); };
     // bits that vary
     for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
         const int e = entry(tile);
@@ -950,7 +1025,7 @@ __global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* k
             const int e = entry(tile);
             const unsigned long long diff = __ldcg(&over[e].diff);
             if (((diff >> (8 * p)) & 0xffull) == 0) continue;
-            const K* src = ((passes_before(diff, p) & 1) ? ka : kb) + over[e].start;
+            const K* src = in_of(passes_before(diff, p), passes_before(diff, P)) + over[e].start;
             const int o0 = (tile - __ldcg(&over[e].first_tile)) * TILE, n = min(TILE, over[e].n - o0);
             if (t < 256) s.dcount[t] = 0;
             __syncthreads();
@@ -992,9 +1067,9 @@ __global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* k
             const int e = entry(tile);
             const unsigned long long diff = __ldcg(&over[e].diff);
             if (((diff >> (8 * p)) & 0xffull) == 0) continue;
-            const bool odd = passes_before(diff, p) & 1;
-            const K* src = (odd ? ka : kb) + over[e].start;
-            K* dst = (odd ? kb : ka) + over[e].start;
+            const int i = passes_before(diff, p), m = passes_before(diff, P);
+            const K* src = in_of(i, m) + over[e].start;
+            K* dst = out_of(i, m) + over[e].start;
             const int ne = over[e].n;
             const int o0 = (tile - __ldcg(&over[e].first_tile)) * TILE, n = min(TILE, ne - o0);
             K key[ITEMS];
@@ -1003,9 +1078,9 @@ __global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* k
             int pos[ITEMS];
 #pragma unroll
             for (int k = 0; k < ITEMS; ++k) {
-                const int i = w * 32 * ITEMS + k * 32 + lane;
-                valid[k] = i < n;
-                key[k] = valid[k] ? __ldcg(src + o0 + i) : (K)0;
+                const int q = w * 32 * ITEMS + k * 32 + lane;
+                valid[k] = q < n;
+                key[k] = valid[k] ? __ldcg(src + o0 + q) : (K)0;
                 dg[k] = (uint32_t)((key[k] >> (8 * p)) & 0xff);
             }
             if (t < 256) s.base[t] = __ldcg(over_cnt + (size_t)tile * 256 + t);
@@ -1019,13 +1094,13 @@ __global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* k
         }
         bar.sync();
     }
-    // bins whose keys are still in keys_b
+    // bins of equal keys
     for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
         const int e = entry(tile);
-        if (passes_before(__ldcg(&over[e].diff), P) & 1) continue;
+        if (__ldcg(&over[e].diff) != 0) continue;
         const int64_t st = over[e].start;
         const int o0 = (tile - __ldcg(&over[e].first_tile)) * TILE, n = min(TILE, over[e].n - o0);
-        for (int i = t; i < n; i += NT) ka[st + o0 + i] = __ldcg(kb + st + o0 + i);
+        for (int i = t; i < n; i += NT) ka[st + o0 + i] = kb[st + o0 + i];
     }
 }
 
@@ -1048,6 +1123,9 @@ static cudaError_t sort_prepare(int max_bins, int n_tiles, WsSortShape* sh) {
     cudaError_t e = cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan_smem(HIST_MAX));
     if (!e) e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ksm);
     if (!e) e = cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ksm);
+    auto *kb0 = k_bin_sort<T, false>, *kb1 = k_bin_sort<T, true>;
+    if (!e) e = cudaFuncSetAttribute(kb0, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BinSmem<T>));
+    if (!e) e = cudaFuncSetAttribute(kb1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BinSmem<T>));
     if (e) return e;
     int dev = 0, sms = 0, np = 0, n1 = 0, no = 0;
     if ((e = cudaGetDevice(&dev))) return e;
@@ -1076,8 +1154,8 @@ cudaError_t ws_sort_prepare(int max_bins, int n_tiles, int samp_max, WsSortShape
 }
 
 template <typename T, typename B>
-static cudaError_t sort_run(const LargeWork<T>& W, const T* values, uint32_t* status, uint64_t spin_limit,
-                            cudaStream_t st) {
+static cudaError_t sort_run(const LargeWork<T>& W, const T* values, bool way_back, uint32_t* status,
+                            uint64_t spin_limit, cudaStream_t st) {
     typedef typename KeyOf<T>::K K;
     cudaError_t e = cudaMemsetAsync(W.ctl, 0, W.sort_zero_bytes, st);
     if (e) return e;
@@ -1103,20 +1181,23 @@ static cudaError_t sort_run(const LargeWork<T>& W, const T* values, uint32_t* st
     const int grid = std::min(sh.part_grid, W.n_sort_tiles);
     WS_LAUNCH(W.prof, WSK_PARTITION, st,
               (k_part<T, B, true><<<grid, WS_SORT_NT, ksm, st>>>(values, nullptr, bins, W.keys_a, W.keys_b, bins2,
+                                                                 way_back ? W.dest1 : nullptr,
                                                                  W.sort_tiles, W.n_sort_tiles, W.lsegs, W.cur1, W.ctl,
                                                                  status)));
     if (W.two_level)
         WS_LAUNCH(W.prof, WSK_PARTITION, st,
                   (k_part<T, B, false><<<grid, WS_SORT_NT, ksm, st>>>(nullptr, W.keys_a, bins2, nullptr, W.keys_b,
-                                                                      nullptr, W.sort_tiles, W.n_sort_tiles, W.lsegs,
+                                                                      nullptr, way_back ? W.dest2 : nullptr, W.sort_tiles, W.n_sort_tiles, W.lsegs,
                                                                       W.cur2, W.ctl, status)));
+    auto* kbin = way_back ? k_bin_sort<T, true> : k_bin_sort<T, false>;
     WS_LAUNCH(W.prof, WSK_BIN_SORT, st,
-              (k_bin_sort<T><<<W.n_bins, BIN_NT, 0, st>>>(W.keys_b, W.keys_a, W.bin_seg, W.lsegs, W.bin_start,
-                                                          W.bin_cnt, W.ctl, W.over, W.n_keys)));
+              (kbin<<<W.n_bins, BIN_NT, sizeof(BinSmem<T>), st>>>(W.keys_b, W.keys_a, W.bin_seg, W.lsegs, W.bin_start,
+                                                                 W.bin_cnt, W.bin_idx, W.ctl, W.over, W.n_keys)));
     {
         K* ka = W.keys_a;
         K* kb = W.keys_b;
-        void* args[] = {&ka, &kb, (void*)&W.ctl, (void*)&W.over, (void*)&W.over_cnt, &spin_limit, &status};
+        K* kt = reinterpret_cast<K*>(W.pairs_b);
+        void* args[] = {&ka, &kb, &kt, (void*)&W.ctl, (void*)&W.over, (void*)&W.over_cnt, &spin_limit, &status};
         WS_LAUNCH(W.prof, WSK_OVERSIZE, st,
                   e = cudaLaunchCooperativeKernel((const void*)k_oversize<T>,
                                                   dim3(std::min(sh.over_grid, W.n_sort_tiles)), dim3(OVER_NT), args, 0,
@@ -1127,18 +1208,18 @@ static cudaError_t sort_run(const LargeWork<T>& W, const T* values, uint32_t* st
 }
 
 template <typename T>
-cudaError_t ws_large_sort(const LargeWork<T>& W, const T* values, uint32_t* status, uint64_t spin_limit,
-                          cudaStream_t st, typename KeyOf<T>::K** sorted) {
+cudaError_t ws_large_sort(const LargeWork<T>& W, const T* values, bool way_back, uint32_t* status,
+                          uint64_t spin_limit, cudaStream_t st, typename KeyOf<T>::K** sorted) {
     *sorted = nullptr;
     if (W.n_sort_tiles == 0) return cudaSuccess;
     *sorted = W.keys_a;
-    return W.sort_shape.wide ? sort_run<T, uint32_t>(W, values, status, spin_limit, st)
-                             : sort_run<T, uint16_t>(W, values, status, spin_limit, st);
+    return W.sort_shape.wide ? sort_run<T, uint32_t>(W, values, way_back, status, spin_limit, st)
+                             : sort_run<T, uint16_t>(W, values, way_back, status, spin_limit, st);
 }
 
 template cudaError_t ws_sort_prepare<float>(int, int, int, WsSortShape*);
 template cudaError_t ws_sort_prepare<double>(int, int, int, WsSortShape*);
-template cudaError_t ws_large_sort<float>(const LargeWork<float>&, const float*, uint32_t*, uint64_t, cudaStream_t,
-                                          uint32_t**);
-template cudaError_t ws_large_sort<double>(const LargeWork<double>&, const double*, uint32_t*, uint64_t,
+template cudaError_t ws_large_sort<float>(const LargeWork<float>&, const float*, bool, uint32_t*, uint64_t,
+                                          cudaStream_t, uint32_t**);
+template cudaError_t ws_large_sort<double>(const LargeWork<double>&, const double*, bool, uint32_t*, uint64_t,
                                            cudaStream_t, uint64_t**);

@@ -96,7 +96,7 @@ cudaError_t ws_large_R(const LargeWork<T>& W, const T* values, double* R_out, do
     typedef typename KeyOf<T>::K K;
     if (W.n_lseg == 0) return cudaSuccess;
     K* sorted = nullptr;
-    cudaError_t e = ws_large_sort<T>(W, values, status, spin_limit, st, &sorted);
+    cudaError_t e = ws_large_sort<T>(W, values, false, status, spin_limit, st, &sorted);
     if (e) return e;
     RPartial* part = reinterpret_cast<RPartial*>(partial);
     WS_LAUNCH(W.prof, WSK_MISC, st,
