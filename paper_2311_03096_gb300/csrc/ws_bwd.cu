@@ -407,19 +407,29 @@ __global__ void __launch_bounds__(BNT) k_bwd_apply(const int32_t* __restrict__ i
     }
 }
 
-// One-CTA segments: the same exact sums in shared memory.  Every thread keeps
-// its CAP / NT elements (grad_out and id) in registers; lanes of a warp with
-// the same cluster add once; each used slot forms its mean once, in place.
+// One-CTA segments: the same exact sums in shared memory, as five signed
+// 19-bit limbs per cluster.  A grad_out value of MANT + 1 bits falls into at
+// most three of them (four for double), each one 32-bit shared-memory add
+// without a returned value (native; a 64-bit shared atomic is a
+// compare-and-swap loop), and 4096 limbs of 19 bits cannot overflow 32 bits.
+// The limbs recombine to the integer that 128-bit additions give.  Bound by
+// those adds and the conversions; 12.6M elements in rows of 3072: 482 us with
+// 64-bit atomics behind a warp match.
+constexpr int LIMBS = 5, LIMB_BITS = 19;   // 95 bits: every ws_bwd_fix value
+
 template <typename T, int NT, int CAP>
-__global__ void __launch_bounds__(NT) k_small_backward(const T* __restrict__ g, const int32_t* __restrict__ ids,
-                                                       const int64_t* __restrict__ offsets,
-                                                       const int32_t* __restrict__ seg_list, T* gin,
-                                                       uint32_t* status) {
+__global__ void __launch_bounds__(NT, 2) k_small_backward(const T* __restrict__ g, const int32_t* __restrict__ ids,
+                                                          const int64_t* __restrict__ offsets,
+                                                          const int32_t* __restrict__ seg_list, T* gin,
+                                                          uint32_t* status) {
+    typedef KeyOf<T> KO;
     constexpr int PER = CAP / NT;
     static_assert(CAP % NT == 0, "whole elements per thread");
+    static_assert(LIMBS * LIMB_BITS >= BwdFix<T>::SH + BwdFix<T>::MANT + 1, "every value fits");
+    static_assert((long long)CAP * ((1 << LIMB_BITS) - 1) < (1ll << 31), "no limb overflows");
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    unsigned long long* acc = reinterpret_cast<unsigned long long*>(smem_raw);   // [CAP][2]
-    int* cnt = reinterpret_cast<int*>(acc + 2 * CAP);                            // [CAP]
+    int* limb = reinterpret_cast<int*>(smem_raw);   // [LIMBS][CAP]
+    int* cnt = limb + LIMBS * CAP;                  // [CAP]
     __shared__ int s_emax;
     const int seg = seg_list[blockIdx.x];
     const int64_t a0 = offsets[seg];
@@ -430,26 +440,25 @@ __global__ void __launch_bounds__(NT) k_small_backward(const T* __restrict__ g, 
     if (t == 0) s_emax = 0;
     T gv[PER];
     int idv[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int i = t + k * NT;
+        gv[k] = i < n ? __ldg(g + a0 + i) : (T)0;
+        idv[k] = i < n ? __ldg(ids + a0 + i) : -1;
+    }
+    for (int i = t; i < (n + 3) / 4; i += NT) {
+#pragma unroll
+        for (int l = 0; l <= LIMBS; ++l) reinterpret_cast<int4*>(limb + l * CAP)[i] = make_int4(0, 0, 0, 0);
+    }
     int e = 0;
     bool bad = false;
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
-        const int i = t + k * NT;
-        gv[k] = (T)0;
-        idv[k] = -1;
-        if (i < n) {
-            gv[k] = g[a0 + i];
-            const int id = ids[a0 + i];
-            if (id >= 0 && id < n) idv[k] = id; else bad = true;
-            acc[2 * i] = 0ull;
-            acc[2 * i + 1] = 0ull;
-            cnt[i] = 0;
-        }
         e = max(e, ws_g_exp(gv[k]));
+        if (idv[k] < 0 || idv[k] >= n) { bad |= t + k * NT < n; idv[k] = -1; }
     }
     if (bad) ws_flag(status, WS_STATUS_INTERNAL);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+    e = __reduce_max_sync(0xffffffffu, e);
     __syncthreads();
     if (lane == 0) atomicMax(&s_emax, e);
     __syncthreads();
@@ -457,27 +466,58 @@ __global__ void __launch_bounds__(NT) k_small_backward(const T* __restrict__ g, 
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
         const int id = idv[k];
-        const i128 q = ws_bwd_fix<T>(gv[k], emax);
-        const unsigned peers = __match_any_sync(0xffffffffu, id);
-        const i128 s = __any_sync(0xffffffffu, __popc(peers) > 1) ? ws_group_sum_i96(peers, q) : q;
-        if (id >= 0 && lane == __ffs((int)peers) - 1) {
-            ws_atomic_add_i128(acc + 2 * id, s);
-            atomicAdd(cnt + id, __popc(peers));
+        if (id < 0) continue;
+        // grad_out = +-m 2^sh in units of the fixed point, as in ws_bwd_fix
+        const uint64_t b = (uint64_t)KO::bits(gv[k]);
+        int ex = (int)((b >> KO::MANT) & KO::EXPMASK);
+        uint64_t m = b & ((1ull << KO::MANT) - 1ull);
+        if (ex == 0) ex = 1; else m |= 1ull << KO::MANT;
+        int sh = ex - emax + BwdFix<T>::SH;
+        if (sh < 0) { m = sh > -64 ? m >> (-sh) : 0ull; sh = 0; }
+        const bool neg = (b >> (KO::BITS - 1)) & 1ull;
+        const int l0 = (sh * 27) >> 9;   // sh / 19 for 0 <= sh <= 94
+        const int r = sh - LIMB_BITS * l0;
+        int* p = limb + l0 * CAP + id;
+        constexpr uint32_t LM = (1u << LIMB_BITS) - 1u;
+        auto add = [&](int l, uint32_t v) {
+            if (v) atomicAdd(p + l * CAP, neg ? -(int)v : (int)v);
+        };
+        const uint64_t w = m << r;   // (float: 42 bits; double: the low 64 of 71)
+        add(0, (uint32_t)w & LM);
+        add(1, (uint32_t)(w >> LIMB_BITS) & LM);
+        if (sizeof(T) == 4) {
+            add(2, (uint32_t)(w >> (2 * LIMB_BITS)));
+        } else {
+            add(2, (uint32_t)(w >> (2 * LIMB_BITS)) & LM);
+            add(3, (uint32_t)((m >> (3 * LIMB_BITS - 18)) >> (18 - r)) & LM);   // (m << r) >> 57, r <= 18
         }
+        atomicAdd(cnt + id, 1);
     }
     __syncthreads();
-    // the mean of slot r replaces its low word (only this thread touches slot r)
+    // the mean of slot r replaces its low limbs (only this thread touches slot r)
     for (int r = t; r < n; r += NT) {
         const int c = cnt[r];
         if (c == 0) continue;
-        const i128 S = (i128)(((u128)acc[2 * r + 1] << 64) | (u128)acc[2 * r]);
-        *reinterpret_cast<T*>(acc + 2 * r) = ws_bwd_mean<T>(S, c, emax);
+        const int64_t A = (int64_t)limb[r] + ((int64_t)limb[CAP + r] << LIMB_BITS);
+        const int64_t B = (int64_t)limb[2 * CAP + r] + ((int64_t)limb[3 * CAP + r] << LIMB_BITS);
+        const i128 S = (i128)A + ((i128)B << (2 * LIMB_BITS)) + ((i128)limb[4 * CAP + r] << (4 * LIMB_BITS));
+        const T mean = ws_bwd_mean<T>(S, c, emax);
+        if (sizeof(T) == 4) limb[r] = __float_as_int((float)mean);
+        else {
+            const long long q = __double_as_longlong((double)mean);
+            limb[r] = (int)(uint32_t)(uint64_t)q;
+            limb[CAP + r] = (int)(uint32_t)((uint64_t)q >> 32);
+        }
     }
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
-        const int i = t + k * NT;
-        if (i < n && idv[k] >= 0) gin[a0 + i] = *reinterpret_cast<const T*>(acc + 2 * idv[k]);
+        const int id = idv[k];
+        if (id < 0) continue;
+        T v;
+        if (sizeof(T) == 4) v = (T)__int_as_float(limb[id]);
+        else v = (T)__longlong_as_double((long long)(((uint64_t)(uint32_t)limb[CAP + id] << 32) | (uint32_t)limb[id]));
+        gin[a0 + t + k * NT] = v;
     }
 }
 
@@ -544,10 +584,10 @@ cudaError_t ws_large_backward(const LargeWork<T>& W, const T* g, const int32_t* 
 template <typename T>
 cudaError_t ws_launch_small_backward(const T* g, const int32_t* ids, const int64_t* offsets, const int32_t* seg_list,
                                      int n_list, T* gin, uint32_t* status, cudaStream_t st, WsProf* prof) {
-    constexpr int NT = 256;
+    constexpr int NT = 512;
     constexpr int CAP = SmallCfg<T>::CAP;
     if (n_list <= 0) return cudaSuccess;
-    const size_t smem = (size_t)CAP * (2 * sizeof(unsigned long long) + sizeof(int));
+    const size_t smem = (size_t)CAP * (LIMBS + 1) * sizeof(int);
     auto k = k_small_backward<T, NT, CAP>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e) return e;
