@@ -28,6 +28,11 @@ __device__ __forceinline__ uint64_t ws_shfl_xor_k(uint64_t v, int o) {
     return (uint64_t)__shfl_xor_sync(WS_FULL_MASK, (unsigned long long)v, o);
 }
 
+__device__ __forceinline__ uint32_t ws_shfl_k(uint32_t v, int l) { return __shfl_sync(WS_FULL_MASK, v, l); }
+__device__ __forceinline__ uint64_t ws_shfl_k(uint64_t v, int l) {
+    return (uint64_t)__shfl_sync(WS_FULL_MASK, (unsigned long long)v, l);
+}
+
 __device__ __forceinline__ void ws_atomic_min_k(uint32_t* p, uint32_t v) { atomicMin(p, v); }
 __device__ __forceinline__ void ws_atomic_max_k(uint32_t* p, uint32_t v) { atomicMax(p, v); }
 __device__ __forceinline__ void ws_atomic_min_k(uint64_t* p, uint64_t v) {

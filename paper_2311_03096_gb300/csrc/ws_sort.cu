@@ -674,18 +674,67 @@ __device__ __forceinline__ void sort_group(K* key, int n) {
         if (i < n) key[i] = v[i];
 }
 
+__device__ __forceinline__ uint32_t warp_min_k(uint32_t v) { return __reduce_min_sync(WS_FULL_MASK, v); }
+__device__ __forceinline__ uint32_t warp_max_k(uint32_t v) { return __reduce_max_sync(WS_FULL_MASK, v); }
+__device__ __forceinline__ uint64_t warp_min_k(uint64_t v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = min(v, ws_shfl_xor_k(v, o));
+    return v;
+}
+__device__ __forceinline__ uint64_t warp_max_k(uint64_t v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = max(v, ws_shfl_xor_k(v, o));
+    return v;
+}
+
 // Sort of n keys or words by one warp: ranks by counting (ties by place).
-// false for more than BIN_WARP_MAX, unless they are equal above the low `low`
-// bits (then any order will do).
-template <typename K>
-__device__ __noinline__ bool sort_warp(K* key, int n, int low) {
+// More than BIN_WARP_MAX words are left alone if they are equal above the
+// place (then any order will do).  Keys of which few differ (weights that are
+// already shared) are written as runs.  false: more than BIN_WARP_MAX and
+// neither.
+template <bool PLACE, typename K>
+__device__ __noinline__ bool sort_warp(K* key, int n) {
     const int lane = threadIdx.x & 31;
     constexpr int PER = BIN_WARP_MAX / 32;
-    if (n > BIN_WARP_MAX) {
-        const K k0 = key[0] >> low;
+    if (PLACE && n > BIN_WARP_MAX) {
+        const K k0 = key[0] >> 12;
         bool same = true;
-        for (int j = lane; j < n; j += 32) same &= (key[j] >> low) == k0;
+        for (int j = lane; j < n; j += 32) same &= (key[j] >> 12) == k0;
         return __all_sync(WS_FULL_MASK, same);
+    }
+    bool runs = false;
+    if (!PLACE && n > 16) {   // (at most 8 different ones among the first 32)
+        const unsigned peers = __match_any_sync(WS_FULL_MASK, (unsigned long long)key[min(lane, n - 1)]);
+        runs = n > BIN_WARP_MAX || __popc(__ballot_sync(WS_FULL_MASK, lane == __ffs((int)peers) - 1)) <= 8;
+    }
+    if (runs) {
+        // lane d gets the d-th smallest value and where its run ends
+        K mine = 0, prev = 0;
+        int end = n, done = 0;
+        for (int d = 0; d < 32 && done < n; ++d) {
+            K lo = ~(K)0;
+            for (int j = lane; j < n; j += 32) {
+                const K x = key[j];
+                if (d == 0 || x > prev) lo = min(lo, x);
+            }
+            lo = warp_min_k(lo);
+            int c = 0;
+            for (int j = lane; j < n; j += 32) c += key[j] == lo;
+            done += __reduce_add_sync(WS_FULL_MASK, c);
+            if (lane == d) { mine = lo; end = done; }
+            prev = lo;
+        }
+        __syncwarp();
+        if (done == n) {
+            for (int d = 0, j0 = 0; d < 32 && j0 < n; ++d) {
+                const K x = ws_shfl_k(mine, d);
+                const int j1 = __shfl_sync(WS_FULL_MASK, end, d);
+                for (int j = j0 + lane; j < j1; j += 32) key[j] = x;
+                j0 = j1;
+            }
+            return true;
+        }
+        if (n > BIN_WARP_MAX) return false;
     }
     K v[PER];
     int r[PER];
@@ -708,19 +757,6 @@ __device__ __noinline__ bool sort_warp(K* key, int n, int low) {
     for (int k = 0; k < PER; ++k)
         if (lane + 32 * k < n) key[r[k]] = v[k];
     return true;
-}
-
-__device__ __forceinline__ uint32_t warp_min_k(uint32_t v) { return __reduce_min_sync(WS_FULL_MASK, v); }
-__device__ __forceinline__ uint32_t warp_max_k(uint32_t v) { return __reduce_max_sync(WS_FULL_MASK, v); }
-__device__ __forceinline__ uint64_t warp_min_k(uint64_t v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = min(v, ws_shfl_xor_k(v, o));
-    return v;
-}
-__device__ __forceinline__ uint64_t warp_max_k(uint64_t v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = max(v, ws_shfl_xor_k(v, o));
-    return v;
 }
 
 // LSD radix passes, 8-bit digits that vary (diff), over a bin's n keys in
@@ -890,7 +926,7 @@ __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>:
     const int nl = s.n_list;
     if (nl > 0) {   // (uniform)
         for (int i = w; i < nl; i += BIN_NT / 32)
-            if (!sort_warp<K>(s.key + (s.list[i] >> 16), (int)(s.list[i] & 0xffffu), PLACE ? 12 : 0) && lane == 0)
+            if (!sort_warp<PLACE, K>(s.key + (s.list[i] >> 16), (int)(s.list[i] & 0xffffu)) && lane == 0)
                 s.radix_needed = 1;
         __syncthreads();
     }

@@ -35,28 +35,44 @@ __global__ void __launch_bounds__(256) k_R_tiles(const typename KeyOf<T>::K* __r
     const int E = ws_fix_scale<T>(max(ws_eff_exp(xlo), ws_eff_exp(xhi)), seg_emin[td.lseg]);
     const K kz = KO::to_key((T)0), knz = KO::to_key(-(T)0);
     const int64_t j0 = (int64_t)td.tin * WS_SORT_TILE;
+    // sum of coef_j q_j over this thread's elements, coef_j = 2j - len + 1
+    // (2k - d - 1 with k = j + 1).  Its elements lie 256 apart, so with c its
+    // last coefficient the sum is c Q - 512 W, Q the sum of its q and W that of
+    // its earlier elements' running sums: 64-bit additions and, every four
+    // elements (the sums stay below 2^61), two 128-bit products.
+    constexpr int U = 4;
     i128 acc = 0;
-    long long dis = 0, nz = 0;
-    for (int i = threadIdx.x; i < td.len; i += 256) {
-        const int64_t j = j0 + i;
-        const K k = seg[j];
-        const bool nonzero = k != kz && k != knz;
-        nz += nonzero;
-        dis += nonzero && (j == 0 || seg[j - 1] != k);
-        const int64_t coef = 2 * j - ls.len + 1;   // 2k - d - 1 with k = j + 1
-        acc += (i128)coef * (i128)ws_fixed<T>(KO::from_key(k), E);
+    int dis = 0, nz = 0;
+    for (int i0 = threadIdx.x; i0 < td.len; i0 += 256 * U) {
+        K k[U], before[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t j = j0 + min(i0 + u * 256, td.len - 1);
+            k[u] = __ldg(seg + j);
+            before[u] = j > 0 ? __ldg(seg + j - 1) : ~k[u];
+        }
+        int64_t Q = 0, Wq = 0;
+        int c = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (i0 + u * 256 < td.len) {
+                const bool nonzero = k[u] != kz && k[u] != knz;
+                nz += nonzero;
+                dis += nonzero && before[u] != k[u];
+                Wq += Q;
+                Q += ws_fixed<T>(KO::from_key(k[u]), E);   // (|Q| <= 2^60, |Wq| <= 6 x 2^58)
+                c = u;
+            }
+        }
+        const int64_t coef = 2 * (j0 + i0 + c * 256) - ls.len + 1;
+        acc += (i128)coef * Q - (i128)512 * Wq;
     }
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    long long packed[2] = {dis, nz};
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        acc += (i128)__shfl_xor_sync(0xffffffffu, (long long)(acc >> 64), o) * ((i128)1 << 64) +
-               (i128)(unsigned long long)__shfl_xor_sync(0xffffffffu, (unsigned long long)acc, o);
-        packed[0] += __shfl_xor_sync(0xffffffffu, packed[0], o);
-        packed[1] += __shfl_xor_sync(0xffffffffu, packed[1], o);
-    }
-    __shared__ long long wsd[8], wsn[8];
-    if (lane == 0) { ws128[w] = acc; wsd[w] = packed[0]; wsn[w] = packed[1]; }
+    acc = ws_warp_reduce_i128(acc);
+    dis = __reduce_add_sync(0xffffffffu, dis);
+    nz = __reduce_add_sync(0xffffffffu, nz);
+    __shared__ int wsd[8], wsn[8];
+    if (lane == 0) { ws128[w] = acc; wsd[w] = dis; wsn[w] = nz; }
     __syncthreads();
     if (threadIdx.x == 0) {
         RPartial p;
@@ -66,20 +82,32 @@ __global__ void __launch_bounds__(256) k_R_tiles(const typename KeyOf<T>::K* __r
     }
 }
 
+// One CTA per segment adds its tiles' partial sums.
 template <typename T>
-__global__ void __launch_bounds__(32) k_R_final(const LargeSeg* __restrict__ lsegs, const TileDesc* __restrict__ tiles,
+__global__ void __launch_bounds__(256) k_R_final(const LargeSeg* __restrict__ lsegs, const TileDesc* __restrict__ tiles,
                                                 const typename KeyOf<T>::K* __restrict__ sorted,
                                                 const int32_t* __restrict__ seg_emin, const RPartial* part,
                                                 double* R_out, double* metric_out, uint32_t* status) {
     typedef KeyOf<T> KO;
-    if (threadIdx.x != 0) return;
+    __shared__ RPartial wp[8];
     const LargeSeg ls = lsegs[blockIdx.x];
     i128 s = 0;
     long long dis = 0, nz = 0;
-    for (int t = 0; t < ls.sort_count; ++t) {
+#pragma unroll 4
+    for (int t = threadIdx.x; t < ls.sort_count; t += 256) {
         const RPartial p = part[ls.sort_first + t];
         s += p.s; dis += p.distinct; nz += p.nonzero;
     }
+    s = ws_warp_reduce_i128(s);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        dis += __shfl_xor_sync(0xffffffffu, dis, o);
+        nz += __shfl_xor_sync(0xffffffffu, nz, o);
+    }
+    if ((threadIdx.x & 31) == 0) { wp[threadIdx.x >> 5].s = s; wp[threadIdx.x >> 5].distinct = dis; wp[threadIdx.x >> 5].nonzero = nz; }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    for (int k = 1; k < 8; ++k) { s += wp[k].s; dis += wp[k].distinct; nz += wp[k].nonzero; }
     const T xlo = KO::from_key(sorted[ls.kpos]), xhi = KO::from_key(sorted[ls.kpos + ls.len - 1]);
     const int E = ws_fix_scale<T>(max(ws_eff_exp(xlo), ws_eff_exp(xhi)), seg_emin[blockIdx.x]);
     ws_note_scale<T>(max(ws_eff_exp(xlo), ws_eff_exp(xhi)), seg_emin[blockIdx.x], status);
@@ -102,7 +130,7 @@ cudaError_t ws_large_R(const LargeWork<T>& W, const T* values, double* R_out, do
     WS_LAUNCH(W.prof, WSK_MISC, st,
               (k_R_tiles<T><<<W.n_sort_tiles, 256, 0, st>>>(sorted, W.sort_tiles, W.lsegs, W.seg_emin, part)));
     WS_LAUNCH(W.prof, WSK_MISC, st,
-              (k_R_final<T><<<W.n_lseg, 32, 0, st>>>(W.lsegs, W.sort_tiles, sorted, W.seg_emin, part, R_out,
+              (k_R_final<T><<<W.n_lseg, 256, 0, st>>>(W.lsegs, W.sort_tiles, sorted, W.seg_emin, part, R_out,
                                                      metric_out, status)));
     return cudaGetLastError();
 }

@@ -40,6 +40,8 @@ def draw(kind, d, dt, seed=5):
         x[rng.random(d) < 0.1] *= -0.0
     elif kind == "few":             # a handful of values, neighbours in the map
         x = np.array([-0.5, 0.25, 0.2500001, 0.2500002, 3.0])[rng.integers(0, 5, d)]
+    elif kind == "shared":          # weights that are already shared: runs of about a thousand equal ones
+        x = rng.standard_normal(1 + d // 1000)[rng.integers(0, 1 + d // 1000, d)]
     elif kind == "binades":         # sixty binades, both signs
         x = np.ldexp(x, rng.integers(-30, 30, d))
     elif kind == "clusters":        # spikes that the cells of the map do not resolve
@@ -72,7 +74,7 @@ def test_bin_edges(ws, ctx, d, dt):
 
 
 @pytest.mark.parametrize("dt", [np.float32, np.float64])
-@pytest.mark.parametrize("kind", ["narrow", "sparse", "few", "binades", "clusters", "sorted", "constant"])
+@pytest.mark.parametrize("kind", ["narrow", "sparse", "few", "shared", "binades", "clusters", "sorted", "constant"])
 def test_distributions(ws, ctx, kind, dt):
     check(ws, ctx, draw(kind, 300007, dt))
 
