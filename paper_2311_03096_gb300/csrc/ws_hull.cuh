@@ -69,17 +69,14 @@ namespace wsh {
 constexpr int NT = 256;                // lanes per tile
 constexpr int M = 16;                  // elements per lane
 constexpr int NW = NT / 32;
-constexpr int WP = 32 * M;             // elements per warp
 constexpr int TILE = NT * M;           // 4096 elements per tile
-constexpr int XSLOT = WP + 1 + WP / M; // prefix slots of one warp (point q stored at q + q / M)
 constexpr uint16_t NONE = 0xffff;
 
 // Shared memory of one tile.
 struct Smem {
-    // X of point p lives in the array of warp own(p) = (p - 1) / WP (p = 0: warp 0),
-    // at slot q + q / M, q = p - own(p) WP in [0, WP]: the lane holding element
-    // p - 1 writes it, so every point has exactly one writer.
-    int64_t X[NW][XSLOT];
+    // X of point p lives at slot p + p / M (lanes with consecutive chunks then
+    // hit distinct banks); the lane holding element p - 1 writes it.
+    int64_t X[TILE + TILE / M + 1];
     uint16_t st[(M + 1) * NT];   // lane stacks (hull vertex points), entry k of lane t at k * NT + t
     uint16_t lo[NT], hi[NT];     // surviving range [lo, hi) of each lane's stack
     uint32_t ne[NW];             // non-empty lanes of every warp
@@ -97,15 +94,8 @@ struct Smem {
 };
 static_assert(NW % 4 == 0, "per-warp words are read four at a time");
 
-__device__ __forceinline__ int own_warp(int p) { return p ? (p - 1) / WP : 0; }
-__device__ __forceinline__ int64_t& xref(Smem& s, int p) {
-    const int w = own_warp(p), q = p - w * WP;
-    return s.X[w][q + q / M];
-}
-__device__ __forceinline__ int64_t xat(const Smem& s, int p) {
-    const int w = own_warp(p), q = p - w * WP;
-    return s.X[w][q + q / M];
-}
+__device__ __forceinline__ int64_t& xref(Smem& s, int p) { return s.X[p + (int)((uint32_t)p / M)]; }
+__device__ __forceinline__ int64_t xat(const Smem& s, int p) { return s.X[p + (int)((uint32_t)p / M)]; }
 
 // The exact hull test on tile-unit prefix values: P_b strictly below the
 // chord from P_a to P_c, i.e. Delta (d - 1) > lambda 2^L K with
@@ -618,6 +608,22 @@ __device__ __forceinline__ bool ic_rounds(Smem& s, const Test& T, int t, int fir
         }
         // decide every boundary to retest against the current blocks
         uint32_t Rm = 0, bits = B & D;
+        if (rounds == 2 && B) {
+            // all of them: a boundary's prefix sums serve its neighbours' tests too
+            bits = 0;
+            uint32_t rest = B;
+            int a = prevS, p = first + __ffs((int)rest) - 1;
+            int64_t Xa = xat(s, a), Xp = xat(s, p);
+            while (rest) {
+                const uint32_t bit = rest & (0u - rest);
+                rest &= rest - 1;
+                const int c = rest ? first + __ffs((int)rest) - 1 : nextS;
+                const int64_t Xc = xat(s, c);
+                if (!T(a, Xa, p, Xp, c, Xc)) Rm |= bit;
+                a = p; Xa = Xp;
+                p = c; Xp = Xc;
+            }
+        }
         while (bits) {
             const int i = __ffs((int)bits) - 1;
             bits &= bits - 1;
