@@ -86,11 +86,9 @@ struct Smem {
     int wsum[NW];
     int general;                 // a bridge walk hit its cap: the tile needs the general kernel
     int all_conc;
-    // IC rounds, per warp: last survivor / removal, first ones (read as int4)
-    __align__(16) int wl[NW];
-    __align__(16) int wlr[NW];
-    __align__(16) int wf[NW];
-    __align__(16) int wfr[NW];
+    // IC rounds, per warp: last and first survivor, for alternate rounds (read as int4)
+    __align__(16) int wl[2][NW];
+    __align__(16) int wf[2][NW];
 };
 static_assert(NW % 4 == 0, "per-warp words are read four at a time");
 
@@ -518,67 +516,60 @@ __device__ __forceinline__ void cta_tree(Smem& s, const Test& T, int t, int cap)
 //   Round r: every surviving block boundary b, with neighbouring boundaries
 //            a < b < c (0 and n at the ends), stays iff the mean of y over
 //            [a, b) is strictly below the mean over [b, c) -- the hull test
-//            at b; all boundaries are decided at once, as the paper's rounds
-//            do.  A boundary whose neighbours did not change keeps last
-//            round's answer, so only boundaries next to a removal are tested
-//            again.
+//            at b.  The lanes decide at once, each for the boundaries of its
+//            own 16 points with the nearest boundaries outside as they were
+//            when the round began; inside a lane a removal is followed up at
+//            once (the stack form of the merge), which saves rounds: a point
+//            on or above the chord of any two other points is no vertex,
+//            whichever of them survive.  After the first such round a lane is
+//            stable in itself and only looks again from an end whose outer
+//            neighbour has changed.
 // When a round removes nothing, every adjacent pair of blocks has increasing
 // means: the blocks are the tile's pool-adjacent-violators partition and
 // their boundaries (with points 0 and n) the vertices of its lower hull.
-// For this lane's range of points: the last set point before it and the first
-// one after it, over the whole CTA, for two point sets at once (B: current
-// boundaries, R: last round's removals; bit i = point first + i).  Inside the
-// warp by ballots and one shuffle each, across warps through one word per
-// warp and set (one barrier).  -1 / BIG when there is none.
-struct Around { int pS, nS, pR, nR; };
-__device__ __forceinline__ Around around(Smem& s, int t, int first, uint32_t B, uint32_t R) {
+// Tile hulls at 2^26, lambda 1e-2: 414 us with one decision per boundary and
+// round (and the removals of the last round exchanged beside the survivors).
+
+// The last boundary of every warp and its first one (bit i of B = point
+// first + i), for this lane's neighbours in other warps; -1 / BIG if none.
+// Written to buffer `buf`; visible after the caller's next barrier.
+constexpr int BIG = 1 << 20;
+__device__ __forceinline__ void post_ends(Smem& s, int t, int first, uint32_t B, int buf) {
+    const unsigned bS = __ballot_sync(WS_FULL_MASK, B != 0);
     const int l = t & 31, w = t >> 5;
-    const int BIG = 1 << 20;
-    const int myLS = B ? first + 31 - __clz((int)B) : -1, myFS = B ? first + __ffs((int)B) - 1 : BIG;
-    const int myLR = R ? first + 31 - __clz((int)R) : -1, myFR = R ? first + __ffs((int)R) - 1 : BIG;
-    const unsigned bS = __ballot_sync(WS_FULL_MASK, B != 0), bR = __ballot_sync(WS_FULL_MASK, R != 0);
-    const unsigned lt = (1u << l) - 1u, gt = l == 31 ? 0u : ~((2u << l) - 1u);
-    auto below = [&](unsigned m, int v) {   // v of the highest lane of m below this one
-        const unsigned mm = m & lt;
-        const int x = __shfl_sync(WS_FULL_MASK, v, mm ? 31 - __clz((int)mm) : l);
-        return mm ? x : -1;
-    };
-    auto above = [&](unsigned m, int v) {   // v of the lowest lane of m above this one
-        const unsigned mm = m & gt;
-        const int x = __shfl_sync(WS_FULL_MASK, v, mm ? __ffs((int)mm) - 1 : l);
-        return mm ? x : BIG;
-    };
-    Around r;
-    r.pS = below(bS, myLS);
-    r.pR = below(bR, myLR);
-    r.nS = above(bS, myFS);
-    r.nR = above(bR, myFR);
-    // the warp's own last / first points of each set
-    const int wLS = __shfl_sync(WS_FULL_MASK, myLS, bS ? 31 - __clz((int)bS) : 0);
-    const int wLR = __shfl_sync(WS_FULL_MASK, myLR, bR ? 31 - __clz((int)bR) : 0);
-    const int wFS = __shfl_sync(WS_FULL_MASK, myFS, bS ? __ffs((int)bS) - 1 : 0);
-    const int wFR = __shfl_sync(WS_FULL_MASK, myFR, bR ? __ffs((int)bR) - 1 : 0);
-    if (l == 0) {
-        s.wl[w] = bS ? wLS : -1;
-        s.wlr[w] = bR ? wLR : -1;
-        s.wf[w] = bS ? wFS : BIG;
-        s.wfr[w] = bR ? wFR : BIG;
+    if (bS == 0) {
+        if (l == 0) { s.wl[buf][w] = -1; s.wf[buf][w] = BIG; }
+        return;
     }
-    __syncthreads();
-    int wl[NW], wlr[NW], wf[NW], wfr[NW];
+    if (l == 31 - __clz((int)bS)) s.wl[buf][w] = first + 31 - __clz((int)B);
+    if (l == __ffs((int)bS) - 1) s.wf[buf][w] = first + __ffs((int)B) - 1;
+}
+
+// For this lane's range of points: the last boundary before it and the first
+// one after it, over the whole CTA: inside the warp by one ballot and two
+// shuffles, across warps from the posted ends.
+struct Around { int pS, nS; };
+__device__ __forceinline__ Around around(const Smem& s, int t, int first, uint32_t B, int buf) {
+    const int l = t & 31, w = t >> 5;
+    const int myL = B ? first + 31 - __clz((int)B) : -1, myF = B ? first + __ffs((int)B) - 1 : BIG;
+    const unsigned bS = __ballot_sync(WS_FULL_MASK, B != 0);
+    const unsigned lo = bS & ((1u << l) - 1u), hi = l == 31 ? 0u : bS & ~((2u << l) - 1u);
+    const int x = __shfl_sync(WS_FULL_MASK, myL, lo ? 31 - __clz((int)lo) : l);
+    const int y = __shfl_sync(WS_FULL_MASK, myF, hi ? __ffs((int)hi) - 1 : l);
+    Around r;
+    r.pS = lo ? x : -1;
+    r.nS = hi ? y : BIG;
+    int wl[NW], wf[NW];
 #pragma unroll
     for (int j = 0; j < NW / 4; ++j) {
-        const int4 a = reinterpret_cast<const int4*>(s.wl)[j], b = reinterpret_cast<const int4*>(s.wlr)[j];
-        const int4 c = reinterpret_cast<const int4*>(s.wf)[j], d = reinterpret_cast<const int4*>(s.wfr)[j];
+        const int4 a = reinterpret_cast<const int4*>(s.wl[buf])[j], c = reinterpret_cast<const int4*>(s.wf[buf])[j];
         wl[4 * j] = a.x; wl[4 * j + 1] = a.y; wl[4 * j + 2] = a.z; wl[4 * j + 3] = a.w;
-        wlr[4 * j] = b.x; wlr[4 * j + 1] = b.y; wlr[4 * j + 2] = b.z; wlr[4 * j + 3] = b.w;
         wf[4 * j] = c.x; wf[4 * j + 1] = c.y; wf[4 * j + 2] = c.z; wf[4 * j + 3] = c.w;
-        wfr[4 * j] = d.x; wfr[4 * j + 1] = d.y; wfr[4 * j + 2] = d.z; wfr[4 * j + 3] = d.w;
     }
 #pragma unroll
     for (int k = 0; k < NW; ++k) {
-        if (k < w) { r.pS = max(r.pS, wl[k]); r.pR = max(r.pR, wlr[k]); }
-        if (k > w) { r.nS = min(r.nS, wf[k]); r.nR = min(r.nR, wfr[k]); }
+        if (k < w) r.pS = max(r.pS, wl[k]);
+        if (k > w) r.nS = min(r.nS, wf[k]);
     }
     return r;
 }
@@ -591,67 +582,71 @@ __device__ __forceinline__ Around around(Smem& s, int t, int first, uint32_t B, 
 __device__ __forceinline__ bool ic_rounds(Smem& s, const Test& T, int t, int first, int n, uint32_t& B, int cap,
                                           int& rounds) {
     rounds = 1;
+    post_ends(s, t, first, B, 0);
     if (!__syncthreads_or(B != 0)) { rounds = 2; return true; }   // one block: the chord (round 2 has nothing to do)
-    uint32_t D = B, Rprev = 0;
-    const int BIG = 1 << 20;
+    int lastP = -1, lastN = -1, buf = 0;
+    auto point = [&](uint32_t bit) { return first + __ffs((int)bit) - 1; };
     while (true) {
         ++rounds;
-        // neighbouring boundaries outside this lane's range, and where last
-        // round's removals were
-        const Around ar = around(s, t, first, B, Rprev);
-        const int pS = ar.pS, nS = ar.nS, pR = ar.pR, nR = ar.nR;
-        const int prevS = pS < 0 ? 0 : pS, nextS = nS >= BIG ? n : nS;
-        // the end survivors' outer neighbours changed if a removal lay between
-        if (B) {
-            if (pR > prevS) D |= B & (0u - B);
-            if (nR < nextS) D |= 1u << (31 - __clz((int)B));
-        }
-        // decide every boundary to retest against the current blocks
-        uint32_t Rm = 0, bits = B & D;
-        if (rounds == 2 && B) {
-            // all of them: a boundary's prefix sums serve its neighbours' tests too
-            bits = 0;
-            uint32_t rest = B;
-            int a = prevS, p = first + __ffs((int)rest) - 1;
-            int64_t Xa = xat(s, a), Xp = xat(s, p);
-            while (rest) {
-                const uint32_t bit = rest & (0u - rest);
-                rest &= rest - 1;
-                const int c = rest ? first + __ffs((int)rest) - 1 : nextS;
-                const int64_t Xc = xat(s, c);
-                if (!T(a, Xa, p, Xp, c, Xc)) Rm |= bit;
-                a = p; Xa = Xp;
-                p = c; Xp = Xc;
+        const Around ar = around(s, t, first, B, buf);
+        const int prevS = ar.pS < 0 ? 0 : ar.pS, nextS = ar.nS >= BIG ? n : ar.nS;
+        const uint32_t B0 = B;
+        if (rounds == 2) {
+            if (B) {
+                // the lane's boundaries from left to right; keep: those that
+                // stand so far, b the last of them and a the one before it
+                uint32_t rest = B, keep = rest & (0u - rest);
+                rest ^= keep;
+                int a = prevS, b = point(keep);
+                int64_t Xa = xat(s, a), Xb = xat(s, b);
+                while (true) {
+                    const uint32_t bit = rest & (0u - rest);
+                    const int c = rest ? point(bit) : nextS;
+                    const int64_t Xc = xat(s, c);
+                    bool empty = false;
+                    while (!T(a, Xa, b, Xb, c, Xc)) {
+                        keep ^= 0x80000000u >> __clz((int)keep);
+                        if (!keep) { empty = true; break; }
+                        b = a; Xb = Xa;
+                        const uint32_t below = keep ^ (0x80000000u >> __clz((int)keep));
+                        a = below ? first + 31 - __clz((int)below) : prevS;
+                        Xa = xat(s, a);
+                    }
+                    if (!rest) break;
+                    rest ^= bit;
+                    keep |= bit;
+                    if (empty) { a = prevS; Xa = xat(s, a); }
+                    else { a = b; Xa = Xb; }
+                    b = c; Xb = Xc;
+                }
+                B = keep;
+            }
+        } else {
+            if (B && prevS != lastP) {   // from the left end
+                const int64_t Xa = xat(s, prevS);
+                while (B) {
+                    const uint32_t bit = B & (0u - B), rest = B ^ bit;
+                    const int b = point(bit), c = rest ? point(rest & (0u - rest)) : nextS;
+                    if (T(prevS, Xa, b, xat(s, b), c, xat(s, c))) break;
+                    B = rest;
+                }
+            }
+            if (B && nextS != lastN) {   // from the right end
+                const int64_t Xc = xat(s, nextS);
+                while (B) {
+                    const uint32_t bit = 0x80000000u >> __clz((int)B), rest = B ^ bit;
+                    const int b = point(bit), a = rest ? first + 31 - __clz((int)rest) : prevS;
+                    if (T(a, xat(s, a), b, xat(s, b), nextS, Xc)) break;
+                    B = rest;
+                }
             }
         }
-        while (bits) {
-            const int i = __ffs((int)bits) - 1;
-            bits &= bits - 1;
-            const int p = first + i;
-            const uint32_t below = B & ((1u << i) - 1u), above = B & ~((2u << i) - 1u);
-            const int a = below ? first + 31 - __clz((int)below) : prevS;
-            const int c = above ? first + __ffs((int)above) - 1 : nextS;
-            if (!T(a, xat(s, a), p, xat(s, p), c, xat(s, c))) Rm |= 1u << i;
-        }
-        if (!__syncthreads_or(Rm != 0)) return true;
+        lastP = prevS;
+        lastN = nextS;
+        buf ^= 1;
+        post_ends(s, t, first, B, buf);
+        if (!__syncthreads_or(B != B0)) return true;
         if (rounds >= cap) return false;
-        // survivors whose in-lane neighbourhood changed
-        const uint32_t B2 = B & ~Rm;
-        D = 0;
-        {
-            uint32_t rest = B2;
-            int pq = -1;
-            while (rest) {
-                const int q = __ffs((int)rest) - 1;
-                rest &= rest - 1;
-                const uint32_t gap = ((1u << q) - 1u) & (pq >= 0 ? ~((2u << pq) - 1u) : 0xffffffffu);
-                if (Rm & gap) { D |= 1u << q; if (pq >= 0) D |= 1u << pq; }
-                pq = q;
-            }
-            if (pq >= 0 && (Rm & ~((2u << pq) - 1u))) D |= 1u << pq;   // removal above the last survivor
-        }
-        Rprev = Rm;
-        B = B2;
     }
 }
 
@@ -669,8 +664,9 @@ __device__ __forceinline__ bool ic_rounds(Smem& s, const Test& T, int t, int fir
 // this.
 __device__ __forceinline__ uint32_t candidate_boundaries(Smem& s, const Test& T, int t, int first, int n,
                                                          uint32_t R, uint32_t G) {
-    const int BIG = 1 << 20;
-    const Around ar = around(s, t, first, R, 0u);
+    post_ends(s, t, first, R, 0);
+    __syncthreads();
+    const Around ar = around(s, t, first, R, 0);
     const int pS = ar.pS, nS = ar.nS;
     const int prevS = pS < 0 ? 0 : pS, nextS = nS >= BIG ? n : nS;
     // interior points of this lane: 1 <= p <= n - 1 and not a run boundary
@@ -690,6 +686,7 @@ __device__ __forceinline__ uint32_t candidate_boundaries(Smem& s, const Test& T,
         const int c = above ? first + __ffs((int)above) - 1 : nextS;
         if (T(a, xat(s, a), p, xat(s, p), c, xat(s, c))) F |= 1u << i;
     }
+    __syncthreads();   // (the posted ends are read; the rounds post theirs in the same place)
     return (R & G) | F;
 }
 
