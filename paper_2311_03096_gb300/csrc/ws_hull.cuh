@@ -579,9 +579,13 @@ __device__ __forceinline__ Around around(const Smem& s, int t, int first, uint32
 // (rounds = rounds run, the final unchanged one included).  Prefix sums of
 // every point must be in s.X (the first barrier here publishes them).  All
 // threads of the CTA call this.
+// prev, next: on convergence the last boundary before the lane's range (0 if
+// none) and the first one after it (n if none).
 __device__ __forceinline__ bool ic_rounds(Smem& s, const Test& T, int t, int first, int n, uint32_t& B, int cap,
-                                          int& rounds) {
+                                          int& rounds, int& prev, int& next) {
     rounds = 1;
+    prev = 0;
+    next = n;
     post_ends(s, t, first, B, 0);
     if (!__syncthreads_or(B != 0)) { rounds = 2; return true; }   // one block: the chord (round 2 has nothing to do)
     int lastP = -1, lastN = -1, buf = 0;
@@ -645,7 +649,7 @@ __device__ __forceinline__ bool ic_rounds(Smem& s, const Test& T, int t, int fir
         lastN = nextS;
         buf ^= 1;
         post_ends(s, t, first, B, buf);
-        if (!__syncthreads_or(B != B0)) return true;
+        if (!__syncthreads_or(B != B0)) { prev = prevS; next = nextS; return true; }
         if (rounds >= cap) return false;
     }
 }

@@ -269,6 +269,11 @@ __global__ void __launch_bounds__(NT, 3) k_small_general(const T* __restrict__ v
 // cluster-start bitmap, values scattered back through the positions.
 // Segments whose prefix sums need 128 bits (or whose bridge walks are too
 // long) are appended to gen_list for the general kernel above.
+// Bound by issue (0.6; 460 thread instructions per weight) and the barriers
+// between its phases.  Rows of the MLP (8202 of 3072 or 4096, lambda 1e-3 .. 1):
+// 809 us with three CTAs per SM (74 KB of shared memory, 80 registers), one
+// decision per boundary and round and a value loop that searched the bitmap;
+// 676 with the rounds of ws_hull.cuh, 601 with four CTAs (57 KB, 64 registers).
 // ---------------------------------------------------------------------------
 template <typename T>
 struct LeanSmem {
@@ -278,21 +283,24 @@ struct LeanSmem {
     // (keys: one slot per 16, 16-bit arrays: two) so those reads do not
     // collide in the shared-memory banks; see kpad / ipad.
     uint16_t idx[CAP + CAP / 8];                        // original position of every sorted element
-    union {
-        K keys[CAP + CAP / 16];                        // the sort, until the hull starts
-        T vals[CAP];                                    // cluster values, after it
-    } kv;
+    // One after the other: the sort; the prefix sums and the rounds.  At the
+    // end the prefix-sum slot of a cluster's first point takes the cluster's
+    // value (FP32: and id), and the lane stacks' storage the first point of
+    // every original position's cluster.  Four CTAs then fit on an SM (FP32).
     union {
         struct {
-            uint32_t whist[(wsh::NT / 32) * 256];
-            uint32_t dcount[256], dstart[256];
+            K keys[CAP + CAP / 16];
+            union {
+                uint32_t cnt[CAP + CAP / 16];   // bucket counts, then starts: two per word (words padded like the keys: kpad)
+                struct {
+                    uint32_t whist[(wsh::NT / 32) * 256];
+                    uint32_t dcount[256], dstart[256];
+                } radix;
+            };
         } sort;
-        struct {
-            int cnt[CAP + CAP / 16];   // bucket counts, then starts (padded like the keys: kpad)
-        } bucket;
         wsh::Smem h;
-        uint16_t cid_of[CAP + CAP / 8];   // cluster of every original position (after the values)
     } u;
+    uint16_t cid[sizeof(T) == 8 ? CAP : 1];   // FP64: cluster id by first point
     K kmin, kmax;
     int bmax;
     int wsumi[wsh::NT / 32];
@@ -301,6 +309,7 @@ struct LeanSmem {
     SegConst sc;    // the segment's global fixed-point scale (cluster values)
     int64_t t11;    // round-1 gap threshold (tile units)
     int flags, emin;
+    int inexact;    // the fixed point truncates some values
 };
 
 // Exclusive scan of one int per thread over the CTA with a single barrier:
@@ -330,7 +339,7 @@ __device__ __forceinline__ int lean_ipad(int p) { return p + ((p >> 4) << 1); } 
 // stays compact in the instruction cache.  All threads of the CTA call each.
 
 // LSD radix sort, 8-bit digits, of the n (key, original position) pairs in
-// s.kv.keys / s.idx (any order on entry; sorted on return).  Every pass takes
+// s.u.sort.keys / s.idx (any order on entry; sorted on return).  Every pass takes
 // position w*32*M + k*32 + l of the previous one, which the stable ranking
 // keeps in order.
 template <typename T>
@@ -349,15 +358,15 @@ __device__ __noinline__ void small_radix(LeanSmem<T>& s, int n) {
         for (int k = 0; k < M; ++k) {
             const int p = w * 32 * M + k * 32 + l;
             valid[k] = p < n;
-            key[k] = valid[k] ? s.kv.keys[lean_kpad(p)] : (K)0;
+            key[k] = valid[k] ? s.u.sort.keys[lean_kpad(p)] : (K)0;
             ii[k] = valid[k] ? s.idx[lean_ipad(p)] : (uint16_t)0;
             dg[k] = (uint32_t)((key[k] >> (8 * pass)) & 0xff);
         }
         __syncthreads();
-        ws_rank_digits<NT, M, 1>(dg, valid, pos, s.u.sort.whist, s.u.sort.dcount, s.u.sort.dstart);
+        ws_rank_digits<NT, M, 1>(dg, valid, pos, s.u.sort.radix.whist, s.u.sort.radix.dcount, s.u.sort.radix.dstart);
 #pragma unroll
         for (int k = 0; k < M; ++k)
-            if (valid[k]) { s.kv.keys[lean_kpad(pos[k])] = key[k]; s.idx[lean_ipad(pos[k])] = ii[k]; }
+            if (valid[k]) { s.u.sort.keys[lean_kpad(pos[k])] = key[k]; s.idx[lean_ipad(pos[k])] = ii[k]; }
         __syncthreads();
     }
 }
@@ -372,15 +381,16 @@ __device__ __noinline__ void small_chain_tree(wsh::Smem& h, const wsh::Test& tst
 // Warm start: the runs of equal earlier cluster ids (low 16 bits; any values
 // are valid) along the sorted order, then candidate_boundaries on the
 // round-1 survivors G.  The earlier
-// ids are staged by original position in `cprev` (the keys' storage: the
-// keys are in registers by now).  Prefix sums of every point must be written
+// ids are staged by original position in `cprev` (the lane stacks' storage,
+// which only a segment whose rounds hit their cap uses, later).  Prefix sums of every point must be written
 // (the barriers here publish them).
 template <typename T>
 __device__ __noinline__ uint32_t small_warm(LeanSmem<T>& s, const wsh::Test& tst, const int32_t* ids_prev,
                                             int64_t a0, int first, int n, uint32_t G) {
     constexpr int M = wsh::M;
     const int t = threadIdx.x;
-    uint16_t* cprev = reinterpret_cast<uint16_t*>(s.kv.keys);
+    uint16_t* cprev = s.u.h.st;   // (st, lo and hi are one run of 16-bit words)
+    static_assert(sizeof(s.u.h.st) + sizeof(s.u.h.lo) + sizeof(s.u.h.hi) >= sizeof(s.idx), "the earlier ids fit");
     if (first < n) {
         const int32_t* src = ids_prev + a0 + first;
         if (first + M <= n && (((uintptr_t)src) & 15) == 0) {
@@ -414,8 +424,16 @@ __device__ __noinline__ uint32_t small_warm(LeanSmem<T>& s, const wsh::Test& tst
     return wsh::candidate_boundaries(s.u.h, tst, t, first, n, R, G);
 }
 
+// A cluster's value from its exact 128-bit sum (FP64 arithmetic or storage).
 template <typename T>
-__global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 3 : 2) k_small(const T* __restrict__ values,
+__device__ __noinline__ T small_value(int64_t xd, int a, int b, int64_t q0, int up, T xs, const SegConst* sc,
+                                      bool fp64, const WsEpi* ep) {
+    const i128 SX = (i128)(b - a) * (i128)q0 + ((i128)xd << up);
+    return ValueOut<T>::value(SX, a, b, xs, *sc, fp64, *ep);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 4 : 2) k_small(const T* __restrict__ values,
                                                    const int64_t* __restrict__ offsets,
                                                    const int32_t* __restrict__ seg_list,
                                                    const double* __restrict__ lambdas, T* out, int32_t* ids,
@@ -499,10 +517,11 @@ __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 3 : 2) k_small(const
     if (l == 0) atomicMin(&s.emin, emin);
 
     // ---- sort (key, original position).  First an interpolation bucket sort:
-    // bucket(x) = floor((x - x_min) n / (x_max - x_min)) in FP32 is monotone
+    // bucket(x) = floor((x - x_min) 2n / (x_max - x_min)) in FP32 is monotone
     // in x (every step rounds monotonically), so equal keys share a bucket and
     // sorting each bucket by key sorts the segment; for the smooth
-    // distributions of weights a bucket holds a few elements.  If a bucket is
+    // distributions of weights a bucket holds half an element on average (n
+    // buckets: more and larger buckets to sort, rows of the MLP 610 us).  If a bucket is
     // larger than BUCKET_MAX the segment takes the LSD radix passes instead.
     constexpr int BUCKET_MAX = 32;
     {
@@ -515,7 +534,7 @@ __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 3 : 2) k_small(const
             lo = min(lo, ws_shfl_xor_k(lo, o));
             hi = max(hi, ws_shfl_xor_k(hi, o));
         }
-        int* cnt = s.u.bucket.cnt;
+        uint32_t* cnt = s.u.sort.cnt;
         for (int i = t; i < n; i += NT) cnt[kpad(i)] = 0;
         if (l == 0) { ws_atomic_min_k(&s.kmin, lo); ws_atomic_max_k(&s.kmax, hi); }
     }
@@ -526,7 +545,11 @@ __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 3 : 2) k_small(const
     const K kfirst = s.kmin, klast = s.kmax;
     const T xlo = KO::from_key(kfirst), xhi = KO::from_key(klast);
     const int emax = ws_fix_scale<T>(max(ws_eff_exp(xlo), ws_eff_exp(xhi)), s.emin);
-    if (t == 0) ws_note_scale<T>(max(ws_eff_exp(xlo), ws_eff_exp(xhi)), s.emin, status);
+    if (t == 0) {
+        const int top = max(ws_eff_exp(xlo), ws_eff_exp(xhi));
+        ws_note_scale<T>(top, s.emin, status);
+        s.inexact = s.emin <= top && top - s.emin > KO::FIX_OFS;
+    }
     int sh;
     const bool bin = ws_tile_binade<T>(kfirst, klast, n, emax, sh);
     const int64_t q0 = ws_fixed<T>(xlo, emax);
@@ -539,63 +562,68 @@ __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 3 : 2) k_small(const
     }
     bool radix = false;
     {
-        int* cnt = s.u.bucket.cnt;
+        uint32_t* cnt = s.u.sort.cnt;
         const float f0 = (float)KO::from_key(s.kmin), f1 = (float)KO::from_key(s.kmax);
         const float span = f1 - f0;
-        const float scale = (span > 0.0f && span <= 3.0e38f) ? (float)n / span : 0.0f;
-        int bk[M], rk[M];
+        const float scale = (span > 0.0f && span <= 3.0e38f) ? (float)(2 * n) / span : 0.0f;
+        uint32_t br[M];   // bucket << 16 | rank
 #pragma unroll
         for (int i = 0; i < M; ++i) {
             if (first + i < n) {
                 const float f = ((float)KO::from_key(key[i]) - f0) * scale;
-                bk[i] = min(n - 1, max(0, (int)f));
-                rk[i] = atomicAdd(&cnt[kpad(bk[i])], 1);
+                const uint32_t b = (uint32_t)min(2 * n - 1, max(0, (int)f));
+                const uint32_t up = (b & 1u) << 4;
+                const uint32_t old = atomicAdd(&cnt[kpad((int)(b >> 1))], 1u << up);
+                br[i] = (b << 16) | ((old >> up) & 0xffffu);
             }
         }
         __syncthreads();
-        // bucket starts: this thread's 16 consecutive buckets, then the CTA scan
-        int c[M], sum = 0, big = 0;
+        // bucket starts: this thread's 32 consecutive buckets, then the CTA scan
+        uint32_t c[M], multi = 0;   // (multi: bit j, bucket 2 first + j holds two or more)
+        int sum = 0, big = 0;
 #pragma unroll
         for (int i = 0; i < M; ++i) {
-            c[i] = (first + i < n) ? cnt[kpad(first + i)] : 0;
-            sum += c[i];
-            big = max(big, c[i]);
+            c[i] = (first + i < n) ? cnt[kpad(first + i)] : 0u;
+            const int c0 = (int)(c[i] & 0xffffu), c1 = (int)(c[i] >> 16);
+            sum += c0 + c1;
+            big = max(big, max(c0, c1));
+            multi |= (c0 >= 2 ? 1u : 0u) << (2 * i) | (c1 >= 2 ? 2u : 0u) << (2 * i);
         }
         int tot;
         int run = lean_excl_scan(sum, s.wsumi, &tot);
 #pragma unroll
         for (int i = 0; i < M; ++i)
-            if (first + i < n) { cnt[kpad(first + i)] = run; run += c[i]; }
+            if (first + i < n) {
+                const uint32_t mid = (uint32_t)run + (c[i] & 0xffffu);
+                cnt[kpad(first + i)] = (uint32_t)run | (mid << 16);
+                run = (int)(mid + (c[i] >> 16));
+            }
         radix = __syncthreads_or(big > BUCKET_MAX);
         if (!radix) {
+            auto start_of_bucket = [&](int b) { return (int)((cnt[kpad(b >> 1)] >> ((b & 1) << 4)) & 0xffffu); };
 #pragma unroll
             for (int i = 0; i < M; ++i)
                 if (first + i < n) {
-                    const int pp = cnt[kpad(bk[i])] + rk[i];
-                    s.kv.keys[kpad(pp)] = key[i];
+                    const int pp = start_of_bucket((int)(br[i] >> 16)) + (int)(br[i] & 0xffffu);
+                    s.u.sort.keys[kpad(pp)] = key[i];
                     s.idx[ipad(pp)] = (uint16_t)(first + i);
                 }
             __syncthreads();
             // each bucket by key (ties may end in any order): up to four
             // elements by a sorting network in registers, larger buckets by
-            // insertion in shared memory.  Bucket ends from the starts (no
-            // indexing of c[] by a loop variable: it would live in local memory).
-            uint32_t multi = 0;
-#pragma unroll
-            for (int i = 0; i < M; ++i)
-                if (first + i < n && c[i] >= 2) multi |= 1u << i;
+            // insertion in shared memory
             while (multi) {
-                const int i = __ffs((int)multi) - 1;
+                const int i = 2 * first + __ffs((int)multi) - 1;
                 multi &= multi - 1;
-                const int b0 = cnt[kpad(first + i)];
-                const int b1 = first + i + 1 < n ? cnt[kpad(first + i + 1)] : n;
+                const int b0 = start_of_bucket(i);
+                const int b1 = i + 1 < 2 * n ? start_of_bucket(i + 1) : n;
                 if (b1 - b0 <= 4) {
                     K k[4];
                     uint16_t x[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         const bool in = b0 + j < b1;
-                        k[j] = in ? s.kv.keys[kpad(b0 + j)] : ~(K)0;
+                        k[j] = in ? s.u.sort.keys[kpad(b0 + j)] : ~(K)0;
                         x[j] = in ? s.idx[ipad(b0 + j)] : (uint16_t)0;
                     }
                     auto cs = [&](int a, int b) {
@@ -607,19 +635,19 @@ __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 3 : 2) k_small(const
                     cs(0, 1); cs(2, 3); cs(0, 2); cs(1, 3); cs(1, 2);
 #pragma unroll
                     for (int j = 0; j < 4; ++j)
-                        if (b0 + j < b1) { s.kv.keys[kpad(b0 + j)] = k[j]; s.idx[ipad(b0 + j)] = x[j]; }
+                        if (b0 + j < b1) { s.u.sort.keys[kpad(b0 + j)] = k[j]; s.idx[ipad(b0 + j)] = x[j]; }
                     continue;
                 }
                 for (int a = b0 + 1; a < b1; ++a) {
-                    const K kk = s.kv.keys[kpad(a)];
+                    const K kk = s.u.sort.keys[kpad(a)];
                     const uint16_t ii = s.idx[ipad(a)];
                     int j = a - 1;
-                    while (j >= b0 && s.kv.keys[kpad(j)] > kk) {
-                        s.kv.keys[kpad(j + 1)] = s.kv.keys[kpad(j)];
+                    while (j >= b0 && s.u.sort.keys[kpad(j)] > kk) {
+                        s.u.sort.keys[kpad(j + 1)] = s.u.sort.keys[kpad(j)];
                         s.idx[ipad(j + 1)] = s.idx[ipad(j)];
                         --j;
                     }
-                    s.kv.keys[kpad(j + 1)] = kk;
+                    s.u.sort.keys[kpad(j + 1)] = kk;
                     s.idx[ipad(j + 1)] = ii;
                 }
             }
@@ -630,7 +658,7 @@ __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 3 : 2) k_small(const
     if (radix) {
 #pragma unroll
         for (int k = 0; k < M; ++k)
-            if (first + k < n) { s.kv.keys[kpad(first + k)] = key[k]; s.idx[ipad(first + k)] = (uint16_t)(first + k); }
+            if (first + k < n) { s.u.sort.keys[kpad(first + k)] = key[k]; s.idx[ipad(first + k)] = (uint16_t)(first + k); }
         __syncthreads();
         small_radix<T>(s, n);
     }
@@ -638,8 +666,9 @@ __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 3 : 2) k_small(const
     // ---- the sorted segment as one hull tile: this thread's 16 sorted keys
     K kr[M];
 #pragma unroll
-    for (int i = 0; i < M; ++i) kr[i] = (first + i < n) ? s.kv.keys[kpad(first + i)] : s.kv.keys[0];
-    const K kprev = (t > 0 && first < n) ? s.kv.keys[kpad(first - 1)] : kfirst;
+    for (int i = 0; i < M; ++i) kr[i] = (first + i < n) ? s.u.sort.keys[kpad(first + i)] : s.u.sort.keys[0];
+    const K kprev = (t > 0 && first < n) ? s.u.sort.keys[kpad(first - 1)] : kfirst;
+    __syncthreads();   // (the keys are read; the prefix sums take their place)
     if (t == 0) {   // (no FP64 on this critical path)
         s.sc = ws_seg_const_f(n, lam, KO::L_BASE - emax, fp64 != 0);
         TileScale& ts = s.ts;
@@ -712,9 +741,9 @@ __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 3 : 2) k_small(const
         }
     }
     if (ids_prev) B = small_warm<T>(s, tst, ids_prev, a0, first, n, B);
-    int rounds = 0;
+    int rounds = 0, prev = 0, next = n;
     bool converged = false;
-    if (ic_cap > 0) converged = wsh::ic_rounds(h, tst, t, first, n, B, ic_cap, rounds);
+    if (ic_cap > 0) converged = wsh::ic_rounds(h, tst, t, first, n, B, ic_cap, rounds, prev, next);
     uint16_t* st16 = reinterpret_cast<uint16_t*>(s.starts);
     if (converged) {
         st16[t] = (uint16_t)(B | (t == 0 ? 1u : 0u));
@@ -732,50 +761,87 @@ __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 3 : 2) k_small(const
     const uint32_t mine = (uint32_t)st16[t] & (first < n ? (n - first >= M ? 0xffffu : ((1u << (n - first)) - 1u)) : 0u);
     int C;
     const int base = lean_excl_scan(__popc(mine), h.wsum, &C);
-    const float x0f = (float)xlo;
-    {
-        uint32_t rest = mine;
-        int r = base;
-        while (rest) {
-            const int i = __ffs((int)rest) - 1;
-            rest &= rest - 1;
-            const int a = first + i;
-            // end of the cluster: the next start (in this thread, else the next set bit of the bitmap), or n
-            int b = n;
-            if (rest) b = first + __ffs((int)rest) - 1;
-            else {
-                for (int wd = (first + M) >> 5; (wd << 5) < n; ++wd) {
-                    uint32_t bits = s.starts[wd];
-                    if ((wd << 5) < first + M) bits &= 0xffffffffu << ((first + M) & 31);
-                    if (bits) { b = min((wd << 5) + __ffs((int)bits) - 1, n); break; }
-                }
-            }
-            const int64_t xd = wsh::xat(h, b) - wsh::xat(h, a);
-            K ki = kr[0];   // kr[i] by selects (a loop-variable index would put kr in local memory)
-#pragma unroll
-            for (int j = 1; j < M; ++j) ki = (i == j) ? kr[j] : ki;
-            if (KO::BITS == 32 && !fp64) {
-                // FP32: mean = x_0 + (deviation sum / count) in tile units; every
-                // term exact but the conversions (a few FP32 ulps of max |w|)
-                const float xa = (float)KO::from_key(ki);
-                const float mean = (b - a == 1) ? xa
-                                                : x0f + ldexpf(ws_u64_to_float((uint64_t)xd) / (float)(b - a), -s.ts.sc.L);
-                s.kv.vals[r] = (T)ws_epilogue<float>(mean, s.sc.mu_f * (float)(n - a - b), ep.beta_f, ep.gamma_f,
-                                                     ep.on != 0);
-            } else {
-                const i128 SX = (i128)(b - a) * (i128)q0 + (bin ? ((i128)xd << sh) : (i128)xd);
-                s.kv.vals[r] = ValueOut<T>::value(SX, a, b, KO::from_key(ki), s.sc, fp64 != 0, ep);
-            }
-            ++r;
+    // neighbouring starts outside this thread's chunk
+    if (!converged) {
+        next = n;
+        for (int wd = (first + M) >> 5; (wd << 5) < n; ++wd) {
+            uint32_t bits = s.starts[wd];
+            if ((wd << 5) < first + M) bits &= 0xffffffffu << ((first + M) & 31);
+            if (bits) { next = min((wd << 5) + __ffs((int)bits) - 1, n); break; }
+        }
+        prev = 0;   // (position 0 is a start)
+        for (int wd = min(first, n) >> 5; wd >= 0; --wd) {
+            uint32_t bits = s.starts[wd];
+            if ((wd << 5) + 31 >= first) bits &= (1u << (first & 31)) - 1u;
+            if (bits) { prev = (wd << 5) + 31 - __clz((int)bits); break; }
         }
     }
-    __syncthreads();   // (the prefix sums are dead: their storage takes the cluster of every position)
-    // ---- the cluster of every original position, then this thread's 16
-    // consecutive outputs (coalesced stores)
+    // ---- the value of every cluster, into the slot of its first point.  That
+    // slot is read as the end of the cluster before it, by this thread except
+    // for its first start, which waits for the barrier.
+    auto put = [&](int a, T val, int r) {
+        if (sizeof(T) == 4) *reinterpret_cast<uint2*>(&wsh::xref(h, a)) = make_uint2(__float_as_uint((float)val), (uint32_t)r);
+        else { *reinterpret_cast<double*>(&wsh::xref(h, a)) = (double)val; s.cid[a] = (uint16_t)r; }
+    };
+    T v0 = (T)0;
+    if (mine) {
+        const int Lt = s.ts.sc.L;
+        // 2^-L as a factor where it is a normal number (then x 2^-L rounds as ldexpf does)
+        const bool fac = Lt >= -126 && Lt <= 126;
+        const float down = fac ? __uint_as_float((uint32_t)(127 - Lt) << 23) : 0.0f;
+        const bool inexact = s.inexact != 0;
+        const float mu_f = s.sc.mu_f, x0f = (float)xlo;
+        uint32_t rest = mine;
+        int a = first + __ffs((int)rest) - 1, r = base;
+        int64_t Xa = wsh::xat(h, a);
+        rest &= rest - 1;
+        while (true) {
+            const int b = rest ? first + __ffs((int)rest) - 1 : next;
+            const int64_t Xb = wsh::xat(h, b), xd = Xb - Xa;
+            T val;
+            if (KO::BITS == 32 && !fp64) {
+                // FP32: mean = x_0 + (deviation sum / count) in tile units; every
+                // term exact but the conversions (a few FP32 ulps of max |w|).
+                // A single weight comes back exactly from its deviation.
+                float mean;
+                if (b - a == 1) {
+                    if (bin) mean = (float)KO::from_key((K)(kfirst + (K)xd));
+                    else if (!inexact && fac && q0 + xd != 0) {   // (zeros keep their sign)
+                        const int64_t q = q0 + xd;
+                        const float f = ws_u64_to_float((uint64_t)(q < 0 ? -q : q));
+                        mean = (q < 0 ? -f : f) * down;
+                    } else mean = (float)values[a0 + s.idx[ipad(a)]];
+                } else {
+                    const float f = ws_u64_to_float((uint64_t)xd) / (float)(b - a);
+                    mean = x0f + (fac ? f * down : ldexpf(f, -Lt));
+                }
+                val = (T)ws_epilogue<float>(mean, mu_f * (float)(n - a - b), ep.beta_f, ep.gamma_f, ep.on != 0);
+            } else {
+                const T xs = b - a == 1 ? values[a0 + s.idx[ipad(a)]] : (T)0;
+                val = small_value<T>(xd, a, b, q0, bin ? sh : 0, xs, &s.sc, fp64 != 0, &ep);
+            }
+            if (r == base) v0 = val;
+            else put(a, val, r);
+            if (!rest) break;
+            rest &= rest - 1;
+            ++r;
+            a = b;
+            Xa = Xb;
+        }
+    }
+    __syncthreads();   // (every prefix sum is read)
+    if (mine) put(first + __ffs((int)mine) - 1, v0, base);
+    // ---- the cluster (its first point) of every original position, then this
+    // thread's 16 consecutive outputs (coalesced stores)
+    uint16_t* start_of = h.st;   // (st, lo and hi are one run of 16-bit words)
+    {
+        int a = prev;
 #pragma unroll
-    for (int i = 0; i < M; ++i) {
-        const int p = first + i;
-        if (p < n) s.u.cid_of[ipad(s.idx[ipad(p)])] = (uint16_t)(base + __popc(mine & ((2u << i) - 1u)) - 1);
+        for (int i = 0; i < M; ++i) {
+            const int p = first + i;
+            if ((mine >> i) & 1u) a = p;
+            if (p < n) start_of[ipad(s.idx[ipad(p)])] = (uint16_t)a;
+        }
     }
     __syncthreads();
     if (first < n) {
@@ -783,9 +849,15 @@ __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 3 : 2) k_small(const
         int32_t oi[M];
 #pragma unroll
         for (int i = 0; i < M; ++i) {
-            const int c = (first + i < n) ? (int)s.u.cid_of[ipad(first + i)] : 0;
-            oi[i] = c;
-            ov[i] = s.kv.vals[c];
+            const int a = (first + i < n) ? (int)start_of[ipad(first + i)] : 0;
+            if (sizeof(T) == 4) {
+                const uint2 q = *reinterpret_cast<const uint2*>(&wsh::xref(h, a));
+                ov[i] = (T)__uint_as_float(q.x);
+                oi[i] = (int32_t)q.y;
+            } else {
+                ov[i] = (T)*reinterpret_cast<const double*>(&wsh::xref(h, a));
+                oi[i] = (int32_t)s.cid[a];
+            }
         }
         T* od = out + a0 + first;
         int32_t* id = ids ? ids + a0 + first : nullptr;
