@@ -566,7 +566,7 @@ __global__ void __launch_bounds__(HNT, 4) k_tile_hull(const typename KeyOf<T>::K
         P.thr = s.hull.thr;
         ws_cta_hull<HNT, HM>(s.hull, n, P, s.sc, &nv);
     } else {
-        const TilePtsWide<HM> P{s.pre.s64, s.pre.base};
+        const TilePtsWide<HM> P{s.pre.s64, s.pre.base, s.muq, s.fast != 0};
         ws_cta_hull<HNT, HM>(s.hull, n, P, s.sc, &nv);
     }
     {

@@ -27,9 +27,11 @@ struct SmallSmem {
             uint32_t whist[(NT / 32) * 256];
             uint32_t dcount[256], dstart[256];
         } sort;
+        uint32_t cnt[CAP];              // bucket counts, then starts: two per word
         struct {
             uint16_t V[CAP + 2];        // hull vertices (points)
             uint32_t mark[CAP / 32];    // bit p: a cluster starts at sorted position p
+            uint16_t multi[CAP / 2];    // clusters of two or more elements
         } ids;
     } r1;
     union {
@@ -38,12 +40,54 @@ struct SmallSmem {
         T val[CAP];
     } r2;
     int wsum_i[NT / 32];
+    K kmin, kmax;
     int flags;
     int emin;
+    int n_multi;
     SegConst sc, sct;
     float muq, muqt;
     int fast, fastt;
 };
+
+// One bucket of the interpolation bucket sort, entries [b0, b1) of (keys, idx)
+// through the slot maps kp and ip, by key (ties may end in any order): up to
+// four entries by a sorting network in registers, more by insertion.
+template <typename K, typename KP, typename IP>
+__device__ __forceinline__ void small_sort_bucket(int b0, int b1, K* keys, uint16_t* idx, KP kp, IP ip) {
+    if (b1 - b0 <= 4) {
+        K k[4];
+        uint16_t x[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const bool in = b0 + j < b1;
+            k[j] = in ? keys[kp(b0 + j)] : ~(K)0;
+            x[j] = in ? idx[ip(b0 + j)] : (uint16_t)0;
+        }
+        auto cs = [&](int a, int b) {
+            const bool sw = k[a] > k[b];
+            const K ka = sw ? k[b] : k[a], kb = sw ? k[a] : k[b];
+            const uint16_t xa = sw ? x[b] : x[a], xb = sw ? x[a] : x[b];
+            k[a] = ka; k[b] = kb; x[a] = xa; x[b] = xb;
+        };
+        cs(0, 1); cs(2, 3); cs(0, 2); cs(1, 3); cs(1, 2);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (b0 + j < b1) { keys[kp(b0 + j)] = k[j]; idx[ip(b0 + j)] = x[j]; }
+        return;
+    }
+    for (int a = b0 + 1; a < b1; ++a) {
+        const K kk = keys[kp(a)];
+        const uint16_t ii = idx[ip(a)];
+        int j = a - 1;
+        while (j >= b0 && keys[kp(j)] > kk) {
+            keys[kp(j + 1)] = keys[kp(j)];
+            idx[ip(j + 1)] = idx[ip(j)];
+            --j;
+        }
+        keys[kp(j + 1)] = kk;
+        idx[ip(j + 1)] = ii;
+    }
+}
 
 // The general one-CTA prox of one segment (every input, including values
 // whose fixed-point sums need 128 bits): used for the segments the lean
@@ -105,8 +149,78 @@ __device__ __forceinline__ void small_general_segment(SmallSmem<T, NT, M>& s, in
         return;
     }
 
-    // ---- LSD radix sort of (key, idx) in shared memory, 8-bit digits
-    for (int pass = 0; pass < KO::BITS / 8; ++pass) {
+    // ---- sort (key, idx) in shared memory: the interpolation bucket sort of
+    // k_small (two buckets per element; eight radix passes took 42 us of a
+    // single FP64 segment of 4096), LSD radix passes where a bucket is large
+    bool radix;
+    {
+        K kk[ITEMS], lo = ~(K)0, hi = 0;
+        if (t == 0) { s.kmin = ~(K)0; s.kmax = 0; }
+        for (int i = t; i < n; i += NT) s.r1.cnt[i] = 0;
+#pragma unroll
+        for (int k = 0; k < ITEMS; ++k) {
+            const int p = t + k * NT;
+            kk[k] = p < n ? s.r2.keys[p] : (K)0;
+            if (p < n) { lo = min(lo, kk[k]); hi = max(hi, kk[k]); }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            lo = min(lo, ws_shfl_xor_k(lo, o));
+            hi = max(hi, ws_shfl_xor_k(hi, o));
+        }
+        __syncthreads();
+        if (lane == 0) { ws_atomic_min_k(&s.kmin, lo); ws_atomic_max_k(&s.kmax, hi); }
+        __syncthreads();
+        const float f0 = (float)KO::from_key(s.kmin), span = (float)KO::from_key(s.kmax) - f0;
+        const float scale = (span > 0.0f && span <= 3.0e38f) ? (float)(2 * n) / span : 0.0f;
+        uint32_t br[ITEMS];   // bucket << 16 | rank
+#pragma unroll
+        for (int k = 0; k < ITEMS; ++k) {
+            if (t + k * NT < n) {
+                const float f = ((float)KO::from_key(kk[k]) - f0) * scale;
+                const uint32_t b = (uint32_t)min(2 * n - 1, max(0, (int)f)), up = (b & 1u) << 4;
+                const uint32_t old = atomicAdd(&s.r1.cnt[b >> 1], 1u << up);
+                br[k] = (b << 16) | ((old >> up) & 0xffffu);
+            }
+        }
+        __syncthreads();
+        int sum = 0, big = 0;
+        uint32_t c[M], multi = 0;   // (multi: bit j, bucket 2 t M + j holds two or more)
+#pragma unroll
+        for (int i = 0; i < M; ++i) {   // (this thread's 32 consecutive buckets)
+            c[i] = t * M + i < n ? s.r1.cnt[t * M + i] : 0u;
+            const int c0 = (int)(c[i] & 0xffffu), c1 = (int)(c[i] >> 16);
+            sum += c0 + c1;
+            big = max(big, max(c0, c1));
+            multi |= (c0 >= 2 ? 1u : 0u) << (2 * i) | (c1 >= 2 ? 2u : 0u) << (2 * i);
+        }
+        int run = ws_block_excl_scan<NT, int>(sum, s.wsum_i, nullptr);
+#pragma unroll
+        for (int i = 0; i < M; ++i) {
+            if (t * M + i < n) s.r1.cnt[t * M + i] = (uint32_t)run | ((uint32_t)(run + (int)(c[i] & 0xffffu)) << 16);
+            run += (int)(c[i] & 0xffffu) + (int)(c[i] >> 16);
+        }
+        radix = __syncthreads_or(big > 32);
+        if (!radix) {
+            auto start = [&](int b) { return (int)((s.r1.cnt[b >> 1] >> ((b & 1) << 4)) & 0xffffu); };
+#pragma unroll
+            for (int k = 0; k < ITEMS; ++k)
+                if (t + k * NT < n) {
+                    const int q = start((int)(br[k] >> 16)) + (int)(br[k] & 0xffffu);
+                    s.r2.keys[q] = kk[k];
+                    s.idx[q] = (uint16_t)(t + k * NT);
+                }
+            __syncthreads();
+            while (multi) {
+                const int b = 2 * t * M + __ffs((int)multi) - 1;
+                multi &= multi - 1;
+                small_sort_bucket<K>(start(b), b + 1 < 2 * n ? start(b + 1) : n, s.r2.keys, s.idx,
+                                     [](int p) { return p; }, [](int p) { return p; });
+            }
+            __syncthreads();
+        }
+    }
+    for (int pass = 0; radix && pass < KO::BITS / 8; ++pass) {
         K kk[ITEMS];
         uint16_t ii[ITEMS];
         uint32_t dg[ITEMS];
@@ -189,7 +303,7 @@ __device__ __forceinline__ void small_general_segment(SmallSmem<T, NT, M>& s, in
         P.thr = s.r2.hull.thr;
         ws_cta_hull<NT, M, TilePtsDev<M>, true>(s.r2.hull, n, P, sc, &nv);
     } else {
-        const TilePtsWide<M> P{s.pre.s64, s.pre.base};
+        const TilePtsWide<M> P{s.pre.s64, s.pre.base, s.muq, s.fast != 0};
         ws_cta_hull<NT, M>(s.r2.hull, n, P, sc, &nv);
     }
     auto X = [&](int p) -> i128 { return ws_tile_X<M>(s.pre.s64, s.pre.base, mode, q0, bsh, p); };
@@ -209,21 +323,44 @@ __device__ __forceinline__ void small_general_segment(SmallSmem<T, NT, M>& s, in
     const bool dev32 = !fp64 && mode != WS_TILE_WIDE;
     const int Ldev = mode == WS_TILE_BINADE ? s.sct.L : sc.L;
     const float x0f = (float)xlo;
-    for (int r = t; r < c; r += NT) {
-        const int a = s.r1.ids.V[r], b = s.r1.ids.V[r + 1];
-        const T xs = (b - a == 1) ? values[a0 + s.idx[a]] : (T)0;
+    // Single weights first, four of a thread's on their way together; the
+    // other clusters from a list, so that no lane waits for a neighbour's
+    // division.
+    if (t == 0) s.n_multi = 0;
+    __syncthreads();
+    constexpr int VU = 4;
+    for (int r0 = t; r0 < c; r0 += NT * VU) {
+        T xv[VU];
+#pragma unroll
+        for (int u = 0; u < VU; ++u) {
+            const int r = min(r0 + u * NT, c - 1), a = s.r1.ids.V[r];
+            xv[u] = s.r1.ids.V[r + 1] - a == 1 ? __ldg(values + a0 + s.idx[a]) : (T)0;
+        }
+#pragma unroll
+        for (int u = 0; u < VU; ++u) {
+            const int r = r0 + u * NT;
+            if (r >= c) break;
+            const int a = s.r1.ids.V[r], b = s.r1.ids.V[r + 1];
+            atomicOr(&s.r1.ids.mark[a >> 5], 1u << (a & 31));
+            if (b - a > 1) { s.r1.ids.multi[atomicAdd(&s.n_multi, 1)] = (uint16_t)r; continue; }
+            s.r2.val[r] = dev32 ? (T)ws_epilogue<float>((float)xv[u], sc.mu_f * (float)(n - a - b), ep.beta_f,
+                                                        ep.gamma_f, ep.on != 0)
+                                : ValueOut<T>::value((i128)0, a, b, xv[u], sc, fp64 != 0, ep);
+        }
+    }
+    __syncthreads();
+    for (int q = t; q < s.n_multi; q += NT) {
+        const int r = s.r1.ids.multi[q], a = s.r1.ids.V[r], b = s.r1.ids.V[r + 1];
         if (dev32) {
-            const float mean = (b - a == 1) ? (float)xs
-                                            : x0f + ldexpf(ws_u64_to_float((uint64_t)(s.pre.s64[ws_sidx<M>(b)] -
-                                                                                   s.pre.s64[ws_sidx<M>(a)])) /
-                                                               (float)(b - a),
-                                                           -Ldev);
+            const float mean = x0f + ldexpf(ws_u64_to_float((uint64_t)(s.pre.s64[ws_sidx<M>(b)] -
+                                                                       s.pre.s64[ws_sidx<M>(a)])) /
+                                                (float)(b - a),
+                                            -Ldev);
             s.r2.val[r] = (T)ws_epilogue<float>(mean, sc.mu_f * (float)(n - a - b), ep.beta_f, ep.gamma_f,
                                                 ep.on != 0);
         } else {
-            s.r2.val[r] = ValueOut<T>::value(X(b) - X(a), a, b, xs, sc, fp64 != 0, ep);
+            s.r2.val[r] = ValueOut<T>::value(X(b) - X(a), a, b, (T)0, sc, fp64 != 0, ep);
         }
-        atomicOr(&s.r1.ids.mark[a >> 5], 1u << (a & 31));
     }
     __syncthreads();
 
@@ -609,47 +746,12 @@ __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 4 : 2) k_small(const
                     s.idx[ipad(pp)] = (uint16_t)(first + i);
                 }
             __syncthreads();
-            // each bucket by key (ties may end in any order): up to four
-            // elements by a sorting network in registers, larger buckets by
-            // insertion in shared memory
             while (multi) {
                 const int i = 2 * first + __ffs((int)multi) - 1;
                 multi &= multi - 1;
                 const int b0 = start_of_bucket(i);
                 const int b1 = i + 1 < 2 * n ? start_of_bucket(i + 1) : n;
-                if (b1 - b0 <= 4) {
-                    K k[4];
-                    uint16_t x[4];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const bool in = b0 + j < b1;
-                        k[j] = in ? s.u.sort.keys[kpad(b0 + j)] : ~(K)0;
-                        x[j] = in ? s.idx[ipad(b0 + j)] : (uint16_t)0;
-                    }
-                    auto cs = [&](int a, int b) {
-                        const bool sw = k[a] > k[b];
-                        const K ka = sw ? k[b] : k[a], kb = sw ? k[a] : k[b];
-                        const uint16_t xa = sw ? x[b] : x[a], xb = sw ? x[a] : x[b];
-                        k[a] = ka; k[b] = kb; x[a] = xa; x[b] = xb;
-                    };
-                    cs(0, 1); cs(2, 3); cs(0, 2); cs(1, 3); cs(1, 2);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (b0 + j < b1) { s.u.sort.keys[kpad(b0 + j)] = k[j]; s.idx[ipad(b0 + j)] = x[j]; }
-                    continue;
-                }
-                for (int a = b0 + 1; a < b1; ++a) {
-                    const K kk = s.u.sort.keys[kpad(a)];
-                    const uint16_t ii = s.idx[ipad(a)];
-                    int j = a - 1;
-                    while (j >= b0 && s.u.sort.keys[kpad(j)] > kk) {
-                        s.u.sort.keys[kpad(j + 1)] = s.u.sort.keys[kpad(j)];
-                        s.idx[ipad(j + 1)] = s.idx[ipad(j)];
-                        --j;
-                    }
-                    s.u.sort.keys[kpad(j + 1)] = kk;
-                    s.idx[ipad(j + 1)] = ii;
-                }
+                small_sort_bucket<K>(b0, b1, s.u.sort.keys, s.idx, kpad, ipad);
             }
             __syncthreads();
         }
