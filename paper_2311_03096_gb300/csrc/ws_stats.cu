@@ -225,39 +225,82 @@ __global__ void __launch_bounds__(256) k_dlam_count(const int32_t* __restrict__ 
     const TileDesc td = tiles[blockIdx.x];
     const LargeSeg ls = lsegs[td.lseg];
     const int64_t slot0 = ls.kpos + td.lseg;
-    for (int i = threadIdx.x; i < td.len; i += 256) {
-        const int id = ids[td.vpos + i];
-        if (id < 0 || id >= ls.len) { ws_flag(status, WS_STATUS_INTERNAL); continue; }
-        atomicAdd(&cnt[slot0 + id], 1);
+    constexpr int U = 8;   // (loads issued together)
+    for (int i0 = threadIdx.x; i0 < td.len; i0 += 256 * U) {
+        int id[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) id[u] = i0 + u * 256 < td.len ? __ldg(ids + td.vpos + i0 + u * 256) : 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (i0 + u * 256 >= td.len) break;
+            if (id[u] < 0 || id[u] >= ls.len) { ws_flag(status, WS_STATUS_INTERNAL); continue; }
+            atomicAdd(&cnt[slot0 + id[u]], 1);
+        }
     }
 }
 
-// exclusive scan of cnt[0..S) in chunks of 4096: pos = chunk-local prefix,
-// csum[b] = total of chunk b
+// Cluster starts in two passes over the counts, in chunks of 4096 slots (one
+// CTA; 16-byte loads, warp w the slots [512 w, 512 w + 512) of its chunk):
+// WRITE false: csum[b] = total of chunk b; then, with csum scanned, WRITE true:
+// key[s] = 2 start(s) + cnt[s], start counted over all slots.  32-bit wrapping
+// arithmetic: len - 2 start - size of a cluster in its segment, which fits, is
+// len + 2 start(first slot of the segment) - key[s].
 constexpr int DL_CHUNK = 4096;
-__global__ void __launch_bounds__(256) k_dlam_scan_chunks(const int32_t* __restrict__ cnt, int64_t S, int32_t* pos,
-                                                          int32_t* csum) {
+template <bool WRITE>
+__global__ void __launch_bounds__(256) k_dlam_starts(const int32_t* __restrict__ cnt, int64_t S, uint32_t* key,
+                                                     int32_t* csum) {
     __shared__ int wsum[8];
-    const int64_t b0 = (int64_t)blockIdx.x * DL_CHUNK;
-    const int t = threadIdx.x;
-    constexpr int PER = DL_CHUNK / 256;
-    int v[PER];
-    int run = 0;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int64_t b0 = (int64_t)blockIdx.x * DL_CHUNK + 512 * w + 4 * lane;
+    int4 v[4];
+    int inc[4], tot = 0;   // inclusive within the warp's rows of 128
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        const int64_t s = b0 + t * PER + k;
-        v[k] = s < S ? cnt[s] : 0;
-        run += v[k];
+    for (int k = 0; k < 4; ++k) {
+        const int64_t s = b0 + 128 * k;
+        if (s + 4 <= S) v[k] = __ldg(reinterpret_cast<const int4*>(cnt + s));
+        else {
+            v[k].x = s < S ? cnt[s] : 0;
+            v[k].y = s + 1 < S ? cnt[s + 1] : 0;
+            v[k].z = s + 2 < S ? cnt[s + 2] : 0;
+            v[k].w = 0;
+        }
     }
-    int tot;
-    int ex = ws_block_excl_scan<256, int>(run, wsum, &tot);
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
-        const int64_t s = b0 + t * PER + k;
-        if (s < S) pos[s] = ex;
-        ex += v[k];
+    for (int k = 0; k < 4; ++k) {
+        const int sum = v[k].x + v[k].y + v[k].z + v[k].w;
+        if (WRITE) {
+            const int i = ws_warp_incl_scan<int>(sum);
+            inc[k] = tot + i - sum;
+            tot += __shfl_sync(0xffffffffu, i, 31);
+        } else {
+            tot += sum;
+        }
     }
-    if (t == 0) csum[blockIdx.x] = tot;
+    if (!WRITE) tot = __reduce_add_sync(0xffffffffu, tot);
+    if (lane == 0) wsum[w] = tot;
+    __syncthreads();
+    if (!WRITE) {
+        if (t == 0) {
+            int all = 0;
+            for (int k = 0; k < 8; ++k) all += wsum[k];
+            csum[blockIdx.x] = all;
+        }
+        return;
+    }
+    int base = csum[blockIdx.x];
+    for (int k = 0; k < w; ++k) base += wsum[k];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int64_t s = b0 + 128 * k;
+        const uint32_t e0 = (uint32_t)(base + inc[k]), e1 = e0 + v[k].x, e2 = e1 + v[k].y, e3 = e2 + v[k].z;
+        const uint4 q = make_uint4(2 * e0 + v[k].x, 2 * e1 + v[k].y, 2 * e2 + v[k].z, 2 * e3 + v[k].w);
+        if (s + 4 <= S) *reinterpret_cast<uint4*>(key + s) = q;
+        else {
+            if (s < S) key[s] = q.x;
+            if (s + 1 < S) key[s + 1] = q.y;
+            if (s + 2 < S) key[s + 2] = q.z;
+        }
+    }
 }
 
 // exclusive scan of the chunk totals, in place (one CTA, carried across rounds)
@@ -278,34 +321,86 @@ __global__ void __launch_bounds__(1024) k_dlam_scan_totals(int32_t* csum, int nb
     }
 }
 
+// Sum of grad_out x (len - 2 start - size) over one sort tile, exactly: every
+// grad_out as a 63-bit integer at the tile's largest exponent (a value more
+// than 39 binades below it, 10 for double, loses the bits below 2^-63 of the
+// largest), the products and the sum in 128 bits, one rounding and one division
+// at the end.  FP64 multiplies and adds per element took 266 us at 2^24 (GB300
+// runs them at a small fraction of the FP32 rate; two gathers per element
+// beside them) and round more.
+constexpr int DL_NT = 512;
 template <typename T>
-__global__ void __launch_bounds__(256) k_dlam_apply(const T* __restrict__ g, const int32_t* __restrict__ ids,
-                                                    const TileDesc* __restrict__ tiles,
-                                                    const LargeSeg* __restrict__ lsegs,
-                                                    const int32_t* __restrict__ cnt, const int32_t* __restrict__ pos,
-                                                    const int32_t* __restrict__ csum, double* out) {
-    __shared__ double wacc[8];
+__global__ void __launch_bounds__(DL_NT) k_dlam_apply(const T* __restrict__ g, const int32_t* __restrict__ ids,
+                                                      const TileDesc* __restrict__ tiles,
+                                                      const LargeSeg* __restrict__ lsegs,
+                                                      const int32_t* __restrict__ cnt,
+                                                      const uint32_t* __restrict__ key, double* out) {
+    typedef KeyOf<T> KO;
+    constexpr int PER = WS_SORT_TILE / DL_NT, UP = 62 - KO::MANT;
+    __shared__ long long wlo[DL_NT / 32], whi[DL_NT / 32];
+    __shared__ int s_emax;
     const TileDesc td = tiles[blockIdx.x];
-    const LargeSeg ls = lsegs[td.lseg];
+    const LargeSeg& ls = lsegs[td.lseg];
     const int64_t slot0 = ls.kpos + td.lseg;
-    const int64_t base = (int64_t)pos[slot0] + csum[slot0 / DL_CHUNK];
-    const double inv = 1.0 / (double)(ls.len - 1);
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < td.len; i += 256) {
-        const int id = ids[td.vpos + i];
-        if (id < 0 || id >= ls.len) continue;
-        const int64_t s = slot0 + id;
-        const int64_t start = (int64_t)pos[s] + csum[s / DL_CHUNK] - base;
-        acc += (double)g[td.vpos + i] * (double)(ls.len - 2 * start - cnt[s]) * inv;
-    }
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    if (t == 0) s_emax = 0;
+    T gv[PER];
+    int id[PER];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) wacc[threadIdx.x >> 5] = acc;
+    for (int k = 0; k < PER; ++k) {
+        const int i = t + k * DL_NT;
+        gv[k] = i < td.len ? __ldg(g + td.vpos + i) : (T)0;
+        id[k] = i < td.len ? __ldg(ids + td.vpos + i) : -1;
+    }
+    // len + 2 start of the segment's first slot, modulo 2^32
+    const uint32_t top = (uint32_t)ls.len + key[slot0] - (uint32_t)cnt[slot0];
+    uint32_t kv[PER];
+    int e = 0;
+    bool odd = false;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        if (id[k] < 0 || (int64_t)id[k] >= ls.len) { id[k] = -1; gv[k] = (T)0; }
+        kv[k] = id[k] >= 0 ? __ldg(key + slot0 + id[k]) : 0u;
+        if (gv[k] != (T)0) e = max(e, ws_eff_exp(gv[k]));
+        odd |= !ws_isfinite(gv[k]);
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    const bool any_odd = __syncthreads_or(odd);
+    if (any_odd) {   // infinities and NaN: as FP64 arithmetic has it
+        double acc = 0.0;
+#pragma unroll
+        for (int k = 0; k < PER; ++k)
+            if (id[k] >= 0) acc += (double)gv[k] * ((double)(int32_t)(top - kv[k]) / (double)(ls.len - 1));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (lane == 0) atomicAdd(&out[ls.seg], acc);
+        return;
+    }
+    if (lane == 0) atomicMax(&s_emax, e);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < 8; ++w) s += wacc[w];
-        atomicAdd(&out[ls.seg], s);
+    const int emax = s_emax;
+    i128 acc = 0;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const uint64_t b = (uint64_t)KO::bits(gv[k]);
+        int ex = (int)((b >> KO::MANT) & KO::EXPMASK);
+        uint64_t m = b & ((1ull << KO::MANT) - 1ull);
+        if (ex == 0) ex = 1; else m |= 1ull << KO::MANT;
+        const int up = UP - (emax - ex);
+        const int64_t q = (int64_t)(up >= 0 ? m << up : (up > -64 ? m >> -up : 0ull));
+        const bool neg = (b >> (KO::BITS - 1)) & 1ull;
+        acc += (i128)(neg ? -q : q) * (int64_t)(int32_t)(top - kv[k]);
+    }
+    acc = ws_warp_reduce_i128(acc);
+    if (lane == 0) { wlo[w] = (long long)(uint64_t)acc; whi[w] = (long long)(uint64_t)((u128)acc >> 64); }
+    __syncthreads();
+    if (t == 0) {
+        i128 S = 0;
+        for (int k = 0; k < DL_NT / 32; ++k) S += (i128)(((u128)(uint64_t)whi[k] << 64) | (u128)(uint64_t)wlo[k]);
+        // grad_out = q 2^(emax - UP - bias - MANT)
+        const int bias = KO::EXPMASK >> 1;
+        const double v = ws_i128_to_double(S) / (double)(ls.len - 1);
+        if (S != 0) atomicAdd(&out[ls.seg], ldexp(v, emax - UP - bias - KO::MANT));
     }
 }
 
@@ -325,18 +420,18 @@ cudaError_t ws_dlambda(const T* g, const int32_t* ids, const int64_t* d_offsets,
     if (W.n_lseg > 0) {
         const int64_t S = W.n_keys + W.n_lseg;
         int32_t* cnt = W.bcnt;
-        int32_t* pos = reinterpret_cast<int32_t*>(W.bsum);
+        uint32_t* key = reinterpret_cast<uint32_t*>(W.bsum);
         int32_t* csum = reinterpret_cast<int32_t*>(partial);
         const int nb = (int)((S + DL_CHUNK - 1) / DL_CHUNK);
         e = cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)S, st);
         if (e) return e;
         WS_LAUNCH(W.prof, WSK_BWD, st,
                   (k_dlam_count<T><<<W.n_sort_tiles, 256, 0, st>>>(ids, W.sort_tiles, W.lsegs, cnt, status)));
-        WS_LAUNCH(W.prof, WSK_BWD, st, (k_dlam_scan_chunks<<<nb, 256, 0, st>>>(cnt, S, pos, csum)));
+        WS_LAUNCH(W.prof, WSK_BWD, st, (k_dlam_starts<false><<<nb, 256, 0, st>>>(cnt, S, key, csum)));
         WS_LAUNCH(W.prof, WSK_BWD, st, (k_dlam_scan_totals<<<1, 1024, 0, st>>>(csum, nb)));
+        WS_LAUNCH(W.prof, WSK_BWD, st, (k_dlam_starts<true><<<nb, 256, 0, st>>>(cnt, S, key, csum)));
         WS_LAUNCH(W.prof, WSK_BWD, st,
-                  (k_dlam_apply<T><<<W.n_sort_tiles, 256, 0, st>>>(g, ids, W.sort_tiles, W.lsegs, cnt, pos, csum,
-                                                                   out)));
+                  (k_dlam_apply<T><<<W.n_sort_tiles, DL_NT, 0, st>>>(g, ids, W.sort_tiles, W.lsegs, cnt, key, out)));
     }
     return cudaGetLastError();
 }
