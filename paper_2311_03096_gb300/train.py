@@ -42,8 +42,10 @@ class ProxMLP:
         return [flat[self.bounds[l]:self.bounds[l + 1]].view(*s) for l, s in enumerate(self.shapes)]
 
     def loss(self, x, y, flat=None):
+        return self._loss(x, y, self.weights(flat))
+
+    def _loss(self, x, y, ws_):
         h = x
-        ws_ = self.weights(flat)
         for l, (w, b) in enumerate(zip(ws_, self.biases)):
             h = torch.nn.functional.linear(h, w, b)
             if l + 1 < len(ws_):
@@ -52,11 +54,14 @@ class ProxMLP:
 
     def sgd(self, x, y):
         """Loss, gradient and the SGD update of the weights (no prox)."""
-        flat = self.flat.detach().requires_grad_(True)
-        loss = self.loss(x, y, flat)
-        (g,) = torch.autograd.grad(loss, flat)
+        # a leaf per layer, not one for the flat buffer: the gradient of a slice of
+        # that is a buffer-sized zero fill and addition per layer
+        ws_ = [w.requires_grad_(True) for w in self.weights(self.flat.detach())]
+        loss = self._loss(x, y, ws_)
+        grads = torch.autograd.grad(loss, ws_)
         with torch.no_grad():
-            self.flat.sub_(self.lr * g)
+            for w, g in zip(self.weights(), grads):
+                w.sub_(g.mul_(self.lr))
         return loss.detach()
 
     def prox(self, stream=None):
