@@ -37,24 +37,6 @@ __device__ __forceinline__ bool ws_lean_x(uint64_t range, int n) {
     return __umul64hi(range, (uint64_t)n) == 0 && range * (uint64_t)n <= ((uint64_t)1 << 62);
 }
 
-// floor(lambda 2^L K / (d - 1)) exactly (the largest D with D (d-1) <= mlam K 2^s),
-// saturated at 2^62.
-static __device__ __noinline__ int64_t ws_floor_muK64(uint64_t K, const SegConst& sc) {
-    if (sc.mlam == 0) return 0;
-    const double est = ldexp((double)sc.mlam * (double)K, sc.s) / (double)sc.dm1;
-    if (!(est < 4.0e18)) return (int64_t)1 << 62;
-    const int64_t q = (int64_t)est;
-    // the estimate is within q 2^-50 + 2 of the answer; bisect a window around it
-    int64_t lo = q > (1 << 14) ? q - (1 << 14) : 0, hi = q + (1 << 14);
-    if (ws_gt_muK(lo, K, sc)) lo = 0;                      // (not reached)
-    if (!ws_gt_muK(hi, K, sc)) return (int64_t)1 << 62;   // (not reached)
-    while (hi - lo > 1) {   // invariant: !gt(lo), gt(hi)
-        const int64_t mid = lo + (hi - lo) / 2;
-        if (ws_gt_muK(mid, K, sc)) hi = mid; else lo = mid;
-    }
-    return lo;
-}
-
 // lambda 2^L / (d - 1) in FP32 for the hull-test filter, without FP64: two
 // roundings (the integer mantissa of lambda, the quotient), covered by the
 // filter's margin.  usable: finite and far from overflow in the filter.

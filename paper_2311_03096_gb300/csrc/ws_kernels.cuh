@@ -132,10 +132,16 @@ struct TileScale {
     uint64_t modd;    // odd part of lambda 2^L (0 when lambda = 0) and its exponent
     int sodd;
     int pad;
-    int64_t t11;      // floor(2 lambda 2^L / (d - 1)), saturated at 2^62: two adjacent
-                      // elements collide at once (IC round 1) iff their gap <= t11 units
+    int64_t t11;      // lower bound of 2 lambda 2^L / (d - 1): two adjacent elements
+                      // collide at once (IC round 1) if their gap <= t11 units
 };
 constexpr int WS_NSCALE = 64;   // per segment: binade shifts 0 .. FIX_OFS, then the segment scale last
+
+// The constants at a segment's own scale (with lambda / (d - 1) in FP64: one
+// division per segment, not one per thread of every later kernel).
+__device__ __forceinline__ SegConst ws_seg_scale(const TileScale* scales, int lseg) {
+    return scales[(size_t)lseg * WS_NSCALE + WS_NSCALE - 1].sc;
+}
 
 // Per-segment run-time values computed on the device.
 struct SegRuntime {
@@ -242,7 +248,7 @@ template <typename T>
 cudaError_t ws_large_hull_fast(const LargeWork<T>& W, const typename KeyOf<T>::K* sorted, const double* lambdas,
                                uint32_t* status, cudaStream_t st);
 template <typename T>
-cudaError_t ws_large_junctions(const LargeWork<T>& W, const double* lambdas, cudaStream_t st);
+cudaError_t ws_large_junctions(const LargeWork<T>& W, cudaStream_t st);
 template <typename T>
 cudaError_t ws_large_prox(const LargeWork<T>& W, const T* values, const double* lambdas, T* out, int32_t* ids,
                           int64_t* n_clusters, int fp64, const WsEpi& ep, uint32_t* status, uint64_t spin_limit,

@@ -602,10 +602,8 @@ struct ClimbSmem {
     SegConst sc;
 };
 
-template <typename T>
 __global__ void __launch_bounds__(HNT) k_climb(const TileDesc* __restrict__ htiles, const LargeSeg* __restrict__ lsegs,
-                                               const double* __restrict__ lambdas,
-                                               const SegRuntime* __restrict__ rt, const uint16_t* vp, const i128* vx,
+                                               const TileScale* __restrict__ scales, const uint16_t* vp, const i128* vx,
                                                const int32_t* __restrict__ nvert, i128* tile_total, Piece* pieces,
                                                int32_t* npieces, int32_t* arrive, int n_hull,
                                                const int32_t* __restrict__ seg_mode) {
@@ -623,9 +621,7 @@ __global__ void __launch_bounds__(HNT) k_climb(const TileDesc* __restrict__ htil
     __syncthreads();   // (the previous tile's shared memory is dead)
     const LargeSeg ls = lsegs[td.lseg];
     if (t == 0) {
-        double lam = lambdas[ls.seg];
-        if (!(lam >= 0.0) || !(lam <= 1.7976931348623157e308)) lam = 0.0;
-        s.sc = ws_seg_const<T>(ls.len, lam, rt[td.lseg].emax);
+        s.sc = ws_seg_scale(scales, td.lseg);
         Piece pc;
         pc.tile = tile; pc.lo = 0; pc.hi = (uint16_t)nvert[tile]; pc.cum = 0; pc.pad = 0; pc.off = 0;
         ws_st_piece(pieces + tile, pc);
@@ -688,7 +684,7 @@ constexpr int SUM_MAX = 8;
 
 template <typename T>
 __global__ void __launch_bounds__(256, 6) k_values(const TileDesc* __restrict__ htiles, const LargeSeg* __restrict__ lsegs,
-                                                const double* __restrict__ lambdas, const SegRuntime* __restrict__ rt,
+                                                const TileScale* __restrict__ scales, const SegRuntime* __restrict__ rt,
                                                 const typename KeyOf<T>::K* __restrict__ sorted,
                                                 const uint16_t* __restrict__ vp, const i128* __restrict__ vx,
                                                 const Piece* __restrict__ pieces,
@@ -743,10 +739,8 @@ __global__ void __launch_bounds__(256, 6) k_values(const TileDesc* __restrict__ 
     }
     __syncthreads();
     if (tp >= 0) {
-        double lam = lambdas[ls.seg];
-        if (!(lam >= 0.0) || !(lam <= 1.7976931348623157e308)) lam = 0.0;
         const int emax = rt[td.lseg].emax;
-        const SegConst sc = ws_seg_const<T>(ls.len, lam, emax);
+        const SegConst sc = ws_seg_scale(scales, td.lseg);
         const Piece pc = P[tp];
         const uint16_t* vpt = vp + (size_t)tile * (HT + 1);
         const i128* vxt = vx + (size_t)tile * (HT + 1);
@@ -1029,12 +1023,12 @@ cudaError_t ws_large_prox(const LargeWork<T>& W, const T* values, const double* 
                                                             W.seg_emin, status)));
     // across tiles: junction bridges and the per-segment resolution, then the
     // tree of merges for the segments that need it
-    e = ws_large_junctions<T>(W, lambdas, st);
+    e = ws_large_junctions<T>(W, st);
     if (e) return e;
     e = cudaMemsetAsync(W.arrive, 0, sizeof(int32_t) * (size_t)n_levels * W.n_hull_tiles, st);
     if (e) return e;
     WS_LAUNCH(W.prof, WSK_CLIMB, st,
-              (k_climb<T><<<small_grid, HNT, 0, st>>>(W.hull_tiles, W.lsegs, lambdas, W.rt, W.vp, W.vx, W.nvert,
+              (k_climb<<<small_grid, HNT, 0, st>>>(W.hull_tiles, W.lsegs, W.scales, W.vp, W.vx, W.nvert,
                                                           W.tile_total, W.pieces, W.npieces, W.arrive,
                                                           W.n_hull_tiles, W.seg_mode)));
     e = cudaMemsetAsync(W.tile_piece, 0xff, sizeof(int32_t) * (size_t)W.n_hull_tiles, st);
@@ -1042,7 +1036,7 @@ cudaError_t ws_large_prox(const LargeWork<T>& W, const T* values, const double* 
     WS_LAUNCH(W.prof, WSK_ROOT, st,
               (k_root<<<W.n_lseg, 256, 0, st>>>(W.lsegs, W.pieces, W.npieces, W.tile_piece, W.rt, n_clusters)));
     WS_LAUNCH(W.prof, WSK_VALUES, st,
-              (k_values<T><<<W.n_hull_tiles, 256, 0, st>>>(W.hull_tiles, W.lsegs, lambdas, W.rt, sorted, W.vp, W.vx,
+              (k_values<T><<<W.n_hull_tiles, 256, 0, st>>>(W.hull_tiles, W.lsegs, W.scales, W.rt, sorted, W.vp, W.vx,
                                                           W.pieces, W.npieces, W.tile_piece, W.cval, W.rank_words,
                                                           fp64, ep, status)));
     // back to the caller's order

@@ -62,12 +62,26 @@ __global__ void __launch_bounds__(WS_NSCALE) k_scales(const typename KeyOf<T>::K
     TileScale ts;
     ts.sc = ws_seg_const_L(ls.len, lamv, KO::L_BASE - emax - (j == WS_NSCALE - 1 ? 0 : j));
     bool f;
-    ts.muq = ws_muq(lamv, ts.sc, f);
+    ts.muq = ws_muq_f(ts.sc, f);
     ts.fast = f ? 1 : 0;
     if (ts.sc.mlam == 0) { ts.modd = 0; ts.sodd = 0; }
     else { const int tz = __ffsll((long long)ts.sc.mlam) - 1; ts.modd = ts.sc.mlam >> tz; ts.sodd = ts.sc.s + tz; }
     ts.pad = 0;
-    ts.t11 = ws_floor_muK64(2, ts.sc);
+    // floor(2 mu), mu = lambda 2^L / (d - 1) in units: muq is within 3e-7
+    // relative of mu, so 2 mu lies between two FP32 bounds; where an integer
+    // lies between them too (lambda = 1, d = 2^24: 2 mu = 1 + 2^-24) one exact
+    // comparison decides.  (A bisection with 192-bit products took 10 us on the
+    // path of every call.)  From 2^20 on the lower bound will do: the rounds
+    // test every boundary that round 1 leaves.
+    const float lo2 = 2.0f * ts.muq * (1.0f - 1.0e-6f), hi2 = 2.0f * ts.muq * (1.0f + 1.0e-6f);
+    if (ts.sc.mlam == 0) ts.t11 = 0;
+    else if (!f) ts.t11 = -1;
+    else if (!(lo2 < 3.9e18f)) ts.t11 = (int64_t)3.9e18;
+    else {
+        ts.t11 = (int64_t)floorf(lo2);
+        const int64_t up = (int64_t)floorf(hi2);
+        if (up == ts.t11 + 1 && !ws_gt_muK(up, 2, ts.sc)) ts.t11 = up;
+    }
     scales[(size_t)lseg * WS_NSCALE + j] = ts;
 }
 
@@ -84,7 +98,8 @@ struct FastSmem {
 // exact tests; a tile that has not converged after ic_cap rounds (or
 // ic_cap = 0) takes the chain and tree merges instead.
 //   Round 1: point p (1 <= p < n) starts a new block iff y_{p-1} < y_p, i.e.
-//            the gap x_p - x_{p-1} exceeds 2 lambda/(d-1): gap > t11 units.
+//            the gap x_p - x_{p-1} exceeds 2 lambda/(d-1): gap > t11 units
+//            (t11 a lower bound; the next round tests what it leaves).
 //   Round r: every surviving block boundary b, with neighbouring boundaries
 //            a < b < c, stays iff the mean of y over [a, b) is strictly below
 //            the mean over [b, c) (the exact hull test at b); all boundaries
@@ -278,9 +293,8 @@ struct JVert {
     i128 X;      // prefix relative to tile T's first point
 };
 
-template <typename T>
 __global__ void __launch_bounds__(256) k_junction(const TileDesc* __restrict__ htiles, const LargeSeg* __restrict__ lsegs,
-                                                  const double* __restrict__ lambdas, const SegRuntime* __restrict__ rt,
+                                                  const TileScale* __restrict__ scales,
                                                   const uint16_t* __restrict__ vp, const i128* __restrict__ vx,
                                                   const int32_t* __restrict__ nvert,
                                                   const i128* __restrict__ tile_total, int32_t* keepR, int32_t* keepL,
@@ -290,9 +304,7 @@ __global__ void __launch_bounds__(256) k_junction(const TileDesc* __restrict__ h
     const TileDesc td = htiles[gw];
     const LargeSeg ls = lsegs[td.lseg];
     if (td.tin + 1 >= ls.hull_count) return;
-    double lam = lambdas[ls.seg];
-    if (!(lam >= 0.0) || !(lam <= 1.7976931348623157e308)) lam = 0.0;
-    const SegConst sc = ws_seg_const<T>(ls.len, lam, rt[td.lseg].emax);
+    const SegConst sc = ws_seg_scale(scales, td.lseg);
     const int TL = gw, TR = gw + 1;
     const int p = nvert[TL] - 1, q = nvert[TR] - 1;
     const size_t bL = (size_t)TL * (HT + 1), bR = (size_t)TR * (HT + 1);
@@ -433,9 +445,8 @@ __global__ void __launch_bounds__(RNT) k_resolve(const LargeSeg* __restrict__ ls
 // One cluster iff no vertex of any tile hull lies strictly below the chord
 // from the segment's first point to its last (every point is on or above its
 // tile's hull).  One warp per hull tile of the segments left undecided.
-template <typename T>
 __global__ void __launch_bounds__(256) k_chord(const TileDesc* __restrict__ htiles, const LargeSeg* __restrict__ lsegs,
-                                               const double* __restrict__ lambdas, const SegRuntime* __restrict__ rt,
+                                               const TileScale* __restrict__ scales,
                                                const uint16_t* __restrict__ vp, const i128* __restrict__ vx,
                                                const int32_t* __restrict__ nvert, const i128* __restrict__ tile_base,
                                                const i128* __restrict__ seg_total,
@@ -447,9 +458,7 @@ __global__ void __launch_bounds__(256) k_chord(const TileDesc* __restrict__ htil
     const TileDesc td = htiles[gw];
     if (seg_mode[td.lseg] != 3) return;
     const LargeSeg ls = lsegs[td.lseg];
-    double lam = lambdas[ls.seg];
-    if (!(lam >= 0.0) || !(lam <= 1.7976931348623157e308)) lam = 0.0;
-    const SegConst sc = ws_seg_const<T>(ls.len, lam, rt[td.lseg].emax);
+    const SegConst sc = ws_seg_scale(scales, td.lseg);
     const i128 base = tile_base[gw], Xd = seg_total[td.lseg];
     const int nv = nvert[gw];
     const size_t b = (size_t)gw * (HT + 1);
@@ -515,11 +524,11 @@ cudaError_t ws_large_hull_fast(const LargeWork<T>& W, const typename KeyOf<T>::K
 }
 
 template <typename T>
-cudaError_t ws_large_junctions(const LargeWork<T>& W, const double* lambdas, cudaStream_t st) {
+cudaError_t ws_large_junctions(const LargeWork<T>& W, cudaStream_t st) {
     const int warps_per_cta = 8;
     const int grid = (W.n_hull_tiles + warps_per_cta - 1) / warps_per_cta;
     WS_LAUNCH(W.prof, WSK_JUNCTION, st,
-              (k_junction<T><<<(W.n_hull_tiles + 127) / 128, 128, 0, st>>>(W.hull_tiles, W.lsegs, lambdas, W.rt, W.vp, W.vx,
+              (k_junction<<<(W.n_hull_tiles + 127) / 128, 128, 0, st>>>(W.hull_tiles, W.lsegs, W.scales, W.vp, W.vx,
                                                                   W.nvert, W.tile_total, W.keepR, W.keepL, W.jflag0,
                                                                   W.n_hull_tiles)));
     WS_LAUNCH(W.prof, WSK_JUNCTION, st,
@@ -527,7 +536,7 @@ cudaError_t ws_large_junctions(const LargeWork<T>& W, const double* lambdas, cud
                                                       W.pieces, W.npieces, W.seg_mode, W.tile_base, W.seg_total,
                                                       W.seg_below)));
     WS_LAUNCH(W.prof, WSK_JUNCTION, st,
-              (k_chord<T><<<grid, 32 * warps_per_cta, 0, st>>>(W.hull_tiles, W.lsegs, lambdas, W.rt, W.vp, W.vx,
+              (k_chord<<<grid, 32 * warps_per_cta, 0, st>>>(W.hull_tiles, W.lsegs, W.scales, W.vp, W.vx,
                                                                W.nvert, W.tile_base, W.seg_total, W.seg_mode,
                                                                W.seg_below, W.n_hull_tiles)));
     WS_LAUNCH(W.prof, WSK_JUNCTION, st,
@@ -539,6 +548,6 @@ cudaError_t ws_large_junctions(const LargeWork<T>& W, const double* lambdas, cud
 #define WS_INST_TILE(T)                                                                                          \
     template cudaError_t ws_large_hull_fast<T>(const LargeWork<T>&, const typename KeyOf<T>::K*, const double*, \
                                                uint32_t*, cudaStream_t);                                         \
-    template cudaError_t ws_large_junctions<T>(const LargeWork<T>&, const double*, cudaStream_t);
+    template cudaError_t ws_large_junctions<T>(const LargeWork<T>&, cudaStream_t);
 WS_INST_TILE(float)
 WS_INST_TILE(double)
