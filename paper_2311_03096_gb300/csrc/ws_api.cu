@@ -51,7 +51,6 @@ struct ws_plan {
     int n_small = 0;
     int32_t* small_gen = nullptr;     // one-CTA segments passed to the general kernel
     int32_t* small_gen_count = nullptr;
-    double* d_lambda1 = nullptr;   // lambda slot for single-vector calls
     // large path
     int n_lseg = 0, n_sort_tiles = 0, n_hull_tiles = 0;
     int64_t n_keys = 0;
@@ -89,7 +88,6 @@ struct ws_plan {
     int32_t* npieces = nullptr;
     int32_t* tile_piece = nullptr;
     int32_t* gen_list = nullptr;
-    int32_t* gen_count = nullptr;
     int32_t* keepR = nullptr;
     int32_t* keepL = nullptr;
     int32_t* jflag0 = nullptr;
@@ -161,7 +159,6 @@ LargeWork<T> make_work(const ws_plan* p) {
     W.npieces = p->npieces;
     W.tile_piece = p->tile_piece;
     W.gen_list = p->gen_list;
-    W.gen_count = p->gen_count;
     W.keepR = p->keepR;
     W.keepL = p->keepL;
     W.jflag0 = p->jflag0;
@@ -307,7 +304,6 @@ ws_status build_plan(ws_plan* p) {
     if ((st = plan_upload(p, &p->d_small, small))) return st;
     if ((st = plan_alloc(p, (void**)&p->small_gen, sizeof(int32_t) * std::max<size_t>(small.size(), 1)))) return st;
     if ((st = plan_alloc(p, (void**)&p->small_gen_count, sizeof(int32_t)))) return st;
-    if ((st = plan_alloc(p, (void**)&p->d_lambda1, sizeof(double)))) return st;
     if (p->n_lseg == 0) return WS_OK;
     if ((st = plan_upload(p, &p->d_lsegs, lsegs))) return st;
     if ((st = plan_upload(p, &p->d_sort_tiles, stiles))) return st;
@@ -317,11 +313,12 @@ ws_status build_plan(ws_plan* p) {
     if ((st = plan_alloc(p, &p->keys_b, ksize * nk))) return st;
     if ((st = plan_alloc(p, (void**)&p->hist, sizeof(uint64_t) * (3 * 256 + 2)))) return st;
     {
-        // one block, cleared before every sort: control words, sampled ranges, cells, bin counts
+        // one block, cleared before every sort: control words, sampled ranges, cells, bin counts,
+        // the merge tree's arrival counters
         const size_t nl = (size_t)p->n_lseg;
         const size_t o_hi = sizeof(SortCtl), o_lo = o_hi + 8 * nl, o_en = o_lo + 8 * nl, o_cells = o_en + 4 * nl,
-                     o_cnt = o_cells + 4 * (size_t)cell_pos;
-        p->sort_zero_bytes = o_cnt + 4 * (size_t)bin_pos;
+                     o_cnt = o_cells + 4 * (size_t)cell_pos, o_arr = o_cnt + 4 * (size_t)bin_pos;
+        p->sort_zero_bytes = o_arr + 4 * (size_t)p->n_levels * nh;
         unsigned char* z = nullptr;
         if ((st = plan_alloc(p, (void**)&z, p->sort_zero_bytes))) return st;
         p->ctl = (SortCtl*)z;
@@ -330,6 +327,7 @@ ws_status build_plan(ws_plan* p) {
         p->seg_en = (uint32_t*)(z + o_en);
         p->cells = (uint32_t*)(z + o_cells);
         p->bin_cnt = (uint32_t*)(z + o_cnt);
+        p->arrive = (int32_t*)(z + o_arr);
         p->n_bins = (int)bin_pos;
     }
     {
@@ -353,12 +351,10 @@ ws_status build_plan(ws_plan* p) {
     if ((st = plan_alloc(p, (void**)&p->vx, sizeof(i128) * nh * (WS_HULL_TILE + 1)))) return st;
     if ((st = plan_alloc(p, (void**)&p->nvert, sizeof(int32_t) * nh))) return st;
     if ((st = plan_alloc(p, (void**)&p->tile_total, sizeof(i128) * nh))) return st;
-    if ((st = plan_alloc(p, (void**)&p->arrive, sizeof(int32_t) * (size_t)p->n_levels * nh))) return st;
     if ((st = plan_alloc(p, (void**)&p->pieces, sizeof(Piece) * nh))) return st;
     if ((st = plan_alloc(p, (void**)&p->npieces, sizeof(int32_t) * nh))) return st;
     if ((st = plan_alloc(p, (void**)&p->tile_piece, sizeof(int32_t) * nh))) return st;
     if ((st = plan_alloc(p, (void**)&p->gen_list, sizeof(int32_t) * nh))) return st;
-    if ((st = plan_alloc(p, (void**)&p->gen_count, sizeof(int32_t)))) return st;
     if ((st = plan_alloc(p, (void**)&p->keepR, sizeof(int32_t) * nh))) return st;
     if ((st = plan_alloc(p, (void**)&p->keepL, sizeof(int32_t) * nh))) return st;
     if ((st = plan_alloc(p, (void**)&p->jflag0, sizeof(int32_t) * nh))) return st;
@@ -390,8 +386,6 @@ ws_status build_plan(ws_plan* p) {
     return WS_OK;
 }
 
-__global__ void k_set_lambda(double* dst, double v) { *dst = v; }
-
 // The one-CTA segments and the device-wide chain touch disjoint elements, so
 // with both present the one-CTA kernel runs on the plan's side stream, after
 // everything already queued on the caller's stream (fork) and before anything
@@ -419,7 +413,7 @@ bool join(ws_plan* p, cudaStream_t st) {
 }
 
 template <typename T>
-ws_status run_forward(ws_plan* p, const void* values, const double* lambdas, void* out, int32_t* ids,
+ws_status run_forward(ws_plan* p, const void* values, WsLambda lambdas, void* out, int32_t* ids,
                       int64_t* n_clusters, ws_prec prec, const WsEpi& ep, cudaStream_t st,
                       const int32_t* ids_prev = nullptr) {
     const int fp64 = prec == WS_PREC_FP64 ? 1 : 0;
@@ -431,7 +425,7 @@ ws_status run_forward(ws_plan* p, const void* values, const double* lambdas, voi
     if (p->n_lseg > 0) {
         LargeWork<T> W = make_work<T>(p);
         e = ws_large_prox<T>(W, (const T*)values, lambdas, (T*)out, ids, n_clusters, fp64, ep, p->ctx->status,
-                             p->ctx->spin_limit, p->n_levels, st);
+                             p->ctx->spin_limit, st);
     }
     if (e) { join(p, st); return map_cuda(e); }
     e = ws_launch_small<T>((const T*)values, p->d_offsets, p->d_small, p->n_small, lambdas, (T*)out, ids, n_clusters,
@@ -579,12 +573,11 @@ static ws_status make_epi(const ws_l1_rewind* epi, WsEpi* ep) {
     return WS_OK;
 }
 
-static ws_status batched_impl(ws_plan* plan, const void* values, const double* lambdas, const ws_l1_rewind* epi, void* out,
+static ws_status batched_impl(ws_plan* plan, const void* values, WsLambda lambdas, const ws_l1_rewind* epi, void* out,
                        int32_t* cluster_ids, int64_t* n_clusters, ws_prec prec, void* stream,
                        const int32_t* ids_prev = nullptr) {
     if (!plan || (prec != WS_PREC_FP32_COMP && prec != WS_PREC_FP64)) return WS_ERR_INVALID;
     if (plan->n > 0 && (!values || !out)) return WS_ERR_INVALID;
-    if (plan->n_seg > 0 && !lambdas) return WS_ERR_INVALID;
     WsEpi ep;
     if (make_epi(epi, &ep) != WS_OK) return WS_ERR_INVALID;
     if (plan->n_seg == 0) return WS_OK;
@@ -605,27 +598,27 @@ static ws_status single_impl(ws_ctx* ctx, const void* w, int64_t d, double lambd
     ws_status st;
     ws_plan* p = cached_plan(ctx, d, dtype, &st);
     if (!p) return st;
-    cudaStream_t s = (cudaStream_t)stream;
-    WS_LAUNCH(&ctx->prof, WSK_MISC, s, (k_set_lambda<<<1, 1, 0, s>>>(p->d_lambda1, lambda)));
-    if (cudaGetLastError() != cudaSuccess) return WS_ERR_CUDA;
-    return batched_impl(p, w, p->d_lambda1, epi, out, cluster_ids, n_clusters, prec, stream);
+    return batched_impl(p, w, WsLambda{nullptr, lambda}, epi, out, cluster_ids, n_clusters, prec, stream);
 }
 
 ws_status ws_prox_batched(ws_plan* plan, const void* values, const double* lambdas, void* out, int32_t* cluster_ids,
                           int64_t* n_clusters, ws_prec prec, void* stream) {
-    return batched_impl(plan, values, lambdas, nullptr, out, cluster_ids, n_clusters, prec, stream);
+    if (plan && plan->n_seg > 0 && !lambdas) return WS_ERR_INVALID;
+    return batched_impl(plan, values, WsLambda{lambdas, 0.0}, nullptr, out, cluster_ids, n_clusters, prec, stream);
 }
 
 ws_status ws_prox_batched_warm(ws_plan* plan, const void* values, const double* lambdas, const int32_t* ids_prev,
                                void* out, int32_t* cluster_ids, int64_t* n_clusters, ws_prec prec, void* stream) {
     if (plan && plan->n > 0 && !ids_prev) return WS_ERR_INVALID;
-    return batched_impl(plan, values, lambdas, nullptr, out, cluster_ids, n_clusters, prec, stream, ids_prev);
+    if (plan && plan->n_seg > 0 && !lambdas) return WS_ERR_INVALID;
+    return batched_impl(plan, values, WsLambda{lambdas, 0.0}, nullptr, out, cluster_ids, n_clusters, prec, stream, ids_prev);
 }
 
 ws_status ws_prox_batched_l1(ws_plan* plan, const void* values, const double* lambdas, const ws_l1_rewind* epi,
                              void* out, int32_t* cluster_ids, int64_t* n_clusters, ws_prec prec, void* stream) {
     if (!epi) return WS_ERR_INVALID;
-    return batched_impl(plan, values, lambdas, epi, out, cluster_ids, n_clusters, prec, stream);
+    if (plan && plan->n_seg > 0 && !lambdas) return WS_ERR_INVALID;
+    return batched_impl(plan, values, WsLambda{lambdas, 0.0}, epi, out, cluster_ids, n_clusters, prec, stream);
 }
 
 ws_status ws_prox(ws_ctx* ctx, const void* w, int64_t d, double lambda, void* out, int32_t* cluster_ids,

@@ -7,6 +7,14 @@ template <typename T> struct SmallCfg;
 template <> struct SmallCfg<float> { static constexpr int M = 16; static constexpr int CAP = 256 * 16; };
 template <> struct SmallCfg<double> { static constexpr int M = 16; static constexpr int CAP = 256 * 16; };
 
+// lambda of every segment: an array in device memory, or one value for the
+// single segment of a vector call.
+struct WsLambda {
+    const double* ptr;
+    double one;
+    __device__ __forceinline__ double at(int seg) const { return ptr ? ptr[seg] : one; }
+};
+
 // Opt-in per-launch timing (CUDA events recorded on the launching stream
 // around every kernel) and a launch counter.  Host-side only.
 enum WsKernelKind {
@@ -31,6 +39,37 @@ struct WsProf {
         ++n;
     }
 };
+// Programmatic dependent launch inside one call's chain: a kernel launched by
+// ws_launch_chain is placed on the SMs while its predecessor's last CTAs run,
+// and waits in ws_chain() for the predecessor's end before it touches memory,
+// so the 1.5 to 2 us between two kernels overlap (d = 40960, 15 launches: 132
+// -> 108 us; 2^26: 2569 -> 2510).  Every kernel launched this way starts with
+// ws_chain().  early = false is a plain launch, for kernels that live off the
+// L1: a CTA that is placed beside a predecessor with a large shared-memory
+// block gets the little L1 that this left.
+__device__ __forceinline__ void ws_chain() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline void ws_launch_if(bool early, void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t st,
+                         A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = early ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+template <typename... P, typename... A>
+inline void ws_launch_chain(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t st, A... args) {
+    ws_launch_if(true, kernel, grid, block, smem, st, args...);
+}
 #define WS_LAUNCH(PROF, KIND, ST, ...) \
     do { (PROF)->begin((ST), (KIND)); __VA_ARGS__; (PROF)->end((ST)); } while (0)
 
@@ -87,7 +126,8 @@ struct SortCtl {
     uint32_t over_count;   // bins above WS_BIN_CAP
     uint32_t over_bar;     // grid barrier of the oversize kernel
     unsigned long long over_diff;   // key bits that vary inside any oversize bin
-    unsigned long long pad;
+    int32_t gen_count;     // hull tiles for the general kernel
+    int32_t pad;
 };
 
 // Map header of a segment: cell = (key - kmin) >> shift.
@@ -153,7 +193,7 @@ struct SegRuntime {
 
 template <typename T>
 cudaError_t ws_launch_small(const T* values, const int64_t* offsets, const int32_t* seg_list, int n_list,
-                            const double* lambdas, T* out, int32_t* ids, int64_t* n_clusters, int fp64,
+                            WsLambda lambdas, T* out, int32_t* ids, int64_t* n_clusters, int fp64,
                             const WsEpi& ep, uint32_t* status, cudaStream_t st, WsProf* prof, int32_t* gen_list,
                             int32_t* gen_count, int ic_cap, const int32_t* ids_prev);
 template <typename T>
@@ -206,16 +246,15 @@ struct LargeWork {
     i128* vx;                // [n_hull_tiles][WS_HULL_TILE + 1] X at vertices (tile-local)
     int32_t* nvert;          // [n_hull_tiles]
     i128* tile_total;        // [n_hull_tiles] node total X, stored at the node's first tile
-    int32_t* arrive;         // [WS_MAX_LEVELS][n_hull_tiles] merge-tree arrival counters
+    int32_t* arrive;         // [levels][n_hull_tiles] merge-tree arrival counters (cleared with the sort's words)
     Piece* pieces;           // [n_hull_tiles]
     int32_t* npieces;        // [n_hull_tiles] pieces of the node whose first tile is this index
     int32_t* tile_piece;     // [n_hull_tiles] piece index in the root list or -1
     int32_t* gen_list;       // [n_hull_tiles] tiles whose hull the general kernel builds
-    int32_t* gen_count;      // [1] their number
     int32_t* keepR;          // [n_hull_tiles] junction results (ws_tile.cu)
     int32_t* keepL;          // [n_hull_tiles]
     int32_t* jflag0;         // [n_hull_tiles]
-    int32_t* seg_mode;       // [n_lseg] 0: junctions resolved, 1: one cluster, 2: tree of merges
+    int32_t* seg_mode;       // [n_lseg] 0: junctions resolved, 3: one cluster unless seg_below (then the tree of merges)
     i128* tile_base;         // [n_hull_tiles] X at every hull tile's first point (segment frame)
     TileScale* scales;       // [n_lseg][WS_NSCALE]
     int32_t* tile_rounds;    // [n_hull_tiles] in-tile IC rounds to converge, -1 chain + trees, -2 general kernel
@@ -245,14 +284,14 @@ cudaError_t ws_large_sort(const LargeWork<T>& W, const T* values, bool way_back,
                           uint64_t spin_limit, cudaStream_t st, typename KeyOf<T>::K** sorted);
 // Lean tile hulls and the junction resolution (ws_tile.cu).
 template <typename T>
-cudaError_t ws_large_hull_fast(const LargeWork<T>& W, const typename KeyOf<T>::K* sorted, const double* lambdas,
+cudaError_t ws_large_hull_fast(const LargeWork<T>& W, const typename KeyOf<T>::K* sorted, WsLambda lambdas,
                                uint32_t* status, cudaStream_t st);
 template <typename T>
 cudaError_t ws_large_junctions(const LargeWork<T>& W, cudaStream_t st);
 template <typename T>
-cudaError_t ws_large_prox(const LargeWork<T>& W, const T* values, const double* lambdas, T* out, int32_t* ids,
+cudaError_t ws_large_prox(const LargeWork<T>& W, const T* values, WsLambda lambdas, T* out, int32_t* ids,
                           int64_t* n_clusters, int fp64, const WsEpi& ep, uint32_t* status, uint64_t spin_limit,
-                          int n_levels, cudaStream_t st);
+                          cudaStream_t st);
 template <typename T>
 cudaError_t ws_large_backward(const LargeWork<T>& W, const T* g, const int32_t* ids, T* gin, uint32_t* status,
                               cudaStream_t st);

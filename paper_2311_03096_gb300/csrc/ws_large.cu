@@ -10,6 +10,8 @@
 // list of "pieces" -- contiguous vertex ranges of tile hulls -- and a merge
 // only edits the two lists where they meet.  The root list is the cluster
 // partition: its consecutive vertices bound the clusters.
+#include <algorithm>
+
 #include "ws_kernels.cuh"
 
 namespace {
@@ -483,7 +485,7 @@ template <typename T>
 __global__ void __launch_bounds__(HNT, 4) k_tile_hull(const typename KeyOf<T>::K* __restrict__ sorted,
                                                    const TileDesc* __restrict__ htiles,
                                                    const LargeSeg* __restrict__ lsegs,
-                                                   const double* __restrict__ lambdas, SegRuntime* rt,
+                                                   WsLambda lambdas, SegRuntime* rt,
                                                    uint16_t* vp, i128* vx, int32_t* nvert, i128* tile_total,
                                                    const int32_t* __restrict__ gen_list,
                                                    const int32_t* __restrict__ gen_count,
@@ -493,13 +495,14 @@ __global__ void __launch_bounds__(HNT, 4) k_tile_hull(const typename KeyOf<T>::K
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TileHullSmem& s = *reinterpret_cast<TileHullSmem*>(smem_raw);
     const int t = threadIdx.x;
+    ws_chain();
     const int n_list = *gen_count;
     for (int li = blockIdx.x; li < n_list; li += gridDim.x) {
     __syncthreads();   // (the previous tile's shared memory is dead)
     const int tile = gen_list[li];
     const TileDesc td = htiles[tile];
     const LargeSeg ls = lsegs[td.lseg];
-    const double lam = lambdas[ls.seg];
+    const double lam = lambdas.at(ls.seg);
     const bool lam_ok = lam >= 0.0 && lam <= 1.7976931348623157e308;
     const double lamv = lam_ok ? lam : 0.0;
     const int n = td.len;
@@ -587,7 +590,7 @@ __global__ void __launch_bounds__(HNT, 4) k_tile_hull(const typename KeyOf<T>::K
 
 // ---------------------------------------------------------------------------
 // 3. the tree of bridge merges across tiles, for segments whose junctions do
-// not resolve locally (seg_mode 2).  All tile hulls are written.  A CTA takes
+// not resolve locally and are not one cluster (seg_mode 3 with seg_below).  All tile hulls are written.  A CTA takes
 // one hull tile after another (a small grid); for each it starts the tile's
 // node list, then climbs: at each level the CTA that arrives second merges
 // the two children of the parent, the first one goes on to its next tile.
@@ -606,18 +609,21 @@ __global__ void __launch_bounds__(HNT) k_climb(const TileDesc* __restrict__ htil
                                                const TileScale* __restrict__ scales, const uint16_t* vp, const i128* vx,
                                                const int32_t* __restrict__ nvert, i128* tile_total, Piece* pieces,
                                                int32_t* npieces, int32_t* arrive, int n_hull,
-                                               const int32_t* __restrict__ seg_mode) {
+                                               const int32_t* __restrict__ seg_mode,
+                                               const int32_t* __restrict__ seg_below) {
     __shared__ ClimbSmem s;
     const int t = threadIdx.x;
+    ws_chain();
+    auto to_climb = [&](int lseg) { return seg_mode[lseg] == 3 && seg_below[lseg] != 0; };
     // Most calls have no segment left for the tree: all threads check this
     // CTA's tiles at once, instead of one tile per round trip in the loop below.
     bool any = false;
     for (int tile = blockIdx.x + t * gridDim.x; tile < n_hull; tile += HNT * gridDim.x)
-        any |= seg_mode[htiles[tile].lseg] == 2;
+        any |= to_climb(htiles[tile].lseg);
     if (!__syncthreads_or(any)) return;
     for (int tile = blockIdx.x; tile < n_hull; tile += gridDim.x) {
     const TileDesc td = htiles[tile];
-    if (seg_mode[td.lseg] != 2) continue;   // (uniform)
+    if (!to_climb(td.lseg)) continue;   // (uniform)
     __syncthreads();   // (the previous tile's shared memory is dead)
     const LargeSeg ls = lsegs[td.lseg];
     if (t == 0) {
@@ -652,15 +658,47 @@ __global__ void __launch_bounds__(HNT) k_climb(const TileDesc* __restrict__ htil
 // ---------------------------------------------------------------------------
 // 4. root of each segment: cluster count, piece index per tile
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_root(const LargeSeg* __restrict__ lsegs, const Piece* pieces,
-                                              const int32_t* npieces, int32_t* tile_piece, SegRuntime* rt,
-                                              int64_t* n_clusters_out) {
-    const int lseg = blockIdx.x;
-    const LargeSeg ls = lsegs[lseg];
-    const Piece* P = pieces + ls.hull_first;
-    const int np = npieces[ls.hull_first];
-    for (int i = threadIdx.x; i < np; i += 256) tile_piece[P[i].tile] = i;
-    if (threadIdx.x == 0) {
+// `parts` CTAs per segment share the numbering; the first also writes the list
+// of a segment that the chord check left as one cluster (its first and its last
+// point).
+__global__ void __launch_bounds__(256) k_root(const LargeSeg* __restrict__ lsegs, const int32_t* __restrict__ nvert,
+                                              const i128* __restrict__ tile_base, const int32_t* __restrict__ seg_mode,
+                                              const int32_t* __restrict__ seg_below, Piece* pieces, int32_t* npieces,
+                                              int32_t* tile_piece, SegRuntime* rt, int64_t* n_clusters_out,
+                                              int parts) {
+    ws_chain();
+    const int lseg = blockIdx.x / parts, part = blockIdx.x % parts;
+    const LargeSeg& ls = lsegs[lseg];
+    const int h0 = ls.hull_first;
+    if (seg_mode[lseg] == 3 && !seg_below[lseg]) {   // (uniform)
+        if (part != 0 || threadIdx.x != 0) return;
+        const int kl = ls.hull_count - 1, nvl = nvert[h0 + kl];
+        Piece a;
+        a.tile = h0; a.lo = 0; a.hi = 1; a.cum = 0; a.pad = 0; a.off = 0;
+        int np = 1;
+        if (kl == 0) {   // one tile: the chord is its hull
+            a.hi = (uint16_t)nvl;
+        } else {
+            Piece z;
+            z.tile = h0 + kl; z.lo = (uint16_t)(nvl - 1); z.hi = (uint16_t)nvl; z.cum = 1; z.pad = 0;
+            z.off = tile_base[h0 + kl];
+            pieces[h0 + 1] = z;
+            tile_piece[h0 + kl] = 1;
+            np = 2;
+        }
+        pieces[h0] = a;
+        npieces[h0] = np;
+        tile_piece[h0] = 0;
+        const int64_t c = kl == 0 ? nvl - 1 : 1;
+        rt[lseg].n_clusters = c;
+        rt[lseg].table_pos = ls.kpos + lseg;
+        if (n_clusters_out) n_clusters_out[ls.seg] = c;
+        return;
+    }
+    const Piece* P = pieces + h0;
+    const int np = npieces[h0];
+    for (int i = part * 256 + threadIdx.x; i < np; i += 256 * parts) tile_piece[P[i].tile] = i;
+    if (part == 0 && threadIdx.x == 0) {
         const Piece last = P[np - 1];
         const int64_t c = (int64_t)last.cum + (last.hi - last.lo) - 1;
         rt[lseg].n_clusters = c;
@@ -697,6 +735,7 @@ __global__ void __launch_bounds__(256, 6) k_values(const TileDesc* __restrict__ 
     __shared__ uint32_t words[HTW];
     __shared__ int wsum[8];
     __shared__ int s_base;
+    ws_chain();
     const int tile = blockIdx.x, t = threadIdx.x;
     const int tp = tile_piece[tile];
     const TileDesc td = htiles[tile];
@@ -850,6 +889,7 @@ __global__ void __launch_bounds__(256, 6) k_bin_out(const LargeSeg* __restrict__
     extern __shared__ __align__(16) unsigned char pair_smem_raw[];
     OutPair<T>* stage = reinterpret_cast<OutPair<T>*>(pair_smem_raw);   // [WS_BIN_CAP]
     const int t = threadIdx.x;
+    ws_chain();
     if ((int)blockIdx.x < n_bins) {
         const int bin = blockIdx.x;
         const int lseg = bin_seg[bin];
@@ -935,6 +975,7 @@ template <typename T>
 __global__ void __launch_bounds__(GNT) k_regroup(const TileDesc* __restrict__ tiles, const LargeSeg* __restrict__ lsegs,
                                                  const SegRuntime* __restrict__ rt, const uint32_t* __restrict__ dest,
                                                  const OutPair<T>* __restrict__ from, OutPair<T>* __restrict__ to) {
+    ws_chain();
     const TileDesc td = tiles[blockIdx.x];
     const LargeSeg& sg = lsegs[td.lseg];
     if (sg.fine_log2 == 0 || rt[td.lseg].n_clusters == 1) return;
@@ -960,6 +1001,7 @@ __global__ void __launch_bounds__(GNT) k_output(const TileDesc* __restrict__ til
                                                 const SegRuntime* __restrict__ rt, const T* __restrict__ cval,
                                                 const uint32_t* __restrict__ dest, const OutPair<T>* __restrict__ pairs_a,
                                                 const OutPair<T>* __restrict__ pairs_b, T* out, int32_t* ids) {
+    ws_chain();
     const TileDesc td = tiles[blockIdx.x];
     const LargeSeg& sg = lsegs[td.lseg];
     if (rt[td.lseg].n_clusters == 1) {   // one cluster (large lambda): every weight gets its value
@@ -1002,9 +1044,9 @@ __global__ void k_copy_sorted(const typename KeyOf<T>::K* __restrict__ sorted, c
 // host-side sequencing of the large path
 // ---------------------------------------------------------------------------
 template <typename T>
-cudaError_t ws_large_prox(const LargeWork<T>& W, const T* values, const double* lambdas, T* out, int32_t* ids,
+cudaError_t ws_large_prox(const LargeWork<T>& W, const T* values, WsLambda lambdas, T* out, int32_t* ids,
                           int64_t* n_clusters, int fp64, const WsEpi& ep, uint32_t* status, uint64_t spin_limit,
-                          int n_levels, cudaStream_t st) {
+                          cudaStream_t st) {
     typedef typename KeyOf<T>::K K;
     if (W.n_lseg == 0) return cudaSuccess;
     K* sorted = nullptr;
@@ -1018,42 +1060,42 @@ cudaError_t ws_large_prox(const LargeWork<T>& W, const T* values, const double* 
     if (e) return e;
     const int small_grid = W.n_hull_tiles < 4 * 152 ? W.n_hull_tiles : 4 * 152;
     WS_LAUNCH(W.prof, WSK_TILE_GENERAL, st,
-              (k_tile_hull<T><<<small_grid, HNT, smem, st>>>(sorted, W.hull_tiles, W.lsegs, lambdas, W.rt, W.vp, W.vx,
-                                                            W.nvert, W.tile_total, W.gen_list, W.gen_count,
-                                                            W.seg_emin, status)));
+              ws_launch_chain(k_tile_hull<T>, small_grid, HNT, smem, st, sorted, W.hull_tiles, W.lsegs, lambdas, W.rt,
+                              W.vp, W.vx, W.nvert, W.tile_total, W.gen_list, &W.ctl->gen_count, W.seg_emin, status));
     // across tiles: junction bridges and the per-segment resolution, then the
     // tree of merges for the segments that need it
     e = ws_large_junctions<T>(W, st);
     if (e) return e;
-    e = cudaMemsetAsync(W.arrive, 0, sizeof(int32_t) * (size_t)n_levels * W.n_hull_tiles, st);
-    if (e) return e;
     WS_LAUNCH(W.prof, WSK_CLIMB, st,
-              (k_climb<<<small_grid, HNT, 0, st>>>(W.hull_tiles, W.lsegs, W.scales, W.vp, W.vx, W.nvert,
-                                                          W.tile_total, W.pieces, W.npieces, W.arrive,
-                                                          W.n_hull_tiles, W.seg_mode)));
-    e = cudaMemsetAsync(W.tile_piece, 0xff, sizeof(int32_t) * (size_t)W.n_hull_tiles, st);
-    if (e) return e;
+              ws_launch_chain(k_climb, small_grid, HNT, 0, st, W.hull_tiles, W.lsegs, W.scales, W.vp, W.vx, W.nvert,
+                              W.tile_total, W.pieces, W.npieces, W.arrive, W.n_hull_tiles, W.seg_mode, W.seg_below));
+    // CTAs per segment of the numbering: one per 1024 tiles of an average segment
+    const int parts = std::max(1, std::min(16, W.n_hull_tiles / W.n_lseg / 1024));
     WS_LAUNCH(W.prof, WSK_ROOT, st,
-              (k_root<<<W.n_lseg, 256, 0, st>>>(W.lsegs, W.pieces, W.npieces, W.tile_piece, W.rt, n_clusters)));
+              ws_launch_chain(k_root, W.n_lseg * parts, 256, 0, st, W.lsegs, W.nvert, W.tile_base, W.seg_mode,
+                              W.seg_below, W.pieces, W.npieces, W.tile_piece, W.rt, n_clusters, parts));
     WS_LAUNCH(W.prof, WSK_VALUES, st,
-              (k_values<T><<<W.n_hull_tiles, 256, 0, st>>>(W.hull_tiles, W.lsegs, W.scales, W.rt, sorted, W.vp, W.vx,
-                                                          W.pieces, W.npieces, W.tile_piece, W.cval, W.rank_words,
-                                                          fp64, ep, status)));
+              ws_launch_chain(k_values<T>, W.n_hull_tiles, 256, 0, st, W.hull_tiles, W.lsegs, W.scales, W.rt, sorted,
+                              W.vp, W.vx, W.pieces, W.npieces, W.tile_piece, W.cval, W.rank_words, fp64, ep, status));
     // back to the caller's order
-    e = cudaFuncSetAttribute(k_bin_out<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(OutPair<T>) * WS_BIN_CAP);
+    const size_t osm = sizeof(OutPair<T>) * WS_BIN_CAP;
+    e = cudaFuncSetAttribute(k_bin_out<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)osm);
     if (e) return e;
     WS_LAUNCH(W.prof, WSK_BIN_OUT, st,
-              (k_bin_out<T><<<W.n_bins + OUT_EXTRA, 256, sizeof(OutPair<T>) * WS_BIN_CAP, st>>>(W.lsegs, W.rt, W.bin_seg, W.bin_start, W.bin_cnt,
-                                                                 W.n_bins, W.bin_idx, W.rank_words, W.cval, sorted,
-                                                                 W.keys_b, W.ctl, W.over, W.pairs_b)));
+              ws_launch_chain(k_bin_out<T>, W.n_bins + OUT_EXTRA, 256, osm, st, W.lsegs, W.rt, W.bin_seg, W.bin_start,
+                              W.bin_cnt, W.n_bins, W.bin_idx, W.rank_words, W.cval, sorted, W.keys_b, W.ctl, W.over,
+                              W.pairs_b));
+    // (the two gathers want their L1: beside the CTAs of k_bin_out they take
+    // twice as long, at 2^24 937 us per call against 810; up to two tiles per
+    // SM the launch counts for more)
+    const bool early = W.n_sort_tiles <= 2 * 152;
     if (W.two_level)
         WS_LAUNCH(W.prof, WSK_REGROUP, st,
-                  (k_regroup<T><<<W.n_sort_tiles, GNT, 0, st>>>(W.sort_tiles, W.lsegs, W.rt, W.dest2, W.pairs_b,
-                                                               W.pairs_a)));
+                  ws_launch_if(early, k_regroup<T>, W.n_sort_tiles, GNT, 0, st, W.sort_tiles, W.lsegs, W.rt, W.dest2,
+                                  W.pairs_b, W.pairs_a));
     WS_LAUNCH(W.prof, WSK_OUTPUT, st,
-              (k_output<T><<<W.n_sort_tiles, GNT, 0, st>>>(W.sort_tiles, W.lsegs, W.rt, W.cval, W.dest1, W.pairs_a,
-                                                          W.pairs_b, out, ids)));
+              ws_launch_if(early, k_output<T>, W.n_sort_tiles, GNT, 0, st, W.sort_tiles, W.lsegs, W.rt, W.cval, W.dest1,
+                              W.pairs_a, W.pairs_b, out, ids));
     return cudaGetLastError();
 }
 
@@ -1066,8 +1108,8 @@ cudaError_t ws_large_copy_sorted(const LargeWork<T>& W, const typename KeyOf<T>:
 }
 
 #define WS_INST(T)                                                                                                  \
-    template cudaError_t ws_large_prox<T>(const LargeWork<T>&, const T*, const double*, T*, int32_t*, int64_t*, int, \
-                                          const WsEpi&, uint32_t*, uint64_t, int, cudaStream_t);                    \
+    template cudaError_t ws_large_prox<T>(const LargeWork<T>&, const T*, WsLambda, T*, int32_t*, int64_t*, int, \
+                                          const WsEpi&, uint32_t*, uint64_t, cudaStream_t);                         \
     template cudaError_t ws_large_copy_sorted<T>(const LargeWork<T>&, const typename KeyOf<T>::K*, T*, cudaStream_t);
 WS_INST(float)
 WS_INST(double)

@@ -95,7 +95,7 @@ __device__ __forceinline__ void small_sort_bucket(int b0, int b1, K* keys, uint1
 template <typename T, int NT, int M>
 __device__ __forceinline__ void small_general_segment(SmallSmem<T, NT, M>& s, int seg, const T* __restrict__ values,
                                                       const int64_t* __restrict__ offsets,
-                                                      const double* __restrict__ lambdas, T* out, int32_t* ids,
+                                                      const WsLambda& lambdas, T* out, int32_t* ids,
                                                       int64_t* n_clusters, int fp64, const WsEpi& ep,
                                                       uint32_t* status) {
     typedef KeyOf<T> KO;
@@ -107,7 +107,7 @@ __device__ __forceinline__ void small_general_segment(SmallSmem<T, NT, M>& s, in
 
     const int64_t a0 = offsets[seg];
     const int n = (int)(offsets[seg + 1] - a0);
-    const double lam = lambdas[seg];
+    const double lam = lambdas.at(seg);
     if (!(lam >= 0.0) || !(lam <= 1.7976931348623157e308)) {
         if (t == 0) ws_flag(status, WS_STATUS_BAD_LAMBDA);
         return;
@@ -386,11 +386,12 @@ __global__ void __launch_bounds__(NT, 3) k_small_general(const T* __restrict__ v
                                                       const int64_t* __restrict__ offsets,
                                                       const int32_t* __restrict__ gen_list,
                                                       const int32_t* __restrict__ gen_count,
-                                                      const double* __restrict__ lambdas, T* out, int32_t* ids,
+                                                      const WsLambda lambdas, T* out, int32_t* ids,
                                                       int64_t* n_clusters, int fp64, const WsEpi ep,
                                                       uint32_t* status) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SmallSmem<T, NT, M>& s = *reinterpret_cast<SmallSmem<T, NT, M>*>(smem_raw);
+    ws_chain();
     const int cnt = *gen_count;
     for (int i = blockIdx.x; i < cnt; i += gridDim.x) {
         small_general_segment<T, NT, M>(s, gen_list[i], values, offsets, lambdas, out, ids, n_clusters, fp64, ep,
@@ -573,7 +574,7 @@ template <typename T>
 __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 4 : 2) k_small(const T* __restrict__ values,
                                                    const int64_t* __restrict__ offsets,
                                                    const int32_t* __restrict__ seg_list,
-                                                   const double* __restrict__ lambdas, T* out, int32_t* ids,
+                                                   const WsLambda lambdas, T* out, int32_t* ids,
                                                    int64_t* n_clusters, int fp64, const WsEpi ep, uint32_t* status,
                                                    int32_t* gen_list, int32_t* gen_count, int ic_cap,
                                                    const int32_t* ids_prev) {   // (may alias ids)
@@ -590,7 +591,7 @@ __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 4 : 2) k_small(const
     const int seg = seg_list[blockIdx.x];
     const int64_t a0 = offsets[seg];
     const int n = (int)(offsets[seg + 1] - a0);
-    const double lam = lambdas[seg];
+    const double lam = lambdas.at(seg);
     if (!(lam >= 0.0) || !(lam <= 1.7976931348623157e308)) {
         if (t == 0) ws_flag(status, WS_STATUS_BAD_LAMBDA);
         return;
@@ -988,7 +989,7 @@ __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 4 : 2) k_small(const
 // ---------------------------------------------------------------------------
 template <typename T>
 cudaError_t ws_launch_small(const T* values, const int64_t* offsets, const int32_t* seg_list, int n_list,
-                            const double* lambdas, T* out, int32_t* ids, int64_t* n_clusters, int fp64,
+                            WsLambda lambdas, T* out, int32_t* ids, int64_t* n_clusters, int fp64,
                             const WsEpi& ep, uint32_t* status, cudaStream_t st, WsProf* prof, int32_t* gen_list,
                             int32_t* gen_count, int ic_cap, const int32_t* ids_prev) {
     constexpr int NT = 256;
@@ -1009,14 +1010,14 @@ cudaError_t ws_launch_small(const T* values, const int64_t* offsets, const int32
     e = cudaFuncSetAttribute(gk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsmem);
     if (e != cudaSuccess) return e;
     WS_LAUNCH(prof, WSK_SMALL, st,
-              (gk<<<n_list < 456 ? n_list : 456, NT, gsmem, st>>>(values, offsets, gen_list, gen_count, lambdas, out, ids,
-                                                               n_clusters, fp64, ep, status)));
+              ws_launch_chain(gk, n_list < 456 ? n_list : 456, NT, gsmem, st, values, offsets, gen_list, gen_count,
+                              lambdas, out, ids, n_clusters, fp64, ep, status));
     return cudaGetLastError();
 }
 
-template cudaError_t ws_launch_small<float>(const float*, const int64_t*, const int32_t*, int, const double*, float*,
+template cudaError_t ws_launch_small<float>(const float*, const int64_t*, const int32_t*, int, WsLambda, float*,
                                             int32_t*, int64_t*, int, const WsEpi&, uint32_t*, cudaStream_t, WsProf*,
                                             int32_t*, int32_t*, int, const int32_t*);
-template cudaError_t ws_launch_small<double>(const double*, const int64_t*, const int32_t*, int, const double*,
+template cudaError_t ws_launch_small<double>(const double*, const int64_t*, const int32_t*, int, WsLambda,
                                              double*, int32_t*, int64_t*, int, const WsEpi&, uint32_t*, cudaStream_t,
                                              WsProf*, int32_t*, int32_t*, int, const int32_t*);

@@ -506,6 +506,7 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
     static_assert(WS_FAN == NT, "one bucket per thread");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     PartSmem<T, B>& s = *reinterpret_cast<PartSmem<T, B>*>(smem_raw);
+    ws_chain();
     if (ctl->abort) return;
     const int t = threadIdx.x;
     // the next tile of this CTA from `tile` on that this pass moves
@@ -817,6 +818,7 @@ __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>:
     typedef typename KO::K K;
     extern __shared__ __align__(16) unsigned char bin_smem_raw[];
     BinSmem<T>& s = *reinterpret_cast<BinSmem<T>*>(bin_smem_raw);
+    ws_chain();
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     if (ctl->abort) {   // the keys were not moved: a sequence that is sorted, so that later steps see a valid one
         for (int64_t i = (int64_t)blockIdx.x * BIN_NT + t; i < n_keys; i += (int64_t)gridDim.x * BIN_NT)
@@ -1215,20 +1217,22 @@ static cudaError_t sort_run(const LargeWork<T>& W, const T* values, bool way_bac
     }
     const size_t ksm = sizeof(PartSmem<T, B>);
     const int grid = std::min(sh.part_grid, W.n_sort_tiles);
+    const T* no_values = nullptr;
+    K* no_keys = nullptr;
+    B* no_bins = nullptr;
     WS_LAUNCH(W.prof, WSK_PARTITION, st,
-              (k_part<T, B, true><<<grid, WS_SORT_NT, ksm, st>>>(values, nullptr, bins, W.keys_a, W.keys_b, bins2,
-                                                                 way_back ? W.dest1 : nullptr,
-                                                                 W.sort_tiles, W.n_sort_tiles, W.lsegs, W.cur1, W.ctl,
-                                                                 status)));
+              ws_launch_chain(k_part<T, B, true>, grid, WS_SORT_NT, ksm, st, values, no_keys, bins, W.keys_a,
+                              W.keys_b, bins2, way_back ? W.dest1 : nullptr, W.sort_tiles, W.n_sort_tiles, W.lsegs,
+                              W.cur1, W.ctl, status));
     if (W.two_level)
         WS_LAUNCH(W.prof, WSK_PARTITION, st,
-                  (k_part<T, B, false><<<grid, WS_SORT_NT, ksm, st>>>(nullptr, W.keys_a, bins2, nullptr, W.keys_b,
-                                                                      nullptr, way_back ? W.dest2 : nullptr, W.sort_tiles, W.n_sort_tiles, W.lsegs,
-                                                                      W.cur2, W.ctl, status)));
-    auto* kbin = way_back ? k_bin_sort<T, true> : k_bin_sort<T, false>;
+                  ws_launch_chain(k_part<T, B, false>, grid, WS_SORT_NT, ksm, st, no_values, W.keys_a, bins2, no_keys,
+                                  W.keys_b, no_bins, way_back ? W.dest2 : nullptr, W.sort_tiles, W.n_sort_tiles,
+                                  W.lsegs, W.cur2, W.ctl, status));
     WS_LAUNCH(W.prof, WSK_BIN_SORT, st,
-              (kbin<<<W.n_bins, BIN_NT, sizeof(BinSmem<T>), st>>>(W.keys_b, W.keys_a, W.bin_seg, W.lsegs, W.bin_start,
-                                                                 W.bin_cnt, W.bin_idx, W.ctl, W.over, W.n_keys)));
+              ws_launch_chain(way_back ? k_bin_sort<T, true> : k_bin_sort<T, false>, W.n_bins, BIN_NT,
+                              sizeof(BinSmem<T>), st, W.keys_b, W.keys_a, W.bin_seg, W.lsegs, W.bin_start, W.bin_cnt,
+                              W.bin_idx, W.ctl, W.over, W.n_keys));
     {
         K* ka = W.keys_a;
         K* kb = W.keys_b;

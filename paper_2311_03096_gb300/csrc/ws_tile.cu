@@ -14,10 +14,10 @@
 //                kept ranges is convex and lies below every point, hence it
 //                is the segment's hull, and it is written as the root piece
 //                list directly.
-//   k_chord,     otherwise: if every tile-hull vertex lies on or above the
-//   k_decide     chord from the segment's first point to its last, the
-//                segment is one cluster; else it takes the tree of bridge
-//                merges (k_climb in ws_large.cu).
+//   k_chord      otherwise: if every tile-hull vertex lies on or above the
+//                chord from the segment's first point to its last, the
+//                segment is one cluster (k_root in ws_large.cu writes its
+//                list); else it takes the tree of bridge merges (k_climb).
 // With small lambda the clusters are short and every tile keeps many
 // vertices, so the first case holds; with a lambda above the collapse
 // threshold (Prop. 4.1) the second does.
@@ -42,13 +42,14 @@ constexpr int CTA_WALK_CAP = 512;
 template <typename T>
 __global__ void __launch_bounds__(WS_NSCALE) k_scales(const typename KeyOf<T>::K* __restrict__ sorted,
                                                       const LargeSeg* __restrict__ lsegs,
-                                                      const double* __restrict__ lambdas,
+                                                      WsLambda lambdas,
                                                       const int32_t* __restrict__ seg_emin, SegRuntime* rt,
                                                       TileScale* scales, uint32_t* status) {
     typedef KeyOf<T> KO;
+    ws_chain();
     const int lseg = blockIdx.x, j = threadIdx.x;
     const LargeSeg ls = lsegs[lseg];
-    const double lam = lambdas[ls.seg];
+    const double lam = lambdas.at(ls.seg);
     const bool lam_ok = lam >= 0.0 && lam <= 1.7976931348623157e308;
     const double lamv = lam_ok ? lam : 0.0;
     const T xlo = KO::from_key(sorted[ls.kpos]), xhi = KO::from_key(sorted[ls.kpos + ls.len - 1]);
@@ -124,10 +125,12 @@ __global__ void __launch_bounds__(NT, 4) k_hull_fast(const typename KeyOf<T>::K*
                                                    const SegRuntime* __restrict__ rt,
                                                    const TileScale* __restrict__ scales, uint16_t* vp, i128* vx,
                                                    int32_t* nvert, i128* tile_total, int32_t* gen_list,
-                                                   int32_t* gen_count, int32_t* tile_rounds, int ic_cap) {
+                                                   int32_t* gen_count, int32_t* tile_rounds, int32_t* tile_piece,
+                                                   int ic_cap) {
     typedef KeyOf<T> KO;
     typedef typename KO::K K;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    ws_chain();
     FastSmem& S = *reinterpret_cast<FastSmem*>(smem_raw);
     wsh::Smem& s = S.h;
     const int t = threadIdx.x, l = t & 31, w = t >> 5;
@@ -145,6 +148,7 @@ __global__ void __launch_bounds__(NT, 4) k_hull_fast(const typename KeyOf<T>::K*
     const bool lean = ws_lean_x(range, n);   // prefix sums in 64 bits
     const bool d64 = ws_lean_tile(range, n);  // every Delta too
     if (t == 0) {
+        tile_piece[tile] = -1;   // (k_root numbers the pieces)
         if (!lean) { gen_list[atomicAdd(gen_count, 1)] = tile; tile_rounds[tile] = -2; }
         else S.ts = scales[(size_t)td.lseg * WS_NSCALE + (bin ? sh : WS_NSCALE - 1)];
         s.general = 0;
@@ -299,6 +303,7 @@ __global__ void __launch_bounds__(256) k_junction(const TileDesc* __restrict__ h
                                                   const int32_t* __restrict__ nvert,
                                                   const i128* __restrict__ tile_total, int32_t* keepR, int32_t* keepL,
                                                   int32_t* jflag0, int n_hull) {
+    ws_chain();
     const int gw = (int)(blockIdx.x * blockDim.x + threadIdx.x);   // one thread per junction
     if (gw >= n_hull) return;
     const TileDesc td = htiles[gw];
@@ -385,6 +390,7 @@ __global__ void __launch_bounds__(RNT) k_resolve(const LargeSeg* __restrict__ ls
                                                  int32_t* npieces, int32_t* seg_mode, i128* tile_base,
                                                  i128* seg_total, int32_t* seg_below) {
     __shared__ ResolveSmem s;
+    ws_chain();
     const int t = threadIdx.x;
     const int lseg = blockIdx.x;
     const LargeSeg ls = lsegs[lseg];
@@ -452,6 +458,7 @@ __global__ void __launch_bounds__(256) k_chord(const TileDesc* __restrict__ htil
                                                const i128* __restrict__ seg_total,
                                                const int32_t* __restrict__ seg_mode, int32_t* seg_below,
                                                int n_hull) {
+    ws_chain();
     const int gw = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5);
     const int lane = threadIdx.x & 31;
     if (gw >= n_hull) return;
@@ -475,51 +482,21 @@ __global__ void __launch_bounds__(256) k_chord(const TileDesc* __restrict__ htil
     if (below) atomicExch(seg_below + td.lseg, 1);
 }
 
-// Per segment left undecided: one cluster (root list = the first and the last
-// point) or the tree of merges.
-__global__ void k_decide(const LargeSeg* __restrict__ lsegs, int n_lseg, const int32_t* __restrict__ nvert,
-                         const i128* __restrict__ tile_base, int32_t* seg_mode, const int32_t* __restrict__ seg_below,
-                         Piece* pieces, int32_t* npieces) {
-    const int lseg = blockIdx.x * blockDim.x + threadIdx.x;
-    if (lseg >= n_lseg || seg_mode[lseg] != 3) return;
-    if (seg_below[lseg]) { seg_mode[lseg] = 2; return; }
-    const LargeSeg ls = lsegs[lseg];
-    const int h0 = ls.hull_first, kl = ls.hull_count - 1;
-    const int nvl = nvert[h0 + kl];
-    Piece a;
-    a.tile = h0; a.lo = 0; a.hi = 1; a.cum = 0; a.pad = 0; a.off = 0;
-    if (kl == 0) {   // one tile: the chord is its hull
-        a.hi = (uint16_t)nvl;
-        pieces[h0] = a;
-        npieces[h0] = 1;
-    } else {
-        Piece z;
-        z.tile = h0 + kl; z.lo = (uint16_t)(nvl - 1); z.hi = (uint16_t)nvl; z.cum = 1; z.pad = 0;
-        z.off = tile_base[h0 + kl];
-        pieces[h0] = a;
-        pieces[h0 + 1] = z;
-        npieces[h0] = 2;
-    }
-    seg_mode[lseg] = 1;
-}
-
 }  // namespace
 
 template <typename T>
-cudaError_t ws_large_hull_fast(const LargeWork<T>& W, const typename KeyOf<T>::K* sorted, const double* lambdas,
+cudaError_t ws_large_hull_fast(const LargeWork<T>& W, const typename KeyOf<T>::K* sorted, WsLambda lambdas,
                                uint32_t* status, cudaStream_t st) {
     WS_LAUNCH(W.prof, WSK_MISC, st,
-              (k_scales<T><<<W.n_lseg, WS_NSCALE, 0, st>>>(sorted, W.lsegs, lambdas, W.seg_emin, W.rt, W.scales,
-                                                           status)));
+              ws_launch_chain(k_scales<T>, W.n_lseg, WS_NSCALE, 0, st, sorted, W.lsegs, lambdas, W.seg_emin, W.rt,
+                              W.scales, status));
     const size_t smem = sizeof(FastSmem);
     cudaError_t e = cudaFuncSetAttribute(k_hull_fast<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e) return e;
-    e = cudaMemsetAsync(W.gen_count, 0, sizeof(int32_t), st);
-    if (e) return e;
     WS_LAUNCH(W.prof, WSK_TILE_HULL, st,
-              (k_hull_fast<T><<<W.n_hull_tiles, NT, smem, st>>>(sorted, W.hull_tiles, W.lsegs, W.rt, W.scales, W.vp,
-                                                                W.vx, W.nvert, W.tile_total, W.gen_list, W.gen_count,
-                                                                W.tile_rounds, W.ic_cap)));
+              ws_launch_chain(k_hull_fast<T>, W.n_hull_tiles, NT, smem, st, sorted, W.hull_tiles, W.lsegs, W.rt,
+                              W.scales, W.vp, W.vx, W.nvert, W.tile_total, W.gen_list, &W.ctl->gen_count,
+                              W.tile_rounds, W.tile_piece, W.ic_cap));
     return cudaGetLastError();
 }
 
@@ -528,25 +505,19 @@ cudaError_t ws_large_junctions(const LargeWork<T>& W, cudaStream_t st) {
     const int warps_per_cta = 8;
     const int grid = (W.n_hull_tiles + warps_per_cta - 1) / warps_per_cta;
     WS_LAUNCH(W.prof, WSK_JUNCTION, st,
-              (k_junction<<<(W.n_hull_tiles + 127) / 128, 128, 0, st>>>(W.hull_tiles, W.lsegs, W.scales, W.vp, W.vx,
-                                                                  W.nvert, W.tile_total, W.keepR, W.keepL, W.jflag0,
-                                                                  W.n_hull_tiles)));
+              ws_launch_chain(k_junction, (W.n_hull_tiles + 127) / 128, 128, 0, st, W.hull_tiles, W.lsegs, W.scales,
+                              W.vp, W.vx, W.nvert, W.tile_total, W.keepR, W.keepL, W.jflag0, W.n_hull_tiles));
     WS_LAUNCH(W.prof, WSK_JUNCTION, st,
-              (k_resolve<T><<<W.n_lseg, RNT, 0, st>>>(W.lsegs, W.nvert, W.tile_total, W.keepR, W.keepL, W.jflag0,
-                                                      W.pieces, W.npieces, W.seg_mode, W.tile_base, W.seg_total,
-                                                      W.seg_below)));
+              ws_launch_chain(k_resolve<T>, W.n_lseg, RNT, 0, st, W.lsegs, W.nvert, W.tile_total, W.keepR, W.keepL,
+                              W.jflag0, W.pieces, W.npieces, W.seg_mode, W.tile_base, W.seg_total, W.seg_below));
     WS_LAUNCH(W.prof, WSK_JUNCTION, st,
-              (k_chord<<<grid, 32 * warps_per_cta, 0, st>>>(W.hull_tiles, W.lsegs, W.scales, W.vp, W.vx,
-                                                               W.nvert, W.tile_base, W.seg_total, W.seg_mode,
-                                                               W.seg_below, W.n_hull_tiles)));
-    WS_LAUNCH(W.prof, WSK_JUNCTION, st,
-              (k_decide<<<(W.n_lseg + 255) / 256, 256, 0, st>>>(W.lsegs, W.n_lseg, W.nvert, W.tile_base,
-                                                                W.seg_mode, W.seg_below, W.pieces, W.npieces)));
+              ws_launch_chain(k_chord, grid, 32 * warps_per_cta, 0, st, W.hull_tiles, W.lsegs, W.scales, W.vp, W.vx,
+                              W.nvert, W.tile_base, W.seg_total, W.seg_mode, W.seg_below, W.n_hull_tiles));
     return cudaGetLastError();
 }
 
 #define WS_INST_TILE(T)                                                                                          \
-    template cudaError_t ws_large_hull_fast<T>(const LargeWork<T>&, const typename KeyOf<T>::K*, const double*, \
+    template cudaError_t ws_large_hull_fast<T>(const LargeWork<T>&, const typename KeyOf<T>::K*, WsLambda, \
                                                uint32_t*, cudaStream_t);                                         \
     template cudaError_t ws_large_junctions<T>(const LargeWork<T>&, cudaStream_t);
 WS_INST_TILE(float)
