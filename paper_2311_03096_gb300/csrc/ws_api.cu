@@ -109,7 +109,7 @@ struct ws_plan {
     void* bsum = nullptr;
     int32_t* bcnt = nullptr;
     unsigned long long* bacc = nullptr;
-    int32_t* bwd_seg = nullptr;
+    BwdWork bwd = {};
     // plans with both one-CTA and device-wide segments: the one-CTA kernel
     // runs on this stream, forked from and joined back into the caller's
     cudaStream_t side = nullptr;
@@ -180,7 +180,7 @@ LargeWork<T> make_work(const ws_plan* p) {
     W.bsum = (T*)p->bsum;
     W.bcnt = p->bcnt;
     W.bacc = p->bacc;
-    W.bwd_seg = p->bwd_seg;
+    W.bwd = p->bwd;
     W.prof = &p->ctx->prof;
     return W;
 }
@@ -232,6 +232,8 @@ ws_status build_plan(ws_plan* p) {
     int64_t kpos = 0;
     int64_t bin_pos = 0, coarse_pos = 0, cell_pos = 0;
     std::vector<int32_t> bin_seg;
+    std::vector<int2> bwd_map;
+    int32_t bwd_coarse = 0;
     int samp_max = 0;
     for (int64_t s = 0; s < p->n_seg; ++s) {
         int64_t a = p->h_offsets[s], len = p->h_offsets[s + 1] - a;
@@ -278,6 +280,19 @@ ws_status build_plan(ws_plan* p) {
         cell_pos += 3 * ls.ncell;   // counts of the cells, then of their parts (at most two per cell on average)
         if (cell_pos > INT32_MAX || bin_pos > INT32_MAX) return WS_ERR_NOMEM;
         p->max_bins = std::max(p->max_bins, (int)ls.nbins);
+        // backward: bins of cluster slots, moved into in one pass or two
+        ls.bb_n = (int32_t)((len + WS_BWD_BIN - 1) >> WS_BWD_BIN_LOG2);
+        ls.bb_fine = 0;
+        if (ls.bb_n > WS_BWD_FAN) {
+            ls.bb_fine = 7;
+            while (((ls.bb_n - 1) >> ls.bb_fine) + 1 > WS_BWD_FAN) ++ls.bb_fine;
+            p->bwd.two_level = 1;
+        }
+        ls.bb_pos = (int32_t)bwd_map.size();
+        ls.bb_cpos = bwd_coarse;
+        for (int b = 0; b < ls.bb_n; ++b)
+            bwd_map.push_back(make_int2(lseg, (b & ((1 << ls.bb_fine) - 1)) == 0 ? ls.bb_cpos + (b >> ls.bb_fine) : -1));
+        bwd_coarse += ((ls.bb_n - 1) >> ls.bb_fine) + 1;
         bin_seg.insert(bin_seg.end(), (size_t)ls.nbins, (int32_t)lseg);
         kpos += (len + 3) & ~(int64_t)3;   // keep every segment's keys 16-byte aligned
         lsegs.push_back(ls);
@@ -381,7 +396,27 @@ ws_status build_plan(ws_plan* p) {
         p->pairs_b = p->bacc;
         p->pairs_a = (unsigned char*)p->pairs_b + pair * nk;   // (two-level plans only)
     }
-    if ((st = plan_alloc(p, (void**)&p->bwd_seg, 2 * sizeof(int32_t) * p->n_lseg))) return st;
+    if (!p->sort_only) {
+        BwdWork& B = p->bwd;
+        B.n_bins = (int)bwd_map.size();
+        bwd_map.resize((bwd_map.size() + 7) & ~(size_t)7, make_int2(0, -1));   // (k_bwd_scan reads eight bins at a time)
+        const size_t nb = bwd_map.size(), nl4 = ((size_t)p->n_lseg + 3) & ~(size_t)3;
+        const size_t words = nl4 + 3 * nb + 1;
+        B.zero_bytes = sizeof(int32_t) * words;
+        if ((st = plan_alloc(p, (void**)&B.emax, B.zero_bytes))) return st;
+        B.cnt = (uint32_t*)B.emax + nl4;
+        B.extra = B.cnt + nb;
+        B.arrive = B.extra + nb;
+        B.n_items = (int32_t*)(B.arrive + nb);
+        int2* map = nullptr;
+        if ((st = plan_upload(p, &map, bwd_map))) return st;
+        B.map = map;
+        if ((st = plan_alloc(p, (void**)&B.start, sizeof(unsigned long long) * (nb + 2)))) return st;
+        if ((st = plan_alloc(p, (void**)&B.cur1, sizeof(unsigned long long) * (size_t)bwd_coarse))) return st;
+        if ((st = plan_alloc(p, (void**)&B.cur2, sizeof(unsigned long long) * nb))) return st;
+        // (a split bin has more than WS_BWD_PIECE pairs, so at most twice its pairs / WS_BWD_PIECE pieces)
+        if ((st = plan_alloc(p, (void**)&B.items, sizeof(uint2) * (2 * nk / WS_BWD_PIECE + 1)))) return st;
+    }
     if (cudaMemset(p->rt, 0, sizeof(SegRuntime) * p->n_lseg) != cudaSuccess) return WS_ERR_CUDA;
     return WS_OK;
 }

@@ -11,28 +11,38 @@
 // order of the additions, and its error does not grow with the cluster size
 // (one rounding when the mean is formed).
 //
-// Large segments: per-segment scale and largest id (k_bwd_prep), the used
-// cluster slots cleared (k_bwd_zero), the sums, the means (k_bwd_mean), the
-// gather (k_bwd_apply).  The sums: the cluster slots are cut into buckets of
-// 2^s consecutive slots, small enough for L2; k_bwd_scatter writes every
-// element as a pair (slot within its bucket, exact fixed-point code) into its
-// bucket's region (the regions sized by k_bwd_prep's bucket counts; each
-// tile's pairs are grouped by bucket in shared memory first, so every run is
-// copied out whole), and the CTAs of k_bwd_pairs take chunks of pairs in
-// order from a counter, so the atomics of the chunks in flight fall into one
-// or two buckets' slots and stay in L2 instead of each costing a random DRAM
-// read and write.  Lanes of a
-// warp with the same slot add once, and a sort tile whose elements all share
-// one cluster adds once per CTA (no pairs), so a single huge cluster costs
-// one atomic per sort tile.  The pairs and the bucket counters borrow the
-// forward's sort buffers, which the backward does not otherwise use.
+// Device-wide segments: the (grad_out, id) pairs are moved into bins of
+// WS_BWD_BIN consecutive cluster slots, whose sums fit the shared memory of one
+// CTA.  k_bwd_prep finds the segment's scale and counts the bins, k_bwd_scan
+// turns the counts into bin starts, k_bwd_part moves the pairs (in one pass up
+// to WS_BWD_FAN bins, in two above, as the forward's sort), k_bwd_bins adds a
+// bin's pairs into limbs in shared memory and writes the means, k_bwd_apply
+// gathers them.  A bin with more than PIECE pairs is added by several CTAs
+// (128-bit global atomics per slot, the last one writes the means).  A tile whose
+// elements all share one cluster adds its sum once and moves no pairs, so a
+// single huge cluster costs one atomic per tile.  The pairs borrow the forward's
+// sort buffers, which the backward does not otherwise use.
+//
+// FP32 2^24, clusters of a few elements, us: prep 52 (issue, the bins' adds),
+// scan 10, moves 71 + 67 (shared-memory wavefronts, 0.67 of the pipe), bins 123
+// (issue, 0.71: half the adds, half the conversions of 15 million means), apply
+// 76 (one line per lane and clock of the L1: 0.75 of that).  Three 64-bit global
+// atomics per pair instead of the bins took 876 in all; in every case measured
+// (from 5000 elements to 2^25, from one cluster to all distinct) the bins are
+// faster: 7 clusters of 2^24 elements 2825 -> 426, one cluster beside short ones
+// 1508 -> 420, 100000 elements 90 -> 30, 2^25 FP64 2201 -> 1492.
 // One-CTA segments: the same arithmetic in shared memory (k_small_backward).
 #include "ws_kernels.cuh"
 
 namespace {
 
-constexpr int BNT = 256;
-constexpr int BTILE = WS_SORT_TILE;   // elements per CTA (the sort tiles of the plan)
+constexpr int BTILE = WS_SORT_TILE;   // elements per tile (the sort tiles of the plan)
+constexpr int PNT = WS_SORT_NT, ITEMS = WS_SORT_ITEMS;
+constexpr int ANT = 256;              // k_bwd_bins
+constexpr int PIECE = WS_BWD_PIECE;
+constexpr int CHUNK = 8 * ANT;        // pairs of one step of k_bwd_bins
+constexpr int EXTRA = 4 * 152;        // CTAs of k_bwd_bins for the split bins
+constexpr int HIST_MAX = 16384;       // bins that k_bwd_prep counts in shared memory
 
 template <typename T> struct BwdFix;
 template <> struct BwdFix<float> { static constexpr int SH = 71, BIAS = 127, MANT = 23; };
@@ -59,42 +69,18 @@ __device__ __forceinline__ i128 ws_bwd_fix(T g, int emax) {
 template <typename T>
 __device__ __forceinline__ T ws_bwd_mean(i128 S, int cnt, int emax) {
     const int Lg = BwdFix<T>::SH - emax + BwdFix<T>::BIAS + BwdFix<T>::MANT;
-    if (sizeof(T) == 4) return (T)ldexpf(ws_i128_to_float_scaled(S, 0) / (float)cnt, -Lg);
+    if (sizeof(T) == 4) {
+        // as ws_i128_to_float_scaled(S, 0) / cnt * 2^-Lg with one scaling: powers of two commute with
+        // the division (no step leaves the normal range), and one multiplication rounds like ldexpf
+        const u128 mag = S < 0 ? (u128)(-S) : (u128)S;
+        const int sh = max(ws_bitlen128(mag) - 62, 0);
+        const float f = ws_u64_to_float((uint64_t)(mag >> sh)) / (float)cnt;
+        const int e = sh - Lg;
+        const float r = e >= -126 && e <= 127 ? f * __int_as_float((e + 127) << 23) : ldexpf(f, e);
+        return (T)(S < 0 ? -r : r);
+    }
     return (T)ldexp(ws_div_i128_n(S, cnt), -Lg);
 }
-
-// A ws_bwd_fix value in one word of the key's width: the significand m
-// (MANT + 1 bits, implicit bit included), the shift sh + MANT + 1 in 7 bits
-// (sh <= SH, and shifts below -(MANT + 1) give 0, stored as m = 0), the sign
-// on top.  Decoding gives back ws_bwd_fix(g, emax) exactly, with no segment
-// at hand.
-template <typename T>
-__device__ __forceinline__ typename KeyOf<T>::K ws_bwd_encode(T g, int emax) {
-    typedef KeyOf<T> KO;
-    typedef typename KO::K K;
-    constexpr int MB = KO::MANT + 1;
-    const uint64_t b = (uint64_t)KO::bits(g);
-    int e = (int)((b >> KO::MANT) & KO::EXPMASK);
-    uint64_t m = b & ((1ull << KO::MANT) - 1ull);
-    if (e == 0) e = 1; else m |= (1ull << KO::MANT);
-    int sh = e - emax + BwdFix<T>::SH;
-    if (sh < -MB) { m = 0; sh = 0; }
-    const uint64_t neg = (b >> (KO::BITS - 1)) & 1ull;
-    return (K)((neg << (KO::BITS - 1)) | ((uint64_t)(sh + MB) << MB) | m);
-}
-template <typename T>
-__device__ __forceinline__ i128 ws_bwd_decode(typename KeyOf<T>::K c) {
-    typedef KeyOf<T> KO;
-    constexpr int MB = KO::MANT + 1;
-    const uint64_t w = (uint64_t)c;
-    const uint64_t m = w & ((1ull << MB) - 1ull);
-    const int sh = (int)((w >> MB) & 127u) - MB;
-    const u128 mag = sh >= 0 ? (u128)m << sh : (u128)(m >> (-sh));
-    return ((w >> (KO::BITS - 1)) & 1ull) ? -(i128)mag : (i128)mag;
-}
-
-constexpr int BK_MAX = 256;   // slot buckets at most
-constexpr int BL = 8;         // elements per thread whose loads are issued together (prep, scatter)
 
 __device__ __forceinline__ void ws_atomic_add_i128(unsigned long long* lo_hi, i128 v) {
     const unsigned long long lo = (unsigned long long)(uint64_t)v;
@@ -104,6 +90,11 @@ __device__ __forceinline__ void ws_atomic_add_i128(unsigned long long* lo_hi, i1
 }
 
 template <typename T> __device__ __forceinline__ int ws_g_exp(T g) { return g != (T)0 ? ws_eff_exp(g) : 0; }
+
+template <typename T> __device__ __forceinline__ T ws_g_of_bits(typename KeyOf<T>::K b) {
+    if (sizeof(T) == 4) return (T)__uint_as_float((uint32_t)b);
+    return (T)__longlong_as_double((long long)b);
+}
 
 // Sum of v over the lanes in `peers` (every one of them calls with the same
 // mask; the groups of a __match_any_sync may call side by side).  |v| < 2^95
@@ -122,301 +113,565 @@ __device__ __forceinline__ i128 ws_group_sum_i96(unsigned peers, i128 v) {
     return (i128)S - (i128)__popc(peers) * ((i128)1 << 95);
 }
 
-// 1. per segment: largest exponent of grad_out and largest cluster id
-// and, for the tiles that are not one cluster, the number of elements in
-// every slot bucket
-template <typename T>
-__global__ void __launch_bounds__(BNT) k_bwd_prep(const T* __restrict__ g, const int32_t* __restrict__ ids,
-                                                  const TileDesc* __restrict__ tiles,
-                                                  const LargeSeg* __restrict__ lsegs, int32_t* seg_emax,
-                                                  int32_t* seg_maxid, int nb, int s, unsigned long long* bk_cnt,
-                                                  uint32_t* status) {
-    __shared__ int h[BK_MAX];
-    const TileDesc td = tiles[blockIdx.x];
-    const LargeSeg ls = lsegs[td.lseg];
-    const int64_t slot0 = ls.kpos + td.lseg;
-    for (int b = threadIdx.x; b < nb; b += BNT) h[b] = 0;
-    __syncthreads();
-    const int id0 = ids[td.vpos];
-    int e = 0, mx = -1;
-    bool bad = false, same = true;
-    for (int i0 = threadIdx.x; i0 < td.len; i0 += BNT * BL) {
-        int idv[BL];
-        T gv[BL];
-#pragma unroll
-        for (int k = 0; k < BL; ++k) {   // (indices clamped into the tile: every load in bounds)
-            const int i = min(i0 + k * BNT, td.len - 1);
-            idv[k] = ids[td.vpos + i];
-            gv[k] = g[td.vpos + i];
-        }
-#pragma unroll
-        for (int k = 0; k < BL; ++k) {
-            if (i0 + k * BNT >= td.len) continue;
-            e = max(e, ws_g_exp(gv[k]));
-            const int id = idv[k];
-            same &= id == id0;
-            if (id < 0 || (int64_t)id >= ls.len) bad = true;
-            else {
-                mx = max(mx, id);
-                atomicAdd(&h[(int)((slot0 + id) >> s)], 1);
-            }
-        }
-    }
-    if (!__syncthreads_and(same))
-        for (int b = threadIdx.x; b < nb; b += BNT)
-            if (h[b]) atomicAdd(bk_cnt + b, (unsigned long long)h[b]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(seg_emax + td.lseg, e);
-        atomicMax(seg_maxid + td.lseg, mx);
-    }
-    if (bad) ws_flag(status, WS_STATUS_INTERNAL);
-}
+// Sums in shared memory, as five signed 19-bit limbs per cluster.  A grad_out
+// value of MANT + 1 bits falls into at most three of them (four for double),
+// each one 32-bit shared-memory add without a returned value (native; a 64-bit
+// shared atomic is a compare-and-swap loop), and 4096 adds of 19 bits cannot
+// overflow 32.  The limbs recombine to the integer that 128-bit additions give.
+constexpr int LIMBS = 5, LIMB_BITS = 19;   // 95 bits: every ws_bwd_fix value
+constexpr uint32_t LIMB_MASK = (1u << LIMB_BITS) - 1u;
 
-// 2. clear the slots of ids 0 .. max id (tile k of a segment clears slots
-// [k BTILE, (k + 1) BTILE): a segment has at most len slots)
-__global__ void __launch_bounds__(BNT) k_bwd_zero(const TileDesc* __restrict__ tiles, const LargeSeg* __restrict__ lsegs,
-                                                  const int32_t* __restrict__ seg_maxid, unsigned long long* acc,
-                                                  int32_t* cnt) {
-    const TileDesc td = tiles[blockIdx.x];
-    const LargeSeg ls = lsegs[td.lseg];
-    const int64_t slot0 = ls.kpos + td.lseg;
-    const int64_t r0 = (int64_t)td.tin * BTILE;
-    const int64_t r1 = min(r0 + BTILE, (int64_t)seg_maxid[td.lseg] + 1);
-    for (int64_t r = r0 + threadIdx.x; r < r1; r += BNT) {
-        acc[2 * (slot0 + r)] = 0ull;
-        acc[2 * (slot0 + r) + 1] = 0ull;
-        cnt[slot0 + r] = 0;
-    }
-}
-
-// 3a. bucket regions: exclusive prefix of the counts (one thread; at most
-// BK_MAX buckets), the scatter cursors and the pairs pass's chunk counter
-__global__ void k_bwd_bscan(const unsigned long long* __restrict__ bk_cnt, int nb, unsigned long long* bk_off,
-                            unsigned long long* bk_cur) {
-    if (threadIdx.x != 0) return;
-    bk_cur[nb] = 0ull;
-    unsigned long long run = 0;
-    for (int b = 0; b < nb; ++b) {
-        bk_off[b] = run;
-        bk_cur[b] = run;
-        run += bk_cnt[b];
-    }
-    bk_off[nb] = run;
-}
-
-// 3b. a tile that is one cluster adds its exact sum once; every other tile
-// writes its elements as (slot within bucket, code) pairs into the bucket
-// regions: first into shared memory grouped by bucket, then each bucket's
-// run copied out to consecutive addresses (whole sectors, not one 4-byte
-// store per scattered element)
-template <typename T>
-size_t ws_bwd_scatter_smem() { return (size_t)BTILE * (sizeof(int32_t) + sizeof(typename KeyOf<T>::K) + 1); }
-
-template <typename T>
-__global__ void __launch_bounds__(BNT) k_bwd_scatter(const T* __restrict__ g, const int32_t* __restrict__ ids,
-                                                     const TileDesc* __restrict__ tiles,
-                                                     const LargeSeg* __restrict__ lsegs,
-                                                     const int32_t* __restrict__ seg_emax, unsigned long long* acc,
-                                                     int32_t* cnt, int nb, int s, unsigned long long* bk_cur,
-                                                     int32_t* pslot, typename KeyOf<T>::K* pcode) {
-    typedef typename KeyOf<T>::K K;
-    __shared__ long long wlo[BNT / 32], whi[BNT / 32];
-    __shared__ int h[BK_MAX], lstart[BK_MAX], wsum[BNT / 32];
-    __shared__ unsigned long long base[BK_MAX];
-    extern __shared__ __align__(16) unsigned char stage_raw[];
-    int32_t* st_slot = reinterpret_cast<int32_t*>(stage_raw);               // [BTILE]
-    K* st_code = reinterpret_cast<K*>(stage_raw + sizeof(int32_t) * BTILE);  // [BTILE]
-    uint8_t* st_b = stage_raw + (sizeof(int32_t) + sizeof(K)) * BTILE;      // [BTILE] bucket (nb <= 256)
-    static_assert(BK_MAX <= BNT && BK_MAX <= 256, "one thread per bucket; buckets fit a byte");
-    const TileDesc td = tiles[blockIdx.x];
-    const LargeSeg ls = lsegs[td.lseg];
-    const int64_t slot0 = ls.kpos + td.lseg;
-    const int emax = seg_emax[td.lseg];
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    auto valid_id = [&](int id) { return id >= 0 && (int64_t)id < ls.len; };
-    for (int b = t; b < nb; b += BNT) h[b] = 0;
-    __syncthreads();
-    const int id0 = ids[td.vpos];
-    bool same = true;
-    for (int i0 = t; i0 < td.len; i0 += BNT * BL) {
-        int idv[BL];
-#pragma unroll
-        for (int k = 0; k < BL; ++k) idv[k] = ids[td.vpos + min(i0 + k * BNT, td.len - 1)];
-#pragma unroll
-        for (int k = 0; k < BL; ++k) {
-            if (i0 + k * BNT >= td.len) continue;
-            same &= idv[k] == id0;
-            if (valid_id(idv[k])) atomicAdd(&h[(int)((slot0 + idv[k]) >> s)], 1);
-        }
-    }
-    if (__syncthreads_and(same)) {
-        if (!valid_id(id0)) return;
-        i128 sum = 0;
-        for (int i0 = t; i0 < td.len; i0 += BNT * BL) {
-            T gv[BL];
-#pragma unroll
-            for (int k = 0; k < BL; ++k) gv[k] = g[td.vpos + min(i0 + k * BNT, td.len - 1)];
-#pragma unroll
-            for (int k = 0; k < BL; ++k)
-                if (i0 + k * BNT < td.len) sum += ws_bwd_fix<T>(gv[k], emax);
-        }
-        sum = ws_warp_reduce_i128(sum);
-        if (lane == 0) { wlo[w] = (long long)(uint64_t)sum; whi[w] = (long long)(uint64_t)((u128)sum >> 64); }
-        __syncthreads();
-        if (t == 0) {
-            i128 tot = 0;
-            for (int k = 0; k < BNT / 32; ++k) tot += (i128)(((u128)(uint64_t)whi[k] << 64) | (u128)(uint64_t)wlo[k]);
-            ws_atomic_add_i128(acc + 2 * (slot0 + id0), tot);
-            atomicAdd(cnt + slot0 + id0, td.len);
-        }
+// p[l * STRIDE] += limb l of ws_bwd_fix(g, emax)
+template <typename T, int STRIDE>
+__device__ __forceinline__ void ws_limb_add(int* p, T g, int emax) {
+    typedef KeyOf<T> KO;
+    static_assert(LIMBS * LIMB_BITS >= BwdFix<T>::SH + BwdFix<T>::MANT + 1, "every value fits");
+    // grad_out = +-m 2^sh in units of the fixed point, as in ws_bwd_fix
+    if (sizeof(T) == 4) {   // (32-bit arithmetic: the integer pipe bounds the kernels)
+        const uint32_t b = (uint32_t)KO::bits(g);
+        const int ex = (int)((b >> 23) & 255u);
+        uint32_t m = (b & 0x7fffffu) | (ex ? 0x800000u : 0u);
+        int sh = max(ex, 1) - emax + BwdFix<T>::SH;
+        if (sh < 0) { m = sh > -32 ? m >> (-sh) : 0u; sh = 0; }
+        const int l0 = (sh * 27) >> 9;   // sh / 19 for 0 <= sh <= 94
+        const int r = sh - LIMB_BITS * l0;
+        const uint32_t lo = m << r, hi = __funnelshift_l(m, 0u, r);   // m << r: 42 bits
+        const int sg = (int)b >> 31;     // 0 or -1: x ^ sg - sg is +-x
+        p += l0 * STRIDE;
+        const uint32_t v0 = lo & LIMB_MASK, v1 = __funnelshift_r(lo, hi, LIMB_BITS) & LIMB_MASK,
+                       v2 = hi >> (2 * LIMB_BITS - 32);
+        if (v0) atomicAdd(p, ((int)v0 ^ sg) - sg);
+        if (v1) atomicAdd(p + STRIDE, ((int)v1 ^ sg) - sg);
+        if (v2) atomicAdd(p + 2 * STRIDE, ((int)v2 ^ sg) - sg);
         return;
     }
-    // each bucket's run in the staging area and its region in the pairs
-    const int cb = t < nb ? h[t] : 0;
-    int total;
-    const int lb = ws_block_excl_scan<BNT, int>(cb, wsum, &total);
-    if (t < nb) {
-        lstart[t] = lb;
-        base[t] = cb ? atomicAdd(bk_cur + t, (unsigned long long)cb) : 0ull;
-        h[t] = 0;
-    }
-    __syncthreads();
-    const int64_t low = ((int64_t)1 << s) - 1;
-    for (int i0 = t; i0 < td.len; i0 += BNT * BL) {
-        int idv[BL];
-        T gv[BL];
-#pragma unroll
-        for (int k = 0; k < BL; ++k) {
-            const int i = min(i0 + k * BNT, td.len - 1);
-            idv[k] = ids[td.vpos + i];
-            gv[k] = g[td.vpos + i];
-        }
-#pragma unroll
-        for (int k = 0; k < BL; ++k) {
-            if (i0 + k * BNT >= td.len || !valid_id(idv[k])) continue;
-            const int64_t slot = slot0 + idv[k];
-            const int b = (int)(slot >> s);
-            const int lp = lstart[b] + atomicAdd(&h[b], 1);
-            st_slot[lp] = (int32_t)(slot & low);
-            st_code[lp] = ws_bwd_encode<T>(gv[k], emax);
-            st_b[lp] = (uint8_t)b;
-        }
-    }
-    __syncthreads();
-    for (int j = t; j < total; j += BNT) {
-        const int b = st_b[j];
-        const unsigned long long pos = base[b] + (unsigned long long)(j - lstart[b]);
-        pslot[pos] = st_slot[j];
-        pcode[pos] = st_code[j];
-    }
+    const uint64_t b = (uint64_t)KO::bits(g);
+    int ex = (int)((b >> KO::MANT) & KO::EXPMASK);
+    uint64_t m = b & ((1ull << KO::MANT) - 1ull);
+    if (ex == 0) ex = 1; else m |= 1ull << KO::MANT;
+    int sh = ex - emax + BwdFix<T>::SH;
+    if (sh < 0) { m = sh > -64 ? m >> (-sh) : 0ull; sh = 0; }
+    const bool neg = (b >> (KO::BITS - 1)) & 1ull;
+    const int l0 = (sh * 27) >> 9;   // sh / 19 for 0 <= sh <= 94
+    const int r = sh - LIMB_BITS * l0;
+    p += l0 * STRIDE;
+    auto add = [&](int l, uint32_t v) {
+        if (v) atomicAdd(p + l * STRIDE, neg ? -(int)v : (int)v);
+    };
+    const uint64_t w = m << r;   // (the low 64 of 71 bits)
+    add(0, (uint32_t)w & LIMB_MASK);
+    add(1, (uint32_t)(w >> LIMB_BITS) & LIMB_MASK);
+    add(2, (uint32_t)(w >> (2 * LIMB_BITS)) & LIMB_MASK);
+    add(3, (uint32_t)((m >> (3 * LIMB_BITS - 18)) >> (18 - r)) & LIMB_MASK);   // (m << r) >> 57, r <= 18
+}
+template <int STRIDE>
+__device__ __forceinline__ i128 ws_limb_sum(const int* p) {
+    const int64_t A = (int64_t)p[0] + ((int64_t)p[STRIDE] << LIMB_BITS);
+    const int64_t B = (int64_t)p[2 * STRIDE] + ((int64_t)p[3 * STRIDE] << LIMB_BITS);
+    return (i128)A + ((i128)B << (2 * LIMB_BITS)) + ((i128)p[4 * STRIDE] << (4 * LIMB_BITS));
 }
 
-// 3c. the pairs, bucket by bucket: the CTAs of a persistent grid take chunks
-// in order from a counter (not a fixed stride, which lets CTAs drift apart),
-// so the slots that the chunks in flight add into span about one bucket
-constexpr int BPER = 8;   // pairs per thread and step
+// Lanes that share the bin (or slot) of the warp's first lane with one: a huge
+// cluster would otherwise serialise the counters' adds.  Returns the mask when
+// it is worth an add of its own (else 0).
+__device__ __forceinline__ unsigned ws_crowd(int v, bool in) {
+    const unsigned act = __ballot_sync(0xffffffffu, in);
+    if (act == 0) return 0;
+    const int lead = __shfl_sync(0xffffffffu, v, __ffs((int)act) - 1);
+    const unsigned eq = __ballot_sync(0xffffffffu, in && v == lead);
+    return __popc(eq) >= 8 ? eq : 0u;
+}
 
+// 1. per segment the largest exponent of grad_out; per bin the elements of the
+// tiles that are not one cluster (cnt) and the tiles that are (extra).  Up to
+// HIST_MAX bins are counted in shared memory by a persistent grid.
 template <typename T>
-__global__ void __launch_bounds__(BNT) k_bwd_pairs(const int32_t* __restrict__ pslot,
-                                                   const typename KeyOf<T>::K* __restrict__ pcode,
-                                                   const unsigned long long* __restrict__ bk_off, int nb, int s,
-                                                   unsigned long long* chunk_ctr, unsigned long long* acc,
-                                                   int32_t* cnt) {
-    typedef typename KeyOf<T>::K K;
-    __shared__ unsigned long long off[BK_MAX + 1];
-    __shared__ unsigned long long s_c0;
-    for (int b = threadIdx.x; b <= nb; b += BNT) off[b] = bk_off[b];
+__global__ void __launch_bounds__(PNT, 3) k_bwd_prep(const T* __restrict__ g, const int32_t* __restrict__ ids,
+                                                     const TileDesc* __restrict__ tiles, int n_tiles,
+                                                     const LargeSeg* __restrict__ lsegs, int n_hist, int32_t* seg_emax,
+                                                     uint32_t* cnt, uint32_t* extra, uint32_t* status) {
+    extern __shared__ uint32_t hist[];   // [n_hist]
+    const int t = threadIdx.x, lane = t & 31;
+    for (int b = t; b < n_hist; b += PNT) hist[b] = 0;
+    bool bad = false;
+    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        const TileDesc td = tiles[tile];
+        const LargeSeg& ls = lsegs[td.lseg];
+        const int64_t slen = ls.len;
+        const int bpos = ls.bb_pos;
+        int idv[ITEMS];
+        T gv[ITEMS];
+#pragma unroll
+        for (int k = 0; k < ITEMS; ++k) {   // (indices clamped into the tile: every load in bounds)
+            const int i = min(t + k * PNT, td.len - 1);
+            idv[k] = __ldg(ids + td.vpos + i);
+            gv[k] = __ldg(g + td.vpos + i);
+        }
+        const int id0 = __ldg(ids + td.vpos);
+        int e = 0;
+        bool same = true;
+#pragma unroll
+        for (int k = 0; k < ITEMS; ++k) {
+            e = max(e, ws_g_exp(gv[k]));
+            same &= idv[k] == id0;
+        }
+        e = __reduce_max_sync(0xffffffffu, e);
+        if (lane == 0 && e > *(volatile int32_t*)(seg_emax + td.lseg)) atomicMax(seg_emax + td.lseg, e);
+        if (__syncthreads_and(same)) {   // (also the barrier after the clearing of hist)
+            if (id0 < 0 || (int64_t)id0 >= slen) bad = true;
+            else if (t == 0) atomicAdd(extra + bpos + (id0 >> WS_BWD_BIN_LOG2), 1u);
+            continue;
+        }
+#pragma unroll
+        for (int k = 0; k < ITEMS; ++k) {
+            const bool here = t + k * PNT < td.len;
+            const bool ok = here && idv[k] >= 0 && (int64_t)idv[k] < slen;
+            bad |= here && !ok;
+            const int b = bpos + (idv[k] >> WS_BWD_BIN_LOG2);
+            const unsigned crowd = ws_crowd(b, ok);
+            uint32_t add = ok ? 1u : 0u;
+            if ((crowd >> lane) & 1u) add = lane == __ffs((int)crowd) - 1 ? (uint32_t)__popc(crowd) : 0u;
+            if (add) {
+                if (n_hist) atomicAdd(&hist[b], add);
+                else atomicAdd(cnt + b, add);
+            }
+        }
+    }
+    if (bad) ws_flag(status, WS_STATUS_INTERNAL);
     __syncthreads();
-    const unsigned long long total = off[nb];
+    for (int b = t; b < n_hist; b += PNT)
+        if (hist[b]) atomicAdd(cnt + b, hist[b]);
+}
+
+// 2. the starts of the bins in the pair buffers and the cursors of the moves
+// (one CTA); the pieces of the bins with more than PIECE pairs
+constexpr int SCAN_NT = 1024, SCAN_PER = 8;
+__global__ void __launch_bounds__(SCAN_NT) k_bwd_scan(const uint32_t* __restrict__ cnt, int n_bins,
+                                                      const int2* __restrict__ map, unsigned long long* start,
+                                                      unsigned long long* cur1, unsigned long long* cur2,
+                                                      uint2* items, int32_t* n_items) {
+    ws_chain();
+    __shared__ long long wsum[SCAN_NT / 32];
+    __shared__ uint2 split[SCAN_NT];   // (bin, first item) of the split bins of one step
+    __shared__ int n_split, s_items;
+    const int t = threadIdx.x;
+    if (t == 0) s_items = 0;
+    long long run = 0;
+    for (int b0 = 0; b0 < n_bins; b0 += SCAN_NT * SCAN_PER) {
+        const int b1 = b0 + t * SCAN_PER;   // (the arrays are padded to whole threads)
+        uint32_t c[SCAN_PER];
+        int first[SCAN_PER];
+        bool big = false;
+        long long mine = 0;
+        if (b1 < n_bins) {
+            const uint4 c0 = __ldg(reinterpret_cast<const uint4*>(cnt + b1)), c1 = __ldg(reinterpret_cast<const uint4*>(cnt + b1) + 1);
+            c[0] = c0.x; c[1] = c0.y; c[2] = c0.z; c[3] = c0.w;
+            c[4] = c1.x; c[5] = c1.y; c[6] = c1.z; c[7] = c1.w;
+#pragma unroll
+            for (int k = 0; k < SCAN_PER; ++k) {
+                first[k] = __ldg(&map[b1 + k].y);
+                mine += c[k];
+                big |= c[k] > (uint32_t)PIECE;
+            }
+        }
+        long long total;
+        long long pos = run + ws_block_excl_scan<SCAN_NT, long long>(mine, wsum, &total);
+        run += total;
+        if (b1 < n_bins) {
+#pragma unroll
+            for (int k = 0; k < SCAN_PER; k += 2) {
+                ulonglong2 q;
+                q.x = (unsigned long long)pos;
+                if (first[k] >= 0) cur1[first[k]] = q.x;   // (the first bin of a bucket of the first move)
+                pos += c[k];
+                q.y = (unsigned long long)pos;
+                if (first[k + 1] >= 0) cur1[first[k + 1]] = q.y;
+                pos += c[k + 1];
+                *reinterpret_cast<ulonglong2*>(start + b1 + k) = q;
+                *reinterpret_cast<ulonglong2*>(cur2 + b1 + k) = q;
+            }
+        }
+        if (!__syncthreads_or(big)) continue;
+#pragma unroll 1
+        for (int k = 0; k < SCAN_PER; ++k) {
+            const int b = b1 + k;
+            const uint32_t ck = b < n_bins ? __ldg(cnt + b) : 0u;
+            if (t == 0) n_split = 0;
+            __syncthreads();
+            if (ck > (uint32_t)PIECE)
+                split[atomicAdd(&n_split, 1)] =
+                    make_uint2((uint32_t)b, (uint32_t)atomicAdd(&s_items, (int)((ck + PIECE - 1) / PIECE)));
+            __syncthreads();
+            for (int i = t >> 5; i < n_split; i += SCAN_NT / 32) {
+                const uint2 sp = split[i];
+                const uint32_t np = (__ldg(cnt + sp.x) + PIECE - 1) / PIECE;
+                for (uint32_t q = t & 31; q < np; q += 32) items[sp.y + q] = make_uint2(sp.x, q);
+            }
+            __syncthreads();
+        }
+    }
+    __syncthreads();
+    if (t == 0) { start[n_bins] = (unsigned long long)run; *n_items = s_items; }
+}
+
+// The bins whose sums are formed in global memory start from zero: split ones,
+// and those that whole tiles add to (a warp per bin).
+__global__ void __launch_bounds__(256) k_bwd_clear(const uint32_t* __restrict__ cnt,
+                                                   const uint32_t* __restrict__ extra, int n_bins,
+                                                   const int2* __restrict__ map, const LargeSeg* __restrict__ lsegs,
+                                                   unsigned long long* acc, int32_t* gcnt) {
+    ws_chain();
     const int lane = threadIdx.x & 31;
-    constexpr unsigned long long CH = (unsigned long long)BNT * BPER;
-    int b = 0;   // bucket of this thread's current pair (pairs only move forward)
-    while (true) {
-        __syncthreads();   // every thread has read the previous chunk's start
-        if (threadIdx.x == 0) s_c0 = atomicAdd(chunk_ctr, 1ull) * CH;
-        __syncthreads();
-        const unsigned long long c0 = s_c0;
-        if (c0 >= total) break;
-        int32_t sl[BPER];
-        K cd[BPER];
-#pragma unroll
-        for (int k = 0; k < BPER; ++k) {
-            const unsigned long long j = c0 + (unsigned long long)k * BNT + threadIdx.x;
-            sl[k] = j < total ? pslot[j] : 0;
-            cd[k] = j < total ? pcode[j] : (K)0;
-        }
-#pragma unroll
-        for (int k = 0; k < BPER; ++k) {
-            const unsigned long long j = c0 + (unsigned long long)k * BNT + threadIdx.x;
-            const bool in = j < total;
-            long long slot = -1 - lane;   // distinct for lanes past the end
-            i128 v = 0;
-            if (in) {
-                while (b + 1 < nb && off[b + 1] <= j) ++b;
-                slot = ((long long)b << s) | (long long)sl[k];
-                v = ws_bwd_decode<T>(cd[k]);
-            }
-            const unsigned peers = __match_any_sync(0xffffffffu, (unsigned long long)slot);
-            const i128 sum = __any_sync(0xffffffffu, __popc(peers) > 1) ? ws_group_sum_i96(peers, v) : v;
-            if (in && lane == __ffs((int)peers) - 1) {
-                ws_atomic_add_i128(acc + 2 * slot, sum);
-                atomicAdd(cnt + slot, __popc(peers));
-            }
+    const int nw = (int)gridDim.x * 8;
+    for (int b = (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5); b < n_bins; b += nw) {
+        if (cnt[b] <= PIECE && extra[b] == 0) continue;
+        const int lseg = map[b].x;
+        const LargeSeg& ls = lsegs[lseg];
+        const int64_t r0 = (int64_t)(b - ls.bb_pos) << WS_BWD_BIN_LOG2;
+        const int64_t r1 = min(r0 + WS_BWD_BIN, ls.len), slot0 = ls.kpos + lseg;
+        for (int64_t r = r0 + lane; r < r1; r += 32) {
+            acc[2 * (slot0 + r)] = 0ull;
+            acc[2 * (slot0 + r) + 1] = 0ull;
+            gcnt[slot0 + r] = 0;
         }
     }
 }
 
-// 4. cluster means (slots 0 .. max id of each segment)
+// 3. moves the pairs into their buckets (FIRST) or, inside the buckets of a
+// long segment, into their bins.  The pairs of one tile are grouped in shared
+// memory (one atomic per pair ranks it), each run reserved with one global
+// atomic and copied out by consecutive threads.
 template <typename T>
-__global__ void __launch_bounds__(BNT) k_bwd_mean(const TileDesc* __restrict__ tiles, const LargeSeg* __restrict__ lsegs,
-                                                  const int32_t* __restrict__ seg_maxid,
-                                                  const int32_t* __restrict__ seg_emax,
-                                                  const unsigned long long* __restrict__ acc,
-                                                  const int32_t* __restrict__ cnt, T* mean) {
-    const TileDesc td = tiles[blockIdx.x];
-    const LargeSeg ls = lsegs[td.lseg];
-    const int64_t slot0 = ls.kpos + td.lseg;
-    const int64_t r0 = (int64_t)td.tin * BTILE;
-    const int64_t r1 = min(r0 + BTILE, (int64_t)seg_maxid[td.lseg] + 1);
-    const int emax = seg_emax[td.lseg];
-    for (int64_t r = r0 + threadIdx.x; r < r1; r += BNT) {
-        const int c = cnt[slot0 + r];
-        if (c == 0) continue;
-        const i128 S = (i128)(((u128)acc[2 * (slot0 + r) + 1] << 64) | (u128)acc[2 * (slot0 + r)]);
-        mean[slot0 + r] = ws_bwd_mean<T>(S, c, emax);
+struct BwdPartSmem {
+    typename KeyOf<T>::K g[BTILE];
+    int32_t id[BTILE];
+    uint32_t cnt[WS_BWD_FAN];
+    uint32_t first[WS_BWD_FAN];              // the run's start inside the tile
+    unsigned long long base[WS_BWD_FAN];     // and its destination
+    int wsum[PNT / 32];
+    long long wlo[PNT / 32], whi[PNT / 32];
+};
+
+template <typename T, bool FIRST>
+__global__ void __launch_bounds__(PNT, 2) k_bwd_part(const typename KeyOf<T>::K* __restrict__ g_in,
+                                                     const int32_t* __restrict__ id_in,
+                                                     typename KeyOf<T>::K* __restrict__ g_a, int32_t* __restrict__ id_a,
+                                                     typename KeyOf<T>::K* __restrict__ g_b, int32_t* __restrict__ id_b,
+                                                     const TileDesc* __restrict__ tiles, int n_tiles,
+                                                     const LargeSeg* __restrict__ lsegs,
+                                                     const unsigned long long* __restrict__ start,
+                                                     unsigned long long* cursor, const int32_t* __restrict__ seg_emax,
+                                                     unsigned long long* acc, int32_t* gcnt, int64_t n_pairs) {
+    typedef KeyOf<T> KO;
+    typedef typename KO::K K;
+    static_assert(WS_BWD_FAN == PNT, "one bucket per thread");
+    extern __shared__ __align__(16) unsigned char part_raw[];
+    BwdPartSmem<T>& s = *reinterpret_cast<BwdPartSmem<T>*>(part_raw);
+    ws_chain();
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    struct Src { int64_t pos; int len; };
+    auto source = [&](int tile) {
+        Src r;
+        const TileDesc& td = tiles[tile];
+        if (FIRST) { r.pos = td.vpos; r.len = td.len; return r; }
+        const LargeSeg& sg = lsegs[td.lseg];
+        r.pos = 0;
+        r.len = 0;
+        if (sg.bb_fine == 0) return r;
+        const int64_t p0 = (int64_t)start[sg.bb_pos] + (int64_t)td.tin * BTILE;
+        const int64_t p1 = (int64_t)start[sg.bb_pos + sg.bb_n];
+        r.pos = p0;
+        r.len = (int)max((int64_t)0, min((int64_t)BTILE, p1 - p0));
+        return r;
+    };
+    K gv[ITEMS];
+    int32_t idv[ITEMS];
+    auto load = [&](const Src& r) {
+#pragma unroll
+        for (int k = 0; k < ITEMS; ++k) {
+            const int p = t + k * PNT;
+            idv[k] = -1;
+            if (p < r.len) {
+                gv[k] = __ldg(g_in + r.pos + p);
+                idv[k] = __ldg(id_in + r.pos + p);
+            }
+        }
+    };
+    int tile = blockIdx.x;
+    if (tile >= n_tiles) return;
+    Src cur = source(tile);
+    load(cur);
+    while (tile < n_tiles) {
+        const int nxt = tile + (int)gridDim.x;
+        const Src ns = nxt < n_tiles ? source(nxt) : Src{0, 0};
+        const int lseg = tiles[tile].lseg;
+        const LargeSeg& sg = lsegs[lseg];
+        const int fl = sg.bb_fine, len = cur.len;
+        bool skip = len == 0;
+        if (FIRST) {
+            const int id0 = __ldg(id_in + cur.pos);
+            const int slen = (int)min(sg.len, (int64_t)INT32_MAX);
+            bool same = true;
+#pragma unroll
+            for (int k = 0; k < ITEMS; ++k) {
+                if (t + k * PNT < len) same &= idv[k] == id0;
+                if (idv[k] >= slen) idv[k] = -1;
+            }
+            if (__syncthreads_and(same)) {
+                // one cluster: the exact sum, once
+                skip = true;
+                if (id0 >= 0 && id0 < slen) {   // (uniform)
+                    const int emax = seg_emax[lseg];
+                    i128 sum = 0;
+#pragma unroll 1
+                    for (int i = t; i < len; i += PNT) sum += ws_bwd_fix<T>(ws_g_of_bits<T>(__ldg(g_in + cur.pos + i)), emax);
+                    sum = ws_warp_reduce_i128(sum);
+                    if (lane == 0) { s.wlo[w] = (long long)(uint64_t)sum; s.whi[w] = (long long)(uint64_t)((u128)sum >> 64); }
+                    __syncthreads();
+                    if (t == 0) {
+                        i128 tot = 0;
+                        for (int k = 0; k < PNT / 32; ++k)
+                            tot += (i128)(((u128)(uint64_t)s.whi[k] << 64) | (u128)(uint64_t)s.wlo[k]);
+                        const int64_t slot = sg.kpos + lseg + id0;
+                        ws_atomic_add_i128(acc + 2 * slot, tot);
+                        atomicAdd(gcnt + slot, len);
+                    }
+                }
+            }
+        }
+        if (skip) {   // (uniform)
+            if (nxt < n_tiles) load(ns);
+            __syncthreads();
+            tile = nxt;
+            cur = ns;
+            continue;
+        }
+        // the tile's buckets: all of the segment's, or the bins of its first to last bucket
+        const int sh = WS_BWD_BIN_LOG2 + (FIRST ? fl : 0);
+        int base = 0, nbk = ((sg.bb_n - 1) >> fl) + 1;
+        if (!FIRST) {
+            base = ((__ldg(id_in + cur.pos) >> WS_BWD_BIN_LOG2) >> fl) << fl;
+            const int hi = (((__ldg(id_in + cur.pos + len - 1) >> WS_BWD_BIN_LOG2) >> fl) + 1) << fl;
+            nbk = max(min(sg.bb_n, hi) - base, 1);
+        }
+        K* go = FIRST && fl != 0 ? g_a : g_b;
+        int32_t* io = FIRST && fl != 0 ? id_a : id_b;
+        for (int r0 = 0; r0 < nbk; r0 += WS_BWD_FAN) {
+            const uint32_t off = (uint32_t)(base + r0);
+            __syncthreads();   // (the previous use of the shared memory is over)
+            s.cnt[t] = 0;
+            __syncthreads();
+            uint32_t rk[ITEMS];
+#pragma unroll
+            for (int k = 0; k < ITEMS; ++k) {
+                const uint32_t b = (uint32_t)(idv[k] >> sh) - off;   // (id -1: above every bucket, or refused below)
+                rk[k] = 0;
+                if (idv[k] >= 0 && b < WS_BWD_FAN) rk[k] = atomicAdd(&s.cnt[b], 1u);
+            }
+            __syncthreads();
+            const uint32_t c = s.cnt[t];
+            s.base[t] = c ? atomicAdd(cursor + (FIRST ? sg.bb_cpos : sg.bb_pos) + off + t, (unsigned long long)c) : 0ull;
+            int total;
+            s.first[t] = (uint32_t)ws_block_excl_scan<PNT, int>((int)c, s.wsum, &total);
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < ITEMS; ++k) {
+                const uint32_t b = (uint32_t)(idv[k] >> sh) - off;
+                if (idv[k] >= 0 && b < WS_BWD_FAN) {
+                    const uint32_t j = s.first[b] + rk[k];
+                    s.g[j] = gv[k];
+                    s.id[j] = idv[k];
+                }
+            }
+            __syncthreads();
+            // (the registers are free: the next tile's loads overlap the copy)
+            if (r0 + WS_BWD_FAN >= nbk && nxt < n_tiles) load(ns);
+#pragma unroll 4
+            for (int j = t; j < total; j += PNT) {
+                const int32_t id = s.id[j];
+                const uint32_t b = (uint32_t)(id >> sh) - off;
+                const int64_t pos = (int64_t)s.base[b] + (int64_t)((uint32_t)j - s.first[b]);
+                if (pos < n_pairs) {   // (always)
+                    go[pos] = s.g[j];
+                    io[pos] = id;
+                }
+            }
+        }
+        tile = nxt;
+        cur = ns;
+    }
+}
+
+// 4. the sums of a bin's slots in shared memory, and its means.  CTA b takes
+// bin b; the last EXTRA CTAs the pieces of the split ones.  Pairs are added in
+// steps of CHUNK; with more than 4096 of them the limbs are normalised after
+// every step (the top limb's carries go to the upper half of the counter, whose
+// lower half holds at most PIECE).
+struct BwdBinSmem {
+    int limb[LIMBS][WS_BWD_BIN];
+    int cnt[WS_BWD_BIN];
+};
+
+template <typename T>
+__global__ void __launch_bounds__(ANT, 4) k_bwd_bins(const typename KeyOf<T>::K* __restrict__ g_b,
+                                                     const int32_t* __restrict__ id_b,
+                                                     const uint32_t* __restrict__ cnt,
+                                                     const uint32_t* __restrict__ extra, int n_bins,
+                                                     const int2* __restrict__ map, const LargeSeg* __restrict__ lsegs,
+                                                     const unsigned long long* __restrict__ start,
+                                                     const uint2* __restrict__ items,
+                                                     const int32_t* __restrict__ n_items, uint32_t* arrive,
+                                                     const int32_t* __restrict__ seg_emax, unsigned long long* acc,
+                                                     int32_t* gcnt, T* mean) {
+    typedef KeyOf<T> KO;
+    typedef typename KO::K K;
+    static_assert(PIECE < 32768, "the counter's lower half");
+    extern __shared__ __align__(16) unsigned char bin_raw[];
+    BwdBinSmem& s = *reinterpret_cast<BwdBinSmem*>(bin_raw);
+    __shared__ int s_last;
+    ws_chain();
+    const int t = threadIdx.x, lane = t & 31;
+    auto run = [&](int bin, int piece) {   // (piece -1: the whole bin)
+        const int nbin = (int)cnt[bin];
+        const bool more = extra[bin] != 0;
+        if (nbin == 0 && !more) return;
+        const int lseg = map[bin].x;
+        const LargeSeg& ls = lsegs[lseg];
+        const int r0 = (bin - ls.bb_pos) << WS_BWD_BIN_LOG2;
+        const int nr = (int)min((int64_t)WS_BWD_BIN, ls.len - r0);
+        const int64_t slot0 = ls.kpos + lseg + r0;
+        const int emax = seg_emax[lseg];
+        const int64_t p0 = (int64_t)start[bin] + (piece > 0 ? (int64_t)piece * PIECE : 0);
+        const int n = piece < 0 ? nbin : min(PIECE, nbin - piece * PIECE);
+        __syncthreads();   // (the previous use of the shared memory is over)
+        for (int i = t; i < (int)(sizeof(BwdBinSmem) / sizeof(int4)); i += ANT)
+            reinterpret_cast<int4*>(&s)[i] = make_int4(0, 0, 0, 0);
+        __syncthreads();
+        for (int c0 = 0; c0 < n; c0 += CHUNK) {
+            K gv[8];
+            int idv[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                if (c0 + k * ANT >= n) break;   // (uniform)
+                const int64_t j = p0 + min(c0 + k * ANT + t, n - 1);
+                gv[k] = __ldg(g_b + j);
+                idv[k] = __ldg(id_b + j);
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                if (c0 + k * ANT >= n) break;
+                const bool in = c0 + k * ANT + t < n;
+                const int r = idv[k] & (WS_BWD_BIN - 1);
+                const T gk = ws_g_of_bits<T>(gv[k]);
+                const unsigned crowd = ws_crowd(r, in);
+                if ((crowd >> lane) & 1u) {
+                    const i128 sum = ws_group_sum_i96(crowd, ws_bwd_fix<T>(gk, emax));
+                    if (lane == __ffs((int)crowd) - 1) {
+#pragma unroll
+                        for (int l = 0; l < LIMBS - 1; ++l)
+                            atomicAdd(&s.limb[l][r], (int)((uint32_t)(uint64_t)((u128)sum >> (l * LIMB_BITS)) & LIMB_MASK));
+                        atomicAdd(&s.limb[LIMBS - 1][r], (int)(sum >> ((LIMBS - 1) * LIMB_BITS)));
+                        atomicAdd(&s.cnt[r], __popc(crowd));
+                    }
+                } else if (in) {
+                    ws_limb_add<T, WS_BWD_BIN>(&s.limb[0][r], gk, emax);
+                    atomicAdd(&s.cnt[r], 1);
+                }
+            }
+            __syncthreads();
+            if (n > 4096) {
+                for (int r = t; r < nr; r += ANT) {
+                    int carry = 0;
+#pragma unroll
+                    for (int l = 0; l < LIMBS; ++l) {
+                        const int v = s.limb[l][r];
+                        // (v + carry stays below 2^31: 2049 values of 19 bits and a carry of 12)
+                        const int x = v + carry;
+                        carry = x >> LIMB_BITS;
+                        s.limb[l][r] = x & (int)LIMB_MASK;
+                    }
+                    s.cnt[r] += carry * 65536;
+                }
+                __syncthreads();
+            }
+        }
+        // the count and the sum of slot r
+        auto slot_cnt = [&](int r) { return s.cnt[r] & 0xffff; };
+        auto slot_sum = [&](int r) {
+            return ws_limb_sum<WS_BWD_BIN>(&s.limb[0][r]) + ((i128)(s.cnt[r] >> 16) << (LIMBS * LIMB_BITS));
+        };
+        if (piece < 0) {
+            for (int r = t; r < nr; r += ANT) {
+                int c = slot_cnt(r);
+                i128 S = slot_sum(r);
+                if (more) {   // (what whole tiles added)
+                    c += gcnt[slot0 + r];
+                    S += (i128)(((u128)acc[2 * (slot0 + r) + 1] << 64) | (u128)acc[2 * (slot0 + r)]);
+                }
+                if (c) mean[slot0 + r] = ws_bwd_mean<T>(S, c, emax);
+            }
+            return;
+        }
+        for (int r = t; r < nr; r += ANT) {
+            const int c = slot_cnt(r);
+            if (c) {
+                ws_atomic_add_i128(acc + 2 * (slot0 + r), slot_sum(r));
+                atomicAdd(gcnt + slot0 + r, c);
+            }
+        }
+        // the piece that comes last forms the means
+        __threadfence();
+        __syncthreads();
+        if (t == 0) s_last = atomicAdd(arrive + bin, 1u) == (uint32_t)((nbin + PIECE - 1) / PIECE) - 1u;
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        for (int r = t; r < nr; r += ANT) {
+            const int c = __ldcg(gcnt + slot0 + r);
+            if (c == 0) continue;
+            const i128 S = (i128)(((u128)__ldcg(acc + 2 * (slot0 + r) + 1) << 64) | (u128)__ldcg(acc + 2 * (slot0 + r)));
+            mean[slot0 + r] = ws_bwd_mean<T>(S, c, emax);
+        }
+    };
+    if ((int)blockIdx.x < n_bins) {
+        if (cnt[blockIdx.x] <= PIECE) run(blockIdx.x, -1);
+        return;
+    }
+    const int ni = *n_items;
+    for (int i = (int)blockIdx.x - n_bins; i < ni; i += EXTRA) {
+        const uint2 it = items[i];
+        run((int)it.x, (int)it.y);
     }
 }
 
 // 5. every element takes its cluster's mean
 template <typename T>
-__global__ void __launch_bounds__(BNT) k_bwd_apply(const int32_t* __restrict__ ids, const TileDesc* __restrict__ tiles,
+__global__ void __launch_bounds__(PNT) k_bwd_apply(const int32_t* __restrict__ ids, const TileDesc* __restrict__ tiles,
                                                    const LargeSeg* __restrict__ lsegs, const T* __restrict__ mean,
                                                    T* gin) {
+    ws_chain();
     const TileDesc td = tiles[blockIdx.x];
-    const LargeSeg ls = lsegs[td.lseg];
-    const int64_t slot0 = ls.kpos + td.lseg;
-    for (int i = threadIdx.x; i < td.len; i += BNT) {
-        const int id = ids[td.vpos + i];
-        if (id < 0 || (int64_t)id >= ls.len) continue;
-        gin[td.vpos + i] = mean[slot0 + id];
+    const LargeSeg& ls = lsegs[td.lseg];
+    const int64_t slot0 = ls.kpos + td.lseg, slen = ls.len;
+    int idv[ITEMS];
+    T v[ITEMS];
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+        const int i = threadIdx.x + k * PNT;
+        idv[k] = i < td.len ? __ldg(ids + td.vpos + i) : -1;
+        if ((int64_t)idv[k] >= slen) idv[k] = -1;
     }
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k)
+        if (idv[k] >= 0) v[k] = __ldg(mean + slot0 + idv[k]);
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k)
+        if (idv[k] >= 0) gin[td.vpos + threadIdx.x + k * PNT] = v[k];
 }
 
-// One-CTA segments: the same exact sums in shared memory, as five signed
-// 19-bit limbs per cluster.  A grad_out value of MANT + 1 bits falls into at
-// most three of them (four for double), each one 32-bit shared-memory add
-// without a returned value (native; a 64-bit shared atomic is a
-// compare-and-swap loop), and 4096 limbs of 19 bits cannot overflow 32 bits.
-// The limbs recombine to the integer that 128-bit additions give.  Bound by
-// those adds and the conversions; 12.6M elements in rows of 3072: 482 us with
-// 64-bit atomics behind a warp match.
-constexpr int LIMBS = 5, LIMB_BITS = 19;   // 95 bits: every ws_bwd_fix value
-
+// One-CTA segments: the same limbs, one CTA per segment.  Bound by the adds and
+// the conversions; 12.6M elements in rows of 3072: 482 us with 64-bit atomics
+// behind a warp match, 90 with the limbs.
 template <typename T, int NT, int CAP>
 __global__ void __launch_bounds__(NT, 2) k_small_backward(const T* __restrict__ g, const int32_t* __restrict__ ids,
                                                           const int64_t* __restrict__ offsets,
@@ -425,7 +680,6 @@ __global__ void __launch_bounds__(NT, 2) k_small_backward(const T* __restrict__ 
     typedef KeyOf<T> KO;
     constexpr int PER = CAP / NT;
     static_assert(CAP % NT == 0, "whole elements per thread");
-    static_assert(LIMBS * LIMB_BITS >= BwdFix<T>::SH + BwdFix<T>::MANT + 1, "every value fits");
     static_assert((long long)CAP * ((1 << LIMB_BITS) - 1) < (1ll << 31), "no limb overflows");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int* limb = reinterpret_cast<int*>(smem_raw);   // [LIMBS][CAP]
@@ -467,30 +721,7 @@ __global__ void __launch_bounds__(NT, 2) k_small_backward(const T* __restrict__ 
     for (int k = 0; k < PER; ++k) {
         const int id = idv[k];
         if (id < 0) continue;
-        // grad_out = +-m 2^sh in units of the fixed point, as in ws_bwd_fix
-        const uint64_t b = (uint64_t)KO::bits(gv[k]);
-        int ex = (int)((b >> KO::MANT) & KO::EXPMASK);
-        uint64_t m = b & ((1ull << KO::MANT) - 1ull);
-        if (ex == 0) ex = 1; else m |= 1ull << KO::MANT;
-        int sh = ex - emax + BwdFix<T>::SH;
-        if (sh < 0) { m = sh > -64 ? m >> (-sh) : 0ull; sh = 0; }
-        const bool neg = (b >> (KO::BITS - 1)) & 1ull;
-        const int l0 = (sh * 27) >> 9;   // sh / 19 for 0 <= sh <= 94
-        const int r = sh - LIMB_BITS * l0;
-        int* p = limb + l0 * CAP + id;
-        constexpr uint32_t LM = (1u << LIMB_BITS) - 1u;
-        auto add = [&](int l, uint32_t v) {
-            if (v) atomicAdd(p + l * CAP, neg ? -(int)v : (int)v);
-        };
-        const uint64_t w = m << r;   // (float: 42 bits; double: the low 64 of 71)
-        add(0, (uint32_t)w & LM);
-        add(1, (uint32_t)(w >> LIMB_BITS) & LM);
-        if (sizeof(T) == 4) {
-            add(2, (uint32_t)(w >> (2 * LIMB_BITS)));
-        } else {
-            add(2, (uint32_t)(w >> (2 * LIMB_BITS)) & LM);
-            add(3, (uint32_t)((m >> (3 * LIMB_BITS - 18)) >> (18 - r)) & LM);   // (m << r) >> 57, r <= 18
-        }
+        ws_limb_add<T, CAP>(limb + id, gv[k], emax);
         atomicAdd(cnt + id, 1);
     }
     __syncthreads();
@@ -498,9 +729,7 @@ __global__ void __launch_bounds__(NT, 2) k_small_backward(const T* __restrict__ 
     for (int r = t; r < n; r += NT) {
         const int c = cnt[r];
         if (c == 0) continue;
-        const int64_t A = (int64_t)limb[r] + ((int64_t)limb[CAP + r] << LIMB_BITS);
-        const int64_t B = (int64_t)limb[2 * CAP + r] + ((int64_t)limb[3 * CAP + r] << LIMB_BITS);
-        const i128 S = (i128)A + ((i128)B << (2 * LIMB_BITS)) + ((i128)limb[4 * CAP + r] << (4 * LIMB_BITS));
+        const i128 S = ws_limb_sum<CAP>(limb + r);
         const T mean = ws_bwd_mean<T>(S, c, emax);
         if (sizeof(T) == 4) limb[r] = __float_as_int((float)mean);
         else {
@@ -527,57 +756,45 @@ template <typename T>
 cudaError_t ws_large_backward(const LargeWork<T>& W, const T* g, const int32_t* ids, T* gin, uint32_t* status,
                               cudaStream_t st) {
     if (W.n_lseg == 0) return cudaSuccess;
-    // seg_emax / seg_maxid live in the backward's per-segment words
-    int32_t* seg_emax = W.bwd_seg;
-    int32_t* seg_maxid = W.bwd_seg + W.n_lseg;
-    cudaError_t e = cudaMemsetAsync(seg_emax, 0, sizeof(int32_t) * W.n_lseg, st);
-    if (e) return e;
-    e = cudaMemsetAsync(seg_maxid, 0xff, sizeof(int32_t) * W.n_lseg, st);
-    if (e) return e;
-    const int nt = W.n_sort_tiles;
-    // slot buckets of 2^s slots (2^21 slots of 20 bytes: about 40 MB, well
-    // inside L2); their counters: 3 nb + 2 words
     typedef typename KeyOf<T>::K K;
-    const int64_t total_slots = W.n_keys + W.n_lseg;
-    int s = 21;
-    while (((total_slots + ((int64_t)1 << s) - 1) >> s) > BK_MAX) ++s;
-    const int nb = (int)((total_slots + ((int64_t)1 << s) - 1) >> s);
-    unsigned long long* bk_cnt = reinterpret_cast<unsigned long long*>(W.hist);
-    unsigned long long* bk_off = bk_cnt + nb;
-    unsigned long long* bk_cur = bk_off + nb + 1;   // nb cursors, then the chunk counter
-    // the pairs borrow the sort's key buffers (n_keys entries each)
-    int32_t* pslot = reinterpret_cast<int32_t*>(W.keys_a);
-    K* pcode = W.keys_b;
-    e = cudaMemsetAsync(bk_cnt, 0, sizeof(unsigned long long) * nb, st);
+    cudaError_t e = cudaMemsetAsync(W.bwd.emax, 0, W.bwd.zero_bytes, st);
     if (e) return e;
-    static const int pairs_grid = [] {
-        int dev = 0, sms = 0, per_sm = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bwd_pairs<T>, BNT, 0) != cudaSuccess) {
-            cudaGetLastError();
-            return 4 * 152;
-        }
-        return std::max(1, sms * std::max(per_sm, 1));
-    }();
+    const BwdWork& B = W.bwd;
+    const int nt = W.n_sort_tiles;
+    // the pairs borrow the sort's buffers (n_keys entries each)
+    K *g_a = W.keys_a, *g_b = W.keys_b;
+    int32_t *id_a = reinterpret_cast<int32_t*>(W.dest1), *id_b = reinterpret_cast<int32_t*>(W.bins);
+    const int n_hist = B.n_bins <= HIST_MAX ? B.n_bins : 0;
+    const size_t hsm = sizeof(uint32_t) * n_hist, psm = sizeof(BwdPartSmem<T>), bsm = sizeof(BwdBinSmem);
+    if ((e = cudaFuncSetAttribute(k_bwd_prep<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * HIST_MAX)) ||
+        (e = cudaFuncSetAttribute(k_bwd_part<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm)) ||
+        (e = cudaFuncSetAttribute(k_bwd_part<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm)) ||
+        (e = cudaFuncSetAttribute(k_bwd_bins<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsm)))
+        return e;
+    const int grid = std::min(nt, 2 * 152);
     WS_LAUNCH(W.prof, WSK_BWD, st,
-              (k_bwd_prep<T><<<nt, BNT, 0, st>>>(g, ids, W.sort_tiles, W.lsegs, seg_emax, seg_maxid, nb, s, bk_cnt,
-                                                 status)));
-    WS_LAUNCH(W.prof, WSK_BWD, st, (k_bwd_zero<<<nt, BNT, 0, st>>>(W.sort_tiles, W.lsegs, seg_maxid, W.bacc, W.bcnt)));
-    WS_LAUNCH(W.prof, WSK_BWD, st, (k_bwd_bscan<<<1, 32, 0, st>>>(bk_cnt, nb, bk_off, bk_cur)));
-    const size_t scatter_smem = ws_bwd_scatter_smem<T>();
-    e = cudaFuncSetAttribute(k_bwd_scatter<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)scatter_smem);
-    if (e) return e;
+              (k_bwd_prep<T><<<std::min(nt, 3 * 152), PNT, hsm, st>>>(g, ids, W.sort_tiles, nt, W.lsegs, n_hist, B.emax, B.cnt, B.extra,
+                                                     status)));
     WS_LAUNCH(W.prof, WSK_BWD, st,
-              (k_bwd_scatter<T><<<nt, BNT, scatter_smem, st>>>(g, ids, W.sort_tiles, W.lsegs, seg_emax, W.bacc, W.bcnt, nb, s,
-                                                    bk_cur, pslot, pcode)));
+              ws_launch_chain(k_bwd_scan, 1, SCAN_NT, 0, st, B.cnt, B.n_bins, B.map, B.start, B.cur1, B.cur2, B.items,
+                              B.n_items));
     WS_LAUNCH(W.prof, WSK_BWD, st,
-              (k_bwd_pairs<T><<<pairs_grid, BNT, 0, st>>>(pslot, pcode, bk_off, nb, s, bk_cur + nb, W.bacc,
-                                                          W.bcnt)));
+              ws_launch_chain(k_bwd_clear, std::min((B.n_bins + 7) / 8, 8 * 152), 256, 0, st, B.cnt, B.extra, B.n_bins,
+                              B.map, W.lsegs, W.bacc, W.bcnt));
     WS_LAUNCH(W.prof, WSK_BWD, st,
-              (k_bwd_mean<T><<<nt, BNT, 0, st>>>(W.sort_tiles, W.lsegs, seg_maxid, seg_emax, W.bacc, W.bcnt,
-                                                 W.bsum)));
-    WS_LAUNCH(W.prof, WSK_BWD, st, (k_bwd_apply<T><<<nt, BNT, 0, st>>>(ids, W.sort_tiles, W.lsegs, W.bsum, gin)));
+              ws_launch_chain(k_bwd_part<T, true>, grid, PNT, psm, st, reinterpret_cast<const K*>(g), ids, g_a, id_a,
+                              g_b, id_b, W.sort_tiles, nt, W.lsegs, B.start, B.cur1, B.emax, W.bacc, W.bcnt,
+                              W.n_keys));
+    if (B.two_level)
+        WS_LAUNCH(W.prof, WSK_BWD, st,
+                  ws_launch_chain(k_bwd_part<T, false>, grid, PNT, psm, st, g_a, id_a, g_a, id_a, g_b, id_b,
+                                  W.sort_tiles, nt, W.lsegs, B.start, B.cur2, B.emax, W.bacc, W.bcnt, W.n_keys));
+    WS_LAUNCH(W.prof, WSK_BWD, st,
+              ws_launch_chain(k_bwd_bins<T>, B.n_bins + EXTRA, ANT, bsm, st, g_b, id_b, B.cnt, B.extra, B.n_bins,
+                              B.map, W.lsegs, B.start, B.items, B.n_items, B.arrive, B.emax, W.bacc, W.bcnt, W.bsum));
+    // (a gather that lives off the caches: a plain launch)
+    WS_LAUNCH(W.prof, WSK_BWD, st,
+              ws_launch_if(nt <= 2 * 152, k_bwd_apply<T>, nt, PNT, 0, st, ids, W.sort_tiles, W.lsegs, W.bsum, gin));
     return cudaGetLastError();
 }
 

@@ -81,6 +81,9 @@ constexpr int WS_SORT_TILE = WS_SORT_NT * WS_SORT_ITEMS;   // 6144 keys per sort
 // one CTA up to WS_BIN_CAP keys.  The ratio 1.6 leaves room for the error of
 // the sampled map (5 to 14 % standard deviation on N(0, 1), the largest bin 1.2
 // to 1.55 times the mean; a mean of 2816 let a few bins of the tails overflow).
+constexpr int WS_BWD_BIN_LOG2 = 11, WS_BWD_BIN = 1 << WS_BWD_BIN_LOG2;   // backward: cluster slots per bin (48 KB of sums)
+constexpr int WS_BWD_PIECE = 16384; // pairs of a bin that one CTA adds
+constexpr int WS_BWD_FAN = 512;    // buckets of one move of the backward
 constexpr int WS_BIN_CAP = 4096;
 constexpr int WS_BIN_MEAN = 2560;
 constexpr int WS_BINS_MAX = 1 << 19;         // per segment (a partition's rank word holds 19 bits of bin)
@@ -117,6 +120,24 @@ struct LargeSeg {
     int32_t ncell;             // cells of the segment's map (a power of two)
     int32_t samp_log2;         // sampled elements per sort tile
     int32_t bin_pos, coarse_pos, cell_pos;   // slices of the per-bin / bucket / cell arrays
+    // backward: bins of cluster slots
+    int32_t bb_n, bb_fine;     // bins of the segment; bucket of the first move = bin >> bb_fine (0: one move only)
+    int32_t bb_pos, bb_cpos;   // slices of the per-bin / bucket arrays
+};
+
+// Work words of the backward (device memory).
+struct BwdWork {
+    int n_bins, two_level;
+    size_t zero_bytes;             // emax .. n_items: one block, cleared by every backward
+    int32_t* emax;                 // [n_lseg] largest grad_out exponent
+    uint32_t* cnt;                 // [n_bins] pairs
+    uint32_t* extra;               // [n_bins] tiles of one cluster (they move no pairs)
+    uint32_t* arrive;              // [n_bins] finished pieces
+    int32_t* n_items;              // pieces of the split bins
+    const int2* map;               // [n_bins] (segment, bucket of the first move that starts here or -1)
+    unsigned long long* start;     // [n_bins + 1]
+    unsigned long long *cur1, *cur2;   // cursors of the moves
+    uint2* items;                  // (bin, piece)
 };
 
 // Sort control words, cleared before every sort.
@@ -274,7 +295,7 @@ struct LargeWork {
     T* bsum;                 // [n_keys + n_lseg] cluster means
     int32_t* bcnt;           // [n_keys + n_lseg] cluster sizes
     unsigned long long* bacc;   // [n_keys + n_lseg][2] exact cluster sums (128-bit, low word first)
-    int32_t* bwd_seg;        // [2 n_lseg] per segment: largest grad exponent, largest cluster id
+    BwdWork bwd;
     WsProf* prof;            // host-side launch accounting
 };
 
