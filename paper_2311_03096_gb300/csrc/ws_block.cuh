@@ -85,6 +85,17 @@ __device__ __forceinline__ V ws_block_excl_scan(V v, V* wsum, V* total) {
     return r;
 }
 
+// The lanes that count into the same slot as the warp's first one with `in`: a
+// huge cluster would otherwise serialise the adds.  Returns their mask when it is
+// worth an add of its own (else 0).
+__device__ __forceinline__ unsigned ws_crowd(int v, bool in) {
+    const unsigned act = __ballot_sync(0xffffffffu, in);
+    if (act == 0) return 0;
+    const int lead = __shfl_sync(0xffffffffu, v, __ffs((int)act) - 1);
+    const unsigned eq = __ballot_sync(0xffffffffu, in && v == lead);
+    return __popc(eq) >= 8 ? eq : 0u;
+}
+
 // ---------------------------------------------------------------------------
 // Fixed-point prefix sums of a sorted tile (points 0..n).
 // Per-point arrays are stored at padded index p + p/M so that the threads of

@@ -171,17 +171,6 @@ __device__ __forceinline__ i128 ws_limb_sum(const int* p) {
     return (i128)A + ((i128)B << (2 * LIMB_BITS)) + ((i128)p[4 * STRIDE] << (4 * LIMB_BITS));
 }
 
-// Lanes that share the bin (or slot) of the warp's first lane with one: a huge
-// cluster would otherwise serialise the counters' adds.  Returns the mask when
-// it is worth an add of its own (else 0).
-__device__ __forceinline__ unsigned ws_crowd(int v, bool in) {
-    const unsigned act = __ballot_sync(0xffffffffu, in);
-    if (act == 0) return 0;
-    const int lead = __shfl_sync(0xffffffffu, v, __ffs((int)act) - 1);
-    const unsigned eq = __ballot_sync(0xffffffffu, in && v == lead);
-    return __popc(eq) >= 8 ? eq : 0u;
-}
-
 // 1. per segment the largest exponent of grad_out; per bin the elements of the
 // tiles that are not one cluster (cnt) and the tiles that are (extra).  Up to
 // HIST_MAX bins are counted in shared memory by a persistent grid.

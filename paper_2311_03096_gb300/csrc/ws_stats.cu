@@ -10,6 +10,8 @@
 // experiment is #distinct nonzero weights / #nonzero weights (0 when every
 // weight is zero); on sorted keys a distinct value is a key that differs
 // from its predecessor.
+#include <algorithm>
+
 #include "ws_kernels.cuh"
 
 namespace {
@@ -218,18 +220,33 @@ __global__ void __launch_bounds__(NT) k_dlam_small(const T* __restrict__ g, cons
     }
 }
 
-template <typename T>
+// Cluster sizes.  Distinct ids: one global atomic each, bound by the L1 (a line
+// per lane and clock; 91 us at 2^24).  Adds to one address go one by one (0.6 ns),
+// so a tile in which at least HOT of 256 sampled ids meet another one of their warp
+// is left to k_dlam_crowded, which adds into a hash table in shared memory first,
+// one global add per id and tile (what finds no place in four probes is added
+// directly).  2^24 elements, dlambda in all, us: one cluster 10740 -> 190, 7
+// clusters 2660 -> 183, one of half the elements 5520 -> 251.  (A kernel of its
+// own: with the table's shared memory the direct adds take 120 us.)
+constexpr int HOT = 3;
 __global__ void __launch_bounds__(256) k_dlam_count(const int32_t* __restrict__ ids, const TileDesc* __restrict__ tiles,
                                                     const LargeSeg* __restrict__ lsegs, int32_t* cnt,
-                                                    uint32_t* status) {
+                                                    uint8_t* crowded, uint32_t* status) {
     const TileDesc td = tiles[blockIdx.x];
     const LargeSeg ls = lsegs[td.lseg];
     const int64_t slot0 = ls.kpos + td.lseg;
     constexpr int U = 8;   // (loads issued together)
-    for (int i0 = threadIdx.x; i0 < td.len; i0 += 256 * U) {
+    bool hot = false;
+    for (int i0 = threadIdx.x, first = 1; i0 - (int)threadIdx.x < td.len; i0 += 256 * U, first = 0) {
         int id[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) id[u] = i0 + u * 256 < td.len ? __ldg(ids + td.vpos + i0 + u * 256) : 0;
+        if (first) {   // (uniform)
+            const unsigned peers = __match_any_sync(0xffffffffu, id[0]);
+            hot = __syncthreads_count(i0 < td.len && __popc(peers) > 1) >= HOT;
+            if (threadIdx.x == 0) crowded[blockIdx.x] = hot ? 1 : 0;
+        }
+        if (hot) return;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             if (i0 + u * 256 >= td.len) break;
@@ -237,6 +254,57 @@ __global__ void __launch_bounds__(256) k_dlam_count(const int32_t* __restrict__ 
             atomicAdd(&cnt[slot0 + id[u]], 1);
         }
     }
+}
+
+constexpr int DC_NT = 512, TAB_LOG2 = 12;
+__device__ __forceinline__ void dlam_crowded_tile(const TileDesc& td, const int32_t* __restrict__ ids,
+                                                  const LargeSeg* __restrict__ lsegs, int32_t* cnt, int* tk, int* tc,
+                                                  uint32_t* status) {
+    constexpr int PER = WS_SORT_TILE / DC_NT, TAB = 1 << TAB_LOG2;
+    const int64_t slot0 = lsegs[td.lseg].kpos + td.lseg, slen = lsegs[td.lseg].len;
+    const int t = threadIdx.x, lane = t & 31;
+    int id[PER];
+    bool bad = false;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int i = t + k * DC_NT;
+        id[k] = i < td.len ? __ldg(ids + td.vpos + i) : -1;
+        if (i < td.len && (id[k] < 0 || (int64_t)id[k] >= slen)) { bad = true; id[k] = -1; }
+    }
+    if (bad) ws_flag(status, WS_STATUS_INTERNAL);
+    __syncthreads();   // (the previous use of the table is over)
+    for (int i = t; i < TAB; i += DC_NT) { tk[i] = -1; tc[i] = 0; }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const unsigned crowd = ws_crowd(id[k], id[k] >= 0);
+        int add = id[k] >= 0 ? 1 : 0;
+        if ((crowd >> lane) & 1u) add = lane == __ffs((int)crowd) - 1 ? __popc(crowd) : 0;
+        if (add == 0) continue;
+        uint32_t h = ((uint32_t)id[k] * 0x9E3779B1u) >> (32 - TAB_LOG2);
+        int probe = 0;
+        for (; probe < 4; ++probe, h = (h + 1) & (TAB - 1)) {
+            int q = *(volatile int*)&tk[h];
+            if (q == -1) {
+                q = atomicCAS(&tk[h], -1, id[k]);
+                if (q == -1) q = id[k];
+            }
+            if (q == id[k]) { atomicAdd(&tc[h], add); break; }
+        }
+        if (probe == 4) atomicAdd(&cnt[slot0 + id[k]], add);
+    }
+    __syncthreads();
+    for (int i = t; i < TAB; i += DC_NT)
+        if (tc[i]) atomicAdd(&cnt[slot0 + tk[i]], tc[i]);
+}
+__global__ void __launch_bounds__(DC_NT) k_dlam_crowded(const int32_t* __restrict__ ids,
+                                                        const TileDesc* __restrict__ tiles, int n_tiles,
+                                                        const LargeSeg* __restrict__ lsegs, int32_t* cnt,
+                                                        const uint8_t* __restrict__ crowded, uint32_t* status) {
+    __shared__ int tk[1 << TAB_LOG2], tc[1 << TAB_LOG2];
+    ws_chain();
+    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x)
+        if (crowded[tile]) dlam_crowded_tile(tiles[tile], ids, lsegs, cnt, tk, tc, status);   // (uniform)
 }
 
 // Cluster starts in two passes over the counts, in chunks of 4096 slots (one
@@ -249,6 +317,7 @@ constexpr int DL_CHUNK = 4096;
 template <bool WRITE>
 __global__ void __launch_bounds__(256) k_dlam_starts(const int32_t* __restrict__ cnt, int64_t S, uint32_t* key,
                                                      int32_t* csum) {
+    ws_chain();
     __shared__ int wsum[8];
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const int64_t b0 = (int64_t)blockIdx.x * DL_CHUNK + 512 * w + 4 * lane;
@@ -305,6 +374,7 @@ __global__ void __launch_bounds__(256) k_dlam_starts(const int32_t* __restrict__
 
 // exclusive scan of the chunk totals, in place (one CTA, carried across rounds)
 __global__ void __launch_bounds__(1024) k_dlam_scan_totals(int32_t* csum, int nb) {
+    ws_chain();
     __shared__ int wsum[32];
     __shared__ int carry;
     if (threadIdx.x == 0) carry = 0;
@@ -335,6 +405,7 @@ __global__ void __launch_bounds__(DL_NT) k_dlam_apply(const T* __restrict__ g, c
                                                       const LargeSeg* __restrict__ lsegs,
                                                       const int32_t* __restrict__ cnt,
                                                       const uint32_t* __restrict__ key, double* out) {
+    ws_chain();
     typedef KeyOf<T> KO;
     constexpr int PER = WS_SORT_TILE / DL_NT, UP = 62 - KO::MANT;
     __shared__ long long wlo[DL_NT / 32], whi[DL_NT / 32];
@@ -422,16 +493,21 @@ cudaError_t ws_dlambda(const T* g, const int32_t* ids, const int64_t* d_offsets,
         int32_t* cnt = W.bcnt;
         uint32_t* key = reinterpret_cast<uint32_t*>(W.bsum);
         int32_t* csum = reinterpret_cast<int32_t*>(partial);
+        uint8_t* crowded = reinterpret_cast<uint8_t*>(W.keys_a);   // (the sort's buffer, free here)
         const int nb = (int)((S + DL_CHUNK - 1) / DL_CHUNK);
         e = cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)S, st);
         if (e) return e;
         WS_LAUNCH(W.prof, WSK_BWD, st,
-                  (k_dlam_count<T><<<W.n_sort_tiles, 256, 0, st>>>(ids, W.sort_tiles, W.lsegs, cnt, status)));
-        WS_LAUNCH(W.prof, WSK_BWD, st, (k_dlam_starts<false><<<nb, 256, 0, st>>>(cnt, S, key, csum)));
-        WS_LAUNCH(W.prof, WSK_BWD, st, (k_dlam_scan_totals<<<1, 1024, 0, st>>>(csum, nb)));
-        WS_LAUNCH(W.prof, WSK_BWD, st, (k_dlam_starts<true><<<nb, 256, 0, st>>>(cnt, S, key, csum)));
+                  (k_dlam_count<<<W.n_sort_tiles, 256, 0, st>>>(ids, W.sort_tiles, W.lsegs, cnt, crowded, status)));
         WS_LAUNCH(W.prof, WSK_BWD, st,
-                  (k_dlam_apply<T><<<W.n_sort_tiles, DL_NT, 0, st>>>(g, ids, W.sort_tiles, W.lsegs, cnt, key, out)));
+                  ws_launch_chain(k_dlam_crowded, std::min(W.n_sort_tiles, 3 * 152), DC_NT, 0, st, ids, W.sort_tiles,
+                                  W.n_sort_tiles, W.lsegs, cnt, crowded, status));
+        WS_LAUNCH(W.prof, WSK_BWD, st, ws_launch_chain(k_dlam_starts<false>, nb, 256, 0, st, cnt, S, key, csum));
+        WS_LAUNCH(W.prof, WSK_BWD, st, ws_launch_chain(k_dlam_scan_totals, 1, 1024, 0, st, csum, nb));
+        WS_LAUNCH(W.prof, WSK_BWD, st, ws_launch_chain(k_dlam_starts<true>, nb, 256, 0, st, cnt, S, key, csum));
+        WS_LAUNCH(W.prof, WSK_BWD, st,
+                  ws_launch_if(W.n_sort_tiles <= 2 * 152, k_dlam_apply<T>, W.n_sort_tiles, DL_NT, 0, st, g, ids,
+                               W.sort_tiles, W.lsegs, cnt, key, out));
     }
     return cudaGetLastError();
 }
