@@ -100,8 +100,7 @@ struct ws_plan {
     SegRuntime* rt = nullptr;
     void* cval = nullptr;
     uint2* rank_words = nullptr;
-    uint32_t* dest1 = nullptr;
-    uint32_t* dest2 = nullptr;
+    PassMap map1 = {}, map2 = {};
     uint16_t* bin_idx = nullptr;
     void* pairs_a = nullptr;
     void* pairs_b = nullptr;
@@ -172,8 +171,8 @@ LargeWork<T> make_work(const ws_plan* p) {
     W.rt = p->rt;
     W.cval = (T*)p->cval;
     W.rank_words = p->rank_words;
-    W.dest1 = p->dest1;
-    W.dest2 = p->dest2;
+    W.map1 = p->map1;
+    W.map2 = p->map2;
     W.bin_idx = p->bin_idx;
     W.pairs_a = (OutPair<T>*)p->pairs_a;
     W.pairs_b = (OutPair<T>*)p->pairs_b;
@@ -382,8 +381,13 @@ ws_status build_plan(ws_plan* p) {
     if ((st = plan_alloc(p, (void**)&p->rt, sizeof(SegRuntime) * p->n_lseg))) return st;
     if ((st = plan_alloc(p, &p->cval, vsize * slots))) return st;
     if ((st = plan_alloc(p, (void**)&p->rank_words, sizeof(uint2) * nh * (WS_HULL_TILE / 32)))) return st;
-    if ((st = plan_alloc(p, (void**)&p->dest1, sizeof(uint32_t) * nk))) return st;
-    if (p->two_level && (st = plan_alloc(p, (void**)&p->dest2, sizeof(uint32_t) * nk))) return st;
+    for (PassMap* m : {&p->map1, &p->map2}) {
+        if (m == &p->map2 && !p->two_level) break;
+        const size_t runs = m == &p->map1 ? (size_t)WS_FAN * p->n_sort_tiles : nk;
+        if ((st = plan_alloc(p, (void**)&m->loc, sizeof(uint16_t) * nk))) return st;
+        if ((st = plan_alloc(p, (void**)&m->starts, sizeof(uint32_t) * (WS_SORT_TILE / 32) * p->n_sort_tiles))) return st;
+        if ((st = plan_alloc(p, (void**)&m->delta, sizeof(uint32_t) * runs))) return st;
+    }
     if ((st = plan_alloc(p, (void**)&p->bin_idx, sizeof(uint16_t) * nk))) return st;
     if ((st = plan_alloc(p, &p->bsum, vsize * slots))) return st;
     if ((st = plan_alloc(p, (void**)&p->bcnt, sizeof(int32_t) * slots))) return st;

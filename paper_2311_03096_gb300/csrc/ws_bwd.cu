@@ -20,8 +20,8 @@
 // gathers them.  A bin with more than PIECE pairs is added by several CTAs
 // (128-bit global atomics per slot, the last one writes the means).  A tile whose
 // elements all share one cluster adds its sum once and moves no pairs, so a
-// single huge cluster costs one atomic per tile.  The pairs borrow the forward's
-// sort buffers, which the backward does not otherwise use.
+// single huge cluster costs one atomic per tile.  The pairs borrow buffers of the
+// forward, which the backward does not otherwise use.
 //
 // FP32 2^24, clusters of a few elements, us: prep 52 (issue, the bins' adds),
 // scan 10, moves 71 + 67 (shared-memory wavefronts, 0.67 of the pipe), bins 123
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(PNT, 2) k_bwd_part(const typename KeyOf<T>::K*
     static_assert(WS_BWD_FAN == PNT, "one bucket per thread");
     extern __shared__ __align__(16) unsigned char part_raw[];
     BwdPartSmem<T>& s = *reinterpret_cast<BwdPartSmem<T>*>(part_raw);
-    ws_chain();
+    ws_chain_wait();
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     struct Src { int64_t pos; int len; };
     auto source = [&](int tile) {
@@ -474,7 +474,10 @@ __global__ void __launch_bounds__(PNT, 2) k_bwd_part(const typename KeyOf<T>::K*
             }
             __syncthreads();
             // (the registers are free: the next tile's loads overlap the copy)
-            if (r0 + WS_BWD_FAN >= nbk && nxt < n_tiles) load(ns);
+            if (r0 + WS_BWD_FAN >= nbk) {
+                if (nxt < n_tiles) load(ns);
+                else ws_chain_go();
+            }
 #pragma unroll 4
             for (int j = t; j < total; j += PNT) {
                 const int32_t id = s.id[j];
@@ -750,9 +753,9 @@ cudaError_t ws_large_backward(const LargeWork<T>& W, const T* g, const int32_t* 
     if (e) return e;
     const BwdWork& B = W.bwd;
     const int nt = W.n_sort_tiles;
-    // the pairs borrow the sort's buffers (n_keys entries each)
+    // the pairs borrow buffers of the forward (n_keys entries each)
     K *g_a = W.keys_a, *g_b = W.keys_b;
-    int32_t *id_a = reinterpret_cast<int32_t*>(W.dest1), *id_b = reinterpret_cast<int32_t*>(W.bins);
+    int32_t *id_a = reinterpret_cast<int32_t*>(W.cval), *id_b = reinterpret_cast<int32_t*>(W.bins);
     const int n_hist = B.n_bins <= HIST_MAX ? B.n_bins : 0;
     const size_t hsm = sizeof(uint32_t) * n_hist, psm = sizeof(BwdPartSmem<T>), bsm = sizeof(BwdBinSmem);
     if ((e = cudaFuncSetAttribute(k_bwd_prep<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * HIST_MAX)) ||

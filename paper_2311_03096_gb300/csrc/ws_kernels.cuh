@@ -42,14 +42,15 @@ struct WsProf {
 // Programmatic dependent launch inside one call's chain: a kernel launched by
 // ws_launch_chain is placed on the SMs while its predecessor's last CTAs run,
 // and waits in ws_chain() for the predecessor's end before it touches memory,
-// so the 1.5 to 2 us between two kernels overlap (d = 40960, 15 launches: 132
-// -> 108 us; 2^26: 2569 -> 2510).  Every kernel launched this way starts with
-// ws_chain().  early = false is a plain launch, for kernels that live off the
-// L1: a CTA that is placed beside a predecessor with a large shared-memory
-// block gets the little L1 that this left.
+// so the 1.5 to 2 us between two kernels overlap (d = 40960, 15 launches: 127
+// -> 104 us).  Every kernel launched this way starts with ws_chain() or
+// ws_chain_wait(); a persistent kernel lets its successor in (ws_chain_go) with
+// its last tile only.  early = false is a plain launch.
+__device__ __forceinline__ void ws_chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void ws_chain_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void ws_chain() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    ws_chain_go();
+    ws_chain_wait();
 }
 template <typename... P, typename... A>
 inline void ws_launch_if(bool early, void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t st,
@@ -123,6 +124,16 @@ struct LargeSeg {
     // backward: bins of cluster slots
     int32_t bb_n, bb_fine;     // bins of the segment; bucket of the first move = bin >> bb_fine (0: one move only)
     int32_t bb_pos, bb_cpos;   // slices of the per-bin / bucket arrays
+};
+
+// What a partition pass leaves to undo it.  A tile's keys lie grouped by bucket
+// in its staging area; run r of them went to place + delta[r] of the segment.
+// 2 bytes per key and a few per run, where a destination per key takes 4, and
+// the pass is undone by runs (coalesced) instead of key by key.
+struct PassMap {
+    uint16_t* loc;      // [n_keys] a key's place in its tile's staging area
+    uint32_t* starts;   // [n_sort_tiles][WS_SORT_TILE / 32] a bit at the first place of every run
+    uint32_t* delta;    // per run; a tile's runs at tile * WS_FAN (first pass), at its first key (second)
 };
 
 // Work words of the backward (device memory).
@@ -286,8 +297,7 @@ struct LargeWork {
     T* cval;                 // [n_keys + n_lseg] cluster values
     uint2* rank_words;       // [n_hull_tiles][WS_HULL_TILE / 32] cluster starts among 32 sorted positions, starts before
     // way back to the caller's order
-    uint32_t* dest1;         // [n_keys] where the first pass put every key (relative to its segment)
-    uint32_t* dest2;         // [n_keys] the same of the second pass (two-level plans)
+    PassMap map1, map2;      // how to undo the first pass and the second (two-level plans)
     uint16_t* bin_idx;       // [n_keys] for every sorted position, its key's place in the unsorted bin
     OutPair<T>* pairs_a;     // [n_keys] in the first pass's order (two-level segments)
     OutPair<T>* pairs_b;     // [n_keys] in bin order; before that, scratch of the oversize bins' sort
@@ -299,7 +309,7 @@ struct LargeWork {
     WsProf* prof;            // host-side launch accounting
 };
 
-// way_back: also record where every key goes (dest1, dest2, bin_idx).
+// way_back: also record where every key goes (map1, map2, bin_idx).
 template <typename T>
 cudaError_t ws_large_sort(const LargeWork<T>& W, const T* values, bool way_back, uint32_t* status,
                           uint64_t spin_limit, cudaStream_t st, typename KeyOf<T>::K** sorted);

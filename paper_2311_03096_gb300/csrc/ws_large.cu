@@ -863,14 +863,15 @@ __device__ __forceinline__ int ws_cluster_at(uint2 rw, uint32_t pos) {
 // single elements all over memory, which is what a lookup of every weight by
 // value costs (one or two random sectors each).  Against a table of clusters
 // with a directory of 2^22 value buckets and such a lookup, us: 2^26 FP32
-// lambda 1e-2: table 449 + lookup 1533 -> values 311, bins 202, regroup 245,
-// output 286; 2^24 lambda 1: 120 + 42 + 212 -> 92, 55, 70, 69; 1024 uneven
-// segments: 878 + 101 + 1241 -> 539, 313, 406 (no second pass).  The sort pays
-// for it by writing where every key goes: 10 bytes per key, 86 + 41 us at 2^26.
+// lambda 1e-2: table 449 + lookup 1533 -> values 289, bins 199, regroup 228,
+// output 233; 2^24 lambda 1: 120 + 42 + 212 -> 82, 53, 65, 61; 1024 uneven
+// segments: 878 + 101 + 1241 -> 498, 309, 340 (no second pass).  The sort pays
+// for it by writing where the keys go: 6 bytes per key and a few per run.
 // ---------------------------------------------------------------------------
 // Bins: value and cluster of every sorted position, put into the order the
-// partition left the bin in (in shared memory).  One CTA per bin; the CTAs after those share the oversize bins,
-// whose elements find their position by bisection in the sorted bin.
+// partition left the bin in (in shared memory).  One CTA per bin; the CTAs after
+// those share the oversize bins, whose elements find their position by bisection
+// in the sorted bin.
 constexpr int OUT_EXTRA = 64;
 
 template <typename T>
@@ -965,42 +966,88 @@ __global__ void __launch_bounds__(256, 6) k_bin_out(const LargeSeg* __restrict__
     }
 }
 
-// One tile per CTA of 1024 threads: two tiles' runs at a time fit an SM's L1,
-// where the neighbours in a run share their sectors (256 threads, eight tiles
-// per SM: output 399 us instead of 286 at 2^26, regroup the same).
-constexpr int GNT = 1024;
+// A pass undone tile by tile: the tile's pairs are read run by run into shared
+// memory, where every element then finds its own.  Bound by DRAM latency and
+// bytes (2^26: 18 bytes per element, 0.78 of the copy rate).  A gather of every
+// pair through a 4-byte destination took one line per lane and clock of the L1
+// and 20 bytes: regroup 245 -> 228 us, output 286 -> 233 at 2^26, 406 -> 340 for
+// 1024 uneven segments.
+constexpr int GNT = WS_SORT_NT;
 
-// Second pass undone: bin order to the first pass's order (two-level segments).
+// The places of this thread's elements t + k GNT, two to a word (loaded first: they
+// arrive while the tile is staged).
+__device__ __forceinline__ void ws_load_places(uint32_t (&pl)[WS_SORT_TILE / GNT / 2], const uint16_t* loc, int len) {
+#pragma unroll
+    for (int k = 0; k < WS_SORT_TILE / GNT; k += 2) {
+        const int a = min((int)threadIdx.x + k * GNT, len - 1), b = min((int)threadIdx.x + (k + 1) * GNT, len - 1);
+        pl[k / 2] = (uint32_t)__ldg(loc + a) | ((uint32_t)__ldg(loc + b) << 16);
+    }
+}
+
+// The tile's pairs, run by run (neighbouring lanes read neighbouring pairs), into
+// the tile's staging order.  Bounds hold whatever the maps contain.
 template <typename T>
-__global__ void __launch_bounds__(GNT) k_regroup(const TileDesc* __restrict__ tiles, const LargeSeg* __restrict__ lsegs,
-                                                 const SegRuntime* __restrict__ rt, const uint32_t* __restrict__ dest,
-                                                 const OutPair<T>* __restrict__ from, OutPair<T>* __restrict__ to) {
+__device__ __forceinline__ void ws_stage_tile(OutPair<T>* stage, uint32_t* words, uint32_t* pre, int* wsum,
+                                              const PassMap& m, int tile, int64_t dpos, int max_run, int len,
+                                              const OutPair<T>* __restrict__ src, uint32_t last) {
+    constexpr int W = WS_SORT_TILE / 32, U = 6;
+    static_assert(W <= GNT && WS_SORT_TILE % (GNT * U) == 0, "a thread per word; whole steps");
+    const int t = threadIdx.x;
+    const uint32_t wd = t < W ? __ldg(m.starts + (int64_t)tile * W + t) : 0u;
+    const int ex = ws_block_excl_scan<GNT, int>(__popc(wd), wsum, nullptr);
+    if (t < W) { words[t] = wd; pre[t] = (uint32_t)ex; }
+    __syncthreads();
+    for (int j0 = t; j0 < len; j0 += GNT * U) {
+        uint32_t p[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int j = min(j0 + u * GNT, len - 1);
+            const int r = (int)pre[j >> 5] + __popc(words[j >> 5] & (0xffffffffu >> (31 - (j & 31)))) - 1;
+            p[u] = min((uint32_t)j + __ldg(m.delta + dpos + max(min(r, max_run - 1), 0)), last);
+        }
+        OutPair<T> o[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) o[u] = src[p[u]];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (j0 + u * GNT < len) stage[j0 + u * GNT] = o[u];
+    }
+    __syncthreads();
+}
+
+template <typename T>
+__global__ void __launch_bounds__(GNT, sizeof(T) == 4 ? 3 : 2) k_regroup(
+    const TileDesc* __restrict__ tiles, const LargeSeg* __restrict__ lsegs, const SegRuntime* __restrict__ rt,
+    const PassMap map, const OutPair<T>* __restrict__ from, OutPair<T>* __restrict__ to) {
+    extern __shared__ __align__(16) unsigned char pair_smem_raw[];
+    __shared__ uint32_t words[WS_SORT_TILE / 32], pre[WS_SORT_TILE / 32];
+    __shared__ int wsum[GNT / 32];
+    OutPair<T>* stage = reinterpret_cast<OutPair<T>*>(pair_smem_raw);   // [WS_SORT_TILE]
     ws_chain();
     const TileDesc td = tiles[blockIdx.x];
     const LargeSeg& sg = lsegs[td.lseg];
     if (sg.fine_log2 == 0 || rt[td.lseg].n_clusters == 1) return;
-    const uint32_t last = (uint32_t)sg.len - 1u;
-    const OutPair<T>* src = from + sg.kpos;
-    constexpr int U = WS_SORT_TILE / GNT;   // (one step: every load of the tile in flight)
-    for (int i0 = threadIdx.x; i0 < td.len; i0 += GNT * U) {
-        uint32_t p[U];
-        OutPair<T> o[U];
+    uint32_t pl[WS_SORT_TILE / GNT / 2];
+    ws_load_places(pl, map.loc + td.kpos, td.len);
+    ws_stage_tile<T>(stage, words, pre, wsum, map, blockIdx.x, td.kpos, td.len, td.len, from + sg.kpos,
+                     (uint32_t)sg.len - 1u);
 #pragma unroll
-        for (int u = 0; u < U; ++u) p[u] = i0 + u * GNT < td.len ? __ldg(dest + td.kpos + i0 + u * GNT) : 0u;
-#pragma unroll
-        for (int u = 0; u < U; ++u) o[u] = src[min(p[u], last)];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (i0 + u * GNT < td.len) to[td.kpos + i0 + u * GNT] = o[u];
+    for (int k = 0; k < WS_SORT_TILE / GNT; ++k) {
+        const int i = threadIdx.x + k * GNT;
+        if (i < td.len) to[td.kpos + i] = stage[min((int)(pl[k / 2] >> (16 * (k & 1)) & 0xffffu), td.len - 1)];
     }
 }
 
 // First pass undone: value and id of every element, in the caller's order.
 template <typename T>
-__global__ void __launch_bounds__(GNT) k_output(const TileDesc* __restrict__ tiles, const LargeSeg* __restrict__ lsegs,
-                                                const SegRuntime* __restrict__ rt, const T* __restrict__ cval,
-                                                const uint32_t* __restrict__ dest, const OutPair<T>* __restrict__ pairs_a,
-                                                const OutPair<T>* __restrict__ pairs_b, T* out, int32_t* ids) {
+__global__ void __launch_bounds__(GNT, sizeof(T) == 4 ? 3 : 2) k_output(
+    const TileDesc* __restrict__ tiles, const LargeSeg* __restrict__ lsegs, const SegRuntime* __restrict__ rt,
+    const T* __restrict__ cval, const PassMap map, const OutPair<T>* __restrict__ pairs_a,
+    const OutPair<T>* __restrict__ pairs_b, T* out, int32_t* ids) {
+    extern __shared__ __align__(16) unsigned char pair_smem_raw[];
+    __shared__ uint32_t words[WS_SORT_TILE / 32], pre[WS_SORT_TILE / 32];
+    __shared__ int wsum[GNT / 32];
+    OutPair<T>* stage = reinterpret_cast<OutPair<T>*>(pair_smem_raw);   // [WS_SORT_TILE]
     ws_chain();
     const TileDesc td = tiles[blockIdx.x];
     const LargeSeg& sg = lsegs[td.lseg];
@@ -1012,22 +1059,17 @@ __global__ void __launch_bounds__(GNT) k_output(const TileDesc* __restrict__ til
         }
         return;
     }
-    const uint32_t last = (uint32_t)sg.len - 1u;
-    const OutPair<T>* src = (sg.fine_log2 ? pairs_a : pairs_b) + sg.kpos;
-    constexpr int U = WS_SORT_TILE / GNT;   // (one step: every load of the tile in flight)
-    for (int i0 = threadIdx.x; i0 < td.len; i0 += GNT * U) {
-        uint32_t p[U];
-        OutPair<T> o[U];
+    uint32_t pl[WS_SORT_TILE / GNT / 2];
+    ws_load_places(pl, map.loc + td.kpos, td.len);
+    ws_stage_tile<T>(stage, words, pre, wsum, map, blockIdx.x, (int64_t)blockIdx.x * WS_FAN, WS_FAN, td.len,
+                     (sg.fine_log2 ? pairs_a : pairs_b) + sg.kpos, (uint32_t)sg.len - 1u);
 #pragma unroll
-        for (int u = 0; u < U; ++u) p[u] = i0 + u * GNT < td.len ? __ldg(dest + td.kpos + i0 + u * GNT) : 0u;
-#pragma unroll
-        for (int u = 0; u < U; ++u) o[u] = src[min(p[u], last)];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (i0 + u * GNT < td.len) {
-                __stcs(out + td.vpos + i0 + u * GNT, o[u].val);
-                if (ids) __stcs(ids + td.vpos + i0 + u * GNT, o[u].id);
-            }
+    for (int k = 0; k < WS_SORT_TILE / GNT; ++k) {
+        const int i = threadIdx.x + k * GNT;
+        if (i >= td.len) break;
+        const OutPair<T> o = stage[min((int)(pl[k / 2] >> (16 * (k & 1)) & 0xffffu), td.len - 1)];
+        __stcs(out + td.vpos + i, o.val);
+        if (ids) __stcs(ids + td.vpos + i, o.id);
     }
 }
 
@@ -1085,16 +1127,20 @@ cudaError_t ws_large_prox(const LargeWork<T>& W, const T* values, WsLambda lambd
               ws_launch_chain(k_bin_out<T>, W.n_bins + OUT_EXTRA, 256, osm, st, W.lsegs, W.rt, W.bin_seg, W.bin_start,
                               W.bin_cnt, W.n_bins, W.bin_idx, W.rank_words, W.cval, sorted, W.keys_b, W.ctl, W.over,
                               W.pairs_b));
-    // (the two gathers want their L1: beside the CTAs of k_bin_out they take
-    // twice as long, at 2^24 937 us per call against 810; up to two tiles per
-    // SM the launch counts for more)
+    const size_t gsm = sizeof(OutPair<T>) * WS_SORT_TILE;
+    if ((e = cudaFuncSetAttribute(k_regroup<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm)) ||
+        (e = cudaFuncSetAttribute(k_output<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm)))
+        return e;
+    // (beside the end of their predecessors the two ways back through large grids lose more than the
+    // launch gains: 2^26 2540 us per call against 2435, 1024 uneven segments 3490 against 3420; up to two
+    // tiles per SM it gains 4 us of 104)
     const bool early = W.n_sort_tiles <= 2 * 152;
     if (W.two_level)
         WS_LAUNCH(W.prof, WSK_REGROUP, st,
-                  ws_launch_if(early, k_regroup<T>, W.n_sort_tiles, GNT, 0, st, W.sort_tiles, W.lsegs, W.rt, W.dest2,
+                  ws_launch_if(early, k_regroup<T>, W.n_sort_tiles, GNT, gsm, st, W.sort_tiles, W.lsegs, W.rt, W.map2,
                                   W.pairs_b, W.pairs_a));
     WS_LAUNCH(W.prof, WSK_OUTPUT, st,
-              ws_launch_if(early, k_output<T>, W.n_sort_tiles, GNT, 0, st, W.sort_tiles, W.lsegs, W.rt, W.cval, W.dest1,
+              ws_launch_if(early, k_output<T>, W.n_sort_tiles, GNT, gsm, st, W.sort_tiles, W.lsegs, W.rt, W.cval, W.map1,
                               W.pairs_a, W.pairs_b, out, ids));
     return cudaGetLastError();
 }

@@ -27,7 +27,7 @@
 //   FP32 2^24     398 -> 271 (68, 2 x 58, 82, 6)
 //   FP64 2^22     319 -> 147 (53, 2 x 23, 41, 6)
 //   1024 FP32 segments of 16 .. 2^20 elements (9.7e7 keys)   2085 -> 1310
-// without the records of the way back; with them 2^26 1010 (2 x 260, bins 334).
+// without the records of the way back; with them 2^26 980 (2 x 249, bins 334).
 // The partition is bound by shared-memory wavefronts (17 per 32 keys: the
 // counters, the staging and the copy out; 0.7 of the pipe), the bin sort by
 // issue (0.65) and the same pipe, the plan by the read of the values (0.104 of
@@ -490,6 +490,7 @@ struct PartSmem {
     B bin[WS_SORT_TILE];
     uint32_t cnt[WS_FAN];
     uint2 run[WS_FAN];        // start of the bucket's run inside the tile, and its destination
+    uint32_t starts[WS_SORT_TILE / 32];   // a bit at the first place of every run
     int wsum[WS_SORT_NT / 32];
 };
 
@@ -497,7 +498,7 @@ template <typename T, typename B, bool FIRST>
 __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
     const T* __restrict__ values, const typename KeyOf<T>::K* __restrict__ keys_in, const B* __restrict__ bins_in,
     typename KeyOf<T>::K* __restrict__ out_a, typename KeyOf<T>::K* __restrict__ out_b, B* __restrict__ bins_out,
-    uint32_t* __restrict__ dest,   // (nullable: where every key goes)
+    PassMap map,   // (map.loc nullable: how to undo the pass)
     const TileDesc* __restrict__ tiles, int n_tiles, const LargeSeg* __restrict__ lsegs, uint32_t* cursor,
     const SortCtl* ctl, uint32_t* status) {
     typedef KeyOf<T> KO;
@@ -506,7 +507,7 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
     static_assert(WS_FAN == NT, "one bucket per thread");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     PartSmem<T, B>& s = *reinterpret_cast<PartSmem<T, B>*>(smem_raw);
-    ws_chain();
+    ws_chain_wait();
     if (ctl->abort) return;
     const int t = threadIdx.x;
     // the next tile of this CTA from `tile` on that this pass moves
@@ -546,6 +547,7 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
             nbk = max(min(sg.nbins, (((int)__ldg(bins_in + k0 + len - 1) >> fl) + 1) << fl) - base, 1);
         }
         const int bsh = FIRST ? 13 + fl : 13;
+        uint32_t jb = 0, rb = 0;   // places and runs of the rounds before
 #pragma unroll
         for (int k = 0; k < ITEMS; ++k) {
             if (FIRST) key[k] = KO::key_of_bits(key[k]);
@@ -555,6 +557,7 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
             const uint32_t off = (uint32_t)(base + r0);
             __syncthreads();   // (the previous use of the shared memory is over)
             s.cnt[t] = 0;
+            if (r0 == 0 && t < WS_SORT_TILE / 32) s.starts[t] = 0;
             __syncthreads();
 #pragma unroll
             for (int k = 0; k < ITEMS; ++k) {
@@ -566,9 +569,18 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
             const uint32_t c = s.cnt[t];
             const uint32_t g =
                 c ? atomicAdd(cursor + (FIRST ? sg.coarse_pos : sg.bin_pos + base) + r0 + t, c) : 0u;
-            int total;
-            const int ex = ws_block_excl_scan<NT, int>((int)c, s.wsum, &total);
-            s.run[t] = make_uint2((uint32_t)ex, g);
+            // (places in the low half, runs in the high one)
+            int tot2;
+            const uint32_t ex2 =
+                (uint32_t)ws_block_excl_scan<NT, int>((int)(c | (c ? 0x10000u : 0u)), s.wsum, &tot2);
+            const uint32_t ex = ex2 & 0xffffu;
+            const int total = tot2 & 0xffff;
+            s.run[t] = make_uint2(ex, g);
+            if (map.loc && c) {
+                const uint32_t j = jb + ex;
+                map.delta[(FIRST ? (int64_t)tile * WS_FAN : tiles[tile].kpos) + rb + (ex2 >> 16)] = g - j;
+                atomicOr(&s.starts[j >> 5], 1u << (j & 31));
+            }
             __syncthreads();
             const int64_t kp = tiles[tile].kpos;
 #pragma unroll
@@ -579,12 +591,15 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
                     const uint32_t rk = br[k] & 0x1fffu, j = run.x + rk;
                     s.key[j] = key[k];
                     s.bin[j] = (B)(br[k] >> 13);
-                    if (dest) dest[kp + t + k * NT] = run.y + rk;
+                    if (map.loc) map.loc[kp + t + k * NT] = (uint16_t)(jb + j);
                 }
             }
             __syncthreads();
             // (the key registers are free: the next tile's loads overlap the copy)
-            if (r0 + WS_FAN >= nbk && nxt < n_tiles) load(tiles[nxt]);
+            if (r0 + WS_FAN >= nbk) {
+                if (nxt < n_tiles) load(tiles[nxt]);
+                else ws_chain_go();
+            }
             // bucket runs, copied out by consecutive threads
             K* dst = (FIRST && fl != 0 ? out_a : out_b) + sg.kpos;
             B* bdst = bins_out + sg.kpos;
@@ -599,7 +614,10 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
                     if (FIRST && fl != 0) bdst[p] = bn;
                 }
             }
+            jb += (uint32_t)total;
+            rb += (uint32_t)tot2 >> 16;
         }
+        if (map.loc && t < WS_SORT_TILE / 32) map.starts[(int64_t)tile * (WS_SORT_TILE / 32) + t] = s.starts[t];
         tile = nxt;
     }
 }
@@ -1222,12 +1240,12 @@ static cudaError_t sort_run(const LargeWork<T>& W, const T* values, bool way_bac
     B* no_bins = nullptr;
     WS_LAUNCH(W.prof, WSK_PARTITION, st,
               ws_launch_chain(k_part<T, B, true>, grid, WS_SORT_NT, ksm, st, values, no_keys, bins, W.keys_a,
-                              W.keys_b, bins2, way_back ? W.dest1 : nullptr, W.sort_tiles, W.n_sort_tiles, W.lsegs,
+                              W.keys_b, bins2, way_back ? W.map1 : PassMap{}, W.sort_tiles, W.n_sort_tiles, W.lsegs,
                               W.cur1, W.ctl, status));
     if (W.two_level)
         WS_LAUNCH(W.prof, WSK_PARTITION, st,
                   ws_launch_chain(k_part<T, B, false>, grid, WS_SORT_NT, ksm, st, no_values, W.keys_a, bins2, no_keys,
-                                  W.keys_b, no_bins, way_back ? W.dest2 : nullptr, W.sort_tiles, W.n_sort_tiles,
+                                  W.keys_b, no_bins, way_back ? W.map2 : PassMap{}, W.sort_tiles, W.n_sort_tiles,
                                   W.lsegs, W.cur2, W.ctl, status));
     WS_LAUNCH(W.prof, WSK_BIN_SORT, st,
               ws_launch_chain(way_back ? k_bin_sort<T, true> : k_bin_sort<T, false>, W.n_bins, BIN_NT,
