@@ -81,6 +81,7 @@ struct ws_plan {
     int32_t* seg_emin = nullptr;
     uint16_t* vp = nullptr;
     i128* vx = nullptr;
+    TileX* hx = nullptr;
     int32_t* nvert = nullptr;
     i128* tile_total = nullptr;
     int32_t* arrive = nullptr;
@@ -151,6 +152,7 @@ LargeWork<T> make_work(const ws_plan* p) {
     W.seg_emin = p->seg_emin;
     W.vp = p->vp;
     W.vx = p->vx;
+    W.hx = p->hx;
     W.nvert = p->nvert;
     W.tile_total = p->tile_total;
     W.arrive = p->arrive;
@@ -363,6 +365,7 @@ ws_status build_plan(ws_plan* p) {
     if ((st = plan_alloc(p, &p->stat_partial, ws_R_partial_bytes(p->n_sort_tiles)))) return st;
     if ((st = plan_alloc(p, (void**)&p->vp, sizeof(uint16_t) * nh * (WS_HULL_TILE + 1)))) return st;
     if ((st = plan_alloc(p, (void**)&p->vx, sizeof(i128) * nh * (WS_HULL_TILE + 1)))) return st;
+    if ((st = plan_alloc(p, (void**)&p->hx, sizeof(TileX) * nh))) return st;
     if ((st = plan_alloc(p, (void**)&p->nvert, sizeof(int32_t) * nh))) return st;
     if ((st = plan_alloc(p, (void**)&p->tile_total, sizeof(i128) * nh))) return st;
     if ((st = plan_alloc(p, (void**)&p->pieces, sizeof(Piece) * nh))) return st;

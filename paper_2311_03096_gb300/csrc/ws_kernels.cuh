@@ -136,6 +136,36 @@ struct PassMap {
     uint32_t* delta;    // per run; a tile's runs at tile * WS_FAN (first pass), at its first key (second)
 };
 
+// X at the vertices of a hull tile: 64-bit sums of deviations from q0 in units of
+// 2^sh (one store of 8 bytes per vertex where 128 bits take a wide product, a
+// shift and 16 bytes: tile hulls of 2^26 elements 415 -> 378 us, of 1024 uneven
+// segments 820 -> 745), or 128-bit values
+// (wide) for the tiles of the general kernel.
+struct TileX {
+    int64_t q0;
+    int32_t sh, wide;
+};
+struct VertX {
+    const i128* x;
+    const TileX* h;
+    // vertex v of `tile`, at the tile's point p
+    __device__ __forceinline__ i128 at(int64_t tile, int v, int p) const {
+        return at(h[tile], tile, v, p);
+    }
+    __device__ __forceinline__ i128 at(const TileX& t, int64_t tile, int v, int p) const {
+        const i128* b = x + tile * (WS_HULL_TILE + 1);
+        if (t.wide) return b[v];
+        return (i128)p * (i128)t.q0 + ((i128)reinterpret_cast<const int64_t*>(b)[v] << t.sh);
+    }
+    // at(tile, v + 1, p + n) - at(tile, v, p), with the tile's TileX at hand
+    __device__ __forceinline__ i128 step(const TileX& t, int64_t tile, int v, int n) const {
+        const i128* b = x + tile * (WS_HULL_TILE + 1);
+        if (t.wide) return b[v + 1] - b[v];
+        const int64_t* q = reinterpret_cast<const int64_t*>(b) + v;
+        return (i128)t.q0 * (int64_t)n + ((i128)(q[1] - q[0]) << t.sh);
+    }
+};
+
 // Work words of the backward (device memory).
 struct BwdWork {
     int n_bins, two_level;
@@ -275,7 +305,8 @@ struct LargeWork {
     uint32_t* hist;          // counters of the backward's slot buckets: >= 3 * 256 + 2 64-bit words
     // hull
     uint16_t* vp;            // [n_hull_tiles][WS_HULL_TILE + 1] vertex points (tile-local)
-    i128* vx;                // [n_hull_tiles][WS_HULL_TILE + 1] X at vertices (tile-local)
+    i128* vx;                // [n_hull_tiles][WS_HULL_TILE + 1] X at vertices (tile-local; see TileX)
+    TileX* hx;               // [n_hull_tiles]
     int32_t* nvert;          // [n_hull_tiles]
     i128* tile_total;        // [n_hull_tiles] node total X, stored at the node's first tile
     int32_t* arrive;         // [levels][n_hull_tiles] merge-tree arrival counters (cleared with the sort's words)

@@ -49,7 +49,7 @@ struct NodeView {
     const Piece* pc;   // piece list
     int np;            // pieces
     const uint16_t* vp;
-    const i128* vx;
+    VertX vx;
     int hull_first;    // global index of the segment's first hull tile
     i128 base;         // X offset of this node's first point in the merge frame
     __device__ __forceinline__ int find(int r) const {   // piece holding rank r
@@ -62,9 +62,9 @@ struct NodeView {
     }
     __device__ __forceinline__ void get(int r, int64_t& pt, i128& X) const {
         const Piece p = ws_ld_piece(pc + find(r));
-        size_t v = (size_t)p.tile * (HT + 1) + p.lo + (r - p.cum);
-        pt = (int64_t)(p.tile - hull_first) * HT + vp[v];
-        X = base + p.off + vx[v];
+        const int v = p.lo + (r - p.cum), at = vp[(size_t)p.tile * (HT + 1) + v];
+        pt = (int64_t)(p.tile - hull_first) * HT + at;
+        X = base + p.off + vx.at(p.tile, v, at);
     }
     __device__ __forceinline__ int count() const {
         if (np == 0) return 0;
@@ -73,11 +73,11 @@ struct NodeView {
     }
 };
 
-__device__ __forceinline__ void ws_piece_vertex(const Piece& q, int v, const uint16_t* vp, const i128* vx,
+__device__ __forceinline__ void ws_piece_vertex(const Piece& q, int v, const uint16_t* vp, const VertX& vx,
                                                 int hull_first, i128 base, int64_t& pt, i128& X) {
-    const size_t idx = (size_t)q.tile * (HT + 1) + v;
-    pt = (int64_t)(q.tile - hull_first) * HT + vp[idx];
-    X = base + q.off + vx[idx];
+    const int at = vp[(size_t)q.tile * (HT + 1) + v];
+    pt = (int64_t)(q.tile - hull_first) * HT + at;
+    X = base + q.off + vx.at(q.tile, v, at);
 }
 
 // Bridge between two node hulls by walking outward from their junction
@@ -85,7 +85,7 @@ __device__ __forceinline__ void ws_piece_vertex(const Piece& q, int v, const uin
 // directly.  Returns false (no result) after too many steps; the caller then
 // runs the galloping search.  Same outputs as ws_bridge.
 __device__ bool ws_bridge_walk(const Piece* PL, int npL, const Piece* PR, int npR, const uint16_t* vp,
-                               const i128* vx, int hull_first, i128 baseR, const SegConst& sc, int& flag, int& istar,
+                               const VertX& vx, int hull_first, i128 baseR, const SegConst& sc, int& flag, int& istar,
                                int& jstar) {
     int lp = npL - 1, rp = 0;
     Piece qL = ws_ld_piece(PL + lp), qR = ws_ld_piece(PR + rp);
@@ -158,7 +158,7 @@ struct MergeSmem {
 };
 
 // Vertex of rank r of a node hull whose piece list is cached in shared memory.
-__device__ __forceinline__ void ws_cached_vertex(const Piece* c, int np, int r, const uint16_t* vp, const i128* vx,
+__device__ __forceinline__ void ws_cached_vertex(const Piece* c, int np, int r, const uint16_t* vp, const VertX& vx,
                                                  int hull_first, i128 base, int64_t& pt, i128& X) {
     int lo = 0, hi = np - 1;   // the last piece whose first rank is <= r
     while (lo < hi) {
@@ -191,7 +191,7 @@ __device__ __forceinline__ int ws_cached_find(const Piece* c, int np, int r) {
 // piece lists are copied into `cache` (capacity >= npL + npR).  All threads
 // call it; it ends synchronised with m.is/js/pl/pr set and m.ok = 1.
 __device__ void ws_parallel_bridge(Piece* cache, MergeSmem& m, const Piece* PL, const Piece* PR, const uint16_t* vp,
-                                   const i128* vx, int hull_first, const SegConst& sc) {
+                                   const VertX& vx, int hull_first, const SegConst& sc) {
     constexpr int NW = HNT / 32;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const int npL = m.npL, npR = m.npR;
@@ -301,7 +301,7 @@ __device__ void ws_parallel_bridge(Piece* cache, MergeSmem& m, const Piece* PL, 
 // walks them in shared memory and falls back to the global search only if
 // the bridge leaves that window.
 __device__ __noinline__ void ws_merge_children(MergeSmem& m, Piece* pieces, int32_t* npieces, i128* ntotal, int Lg, int Rg,
-                                  const uint16_t* vp, const i128* vx, int hull_first, const SegConst& sc,
+                                  const uint16_t* vp, const VertX& vx, int hull_first, const SegConst& sc,
                                   Piece* cache, int cache_cap) {
     const int t = threadIdx.x;
     Piece* PL = pieces + Lg;
@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(HNT, 4) k_tile_hull(const typename KeyOf<T>::K
                                                    const TileDesc* __restrict__ htiles,
                                                    const LargeSeg* __restrict__ lsegs,
                                                    WsLambda lambdas, SegRuntime* rt,
-                                                   uint16_t* vp, i128* vx, int32_t* nvert, i128* tile_total,
+                                                   uint16_t* vp, i128* vx, TileX* hx, int32_t* nvert, i128* tile_total,
                                                    const int32_t* __restrict__ gen_list,
                                                    const int32_t* __restrict__ gen_count,
                                                    const int32_t* __restrict__ seg_emin, uint32_t* status) {
@@ -583,6 +583,7 @@ __global__ void __launch_bounds__(HNT, 4) k_tile_hull(const typename KeyOf<T>::K
     }
     if (t == 0) {
         nvert[tile] = nv;
+        hx[tile] = TileX{0, 0, 1};
         __stcg(reinterpret_cast<uint4*>(tile_total + tile), *reinterpret_cast<const uint4*>(&total));
     }
     }
@@ -606,7 +607,7 @@ struct ClimbSmem {
 };
 
 __global__ void __launch_bounds__(HNT) k_climb(const TileDesc* __restrict__ htiles, const LargeSeg* __restrict__ lsegs,
-                                               const TileScale* __restrict__ scales, const uint16_t* vp, const i128* vx,
+                                               const TileScale* __restrict__ scales, const uint16_t* vp, const VertX vx,
                                                const int32_t* __restrict__ nvert, i128* tile_total, Piece* pieces,
                                                int32_t* npieces, int32_t* arrive, int n_hull,
                                                const int32_t* __restrict__ seg_mode,
@@ -724,7 +725,7 @@ template <typename T>
 __global__ void __launch_bounds__(256, 6) k_values(const TileDesc* __restrict__ htiles, const LargeSeg* __restrict__ lsegs,
                                                 const TileScale* __restrict__ scales, const SegRuntime* __restrict__ rt,
                                                 const typename KeyOf<T>::K* __restrict__ sorted,
-                                                const uint16_t* __restrict__ vp, const i128* __restrict__ vx,
+                                                const uint16_t* __restrict__ vp, const VertX vx,
                                                 const Piece* __restrict__ pieces,
                                                 const int32_t* __restrict__ npieces,
                                                 const int32_t* __restrict__ tile_piece, T* cval, uint2* rank_words,
@@ -739,6 +740,7 @@ __global__ void __launch_bounds__(256, 6) k_values(const TileDesc* __restrict__ 
     const int tile = blockIdx.x, t = threadIdx.x;
     const int tp = tile_piece[tile];
     const TileDesc td = htiles[tile];
+    const TileX tx = vx.h[tile];
     const LargeSeg& ls = lsegs[td.lseg];
     const int h0 = ls.hull_first;
     const int64_t kpos = ls.kpos, n_clusters = rt[td.lseg].n_clusters, table_pos = rt[td.lseg].table_pos;
@@ -782,7 +784,6 @@ __global__ void __launch_bounds__(256, 6) k_values(const TileDesc* __restrict__ 
         const SegConst sc = ws_seg_scale(scales, td.lseg);
         const Piece pc = P[tp];
         const uint16_t* vpt = vp + (size_t)tile * (HT + 1);
-        const i128* vxt = vx + (size_t)tile * (HT + 1);
         const int64_t p0 = (int64_t)td.tin * HT;
         int sh = 0;
         const bool bin = n_clusters != 1 && ws_tile_binade<T>(key[0], key[td.len - 1], td.len, emax, sh);
@@ -818,22 +819,19 @@ __global__ void __launch_bounds__(256, 6) k_values(const TileDesc* __restrict__ 
                     }
                     SX = (i128)q;
                 } else {
-                    i128 Xb;
                     bool ok = true;
                     if (bl >= 0) {
-                        Xb = pc.off + vxt[i + 1];
+                        SX = vx.step(tx, tile, i, bl - al);
                     } else if (tp + 1 < np) {
                         const Piece q = P[tp + 1];
-                        const size_t v = (size_t)q.tile * (HT + 1) + q.lo;
-                        b = (int64_t)(q.tile - h0) * HT + vp[v];
-                        Xb = q.off + vx[v];
+                        const int at = vp[(size_t)q.tile * (HT + 1) + q.lo];
+                        b = (int64_t)(q.tile - h0) * HT + at;
+                        SX = q.off + vx.at(q.tile, q.lo, at) - (pc.off + vx.at(tile, i, al));
                     } else {
                         ok = false;
                         ws_flag(status, WS_STATUS_INTERNAL);
-                        Xb = 0;
                     }
                     if (ok) {
-                        SX = Xb - (pc.off + vxt[i]);
                         if (b - a == 1) xs = KO::from_key(sorted[kpos + a]);
                     } else b = a + 1;
                 }
@@ -1103,13 +1101,13 @@ cudaError_t ws_large_prox(const LargeWork<T>& W, const T* values, WsLambda lambd
     const int small_grid = W.n_hull_tiles < 4 * 152 ? W.n_hull_tiles : 4 * 152;
     WS_LAUNCH(W.prof, WSK_TILE_GENERAL, st,
               ws_launch_chain(k_tile_hull<T>, small_grid, HNT, smem, st, sorted, W.hull_tiles, W.lsegs, lambdas, W.rt,
-                              W.vp, W.vx, W.nvert, W.tile_total, W.gen_list, &W.ctl->gen_count, W.seg_emin, status));
+                              W.vp, W.vx, W.hx, W.nvert, W.tile_total, W.gen_list, &W.ctl->gen_count, W.seg_emin, status));
     // across tiles: junction bridges and the per-segment resolution, then the
     // tree of merges for the segments that need it
     e = ws_large_junctions<T>(W, st);
     if (e) return e;
     WS_LAUNCH(W.prof, WSK_CLIMB, st,
-              ws_launch_chain(k_climb, small_grid, HNT, 0, st, W.hull_tiles, W.lsegs, W.scales, W.vp, W.vx, W.nvert,
+              ws_launch_chain(k_climb, small_grid, HNT, 0, st, W.hull_tiles, W.lsegs, W.scales, W.vp, VertX{W.vx, W.hx}, W.nvert,
                               W.tile_total, W.pieces, W.npieces, W.arrive, W.n_hull_tiles, W.seg_mode, W.seg_below));
     // CTAs per segment of the numbering: one per 1024 tiles of an average segment
     const int parts = std::max(1, std::min(16, W.n_hull_tiles / W.n_lseg / 1024));
@@ -1118,7 +1116,7 @@ cudaError_t ws_large_prox(const LargeWork<T>& W, const T* values, WsLambda lambd
                               W.seg_below, W.pieces, W.npieces, W.tile_piece, W.rt, n_clusters, parts));
     WS_LAUNCH(W.prof, WSK_VALUES, st,
               ws_launch_chain(k_values<T>, W.n_hull_tiles, 256, 0, st, W.hull_tiles, W.lsegs, W.scales, W.rt, sorted,
-                              W.vp, W.vx, W.pieces, W.npieces, W.tile_piece, W.cval, W.rank_words, fp64, ep, status));
+                              W.vp, VertX{W.vx, W.hx}, W.pieces, W.npieces, W.tile_piece, W.cval, W.rank_words, fp64, ep, status));
     // back to the caller's order
     const size_t osm = sizeof(OutPair<T>) * WS_BIN_CAP;
     e = cudaFuncSetAttribute(k_bin_out<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)osm);

@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(NT, 4) k_hull_fast(const typename KeyOf<T>::K*
                                                    const LargeSeg* __restrict__ lsegs,
                                                    const SegRuntime* __restrict__ rt,
                                                    const TileScale* __restrict__ scales, uint16_t* vp, i128* vx,
-                                                   int32_t* nvert, i128* tile_total, int32_t* gen_list,
+                                                   TileX* hx, int32_t* nvert, i128* tile_total, int32_t* gen_list,
                                                    int32_t* gen_count, int32_t* tile_rounds, int32_t* tile_piece,
                                                    int ic_cap) {
     typedef KeyOf<T> KO;
@@ -237,16 +237,15 @@ __global__ void __launch_bounds__(NT, 4) k_hull_fast(const typename KeyOf<T>::K*
         c = (int)s.hi[t] - lo;
     }
 
-    // ---- write the hull: tile-local points and tile-local X in the segment's
-    // fixed point (binade tiles: X = p q0 + (deviation sum << sh))
+    // ---- write the hull: tile-local points and X in the tile's units (in the
+    // segment's fixed point X = p q0 + (deviation sum << sh))
     int nv;
     const int o = ws_block_excl_scan<NT, int>(c, s.wsum, &nv);
-    i128* vxo = vx + (size_t)tile * (HT + 1) + o;
+    int64_t* vxt = reinterpret_cast<int64_t*>(vx + (size_t)tile * (HT + 1));
     uint16_t* vpo = vp + (size_t)tile * (HT + 1) + o;
     auto put = [&](int k, int p) {
-        const int64_t xu = wsh::xat(s, p);
         vpo[k] = (uint16_t)p;
-        vxo[k] = (i128)p * (i128)q0 + (bin ? ((i128)xu << sh) : (i128)xu);
+        vxt[o + k] = wsh::xat(s, p);
     };
     if (converged) {
         // the vertex points staged in the (idle) lane-stack storage, then both
@@ -263,19 +262,18 @@ __global__ void __launch_bounds__(NT, 4) k_hull_fast(const typename KeyOf<T>::K*
         }
         if (first < n && last == n) stage[k++] = (uint16_t)n;
         __syncthreads();
-        i128* vxt = vx + (size_t)tile * (HT + 1);
         uint16_t* vpt = vp + (size_t)tile * (HT + 1);
         for (int i = t; i < nv; i += NT) {
             const int p = stage[i];
-            const int64_t xu = wsh::xat(s, p);
             vpt[i] = (uint16_t)p;
-            vxt[i] = (i128)p * (i128)q0 + (bin ? ((i128)xu << sh) : (i128)xu);
+            vxt[i] = wsh::xat(s, p);
         }
     } else {
         for (int k = 0; k < c; ++k) put(k, s.st[(lo + k) * NT + t]);
     }
     if (t == 0) {
         nvert[tile] = nv;
+        hx[tile] = TileX{q0, bin ? sh : 0, 0};
         const int64_t xu = wsh::xat(s, n);
         const i128 tot = (i128)n * (i128)q0 + (bin ? ((i128)xu << sh) : (i128)xu);
         __stcg(reinterpret_cast<uint4*>(tile_total + tile), *reinterpret_cast<const uint4*>(&tot));
@@ -299,7 +297,7 @@ struct JVert {
 
 __global__ void __launch_bounds__(256) k_junction(const TileDesc* __restrict__ htiles, const LargeSeg* __restrict__ lsegs,
                                                   const TileScale* __restrict__ scales,
-                                                  const uint16_t* __restrict__ vp, const i128* __restrict__ vx,
+                                                  const uint16_t* __restrict__ vp, const VertX vx,
                                                   const int32_t* __restrict__ nvert,
                                                   const i128* __restrict__ tile_total, int32_t* keepR, int32_t* keepL,
                                                   int32_t* jflag0, int n_hull) {
@@ -311,12 +309,13 @@ __global__ void __launch_bounds__(256) k_junction(const TileDesc* __restrict__ h
     if (td.tin + 1 >= ls.hull_count) return;
     const SegConst sc = ws_seg_scale(scales, td.lseg);
     const int TL = gw, TR = gw + 1;
+    const TileX hL = vx.h[TL], hR = vx.h[TR];
     const int p = nvert[TL] - 1, q = nvert[TR] - 1;
     const size_t bL = (size_t)TL * (HT + 1), bR = (size_t)TR * (HT + 1);
     const i128 baseR = tile_total[TL];
     const int64_t offR = td.len;   // (a tile that has a right neighbour is whole)
-    auto L = [&](int i) -> JVert { return JVert{(int64_t)vp[bL + i], vx[bL + i]}; };
-    auto R = [&](int j) -> JVert { return JVert{offR + (int64_t)vp[bR + j], baseR + vx[bR + j]}; };
+    auto L = [&](int i) -> JVert { const int pt = vp[bL + i]; return JVert{(int64_t)pt, vx.at(hL, TL, i, pt)}; };
+    auto R = [&](int j) -> JVert { const int pt = vp[bR + j]; return JVert{offR + (int64_t)pt, baseR + vx.at(hR, TR, j, pt)}; };
     auto cvx = [&](const JVert& a, const JVert& b, const JVert& c) { return ws_convex(a.X, b.X, c.X, a.p, b.p, c.p, sc); };
     // L_p = R_0 is the junction point
     int i = p - 1, j = 1;
@@ -453,7 +452,7 @@ __global__ void __launch_bounds__(RNT) k_resolve(const LargeSeg* __restrict__ ls
 // tile's hull).  One warp per hull tile of the segments left undecided.
 __global__ void __launch_bounds__(256) k_chord(const TileDesc* __restrict__ htiles, const LargeSeg* __restrict__ lsegs,
                                                const TileScale* __restrict__ scales,
-                                               const uint16_t* __restrict__ vp, const i128* __restrict__ vx,
+                                               const uint16_t* __restrict__ vp, const VertX vx,
                                                const int32_t* __restrict__ nvert, const i128* __restrict__ tile_base,
                                                const i128* __restrict__ seg_total,
                                                const int32_t* __restrict__ seg_mode, int32_t* seg_below,
@@ -468,6 +467,7 @@ __global__ void __launch_bounds__(256) k_chord(const TileDesc* __restrict__ htil
     const SegConst sc = ws_seg_scale(scales, td.lseg);
     const i128 base = tile_base[gw], Xd = seg_total[td.lseg];
     const int nv = nvert[gw];
+    const TileX hx = vx.h[gw];
     const size_t b = (size_t)gw * (HT + 1);
     const int64_t p0 = (int64_t)td.tin * HT;
     bool below = false;
@@ -475,9 +475,10 @@ __global__ void __launch_bounds__(256) k_chord(const TileDesc* __restrict__ htil
         // decided elsewhere?  (an L2 round trip: every eighth step only, so that
         // the two tail tiles' thousands of vertices do not wait on it each step)
         if ((it & 7) == 0 && *(volatile const int32_t*)(seg_below + td.lseg)) break;
-        const int64_t pos = p0 + vp[b + v];
+        const int at = vp[b + v];
+        const int64_t pos = p0 + at;
         if (pos == 0 || pos == ls.len) continue;
-        if (ws_convex((i128)0, base + vx[b + v], Xd, 0, pos, ls.len, sc)) { below = true; break; }
+        if (ws_convex((i128)0, base + vx.at(hx, gw, v, at), Xd, 0, pos, ls.len, sc)) { below = true; break; }
     }
     if (below) atomicExch(seg_below + td.lseg, 1);
 }
@@ -495,7 +496,7 @@ cudaError_t ws_large_hull_fast(const LargeWork<T>& W, const typename KeyOf<T>::K
     if (e) return e;
     WS_LAUNCH(W.prof, WSK_TILE_HULL, st,
               ws_launch_chain(k_hull_fast<T>, W.n_hull_tiles, NT, smem, st, sorted, W.hull_tiles, W.lsegs, W.rt,
-                              W.scales, W.vp, W.vx, W.nvert, W.tile_total, W.gen_list, &W.ctl->gen_count,
+                              W.scales, W.vp, W.vx, W.hx, W.nvert, W.tile_total, W.gen_list, &W.ctl->gen_count,
                               W.tile_rounds, W.tile_piece, W.ic_cap));
     return cudaGetLastError();
 }
@@ -506,12 +507,12 @@ cudaError_t ws_large_junctions(const LargeWork<T>& W, cudaStream_t st) {
     const int grid = (W.n_hull_tiles + warps_per_cta - 1) / warps_per_cta;
     WS_LAUNCH(W.prof, WSK_JUNCTION, st,
               ws_launch_chain(k_junction, (W.n_hull_tiles + 127) / 128, 128, 0, st, W.hull_tiles, W.lsegs, W.scales,
-                              W.vp, W.vx, W.nvert, W.tile_total, W.keepR, W.keepL, W.jflag0, W.n_hull_tiles));
+                              W.vp, VertX{W.vx, W.hx}, W.nvert, W.tile_total, W.keepR, W.keepL, W.jflag0, W.n_hull_tiles));
     WS_LAUNCH(W.prof, WSK_JUNCTION, st,
               ws_launch_chain(k_resolve<T>, W.n_lseg, RNT, 0, st, W.lsegs, W.nvert, W.tile_total, W.keepR, W.keepL,
                               W.jflag0, W.pieces, W.npieces, W.seg_mode, W.tile_base, W.seg_total, W.seg_below));
     WS_LAUNCH(W.prof, WSK_JUNCTION, st,
-              ws_launch_chain(k_chord, grid, 32 * warps_per_cta, 0, st, W.hull_tiles, W.lsegs, W.scales, W.vp, W.vx,
+              ws_launch_chain(k_chord, grid, 32 * warps_per_cta, 0, st, W.hull_tiles, W.lsegs, W.scales, W.vp, VertX{W.vx, W.hx},
                               W.nvert, W.tile_base, W.seg_total, W.seg_mode, W.seg_below, W.n_hull_tiles));
     return cudaGetLastError();
 }
