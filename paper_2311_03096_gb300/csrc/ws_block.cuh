@@ -230,14 +230,6 @@ __device__ __forceinline__ i128 ws_tile_X(const int64_t* s64, const i128* base, 
     return base[p / M] + (i128)v;
 }
 
-// lambda * 2^L / (d - 1) as float for the FP32 filter; usable if finite and
-// small enough that muq * (c - a) * n1 * n2 stays far from overflow.
-__device__ __forceinline__ float ws_muq(double lam, const SegConst& sc, bool& usable) {
-    double m = (sc.d > 1) ? ldexp(lam, sc.L) / (double)(sc.d - 1) : 0.0;
-    usable = (m == m) && m < 1.0e26;
-    return usable ? (float)m : 0.0f;
-}
-
 // ---------------------------------------------------------------------------
 // Stable ranking of a CTA's keys by one 8-bit digit.
 // Arrangement: warp w owns positions [w*32*ITEMS, (w+1)*32*ITEMS); item k of
@@ -377,21 +369,26 @@ struct TilePtsWide {
     bool fast;
     __device__ __forceinline__ int64_t v(int p) const { return s64[ws_sidx<M>(p)]; }
     __device__ __forceinline__ i128 Xv(int p, int64_t vp) const { return base[p / M] + (i128)vp; }
-    // An FP32 filter first: |fB - B n1| <= 2.4e-7 |B n1| (three roundings of the
-    // conversion, one product), the same for A; the right-hand side, the two
-    // subtractions: < 5e-7 of the terms in all.  One FP64 segment of 4096
-    // N(0, 1) weights, one CTA: hull 50 us (lambda 0.1) and 132 us (1) with the
-    // exact 128/192-bit test alone.
+    // Delta = B n1 - A n2 exact in 128 bits (|X| < 2^75: elements below 2^62, at
+    // most 2^12 of them), then an FP32 comparison with mu (c - a) n1 n2 whose error
+    // is relative to Delta + rhs, as in TilePtsDev: < 6e-7, three roundings of the
+    // conversion and four of the right-hand side.  (A filter on the rounded terms
+    // B n1 and A n2, which nearly cancel, left most tests to the 192-bit
+    // comparison: hull of one such tile of 2^22 N(0, 1) weights 39 us, 18 with this
+    // one.)
     __device__ __forceinline__ bool convex_v(int a, int64_t va, int b, int64_t vb, int c, int64_t vc,
                                              const SegConst& sc) const {
-        const i128 Xa = Xv(a, va), Xb = Xv(b, vb), Xc = Xv(c, vc);
+        return convex_X(a, Xv(a, va), b, Xv(b, vb), c, Xv(c, vc), sc);
+    }
+    __device__ __forceinline__ bool convex_X(int a, i128 Xa, int b, i128 Xb, int c, i128 Xc, const SegConst& sc) const {
+        const int n1 = b - a, n2 = c - b;
+        const i128 D = (Xc - Xb) * (i128)n1 - (Xb - Xa) * (i128)n2;
+        if (D <= 0) return false;
+        if (sc.mlam == 0) return true;
         if (fast) {
-            const float n1 = (float)(b - a), n2 = (float)(c - b);
-            const float fB = ws_i128_to_float_scaled(Xc - Xb, 0) * n1;
-            const float fA = ws_i128_to_float_scaled(Xb - Xa, 0) * n2;
-            const float rhs = muq * (float)(c - a) * n1 * n2;
-            const float diff = (fB - fA) - rhs;
-            const float err = 6.0e-7f * (fabsf(fB) + fabsf(fA) + rhs);
+            const float Df = ws_i128_to_float_scaled(D, 0);
+            const float rhs = muq * ((float)(c - a) * (float)(n1 * n2));
+            const float diff = Df - rhs, err = 6.0e-7f * (Df + rhs);
             if (diff > err) return true;
             if (diff < -err) return false;
         }

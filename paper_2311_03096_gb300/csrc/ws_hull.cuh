@@ -54,6 +54,12 @@ constexpr int NW = NT / 32;
 constexpr int TILE = NT * M;           // 4096 elements per tile
 constexpr uint16_t NONE = 0xffff;
 
+// IC rounds, per warp: last and first survivor, for alternate rounds (read as int4)
+struct Ends {
+    __align__(16) int wl[2][NW];
+    __align__(16) int wf[2][NW];
+};
+
 // Shared memory of one tile.
 struct Smem {
     // X of point p lives at slot p + p / M (lanes with consecutive chunks then
@@ -68,9 +74,7 @@ struct Smem {
     int wsum[NW];
     int general;                 // a bridge walk hit its cap: the tile needs the general kernel
     int all_conc;
-    // IC rounds, per warp: last and first survivor, for alternate rounds (read as int4)
-    __align__(16) int wl[2][NW];
-    __align__(16) int wf[2][NW];
+    Ends e;
 };
 static_assert(NW % 4 == 0, "per-warp words are read four at a time");
 
@@ -516,7 +520,7 @@ __device__ __forceinline__ void cta_tree(Smem& s, const Test& T, int t, int cap)
 // first + i), for this lane's neighbours in other warps; -1 / BIG if none.
 // Written to buffer `buf`; visible after the caller's next barrier.
 constexpr int BIG = 1 << 20;
-__device__ __forceinline__ void post_ends(Smem& s, int t, int first, uint32_t B, int buf) {
+__device__ __forceinline__ void post_ends(Ends& s, int t, int first, uint32_t B, int buf) {
     const unsigned bS = __ballot_sync(WS_FULL_MASK, B != 0);
     const int l = t & 31, w = t >> 5;
     if (bS == 0) {
@@ -531,7 +535,7 @@ __device__ __forceinline__ void post_ends(Smem& s, int t, int first, uint32_t B,
 // one after it, over the whole CTA: inside the warp by one ballot and two
 // shuffles, across warps from the posted ends.
 struct Around { int pS, nS; };
-__device__ __forceinline__ Around around(const Smem& s, int t, int first, uint32_t B, int buf) {
+__device__ __forceinline__ Around around(const Ends& s, int t, int first, uint32_t B, int buf) {
     const int l = t & 31, w = t >> 5;
     const int myL = B ? first + 31 - __clz((int)B) : -1, myF = B ? first + __ffs((int)B) - 1 : BIG;
     const unsigned bS = __ballot_sync(WS_FULL_MASK, B != 0);
@@ -558,13 +562,14 @@ __device__ __forceinline__ Around around(const Smem& s, int t, int first, uint32
 
 // B: this lane's round-1 boundaries (bit i = point first + i); on return the
 // surviving ones.  Returns true if the rounds converged within `cap` rounds
-// (rounds = rounds run, the final unchanged one included).  Prefix sums of
-// every point must be in s.X (the first barrier here publishes them).  All
-// threads of the CTA call this.
+// (rounds = rounds run, the final unchanged one included).  x(p) is the prefix
+// sum of point p in shared memory (the first barrier here publishes them), T the
+// exact test on points and prefix sums.  All threads of the CTA call this.
 // prev, next: on convergence the last boundary before the lane's range (0 if
 // none) and the first one after it (n if none).
-__device__ __forceinline__ bool ic_rounds(Smem& s, const Test& T, int t, int first, int n, uint32_t& B, int cap,
-                                          int& rounds, int& prev, int& next) {
+template <class XF, class TF>
+__device__ __forceinline__ bool ic_rounds(Ends& s, const XF& x, const TF& T, int t, int first, int n, uint32_t& B,
+                                          int cap, int& rounds, int& prev, int& next) {
     rounds = 1;
     prev = 0;
     next = n;
@@ -584,11 +589,11 @@ __device__ __forceinline__ bool ic_rounds(Smem& s, const Test& T, int t, int fir
                 uint32_t rest = B, keep = rest & (0u - rest);
                 rest ^= keep;
                 int a = prevS, b = point(keep);
-                int64_t Xa = xat(s, a), Xb = xat(s, b);
+                auto Xa = x(a), Xb = x(b);
                 while (true) {
                     const uint32_t bit = rest & (0u - rest);
                     const int c = rest ? point(bit) : nextS;
-                    const int64_t Xc = xat(s, c);
+                    const auto Xc = x(c);
                     bool empty = false;
                     while (!T(a, Xa, b, Xb, c, Xc)) {
                         keep ^= 0x80000000u >> __clz((int)keep);
@@ -596,12 +601,12 @@ __device__ __forceinline__ bool ic_rounds(Smem& s, const Test& T, int t, int fir
                         b = a; Xb = Xa;
                         const uint32_t below = keep ^ (0x80000000u >> __clz((int)keep));
                         a = below ? first + 31 - __clz((int)below) : prevS;
-                        Xa = xat(s, a);
+                        Xa = x(a);
                     }
                     if (!rest) break;
                     rest ^= bit;
                     keep |= bit;
-                    if (empty) { a = prevS; Xa = xat(s, a); }
+                    if (empty) { a = prevS; Xa = x(a); }
                     else { a = b; Xa = Xb; }
                     b = c; Xb = Xc;
                 }
@@ -609,20 +614,20 @@ __device__ __forceinline__ bool ic_rounds(Smem& s, const Test& T, int t, int fir
             }
         } else {
             if (B && prevS != lastP) {   // from the left end
-                const int64_t Xa = xat(s, prevS);
+                const auto Xa = x(prevS);
                 while (B) {
                     const uint32_t bit = B & (0u - B), rest = B ^ bit;
                     const int b = point(bit), c = rest ? point(rest & (0u - rest)) : nextS;
-                    if (T(prevS, Xa, b, xat(s, b), c, xat(s, c))) break;
+                    if (T(prevS, Xa, b, x(b), c, x(c))) break;
                     B = rest;
                 }
             }
             if (B && nextS != lastN) {   // from the right end
-                const int64_t Xc = xat(s, nextS);
+                const auto Xc = x(nextS);
                 while (B) {
                     const uint32_t bit = 0x80000000u >> __clz((int)B), rest = B ^ bit;
                     const int b = point(bit), a = rest ? first + 31 - __clz((int)rest) : prevS;
-                    if (T(a, xat(s, a), b, xat(s, b), nextS, Xc)) break;
+                    if (T(a, x(a), b, x(b), nextS, Xc)) break;
                     B = rest;
                 }
             }
@@ -650,9 +655,9 @@ __device__ __forceinline__ bool ic_rounds(Smem& s, const Test& T, int t, int fir
 // this.
 __device__ __forceinline__ uint32_t candidate_boundaries(Smem& s, const Test& T, int t, int first, int n,
                                                          uint32_t R, uint32_t G) {
-    post_ends(s, t, first, R, 0);
+    post_ends(s.e, t, first, R, 0);
     __syncthreads();
-    const Around ar = around(s, t, first, R, 0);
+    const Around ar = around(s.e, t, first, R, 0);
     const int pS = ar.pS, nS = ar.nS;
     const int prevS = pS < 0 ? 0 : pS, nextS = nS >= BIG ? n : nS;
     // interior points of this lane: 1 <= p <= n - 1 and not a run boundary
@@ -717,6 +722,41 @@ __device__ __forceinline__ bool chain_tree_hull(Smem& s, const Test& T, int t, i
     }
     cta_tree(s, T, t, cta_cap);
     return !s.general;   // (uniform after cta_tree's barrier)
+}
+
+// The same rounds for a tile whose prefix sums need 128 bits, into the chunk
+// lists of `h` (each vertex once).  One CTA per tile, so the latency of its
+// chain of decisions counts: one FP64 segment of 4096
+// N(0, 1) weights 90 us with the chain and the tree of merges, 79 with the rounds.
+static __device__ __noinline__ bool wide_rounds(HullSmem<NT, M>& h, Ends& e, int n, const TilePtsWide<M>& P,
+                                                const SegConst& sc, int cap, int* nv) {
+    const int t = threadIdx.x, first = t * M, last = min(first + M, n);
+    auto x = [&](int p) -> i128 { return P.Xv(p, P.v(p)); };
+    auto T = [&](int a, i128 Xa, int b, i128 Xb, int c, i128 Xc) { return P.convex_X(a, Xa, b, Xb, c, Xc, sc); };
+    uint32_t B = 0;
+    if (first < n) {
+        i128 Xa = x(max(first - 1, 0)), Xb = x(first);
+#pragma unroll 1
+        for (int p = first; p < last; ++p) {   // (p <= n - 1)
+            const i128 Xc = x(p + 1);
+            if (p >= 1 && T(p - 1, Xa, p, Xb, p + 1, Xc)) B |= 1u << (p - first);
+            Xa = Xb;
+            Xb = Xc;
+        }
+    }
+    int rounds, prev, next;
+    if (!ic_rounds(e, x, T, t, first, n, B, cap, rounds, prev, next)) return false;
+    int c = 0;
+    if (t == 0) h.H[NT * c++] = 0;
+    while (B) {
+        h.H[NT * c++ + t] = (uint16_t)(first + __ffs((int)B) - 1);
+        B &= B - 1;
+    }
+    if (first < n && last == n) h.H[NT * c++ + t] = (uint16_t)n;
+    h.lo[t] = 0;
+    h.hi[t] = (uint16_t)c;
+    h.cum[t] = ws_block_excl_scan<NT, int>(c, h.wsum_i, nv);
+    return true;
 }
 
 }  // namespace wsh

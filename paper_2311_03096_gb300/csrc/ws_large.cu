@@ -12,6 +12,7 @@
 // partition: its consecutive vertices bound the clusters.
 #include <algorithm>
 
+#include "ws_hull.cuh"
 #include "ws_kernels.cuh"
 
 namespace {
@@ -471,6 +472,7 @@ __device__ __noinline__ void ws_merge_children(MergeSmem& m, Piece* pieces, int3
 struct TileHullSmem {
     TilePrefix<HNT, HM> pre;
     HullSmem<HNT, HM> hull;
+    wsh::Ends ends;
     SegConst sc;     // global fixed-point scale of the segment
     SegConst sct;    // scale of this tile when it lies in one binade
     float muq, muqt;
@@ -489,7 +491,7 @@ __global__ void __launch_bounds__(HNT, 4) k_tile_hull(const typename KeyOf<T>::K
                                                    uint16_t* vp, i128* vx, TileX* hx, int32_t* nvert, i128* tile_total,
                                                    const int32_t* __restrict__ gen_list,
                                                    const int32_t* __restrict__ gen_count,
-                                                   const int32_t* __restrict__ seg_emin, uint32_t* status) {
+                                                   const int32_t* __restrict__ seg_emin, int ic_cap, uint32_t* status) {
     typedef KeyOf<T> KO;
     typedef typename KO::K K;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -515,11 +517,14 @@ __global__ void __launch_bounds__(HNT, 4) k_tile_hull(const typename KeyOf<T>::K
         if (td.tin == 0) rt[td.lseg].emax = emax;
         s.sc = ws_seg_const<T>(ls.len, lamv, emax);
         bool f;
-        s.muq = ws_muq(lamv, s.sc, f);
+        s.muq = ws_muq_f(s.sc, f);
         s.fast = f ? 1 : 0;
+    }
+    if (t == 32) {   // (two warps: FP64 divisions take a few microseconds each)
         const int sh = ws_eff_exp(KO::from_key(kfirst)) - emax + KO::FIX_OFS;
-        s.sct = ws_seg_const_L(ls.len, lamv, s.sc.L - (sh > 0 ? sh : 0));
-        s.muqt = ws_muq(lamv, s.sct, f);
+        s.sct = ws_seg_const_L(ls.len, lamv, KO::L_BASE - emax - (sh > 0 ? sh : 0));
+        bool f;
+        s.muqt = ws_muq_f(s.sct, f);
         s.fastt = f ? 1 : 0;
     }
     // this thread's 16 consecutive sorted keys (vector loads when whole and aligned)
@@ -570,7 +575,8 @@ __global__ void __launch_bounds__(HNT, 4) k_tile_hull(const typename KeyOf<T>::K
         ws_cta_hull<HNT, HM>(s.hull, n, P, s.sc, &nv);
     } else {
         const TilePtsWide<HM> P{s.pre.s64, s.pre.base, s.muq, s.fast != 0};
-        ws_cta_hull<HNT, HM>(s.hull, n, P, s.sc, &nv);
+        if (ic_cap <= 0 || !wsh::wide_rounds(s.hull, s.ends, n, P, s.sc, ic_cap, &nv))
+            ws_cta_hull<HNT, HM>(s.hull, n, P, s.sc, &nv);
     }
     {
         const int l = s.hull.lo[t], h = s.hull.hi[t], o = s.hull.cum[t];
@@ -1101,7 +1107,8 @@ cudaError_t ws_large_prox(const LargeWork<T>& W, const T* values, WsLambda lambd
     const int small_grid = W.n_hull_tiles < 4 * 152 ? W.n_hull_tiles : 4 * 152;
     WS_LAUNCH(W.prof, WSK_TILE_GENERAL, st,
               ws_launch_chain(k_tile_hull<T>, small_grid, HNT, smem, st, sorted, W.hull_tiles, W.lsegs, lambdas, W.rt,
-                              W.vp, W.vx, W.hx, W.nvert, W.tile_total, W.gen_list, &W.ctl->gen_count, W.seg_emin, status));
+                              W.vp, W.vx, W.hx, W.nvert, W.tile_total, W.gen_list, &W.ctl->gen_count, W.seg_emin, W.ic_cap,
+                              status));
     // across tiles: junction bridges and the per-segment resolution, then the
     // tree of merges for the segments that need it
     e = ws_large_junctions<T>(W, st);

@@ -40,6 +40,7 @@ struct SmallSmem {
         T val[CAP];
     } r2;
     int wsum_i[NT / 32];
+    wsh::Ends ends;
     K kmin, kmax;
     int flags;
     int emin;
@@ -97,7 +98,7 @@ __device__ __forceinline__ void small_general_segment(SmallSmem<T, NT, M>& s, in
                                                       const int64_t* __restrict__ offsets,
                                                       const WsLambda& lambdas, T* out, int32_t* ids,
                                                       int64_t* n_clusters, int fp64, const WsEpi& ep,
-                                                      uint32_t* status) {
+                                                      int ic_cap, uint32_t* status) {
     typedef KeyOf<T> KO;
     typedef typename KO::K K;
     typedef SmallSmem<T, NT, M> S;
@@ -119,7 +120,7 @@ __device__ __forceinline__ void small_general_segment(SmallSmem<T, NT, M>& s, in
     }
 
     // ---- load (striped per warp, coalesced), map to keys, check finiteness
-    if (t == 0) { s.flags = 0; s.emin = 0x7fffffff; }
+    if (t == 0) { s.flags = 0; s.emin = 0x7fffffff; s.n_multi = 0; }
     __syncthreads();
     bool bad = false;
 #pragma unroll
@@ -211,9 +212,16 @@ __device__ __forceinline__ void small_general_segment(SmallSmem<T, NT, M>& s, in
                     s.idx[q] = (uint16_t)(t + k * NT);
                 }
             __syncthreads();
-            while (multi) {
-                const int b = 2 * t * M + __ffs((int)multi) - 1;
-                multi &= multi - 1;
+            // (spread over the CTA: the fullest buckets are neighbours)
+            uint16_t* list = reinterpret_cast<uint16_t*>(&s.pre);   // (not in use yet; at most n / 2 entries)
+            static_assert(sizeof(s.pre) >= sizeof(uint16_t) * CAP / 2, "the list fits");
+            if (multi) {
+                int at = atomicAdd(&s.n_multi, __popc(multi));
+                for (; multi; multi &= multi - 1) list[at++] = (uint16_t)(2 * t * M + __ffs((int)multi) - 1);
+            }
+            __syncthreads();
+            for (int i = t; i < s.n_multi; i += NT) {
+                const int b = list[i];
                 small_sort_bucket<K>(start(b), b + 1 < 2 * n ? start(b + 1) : n, s.r2.keys, s.idx,
                                      [](int p) { return p; }, [](int p) { return p; });
             }
@@ -261,17 +269,18 @@ __device__ __forceinline__ void small_general_segment(SmallSmem<T, NT, M>& s, in
     const K kfirst = s.r2.keys[0], klast = s.r2.keys[n - 1];
     const T xlo = KO::from_key(kfirst), xhi = KO::from_key(klast);
     const int emax = ws_fix_scale<T>(max(ws_eff_exp(xlo), ws_eff_exp(xhi)), s.emin);
+    // (two warps: FP64 divisions take a few microseconds each)
     if (t == 0) {
         s.sc = ws_seg_const<T>(n, lam, emax);
         bool f;
-        s.muq = ws_muq(lam, s.sc, f);
+        s.muq = ws_muq_f(s.sc, f);
         s.fast = f ? 1 : 0;
     }
-    if (t == 0) {
+    if (t == 32) {
         const int sh0 = ws_eff_exp(xlo) - emax + KO::FIX_OFS;
-        s.sct = ws_seg_const_L(n, lam, s.sc.L - (sh0 > 0 ? sh0 : 0));
+        s.sct = ws_seg_const_L(n, lam, KO::L_BASE - emax - (sh0 > 0 ? sh0 : 0));
         bool f;
-        s.muqt = ws_muq(lam, s.sct, f);
+        s.muqt = ws_muq_f(s.sct, f);
         s.fastt = f ? 1 : 0;
     }
     // (the prefix sums end with a barrier; the keys' storage is reused from here on)
@@ -303,8 +312,10 @@ __device__ __forceinline__ void small_general_segment(SmallSmem<T, NT, M>& s, in
         P.thr = s.r2.hull.thr;
         ws_cta_hull<NT, M, TilePtsDev<M>, true>(s.r2.hull, n, P, sc, &nv);
     } else {
+        static_assert(NT == wsh::NT && M == wsh::M, "the rounds' tile");
         const TilePtsWide<M> P{s.pre.s64, s.pre.base, s.muq, s.fast != 0};
-        ws_cta_hull<NT, M>(s.r2.hull, n, P, sc, &nv);
+        if (ic_cap <= 0 || !wsh::wide_rounds(s.r2.hull, s.ends, n, P, sc, ic_cap, &nv))
+            ws_cta_hull<NT, M>(s.r2.hull, n, P, sc, &nv);
     }
     auto X = [&](int p) -> i128 { return ws_tile_X<M>(s.pre.s64, s.pre.base, mode, q0, bsh, p); };
     {
@@ -388,14 +399,14 @@ __global__ void __launch_bounds__(NT, 3) k_small_general(const T* __restrict__ v
                                                       const int32_t* __restrict__ gen_count,
                                                       const WsLambda lambdas, T* out, int32_t* ids,
                                                       int64_t* n_clusters, int fp64, const WsEpi ep,
-                                                      uint32_t* status) {
+                                                      int ic_cap, uint32_t* status) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SmallSmem<T, NT, M>& s = *reinterpret_cast<SmallSmem<T, NT, M>*>(smem_raw);
     ws_chain();
     const int cnt = *gen_count;
     for (int i = blockIdx.x; i < cnt; i += gridDim.x) {
         small_general_segment<T, NT, M>(s, gen_list[i], values, offsets, lambdas, out, ids, n_clusters, fp64, ep,
-                                        status);
+                                        ic_cap, status);
         __syncthreads();
     }
 }
@@ -846,7 +857,8 @@ __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 4 : 2) k_small(const
     if (ids_prev) B = small_warm<T>(s, tst, ids_prev, a0, first, n, B);
     int rounds = 0, prev = 0, next = n;
     bool converged = false;
-    if (ic_cap > 0) converged = wsh::ic_rounds(h, tst, t, first, n, B, ic_cap, rounds, prev, next);
+    if (ic_cap > 0) converged = wsh::ic_rounds(h.e, [&](int p) { return wsh::xat(h, p); }, tst, t, first, n, B,
+                                                    ic_cap, rounds, prev, next);
     uint16_t* st16 = reinterpret_cast<uint16_t*>(s.starts);
     if (converged) {
         st16[t] = (uint16_t)(B | (t == 0 ? 1u : 0u));
@@ -1011,7 +1023,7 @@ cudaError_t ws_launch_small(const T* values, const int64_t* offsets, const int32
     if (e != cudaSuccess) return e;
     WS_LAUNCH(prof, WSK_SMALL, st,
               ws_launch_chain(gk, n_list < 456 ? n_list : 456, NT, gsmem, st, values, offsets, gen_list, gen_count,
-                              lambdas, out, ids, n_clusters, fp64, ep, status));
+                              lambdas, out, ids, n_clusters, fp64, ep, ic_cap, status));
     return cudaGetLastError();
 }
 

@@ -222,7 +222,8 @@ __global__ void __launch_bounds__(NT, 4) k_hull_fast(const typename KeyOf<T>::K*
     }
     int rounds = 0, prev, next;
     bool converged = false;
-    if (ic_cap > 0) converged = wsh::ic_rounds(s, tst, t, first, n, B, ic_cap, rounds, prev, next);
+    if (ic_cap > 0) converged = wsh::ic_rounds(s.e, [&](int p) { return wsh::xat(s, p); }, tst, t, first, n, B,
+                                                    ic_cap, rounds, prev, next);
     if (t == 0) tile_rounds[tile] = converged ? rounds : -1;
     int c;      // vertices this lane writes
     int lo = 0;
