@@ -418,11 +418,12 @@ __global__ void __launch_bounds__(NT, 3) k_small_general(const T* __restrict__ v
 // cluster-start bitmap, values scattered back through the positions.
 // Segments whose prefix sums need 128 bits (or whose bridge walks are too
 // long) are appended to gen_list for the general kernel above.
-// Bound by issue (0.6; 460 thread instructions per weight) and the barriers
-// between its phases.  Rows of the MLP (8202 of 3072 or 4096, lambda 1e-3 .. 1):
+// Bound by issue (0.64; 470 thread instructions per weight), instruction fetches
+// and the barriers between its phases.  Rows of the MLP (8202 of 3072 or 4096, lambda 1e-3 .. 1):
 // 809 us with three CTAs per SM (74 KB of shared memory, 80 registers), one
 // decision per boundary and round and a value loop that searched the bitmap;
-// 676 with the rounds of ws_hull.cuh, 601 with four CTAs (57 KB, 64 registers).
+// 676 with the rounds of ws_hull.cuh, 601 with four CTAs (57 KB, 64 registers), 579
+// with the loops over shared memory rolled (fetching instructions is the first stall).
 // ---------------------------------------------------------------------------
 template <typename T>
 struct LeanSmem {
@@ -840,7 +841,7 @@ __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 4 : 2) k_small(const
     if (first < n) {
         const int64_t t11 = s.t11;
         int64_t dprev = devk(kprev), prevX = 0;
-#pragma unroll
+#pragma unroll 4
         for (int i = 0; i < M; ++i) {
             const int p = first + i;
             if (p < n) {
@@ -951,7 +952,7 @@ __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 4 : 2) k_small(const
     uint16_t* start_of = h.st;   // (st, lo and hi are one run of 16-bit words)
     {
         int a = prev;
-#pragma unroll
+#pragma unroll 4
         for (int i = 0; i < M; ++i) {
             const int p = first + i;
             if ((mine >> i) & 1u) a = p;
@@ -960,34 +961,38 @@ __global__ void __launch_bounds__(wsh::NT, sizeof(T) == 4 ? 4 : 2) k_small(const
     }
     __syncthreads();
     if (first < n) {
-        T ov[M];
-        int32_t oi[M];
-#pragma unroll
-        for (int i = 0; i < M; ++i) {
-            const int a = (first + i < n) ? (int)start_of[ipad(first + i)] : 0;
-            if (sizeof(T) == 4) {
-                const uint2 q = *reinterpret_cast<const uint2*>(&wsh::xref(h, a));
-                ov[i] = (T)__uint_as_float(q.x);
-                oi[i] = (int32_t)q.y;
-            } else {
-                ov[i] = (T)*reinterpret_cast<const double*>(&wsh::xref(h, a));
-                oi[i] = (int32_t)s.cid[a];
-            }
-        }
         T* od = out + a0 + first;
         int32_t* id = ids ? ids + a0 + first : nullptr;
-        if (first + M <= n && (((uintptr_t)od) & 15) == 0 && (!id || (((uintptr_t)id) & 15) == 0)) {
-            constexpr int VT = 16 / (int)sizeof(T);
+        const bool whole = first + M <= n && (((uintptr_t)od) & 15) == 0 && (!id || (((uintptr_t)id) & 15) == 0);
+        // (four at a time: the loop is rolled for the instruction cache)
+#pragma unroll 1
+        for (int j = 0; j < M; j += 4) {
+            __align__(16) T ov[4];
+            __align__(16) int32_t oi[4];
 #pragma unroll
-            for (int i = 0; i < M; i += VT) __stcs(reinterpret_cast<uint4*>(od + i), *reinterpret_cast<const uint4*>(ov + i));
-            if (id) {
-#pragma unroll
-                for (int i = 0; i < M; i += 4) __stcs(reinterpret_cast<uint4*>(id + i), *reinterpret_cast<const uint4*>(oi + i));
+            for (int i = 0; i < 4; ++i) {
+                const int a = (first + j + i < n) ? (int)start_of[ipad(first + j + i)] : 0;
+                if (sizeof(T) == 4) {
+                    const uint2 q = *reinterpret_cast<const uint2*>(&wsh::xref(h, a));
+                    ov[i] = (T)__uint_as_float(q.x);
+                    oi[i] = (int32_t)q.y;
+                } else {
+                    ov[i] = (T)*reinterpret_cast<const double*>(&wsh::xref(h, a));
+                    oi[i] = (int32_t)s.cid[a];
+                }
             }
-        } else {
-            for (int i = 0; i < M && first + i < n; ++i) {
-                od[i] = ov[i];
-                if (id) id[i] = oi[i];
+            if (whole) {
+#pragma unroll
+                for (int i = 0; i < (int)sizeof(T) / 4; ++i)
+                    __stcs(reinterpret_cast<uint4*>(od + j) + i, reinterpret_cast<const uint4*>(ov)[i]);
+                if (id) __stcs(reinterpret_cast<uint4*>(id + j), *reinterpret_cast<const uint4*>(oi));
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (first + j + i < n) {
+                        od[j + i] = ov[i];
+                        if (id) id[j + i] = oi[i];
+                    }
             }
         }
     }
