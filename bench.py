@@ -3,7 +3,7 @@
 Workload (the single-large-vector configuration): d = 2^26 FP32 weights,
 w_i ~ N(0, 1) with 10% of positions overwritten by exact duplicates, seeded;
 each step is one prox (the whole hot path: sort, shift, exact merge, cluster
-values, lookup back to the caller's order) with lambda cycling through
+values, the way back to the caller's order) with lambda cycling through
 {1e-2, 1, 1e2}.  The input (256 MiB) is larger than L2 and resident in HBM
 before the timed region.
 
@@ -48,10 +48,10 @@ ALGO_BYTES_PER_ELEM_F32 = {
 }
 
 # Whole-step byte models per element (FP32 storage), fixed before tuning:
-# the I/O floor (read w, write out and cluster id), this library's key-only
-# sort pipeline (histogram read 4 + four 8-bit passes x (read + write key) 32 +
-# merge read of the sorted keys 4 + lookup 12) and the sort-with-index-payload
-# pipeline of the design survey (80 B).  One-CTA segments of a batch move the
+# the I/O floor (read w, write out and cluster id), a key-only radix sort
+# pipeline (histogram read 4 + four 8-bit passes x (read + write key) 32 +
+# merge read of the sorted keys 4 + lookup 12) and a sort with an index
+# payload (80 B).  One-CTA segments of a batch move the
 # I/O floor only.
 IO_FLOOR_B = 12
 ONE_CTA_MAX_F32 = 4096   # FP32 segments up to this length run one CTA each

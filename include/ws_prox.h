@@ -35,7 +35,7 @@
  *     nothing is enqueued.  Errors found on the device (a NaN/Inf input, a
  *     bounded wait that gave up) are OR-ed into the context's status word and
  *     reported by ws_get_status; outputs of that call are then unspecified.
- *   - Concurrency: a plan's scratch (sort buffers, look-back words, hull and
+ *   - Concurrency: a plan's scratch (sort buffers, control words, hull and
  *     cluster tables) is reused by every call made with that plan.  The
  *     single-vector calls (ws_prox, ws_prox_l1, ws_prox_backward,
  *     ws_prox_dlambda, ws_R) share one plan per (d, dtype) cached in the
@@ -243,8 +243,8 @@ ws_status ws_get_inexact(ws_ctx* ctx, int* inexact, void* stream);
 /* Human-readable name of a status code (static string). */
 const char* ws_status_string(ws_status s);
 
-/* Set the iteration bound of every device-side spin-wait (decoupled
- * look-back).  A wait that exceeds it gives up, sets WS_ERR_TIMEOUT and lets
+/* Set the iteration bound of every device-side spin-wait (the sort's grid
+ * barriers).  A wait that exceeds it gives up, sets WS_ERR_TIMEOUT and lets
  * its kernel exit.  0 restores the default.  Test hook. */
 void ws_debug_set_spin_limit(ws_ctx* ctx, int64_t limit);
 

@@ -99,3 +99,26 @@ def test_segments(ws, ctx):
         got = np.split(s.cpu().numpy(), np.cumsum(lens)[:-1])
         for g, p in zip(got, parts):
             assert np.array_equal(np.sort(g), g) and np.array_equal(np.sort(p), g)
+
+
+def test_more_bins_than_16_bits_number(ws, ctx):
+    """A segment of more than 65536 bins (their numbers take 32 bits), sorted and brought back to its order."""
+    d = 65537 * 2560 + 12345
+    g = torch.Generator(device="cuda").manual_seed(11)
+    w = torch.randn(d, generator=g, device="cuda")
+    w[::10] = w[1]
+    want, order = torch.sort(w)
+    plan = ws.Plan([0, d])
+    s = torch.zeros_like(w)
+    plan.debug_sort(w, s)
+    ctx.check(what="debug_sort")
+    assert torch.equal(s, want)
+    out, ids, _ = plan.forward(w, torch.zeros(1, dtype=torch.float64, device="cuda"))
+    ctx.check(what="prox")
+    # lambda 0: equal weights are one cluster; a weight alone is its own value, the mean of several equal ones has
+    # the four roundings of the FP32 value at most (it is not promised to be the weight itself)
+    alone = torch.bincount(ids)[ids] == 1
+    assert torch.equal(out[alone], w[alone])
+    assert torch.all((out - w).abs() <= 2.0 ** -22 * w.abs())
+    step = (ids[order][1:] - ids[order][:-1])
+    assert torch.equal(step, (want[1:] != want[:-1]).int())
