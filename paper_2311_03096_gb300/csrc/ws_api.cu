@@ -332,7 +332,7 @@ ws_status build_plan(ws_plan* p) {
         // one block, cleared before every sort: control words, sampled ranges, cells, bin counts,
         // the merge tree's arrival counters
         const size_t nl = (size_t)p->n_lseg;
-        const size_t o_hi = sizeof(SortCtl), o_lo = o_hi + 8 * nl, o_en = o_lo + 8 * nl, o_cells = o_en + 4 * nl,
+        const size_t o_hi = sizeof(SortCtl), o_lo = o_hi + 8 * nl, o_en = o_lo + 16 * nl, o_cells = o_en + 4 * nl,
                      o_cnt = o_cells + 4 * (size_t)cell_pos, o_arr = o_cnt + 4 * (size_t)bin_pos;
         p->sort_zero_bytes = o_arr + 4 * (size_t)p->n_levels * nh;
         unsigned char* z = nullptr;

@@ -195,6 +195,8 @@ struct SortCtl {
 // Map header of a segment: cell = (key - kmin) >> shift.
 struct SortHdr {
     uint64_t kmin;
+    uint64_t mag;     // FP64: magnitudes below this count as it (see squeeze)
+    uint64_t dlo, dhi;   // smallest and largest sample above kmin
     int32_t shift;
 };
 
@@ -287,7 +289,7 @@ struct LargeWork {
     SortCtl* ctl;
     size_t sort_zero_bytes;
     unsigned long long* seg_hi;   // [n_lseg] largest sampled key
-    unsigned long long* seg_lo;   // [n_lseg] complement of the smallest sampled key
+    unsigned long long* seg_lo;   // [2][n_lseg] complements of the smallest sampled key and nonzero magnitude
     uint32_t* seg_en;        // [n_lseg] INT_MAX - smallest effective exponent of a nonzero value
     uint32_t* cells;         // [3 cells] sampled keys per cell, then per part of a cell
     uint32_t* bin_cnt;       // [n_bins]

@@ -97,14 +97,31 @@ struct MapTab {
     float2 knots[2 * WS_CELLS + 1];     // map value at the start of the part, its slope
 };
 
+// FP64 keys as the map sees them: magnitudes below m (the binade of the
+// smallest sampled one) count as m, and the gap between -m and m closes.  The
+// key range of values of both signs spans 2 x 1023 binades, nearly all of them
+// between -m and m and empty; cells cut from all of it were two or four binades
+// wide, their parts too coarse at the ends of a distribution, and bins overflowed
+// (1 to 4 of them cost the oversize kernel's 115 us and 60 us on the way back:
+// 700001 N(0, 1) weights 392 us with them, 222 without).  Monotone in the key.
+template <typename T>
+__device__ __forceinline__ typename KeyOf<T>::K squeeze(typename KeyOf<T>::K k, uint64_t m) {
+    typedef typename KeyOf<T>::K K;
+    if (sizeof(K) == 4) return k;   // (512 binades of keys: cells of half a binade)
+    const K z = (K)1 << (KeyOf<T>::BITS - 1);   // the key of +0
+    return k >= z ? z + (max(k - z, (K)m) - (K)m) : z - 1 - (max(z - 1 - k, (K)m) - (K)m);
+}
+
 template <typename T>
 struct KeyMap {
     typedef typename KeyOf<T>::K K;
     K kmin;
+    uint64_t mag;
     int shift;
     uint32_t ncell, last;
     __device__ __forceinline__ void init(const SortHdr& h, int ncell_, int nbins) {
         kmin = (K)h.kmin;
+        mag = h.mag;
         shift = h.shift;
         ncell = (uint32_t)ncell_;
         last = (uint32_t)(nbins - 1);
@@ -118,14 +135,15 @@ struct KeyMap {
     __device__ __forceinline__ static float slope(float db, int s2) {
         return ldexpf(db * (1.0f - 1.0f / 1048576.0f), -(sizeof(K) == 4 ? s2 : min(s2, 24)));
     }
-    __device__ __forceinline__ uint32_t bin(K k, const MapTab& m) const {
+    __device__ __forceinline__ uint32_t bin(K key, const MapTab& m) const {
+        const K k = squeeze<T>(key, mag);
         const K d = max(k, kmin) - kmin;
         const uint32_t e = m.split[(uint32_t)min(d >> shift, (K)ncell)];
         const int s2 = (int)(e >> 16);
         const K in = d & (((K)1 << shift) - 1);
         const uint32_t i = min((e & 0xffffu) + (uint32_t)(in >> s2), 2u * WS_CELLS);
         const float2 kn = m.knots[i];
-        return min((uint32_t)(int)fmaf((float)low(d, s2), kn.y, kn.x), last);
+        return min(__float2uint_rz(fmaf((float)low(d, s2), kn.y, kn.x)), last);   // (below 0: bin 0)
     }
 };
 
@@ -146,7 +164,7 @@ __device__ __forceinline__ int sample_pos(int tile, int j, int len, int mlog) {
 // and, for short segments, by the barriers (about 2 us each).
 // ---------------------------------------------------------------------------
 struct PlanSmem {
-    unsigned long long hi, lo;
+    unsigned long long hi, lo, mag;
     int emin, parts;
     int wsum[PLAN_NT / 32];
 };
@@ -179,13 +197,13 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
 
     // 1. range of the sampled keys (one warp per tile; the CTA's first segment
     // is combined in shared memory)
-    if (t == 0) { S.hi = 0; S.lo = 0; }
+    if (t == 0) { S.hi = 0; S.lo = 0; S.mag = 0; }
     __syncthreads();
     for (int tile = t0 + w; tile < t1; tile += PLAN_NT / 32) {
         const TileDesc td = tiles[tile];
         const int ml = lsegs[td.lseg].samp_log2;
         const int m = min(td.len, 1 << ml);
-        K hi = 0, lo = 0;   // (lo: complement, so that 0 is neutral)
+        K hi = 0, lo = 0, mg = 0;   // (lo, mg: complements, so that 0 is neutral)
         K* keep = cache + ((size_t)(tile - t0) << samp_max);
 #pragma unroll 4
         for (int j = lane; j < m; j += 32) {
@@ -193,19 +211,26 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
             if (cached) keep[j] = k;
             hi = max(hi, k);
             lo = max(lo, (K)~k);
+            if (sizeof(K) == 8) {
+                const K z = (K)1 << (KO::BITS - 1), a = k >= z ? k - z : z - 1 - k;
+                if (a != 0) mg = max(mg, (K)~a);
+            }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             hi = max(hi, ws_shfl_xor_k(hi, o));
             lo = max(lo, ws_shfl_xor_k(lo, o));
+            if (sizeof(K) == 8) mg = max(mg, ws_shfl_xor_k(mg, o));
         }
         if (lane == 0) {
             if (td.lseg == seg0) {
                 atomicMax(&S.hi, (unsigned long long)hi);
                 atomicMax(&S.lo, (unsigned long long)lo);
+                if (sizeof(K) == 8) atomicMax(&S.mag, (unsigned long long)mg);
             } else {
                 atomicMax(seg_hi + td.lseg, (unsigned long long)hi);
                 atomicMax(seg_lo + td.lseg, (unsigned long long)lo);
+                if (sizeof(K) == 8) atomicMax(seg_lo + n_lseg + td.lseg, (unsigned long long)mg);
             }
         }
     }
@@ -213,13 +238,20 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
     if (t == 0 && seg0 >= 0) {
         atomicMax(seg_hi + seg0, S.hi);
         atomicMax(seg_lo + seg0, S.lo);
+        if (sizeof(K) == 8) atomicMax(seg_lo + n_lseg + seg0, S.mag);
     }
     bar.sync();
 
     // header of a segment from its sampled range
     auto header = [&](int lseg, const LargeSeg& sg) {
         SortHdr h;
-        const K hi = (K)__ldcg(seg_hi + lseg), lo = (K)~(K)__ldcg(seg_lo + lseg);
+        h.mag = 0;
+        if (sizeof(K) == 8) {   // (a whole binade: cells stay aligned with the binades)
+            const unsigned long long c = __ldcg(seg_lo + n_lseg + lseg);
+            h.mag = c ? (~c >> KO::MANT) << KO::MANT : 0ull;
+        }
+        const K hi = squeeze<T>((K)__ldcg(seg_hi + lseg), h.mag),
+                lo = squeeze<T>((K)~(K)__ldcg(seg_lo + lseg), h.mag);
         // cells aligned in the key space, so that no cell (or part of one)
         // straddles a binade, where the density per key jumps by two
         const K range = hi > lo ? hi - lo : (K)0;
@@ -228,6 +260,8 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
         h.shift = max(bl - cl, 0);
         if (hi > lo && (hi >> h.shift) - (lo >> h.shift) >= (K)sg.ncell) ++h.shift;
         h.kmin = (uint64_t)((lo >> h.shift) << h.shift);
+        h.dlo = (uint64_t)lo - h.kmin;
+        h.dhi = (uint64_t)max(hi, lo) - h.kmin;
         return h;
     };
     // f(offset above kmin) for every sample of tiles [ta, tb) of one segment
@@ -239,8 +273,10 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
             const int64_t o = (int64_t)(tile - sg.sort_first) * WS_SORT_TILE;
             const int len = (int)min((int64_t)WS_SORT_TILE, sg.len - o);
             if (j < len) {
-                const K k = cached ? cache[((size_t)(tile - t0) << samp_max) + j]
-                                   : KO::to_key(__ldg(values + sg.vpos + o + sample_pos(tile, j, len, sg.samp_log2)));
+                const K k = squeeze<T>(
+                    cached ? cache[((size_t)(tile - t0) << samp_max) + j]
+                           : KO::to_key(__ldg(values + sg.vpos + o + sample_pos(tile, j, len, sg.samp_log2))),
+                    h.mag);
                 f(k > (K)h.kmin ? k - (K)h.kmin : (K)0);
             }
         }
@@ -373,6 +409,30 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
                 const int q1 = min((int)(e & 0xffffu) + (1 << (h.shift - s2)), parts);
                 for (int q = (int)(e & 0xffffu); q < q1; ++q)
                     tab.knots[q].y = KeyMap<T>::slope(tab.knots[q + 1].x - tab.knots[q].x, s2);
+            }
+            __syncthreads();
+            if (t == 0) {
+                // The parts of the smallest and the largest sample are filled from and up to these
+                // only (a distribution with a hard edge: the bins there held two times the mean and
+                // more).  Below the first: bin 0; above the last: the last bin.
+                auto part_at = [&](K d, int& s2) {
+                    const uint32_t e = tab.split[(uint32_t)min(d >> h.shift, (K)(sg.ncell - 1))];
+                    s2 = (int)(e >> 16);
+                    return (int)min((e & 0xffffu) + (uint32_t)((d & (((K)1 << h.shift) - 1)) >> s2), (uint32_t)(parts - 1));
+                };
+                int s0, s1;
+                const int q0 = part_at((K)h.dlo, s0), q1 = part_at((K)h.dhi, s1);
+                const float w0 = ldexpf(1.0f, sizeof(K) == 4 ? s0 : min(s0, 24)), l0 = (float)KeyMap<T>::low((K)h.dlo, s0);
+                const float l1 = (float)KeyMap<T>::low((K)h.dhi, s1) + 1.0f;
+                if (q0 < q1) {
+                    // (the start moves by at most 64 times the part's bins: its rounding, 2^-18 of them, stays
+                    // inside the slope's 2^-16)
+                    if ((w0 - l0) * 64.0f >= w0) {
+                        const float y = (tab.knots[q0 + 1].x - tab.knots[q0].x) * (1.0f - 1.0f / 65536.0f) / (w0 - l0);
+                        tab.knots[q0] = make_float2(tab.knots[q0].x - l0 * y, y);
+                    }
+                    tab.knots[q1].y = (tab.knots[q1 + 1].x - tab.knots[q1].x) / l1;
+                }
             }
         }
         KeyMap<T> map;

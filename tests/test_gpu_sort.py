@@ -122,3 +122,26 @@ def test_more_bins_than_16_bits_number(ws, ctx):
     assert torch.all((out - w).abs() <= 2.0 ** -22 * w.abs())
     step = (ids[order][1:] - ids[order][:-1])
     assert torch.equal(step, (want[1:] != want[:-1]).int())
+
+
+@pytest.mark.parametrize("dt", [np.float32, np.float64])
+@pytest.mark.parametrize("kind", ["uniform", "one side", "with zeros", "tiny outliers", "two spikes"])
+@pytest.mark.parametrize("d", [4097, 50000, 700001, 3000001])
+def test_hard_edges_and_the_gap_around_zero(ws, ctx, dt, kind, d):
+    """The map's ends (the parts of the smallest and the largest sample) and, in FP64, its closed gap
+    around zero: magnitudes below the sampled ones, on both sides, zeros of both signs, denormals."""
+    rng = np.random.default_rng(d)
+    x = rng.uniform(-0.038, 0.038, d)
+    if kind == "one side":
+        x = np.abs(x) + 1.0
+    elif kind == "with zeros":
+        x[rng.random(d) < 0.01] = 0.0
+        x[rng.random(d) < 0.01] *= -0.0
+    elif kind == "tiny outliers":
+        tiny = np.finfo(dt).smallest_subnormal
+        x[:64] = np.arange(-32, 32) * float(tiny)
+        x[64:70] = [1e30, -1e30, 1e-30, -1e-30, 3e-38, -3e-38]
+        rng.shuffle(x)
+    elif kind == "two spikes":
+        x = np.where(x < 0, -1.0, 1.0) + 1e-6 * x
+    check(ws, ctx, x.astype(dt))
