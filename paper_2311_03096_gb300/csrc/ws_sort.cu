@@ -1010,14 +1010,18 @@ __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>:
                 s.radix_needed = 1;
         __syncthreads();
     }
-    if (PLACE && cut > 0 && !s.radix_needed) {   // (uniform)
+    bool radix = s.radix_needed != 0;   // (uniform: the last write is before the barrier above)
+    if (PLACE && cut > 0 && !radix) {
         // runs with the same top bits: the thread of a run's first word orders it by the whole keys
+        // (a run too long for that is a word of the barrier, not of shared memory: a warp that
+        // has found one must not change the condition above for a warp that comes to it later)
+        bool long_run = false;
         for (int i = t; i < n; i += BIN_NT) {
             const K top = s.key[i] >> 12;
             if (i > 0 && (s.key[i - 1] >> 12) == top) continue;
             int e = i + 1;
             while (e < n && e - i <= BIN_RUN_MAX && (s.key[e] >> 12) == top) ++e;
-            if (e - i > BIN_RUN_MAX) { s.radix_needed = 1; continue; }
+            if (e - i > BIN_RUN_MAX) { long_run = true; continue; }
             for (int a = i + 1; a < e; ++a) {
                 const K wa = s.key[a], ka = __ldg(src + ((uint32_t)wa & 0xfffu));
                 int j = a - 1;
@@ -1025,11 +1029,9 @@ __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>:
                 s.key[j + 1] = wa;
             }
         }
-        __syncthreads();
+        radix = __syncthreads_or(long_run) != 0;
     }
-    const bool radix = s.radix_needed != 0;   // (uniform)
-    if (radix) {
-        __syncthreads();
+    if (radix) {   // (uniform; every word of the steps above has been read)
         bin_radix<T, PLACE>(s, src, n, (K)(~(uint64_t)0 >> (64 - range_bits)) | (lo ^ hi));
     }
     K* dst = sorted + start;
