@@ -348,7 +348,7 @@ cudaError_t ws_large_sort(const LargeWork<T>& W, const T* values, bool way_back,
                           uint64_t spin_limit, cudaStream_t st, typename KeyOf<T>::K** sorted);
 // Lean tile hulls and the junction resolution (ws_tile.cu).
 template <typename T>
-cudaError_t ws_large_hull_fast(const LargeWork<T>& W, const typename KeyOf<T>::K* sorted, WsLambda lambdas,
+cudaError_t ws_large_hull_fast(const LargeWork<T>& W, typename KeyOf<T>::K* sorted, WsLambda lambdas,
                                uint32_t* status, cudaStream_t st);
 template <typename T>
 cudaError_t ws_large_junctions(const LargeWork<T>& W, cudaStream_t st);

@@ -50,8 +50,11 @@ __device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
 
 // Barrier over a cooperative grid: arrivals are counted in *ctr (cleared
 // before the launch).  A wait that gives up sets the timeout status and the
-// abort word; the CTA then goes on without waiting (every access of the
-// kernels below is in bounds whatever the other CTAs have written).
+// abort word, and sync() is false then, for the whole CTA: what the other CTAs
+// were to write before the barrier may be missing.  The plan kernel goes on
+// without waiting (it indexes with nothing from another CTA but what it clamps);
+// the oversize kernel leaves (it indexes with other CTAs' tile numbers, which
+// may be an earlier call's).
 struct GridBarrier {
     uint32_t* ctr;
     uint32_t* abort;
@@ -59,7 +62,7 @@ struct GridBarrier {
     uint64_t limit;
     uint32_t target;
     bool dead;   // (thread 0)
-    __device__ __forceinline__ void sync() {
+    __device__ __forceinline__ bool sync() {
         __syncthreads();
         if (threadIdx.x == 0) {
             target += gridDim.x;
@@ -77,7 +80,7 @@ struct GridBarrier {
             }
             __threadfence();
         }
-        __syncthreads();
+        return !__syncthreads_or(dead);   // (dead: thread 0's, false elsewhere)
     }
 };
 
@@ -1092,7 +1095,7 @@ __global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* k
             __syncthreads();
         }
     }
-    bar.sync();
+    if (!bar.sync()) return;
     const int n_tiles = __ldcg(&over[cnt - 1].first_tile) + (over[cnt - 1].n + TILE - 1) / TILE;
     // entry of a tile (all threads; ends synchronised)
     auto entry = [&](int tile) -> int {
@@ -1134,7 +1137,7 @@ __global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* k
             atomicOr(&ctl->over_diff, s.diff);
         }
     }
-    bar.sync();
+    if (!bar.sync()) return;
     const unsigned long long all = __ldcg(&ctl->over_diff);
     for (int p = 0; p < P; ++p) {
         if (((all >> (8 * p)) & 0xffull) == 0) continue;   // (uniform over the grid)
@@ -1151,7 +1154,7 @@ __global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* k
             __syncthreads();
             if (t < 256) __stcg(over_cnt + (size_t)tile * 256 + t, s.dcount[t]);
         }
-        bar.sync();
+        if (!bar.sync()) return;
         // counts -> first position of every (tile, digit), one CTA per bin
         for (int e = blockIdx.x; e < cnt; e += gridDim.x) {
             const unsigned long long diff = __ldcg(&over[e].diff);
@@ -1179,7 +1182,7 @@ __global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* k
             if (t < 256)
                 for (int i = 0; i < nt; ++i) __stcg(c + (size_t)i * 256 + t, __ldcg(c + (size_t)i * 256 + t) + (uint32_t)ex);
         }
-        bar.sync();
+        if (!bar.sync()) return;
         // stable scatter
         for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
             const int e = entry(tile);
@@ -1210,7 +1213,7 @@ __global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* k
                     if (q < (uint32_t)ne) dst[q] = key[k];
                 }
         }
-        bar.sync();
+        if (!bar.sync()) return;
     }
     // bins of equal keys
     for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {

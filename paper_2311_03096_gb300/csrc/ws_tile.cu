@@ -40,7 +40,7 @@ constexpr int CTA_WALK_CAP = 512;
 // Per-segment scale constants (one CTA of WS_NSCALE threads per segment)
 // ---------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(WS_NSCALE) k_scales(const typename KeyOf<T>::K* __restrict__ sorted,
+__global__ void __launch_bounds__(WS_NSCALE) k_scales(typename KeyOf<T>::K* sorted, const SortCtl* __restrict__ ctl,
                                                       const LargeSeg* __restrict__ lsegs,
                                                       WsLambda lambdas,
                                                       const int32_t* __restrict__ seg_emin, SegRuntime* rt,
@@ -52,6 +52,10 @@ __global__ void __launch_bounds__(WS_NSCALE) k_scales(const typename KeyOf<T>::K
     const double lam = lambdas.at(ls.seg);
     const bool lam_ok = lam >= 0.0 && lam <= 1.7976931348623157e308;
     const double lamv = lam_ok ? lam : 0.0;
+    if (ctl->abort) {   // (uniform) a wait of the sort gave up: keys in order for the kernels that follow
+        for (int64_t i = j; i < ls.len; i += WS_NSCALE) sorted[ls.kpos + i] = KO::to_key((T)0);
+        __syncthreads();
+    }
     const T xlo = KO::from_key(sorted[ls.kpos]), xhi = KO::from_key(sorted[ls.kpos + ls.len - 1]);
     const int emax = ws_fix_scale<T>(max(ws_eff_exp(xlo), ws_eff_exp(xhi)), seg_emin[lseg]);
     if (j == 0) {
@@ -513,10 +517,10 @@ __global__ void __launch_bounds__(256) k_chord(const TileDesc* __restrict__ htil
 }  // namespace
 
 template <typename T>
-cudaError_t ws_large_hull_fast(const LargeWork<T>& W, const typename KeyOf<T>::K* sorted, WsLambda lambdas,
+cudaError_t ws_large_hull_fast(const LargeWork<T>& W, typename KeyOf<T>::K* sorted, WsLambda lambdas,
                                uint32_t* status, cudaStream_t st) {
     WS_LAUNCH(W.prof, WSK_MISC, st,
-              ws_launch_chain(k_scales<T>, W.n_lseg, WS_NSCALE, 0, st, sorted, W.lsegs, lambdas, W.seg_emin, W.rt,
+              ws_launch_chain(k_scales<T>, W.n_lseg, WS_NSCALE, 0, st, sorted, W.ctl, W.lsegs, lambdas, W.seg_emin, W.rt,
                               W.scales, status));
     const size_t smem = sizeof(FastSmem);
     cudaError_t e = cudaFuncSetAttribute(k_hull_fast<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -545,7 +549,7 @@ cudaError_t ws_large_junctions(const LargeWork<T>& W, cudaStream_t st) {
 }
 
 #define WS_INST_TILE(T)                                                                                          \
-    template cudaError_t ws_large_hull_fast<T>(const LargeWork<T>&, const typename KeyOf<T>::K*, WsLambda, \
+    template cudaError_t ws_large_hull_fast<T>(const LargeWork<T>&, typename KeyOf<T>::K*, WsLambda, \
                                                uint32_t*, cudaStream_t);                                         \
     template cudaError_t ws_large_junctions<T>(const LargeWork<T>&, cudaStream_t);
 WS_INST_TILE(float)
