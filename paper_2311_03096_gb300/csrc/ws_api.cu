@@ -77,6 +77,9 @@ struct ws_plan {
     uint32_t* cur2 = nullptr;
     int32_t* bin_seg = nullptr;
     OverBin* over = nullptr;
+    void* over_tabs = nullptr;
+    OverClass* over_items = nullptr;
+    OverClass* over_big = nullptr;
     uint32_t* over_cnt = nullptr;
     int32_t* seg_emin = nullptr;
     uint16_t* vp = nullptr;
@@ -148,6 +151,9 @@ LargeWork<T> make_work(const ws_plan* p) {
     W.cur2 = p->cur2;
     W.bin_seg = p->bin_seg;
     W.over = p->over;
+    W.over_tabs = p->over_tabs;
+    W.over_items = p->over_items;
+    W.over_big = p->over_big;
     W.over_cnt = p->over_cnt;
     W.seg_emin = p->seg_emin;
     W.vp = p->vp;
@@ -357,8 +363,14 @@ ws_status build_plan(ws_plan* p) {
     if ((st = plan_alloc(p, (void**)&p->cur1, sizeof(uint32_t) * (size_t)coarse_pos))) return st;
     if ((st = plan_alloc(p, (void**)&p->cur2, sizeof(uint32_t) * (size_t)bin_pos))) return st;
     if ((st = plan_alloc(p, (void**)&p->over, sizeof(OverBin) * (size_t)bin_pos))) return st;
-    // (a bin of n > WS_BIN_CAP keys has at most n / (WS_SORT_TILE / 2) + 1 tiles, all of them at most this many)
-    static_assert(WS_BIN_CAP >= WS_SORT_TILE / 2, "oversize bins average at least half a tile's keys per tile");
+    {
+        const size_t no = nk / WS_BIN_CAP + 1;   // (at most: an oversize bin has more than WS_BIN_CAP keys)
+        if ((st = plan_alloc(p, &p->over_tabs, (f64 ? sizeof(OverTab<uint64_t>) : sizeof(OverTab<uint32_t>)) * no))) return st;
+        if ((st = plan_alloc(p, (void**)&p->over_items, sizeof(OverClass) * (OVER_SPL + 1) * no))) return st;
+        if ((st = plan_alloc(p, (void**)&p->over_big, sizeof(OverClass) * no))) return st;
+    }
+    // (a class of n > WS_BIN_CAP keys has at most n / (WS_SORT_TILE / 2) tiles, all of them at most this many)
+    static_assert(WS_BIN_CAP >= WS_SORT_TILE / 2, "such classes average at least half a tile's keys per tile");
     if ((st = plan_alloc(p, (void**)&p->over_cnt,
                          sizeof(uint32_t) * 256 * ((size_t)p->n_keys / (WS_SORT_TILE / 2) + 1)))) return st;
     if ((st = plan_alloc(p, (void**)&p->seg_emin, sizeof(int32_t) * p->n_lseg))) return st;

@@ -145,24 +145,37 @@ struct TileX {
     int64_t q0;
     int32_t sh, wide;
 };
+__device__ __forceinline__ i128 ws_i128(int64_t hi, uint64_t lo) { return (i128)(((u128)(uint64_t)hi << 64) | lo); }
+// a b, and a 2^s for 0 <= s < 64, in two words each (the 128-bit operators take wide
+// products and shifts of both words)
+__device__ __forceinline__ i128 ws_mul_i64(int64_t a, int64_t b) { return ws_i128(__mul64hi(a, b), (uint64_t)a * (uint64_t)b); }
+__device__ __forceinline__ i128 ws_shl_i64(int64_t a, int s) { return ws_i128((a >> 1) >> (63 - s), (uint64_t)a << s); }
 struct VertX {
     const i128* x;
     const TileX* h;
     // vertex v of `tile`, at the tile's point p
+    // (for searches, which wait for one load after the other: all that a vertex needs is loaded side by
+    // side and picked without a branch, so that the loads of two vertices overlap as well)
     __device__ __forceinline__ i128 at(int64_t tile, int v, int p) const {
-        return at(h[tile], tile, v, p);
+        const i128* b = x + tile * (WS_HULL_TILE + 1);
+        const ulonglong2 w = __ldg(reinterpret_cast<const ulonglong2*>(b + v));
+        const int64_t s = __ldg(reinterpret_cast<const int64_t*>(b) + v);
+        const TileX t = h[tile];
+        const i128 q = ws_mul_i64(p, t.q0) + ws_shl_i64(s, t.sh);
+        const uint64_t m = t.wide ? ~0ull : 0ull;
+        return ws_i128((int64_t)((w.y & m) | ((uint64_t)(q >> 64) & ~m)), (w.x & m) | ((uint64_t)q & ~m));
     }
     __device__ __forceinline__ i128 at(const TileX& t, int64_t tile, int v, int p) const {
         const i128* b = x + tile * (WS_HULL_TILE + 1);
         if (t.wide) return b[v];
-        return (i128)p * (i128)t.q0 + ((i128)reinterpret_cast<const int64_t*>(b)[v] << t.sh);
+        return ws_mul_i64(p, t.q0) + ws_shl_i64(reinterpret_cast<const int64_t*>(b)[v], t.sh);
     }
     // at(tile, v + 1, p + n) - at(tile, v, p), with the tile's TileX at hand
     __device__ __forceinline__ i128 step(const TileX& t, int64_t tile, int v, int n) const {
         const i128* b = x + tile * (WS_HULL_TILE + 1);
         if (t.wide) return b[v + 1] - b[v];
         const int64_t* q = reinterpret_cast<const int64_t*>(b) + v;
-        return (i128)t.q0 * (int64_t)n + ((i128)(q[1] - q[0]) << t.sh);
+        return ws_mul_i64(n, t.q0) + ws_shl_i64(q[1] - q[0], t.sh);
     }
 };
 
@@ -187,7 +200,9 @@ struct SortCtl {
     uint32_t abort;        // a barrier gave up: the keys are not moved
     uint32_t over_count;   // bins above WS_BIN_CAP
     uint32_t over_bar;     // grid barrier of the oversize kernel
-    unsigned long long over_diff;   // key bits that vary inside any oversize bin
+    unsigned long long over_diff;   // key bits that vary inside any class above WS_BIN_CAP
+    uint32_t over_items;   // classes to sort, up to WS_BIN_CAP keys
+    uint32_t over_big;     // and above
     int32_t gen_count;     // hull tiles for the general kernel
     int32_t pad;
 };
@@ -205,8 +220,39 @@ struct OverBin {
     int64_t start;          // first key
     int32_t n;
     int32_t first_tile;     // of the oversize kernel's tiles
-    unsigned long long diff;   // key bits that vary inside the bin
-    int32_t lseg, pad;
+    int32_t lseg;
+    int32_t nspl;           // splitters of its classes
+};
+
+// Its classes: 2 i + 1 the keys equal to splitter i, 2 i those between splitters
+// i - 1 and i (see ws_sort.cu).
+constexpr int OVER_SPL = 255;
+template <typename K>
+struct OverTab {
+    K spl[OVER_SPL];                  // ascending, different
+    uint32_t cnt[2 * OVER_SPL + 1];   // keys per class
+    uint32_t cur[OVER_SPL + 1];       // write cursors of the classes between splitters
+};
+// Classes of N keys; spl: OVER_SPL + 1 entries, ~0 beyond the splitters.  The searches
+// take one step after the other side by side (their loads overlap).
+template <typename K, int N>
+__device__ __forceinline__ void ws_over_classes(const K* spl, int n, const K (&key)[N], int (&cls)[N]) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) cls[k] = 0;   // splitters below the key, so far
+    for (int step = 1 << (31 - __clz(n | 1)); step > 0; step >>= 1) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) cls[k] += spl[cls[k] + step - 1] < key[k] ? step : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < N; ++k) cls[k] = 2 * cls[k] + (cls[k] < n && spl[cls[k]] == key[k] ? 1 : 0);
+}
+
+// A class between splitters that is to be sorted.
+struct OverClass {
+    int64_t start;
+    int32_t n;
+    int32_t first_tile;        // above WS_BIN_CAP keys: of the radix passes' tiles
+    unsigned long long diff;   // and the key bits that vary inside it
 };
 
 // A piece of a node hull: vertices [lo, hi) of hull tile `tile`; cum = rank of
@@ -271,6 +317,7 @@ struct WsSortShape {
     int max_bins = 0;                                  // of the longest segment
     int samp_max = 0;                                  // log2 of the most samples per tile
     int plan_grid = 1, part_grid = 1, over_grid = 1;   // CTAs resident at once
+    int out_extra = 1;                                 // CTAs of the way back for the oversize bins
 };
 template <typename T> cudaError_t ws_sort_prepare(int max_bins, int n_tiles, int samp_max, WsSortShape* sh);
 
@@ -302,6 +349,9 @@ struct LargeWork {
     uint32_t* cur2;          // [n_bins] write cursors of the second pass
     const int32_t* bin_seg;  // [n_bins] segment of every bin
     OverBin* over;           // [n_bins] oversize bins
+    void* over_tabs;         // [n_keys / WS_BIN_CAP + 1] OverTab: their classes
+    OverClass* over_items;   // [n_keys / WS_BIN_CAP + 1][OVER_SPL + 1] classes to sort
+    OverClass* over_big;     // [n_keys / WS_BIN_CAP + 1] those above WS_BIN_CAP keys
     uint32_t* over_cnt;      // [n_keys / (WS_SORT_TILE / 2) + 1][256] digit counts of their tiles
     int32_t* seg_emin;       // [n_lseg] smallest effective exponent of a nonzero value
     uint32_t* hist;          // counters of the backward's slot buckets: >= 3 * 256 + 2 64-bit words

@@ -874,9 +874,100 @@ __device__ __forceinline__ int ws_cluster_at(uint2 rw, uint32_t pos) {
 // ---------------------------------------------------------------------------
 // Bins: value and cluster of every sorted position, put into the order the
 // partition left the bin in (in shared memory).  One CTA per bin; the CTAs after
-// those share the oversize bins, whose elements find their position by bisection
-// in the sorted bin.
-constexpr int OUT_EXTRA = 64;
+// those share the tiles of the oversize bins.
+
+// Oversize bins, elements [o0, o0 + n) of a bin at a time: an element takes its
+// place from the classes that the sort cut the bin into.  One cluster holds a tie,
+// so the ties' values are looked up once per bin, and only the elements between
+// splitters look for their key (by bisection, in their class).
+template <typename T>
+struct OverOutSmem {
+    typename KeyOf<T>::K spl[OVER_SPL + 1];
+    uint32_t start[2 * OVER_SPL + 2];
+    OutPair<T> tie[OVER_SPL];
+    int wsum[8];
+};
+template <typename T>
+__device__ __noinline__ void bin_out_oversize(OverOutSmem<T>& s, int cta, int n_ctas, int cnt,
+                                              const LargeSeg* __restrict__ lsegs, const SegRuntime* __restrict__ rt,
+                                              const uint2* __restrict__ rank_words, const T* __restrict__ cval,
+                                              const typename KeyOf<T>::K* __restrict__ sorted,
+                                              const typename KeyOf<T>::K* __restrict__ keys,
+                                              const OverBin* __restrict__ over,
+                                              const OverTab<typename KeyOf<T>::K>* __restrict__ tabs, OutPair<T>* pairs) {
+    typedef typename KeyOf<T>::K K;
+    constexpr int TILE = WS_SORT_TILE, U = 4;
+    const int t = threadIdx.x;
+    // this CTA's tiles, contiguous: a table serves all tiles of its bin
+    const int n_tiles = over[cnt - 1].first_tile + (over[cnt - 1].n + TILE - 1) / TILE;
+    int tile = (int)((int64_t)n_tiles * cta / n_ctas);
+    const int t1 = (int)((int64_t)n_tiles * (cta + 1) / n_ctas);
+    int e = 0;
+    for (int hi = cnt - 1; e < hi;) {
+        const int mid = (e + hi + 1) >> 1;
+        if (over[mid].first_tile <= tile) e = mid; else hi = mid - 1;
+    }
+    for (; tile < t1; ++e) {
+        const OverBin ob = over[e];
+        const int te = min(t1, ob.first_tile + (ob.n + TILE - 1) / TILE);
+        const LargeSeg& sg = lsegs[ob.lseg];
+        const int64_t c = rt[ob.lseg].n_clusters;
+        if (c == 1) { tile = te; continue; }   // (one cluster: every element has it)
+        const uint2* sw = rank_words + (size_t)sg.hull_first * HTW;
+        const T* cv = cval + rt[ob.lseg].table_pos;
+        const uint32_t pos0 = (uint32_t)(ob.start - sg.kpos);   // the bin's first sorted position
+        auto pair_at = [&](uint32_t r) {
+            const uint32_t p = pos0 + min(r, (uint32_t)ob.n - 1u);
+            OutPair<T> o = {};
+            o.id = ws_cluster_at(__ldg(sw + (p >> 5)), p);
+            o.val = __ldg(cv + min(max((int64_t)o.id, (int64_t)0), c - 1));
+            return o;
+        };
+        const int S = ob.nspl;
+        __syncthreads();   // (the previous bin's table is dead)
+        // (two classes a thread: between splitters, and equal to the next one)
+        static_assert(OVER_SPL < 256, "a thread per splitter");
+        const int between = t <= S ? (int)tabs[e].cnt[2 * t] : 0, tie = t < S ? (int)tabs[e].cnt[2 * t + 1] : 0;
+        const int ex = ws_block_excl_scan<256, int>(between + tie, s.wsum, nullptr);
+        if (t <= S) {
+            s.start[2 * t] = (uint32_t)ex;
+            s.start[2 * t + 1] = (uint32_t)(ex + between);
+            if (tie > 0) s.tie[t] = pair_at((uint32_t)(ex + between));
+        }
+        if (t <= OVER_SPL) s.spl[t] = t < S ? tabs[e].spl[t] : ~(K)0;
+        __syncthreads();
+        const K* sk = sorted + ob.start;
+        const int o0 = (tile - ob.first_tile) * TILE, o1 = min((te - ob.first_tile) * TILE, ob.n);
+        for (int i0 = o0 + t; i0 < o1; i0 += 256 * U) {
+            K k[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) k[u] = __ldg(keys + ob.start + min(i0 + u * 256, o1 - 1));
+            int cl[U];
+            ws_over_classes<K, U>(s.spl, S, k, cl);
+            // (first position whose key is not below the element's; the searches go side by side)
+            uint32_t r[U], m[U], more = 0;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                r[u] = s.start[cl[u]];
+                m[u] = cl[u] & 1 ? 0u : s.start[cl[u] + 1] - r[u];
+                more |= m[u];
+            }
+            for (; more != 0; more >>= 1) {
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const uint32_t half = m[u] >> 1;
+                    const bool below = m[u] != 0 && sk[min(r[u] + half, (uint32_t)ob.n - 1u)] < k[u];
+                    if (below) r[u] += half + 1;
+                    m[u] = below ? m[u] - half - 1 : half;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (i0 + u * 256 < o1) pairs[ob.start + i0 + u * 256] = cl[u] & 1 ? s.tie[cl[u] >> 1] : pair_at(r[u]);
+        }
+        tile = te;
+    }
+}
 
 template <typename T>
 __global__ void __launch_bounds__(256, 6) k_bin_out(const LargeSeg* __restrict__ lsegs, const SegRuntime* __restrict__ rt,
@@ -888,7 +979,7 @@ __global__ void __launch_bounds__(256, 6) k_bin_out(const LargeSeg* __restrict__
                                                  const typename KeyOf<T>::K* __restrict__ sorted,
                                                  const typename KeyOf<T>::K* __restrict__ keys,
                                                  const SortCtl* __restrict__ ctl, const OverBin* __restrict__ over,
-                                                 OutPair<T>* pairs) {
+                                                 const OverTab<typename KeyOf<T>::K>* __restrict__ tabs, OutPair<T>* pairs) {
     typedef typename KeyOf<T>::K K;
     __shared__ uint2 rw[HTW + 2];
     extern __shared__ __align__(16) unsigned char pair_smem_raw[];
@@ -936,38 +1027,8 @@ __global__ void __launch_bounds__(256, 6) k_bin_out(const LargeSeg* __restrict__
     }
     const int cnt = (int)ctl->over_count;
     if (cnt == 0 || ctl->abort) return;
-    const int n_tiles = over[cnt - 1].first_tile + (over[cnt - 1].n + WS_SORT_TILE - 1) / WS_SORT_TILE;
-    for (int tile = (int)blockIdx.x - n_bins; tile < n_tiles; tile += OUT_EXTRA) {
-        int lo = 0, hi = cnt - 1;   // (uniform)
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (over[mid].first_tile <= tile) lo = mid; else hi = mid - 1;
-        }
-        const OverBin ob = over[lo];
-        const int lseg = ob.lseg;
-        const LargeSeg& sg = lsegs[lseg];
-        const int64_t c = rt[lseg].n_clusters;
-        if (c == 1) continue;
-        const uint2* sw = rank_words + (size_t)sg.hull_first * HTW;
-        const T* cv = cval + rt[lseg].table_pos;
-        const K* sk = sorted + ob.start;
-        const int e0 = (tile - ob.first_tile) * WS_SORT_TILE, e1 = min(e0 + WS_SORT_TILE, ob.n);
-        for (int i = e0 + t; i < e1; i += 256) {
-            const K k = keys[ob.start + i];
-            int r = 0, m = ob.n;   // first position whose key is not below k
-            if (ob.diff != 0)
-                while (m > 0) {
-                    const int half = m >> 1;
-                    if (sk[r + half] < k) { r += half + 1; m -= half + 1; } else m = half;
-                }
-            const uint32_t p = (uint32_t)(ob.start - sg.kpos) + (uint32_t)min(r, ob.n - 1);
-            const int id = ws_cluster_at(sw[p >> 5], p);
-            OutPair<T> o = {};
-            o.val = __ldg(cv + min(max((int64_t)id, (int64_t)0), c - 1));
-            o.id = id;
-            pairs[ob.start + i] = o;
-        }
-    }
+    bin_out_oversize<T>(*reinterpret_cast<OverOutSmem<T>*>(pair_smem_raw), (int)blockIdx.x - n_bins,
+                        (int)gridDim.x - n_bins, cnt, lsegs, rt, rank_words, cval, sorted, keys, over, tabs, pairs);
 }
 
 // A pass undone tile by tile: the tile's pairs are read run by run into shared
@@ -1126,12 +1187,13 @@ cudaError_t ws_large_prox(const LargeWork<T>& W, const T* values, WsLambda lambd
                               W.vp, VertX{W.vx, W.hx}, W.pieces, W.npieces, W.tile_piece, W.cval, W.rank_words, fp64, ep, status));
     // back to the caller's order
     const size_t osm = sizeof(OutPair<T>) * WS_BIN_CAP;
+    static_assert(sizeof(OverOutSmem<T>) <= sizeof(OutPair<T>) * WS_BIN_CAP, "in the same shared memory");
     e = cudaFuncSetAttribute(k_bin_out<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)osm);
     if (e) return e;
     WS_LAUNCH(W.prof, WSK_BIN_OUT, st,
-              ws_launch_chain(k_bin_out<T>, W.n_bins + OUT_EXTRA, 256, osm, st, W.lsegs, W.rt, W.bin_seg, W.bin_start,
+              ws_launch_chain(k_bin_out<T>, W.n_bins + W.sort_shape.out_extra, 256, osm, st, W.lsegs, W.rt, W.bin_seg, W.bin_start,
                               W.bin_cnt, W.n_bins, W.bin_idx, W.rank_words, W.cval, sorted, W.keys_b, W.ctl, W.over,
-                              W.pairs_b));
+                              reinterpret_cast<const OverTab<K>*>(W.over_tabs), W.pairs_b));
     const size_t gsm = sizeof(OutPair<T>) * WS_SORT_TILE;
     if ((e = cudaFuncSetAttribute(k_regroup<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm)) ||
         (e = cudaFuncSetAttribute(k_output<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm)))

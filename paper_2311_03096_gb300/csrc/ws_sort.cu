@@ -14,9 +14,9 @@
 //                 tile ranks its keys with one shared-memory atomic each and
 //                 reserves its runs with one global atomic per bucket;
 //   k_bin_sort    sorts every bin in one CTA;
-//   k_oversize    an LSD radix sort of the bins that do not fit one CTA (heavy
-//                 ties, or a distribution that the map does not resolve),
-//                 returns at once when there are none.
+//   k_oversize    sorts the bins that do not fit one CTA (heavy ties, or a
+//                 distribution that the map does not resolve), returns at once
+//                 when there are none.
 // The map only decides how even the bins are: it is monotone in the key by
 // construction, so the result is the sorted sequence for any input.
 //
@@ -557,6 +557,28 @@ struct PartSmem {
     int wsum[WS_SORT_NT / 32];
 };
 
+// Ranks of a warp's keys (w: bin << 13 per key, the rank goes below) where many are in
+// bucket `tie`: these are counted by votes, and added once.
+__device__ __noinline__ void part_rank_tied(uint32_t* w, uint32_t* cnt, uint32_t tie, int bsh, uint32_t off, int len) {
+    const int t = threadIdx.x, lane = t & 31;
+    uint32_t met = 0;
+#pragma unroll 1
+    for (int p = t; p < WS_SORT_TILE; p += WS_SORT_NT) {
+        const uint32_t x = w[p], b = (x >> bsh) - off;
+        const bool in = p < len && b < WS_FAN;
+        const unsigned m = __ballot_sync(WS_FULL_MASK, in && b == tie);
+        if (in)
+            w[p] = (x & ~0x1fffu) |
+                   (b == tie ? met + (uint32_t)__popc(m & ((1u << lane) - 1u)) : atomicAdd(&cnt[b], 1u));
+        met += (uint32_t)__popc(m);
+    }
+    uint32_t at = lane == 0 ? atomicAdd(&cnt[tie], met) : 0u;
+    at = __shfl_sync(WS_FULL_MASK, at, 0);
+#pragma unroll 1
+    for (int p = t; p < len; p += WS_SORT_NT)
+        if ((w[p] >> bsh) - off == tie) w[p] += at;
+}
+
 template <typename T, typename B, bool FIRST>
 __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
     const T* __restrict__ values, const typename KeyOf<T>::K* __restrict__ keys_in, const B* __restrict__ bins_in,
@@ -622,10 +644,29 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
             s.cnt[t] = 0;
             if (r0 == 0 && t < WS_SORT_TILE / 32) s.starts[t] = 0;
             __syncthreads();
+            // (a heavy tie's adds to its bucket would go one by one: in a warp whose first keys meet in a
+            // bucket its lanes are counted by votes, and added once.  2^26 weights: 99 % zeros 835 -> 600 us for
+            // both passes, one value 779 -> 546, N(0, 1) as before.  With few buckets every warp's keys meet, and
+            // the adds are as fast: 8192 segments of 4097 183 us, by votes 207)
+            uint32_t tie = 0xffffffffu;
+            if (nbk >= 8) {   // (uniform)
+                const uint32_t b = (br[0] >> bsh) - off;
+                const unsigned crowd = ws_crowd((int)b, t < len && b < WS_FAN);
+                if (crowd) tie = __shfl_sync(WS_FULL_MASK, b, __ffs((int)crowd) - 1);
+            }
+            if (tie == 0xffffffffu) {
 #pragma unroll
-            for (int k = 0; k < ITEMS; ++k) {
-                const uint32_t b = (br[k] >> bsh) - off;
-                if (t + k * NT < len && b < WS_FAN) br[k] = (br[k] & ~0x1fffu) | atomicAdd(&s.cnt[b], 1u);
+                for (int k = 0; k < ITEMS; ++k) {
+                    const uint32_t b = (br[k] >> bsh) - off;
+                    if (t + k * NT < len && b < WS_FAN) br[k] = (br[k] & ~0x1fffu) | atomicAdd(&s.cnt[b], 1u);
+                }
+            } else {   // (through the staging area: out of line, and the loop above keeps its registers)
+                uint32_t* w = reinterpret_cast<uint32_t*>(s.key);
+#pragma unroll
+                for (int k = 0; k < ITEMS; ++k) w[t + k * NT] = br[k];
+                part_rank_tied(w, s.cnt, tie, bsh, off, len);
+#pragma unroll
+                for (int k = 0; k < ITEMS; ++k) br[k] = w[t + k * NT];
             }
             __syncthreads();
             // start inside the tile, and the run's destination
@@ -770,19 +811,19 @@ __device__ __forceinline__ uint64_t warp_max_k(uint64_t v) {
 }
 
 // Sort of n keys or words by one warp: ranks by counting (ties by place).
-// More than BIN_WARP_MAX words are left alone if they are equal above the
-// place (then any order will do).  Keys of which few differ (weights that are
-// already shared) are written as runs.  false: more than BIN_WARP_MAX and
-// neither.
+// Words that are equal above the place are left alone (any order will do).
+// Keys of which few differ (weights that are already shared) are written as
+// runs.  false: more than BIN_WARP_MAX and neither.
 template <bool PLACE, typename K>
 __device__ __noinline__ bool sort_warp(K* key, int n) {
     const int lane = threadIdx.x & 31;
     constexpr int PER = BIN_WARP_MAX / 32;
-    if (PLACE && n > BIN_WARP_MAX) {
+    if (PLACE && n > 16) {
         const K k0 = key[0] >> 12;
         bool same = true;
         for (int j = lane; j < n; j += 32) same &= (key[j] >> 12) == k0;
-        return __all_sync(WS_FULL_MASK, same);
+        if (__all_sync(WS_FULL_MASK, same)) return true;
+        if (n > BIN_WARP_MAX) return false;
     }
     bool runs = false;
     if (!PLACE && n > 16) {   // (at most 8 different ones among the first 32)
@@ -831,7 +872,7 @@ __device__ __noinline__ bool sort_warp(K* key, int n) {
 #pragma unroll
         for (int k = 0; k < PER; ++k) {
             if (32 * k >= n) break;   // (uniform)
-            r[k] += (x < v[k] || (x == v[k] && j < lane + 32 * k)) ? 1 : 0;
+            r[k] += (x < v[k] || (!PLACE && x == v[k] && j < lane + 32 * k)) ? 1 : 0;   // (places: all words differ)
         }
     }
     __syncwarp();
@@ -842,15 +883,18 @@ __device__ __noinline__ bool sort_warp(K* key, int n) {
 }
 
 // LSD radix passes, 8-bit digits that vary (diff), over a bin's n keys in
-// s.key; with PLACE over the keys src[place], s.key holding the places.  The
-// rare path: out of line.
+// s.key; with PLACE over the words that are there already (words: they hold every
+// bit that varies), or else over the keys src[place], s.key holding the places.
+// The rare path: out of line.
 template <typename T, bool PLACE>
 __device__ __noinline__ void bin_radix(BinSmem<T>& s, const typename KeyOf<T>::K* src, int n,
-                                       typename KeyOf<T>::K diff) {
+                                       typename KeyOf<T>::K diff, bool words) {
     typedef typename KeyOf<T>::K K;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    for (int i = t; i < n; i += BIN_NT) s.key[i] = PLACE ? (K)i : src[i];
-    __syncthreads();
+    if (!words) {
+        for (int i = t; i < n; i += BIN_NT) s.key[i] = PLACE ? (K)i : src[i];
+        __syncthreads();
+    }
     for (int pass = 0; pass < KeyOf<T>::BITS / 8; ++pass) {
         if (((diff >> (8 * pass)) & 0xff) == 0) continue;
         K key[BIN_ITEMS];
@@ -862,7 +906,7 @@ __device__ __noinline__ void bin_radix(BinSmem<T>& s, const typename KeyOf<T>::K
             const int p = w * 32 * BIN_ITEMS + k * 32 + lane;
             valid[k] = p < n;
             key[k] = valid[k] ? s.key[p] : (K)0;
-            const K kk = PLACE ? (valid[k] ? __ldg(src + (uint32_t)key[k]) : (K)0) : key[k];
+            const K kk = PLACE && !words ? (valid[k] ? __ldg(src + (uint32_t)key[k]) : (K)0) : key[k];
             dg[k] = (uint32_t)((kk >> (8 * pass)) & 0xff);
         }
         __syncthreads();
@@ -886,6 +930,62 @@ __device__ __forceinline__ float ws_trunc_f32(double v) {
     return __uint_as_float(sign | ((uint32_t)e << 23) | m);
 }
 
+constexpr int OVER_SAMPLE = 1024;   // keys at most
+// Splitters of a bin, by one warp: quantiles of a sorted sample, each value once.
+// (A value of more than two gaps between them is among them, so a class between
+// splitters holds less than 3 / (quantiles + 1) of the bin, but for the sample's error.)
+// Enters the bin in the list; the counts of its classes are cleared.
+template <typename K>
+__device__ __noinline__ void over_sample(K* s, const K* __restrict__ src, int n, int64_t start, int lseg, SortCtl* ctl,
+                                         OverBin* over, OverTab<K>* tabs) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t entry = lane == 0 ? atomicAdd(&ctl->over_count, 1u) : 0u;   // (back with the sample)
+    int ns = 0;
+    OverTab<K>* tab = nullptr;
+    // a small sample for a bin that a few classes cut; a large one for a large bin of many different values
+    for (int m = n < 16384 ? 64 : 256;; m = OVER_SAMPLE) {
+#pragma unroll 4
+        for (int j = lane; j < m; j += 32) s[j] = __ldg(src + ((uint64_t)(2 * j + 1) * (uint64_t)n) / (uint32_t)(2 * m));
+        __syncwarp();
+        for (int k = 2; k <= m; k <<= 1)
+            for (int d = k >> 1; d > 0; d >>= 1) {
+#pragma unroll 4
+                for (int q = lane; q < m / 2; q += 32) {
+                    const int i = 2 * q - (q & (d - 1)), j = i + d;
+                    const K a = s[i], b = s[j];
+                    if ((a > b) == ((i & k) == 0)) { s[i] = b; s[j] = a; }
+                }
+                __syncwarp();
+            }
+        tab = tabs + __shfl_sync(WS_FULL_MASK, entry, 0);
+        // a splitter for every 256 keys (classes that one CTA sorts in a microsecond or two)
+        const int q = min(min(OVER_SPL, m - 1), n / 256);
+        ns = 0;
+        for (int c0 = 1; c0 <= q; c0 += 32) {
+            const int c = c0 + lane;
+            const bool in = c <= q;
+            const K v = s[in ? c * m / (q + 1) : 0];
+            const bool take = in && (c == 1 || v != s[(c - 1) * m / (q + 1)]);
+            const unsigned vote = __ballot_sync(WS_FULL_MASK, take);
+            if (take) tab->spl[ns + __popc(vote & ((1u << lane) - 1u))] = v;
+            ns += __popc(vote);
+        }
+        if (m == OVER_SAMPLE || n < (1 << 17) || ns < 64) break;   // (uniform)
+        __syncwarp();
+    }
+    for (int j = lane; j < 2 * ns + 1; j += 32) tab->cnt[j] = 0;
+    for (int j = lane; j < ns + 1; j += 32) tab->cur[j] = 0;
+    if (lane == 0) {
+        OverBin ob;
+        ob.start = start;
+        ob.n = n;
+        ob.first_tile = 0;
+        ob.lseg = lseg;
+        ob.nspl = ns;
+        over[entry] = ob;
+    }
+}
+
 template <typename T, bool PLACE>
 __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>::K* __restrict__ keys,
                                                         typename KeyOf<T>::K* __restrict__ sorted,
@@ -894,7 +994,8 @@ __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>:
                                                         const uint32_t* __restrict__ bin_start,
                                                         const uint32_t* __restrict__ bin_cnt,
                                                         uint16_t* __restrict__ bin_idx,   // (PLACE)
-                                                        SortCtl* ctl, OverBin* over, int64_t n_keys) {
+                                                        SortCtl* ctl, OverBin* over,
+                                                        OverTab<typename KeyOf<T>::K>* tabs, int64_t n_keys) {
     typedef KeyOf<T> KO;
     typedef typename KO::K K;
     extern __shared__ __align__(16) unsigned char bin_smem_raw[];
@@ -911,13 +1012,8 @@ __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>:
     const int n = (int)bin_cnt[bin];
     if (n <= 0) return;
     if (n > WS_BIN_CAP) {
-        if (t == 0) {
-            const uint32_t i = atomicAdd(&ctl->over_count, 1u);
-            over[i].start = start;
-            over[i].n = n;
-            over[i].diff = 0;
-            over[i].lseg = bin_seg[bin];
-        }
+        // to the oversize kernel, with the splitters that it needs (here they cost no time of their own)
+        if (t < 32) over_sample<K>(s.key, keys + start, n, start, bin_seg[bin], ctl, over, tabs);
         return;
     }
     const K* src = keys + start;
@@ -1033,9 +1129,21 @@ __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>:
             }
         }
         radix = __syncthreads_or(long_run) != 0;
+        if (radix) {
+            // (a long run of ties is in order as it is: one pass looks for a key below its neighbour)
+            bool inverted = false;
+            for (int i = t + 1; i < n; i += BIN_NT) {
+                const K a = s.key[i - 1], b = s.key[i];
+                if ((a >> 12) == (b >> 12))
+                    inverted |= __ldg(src + ((uint32_t)a & 0xfffu)) > __ldg(src + ((uint32_t)b & 0xfffu));
+            }
+            radix = __syncthreads_or(inverted) != 0;
+        }
     }
     if (radix) {   // (uniform; every word of the steps above has been read)
-        bin_radix<T, PLACE>(s, src, n, (K)(~(uint64_t)0 >> (64 - range_bits)) | (lo ^ hi));
+        const K vary = (K)(~(uint64_t)0 >> (64 - range_bits));
+        if (PLACE && cut == 0) bin_radix<T, PLACE>(s, src, n, (K)(vary << 12), true);
+        else bin_radix<T, PLACE>(s, src, n, vary | (lo ^ hi), false);
     }
     K* dst = sorted + start;
 #pragma unroll 4
@@ -1052,59 +1160,260 @@ __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>:
 }
 
 // ---------------------------------------------------------------------------
-// Oversize bins: LSD radix passes over the digits that vary, all bins side by
-// side, as a cooperative grid with a barrier between the steps.  A bin's keys
-// stay in keys_b (the way back needs them); its passes alternate between
-// keys_a and a scratch buffer so that the last one writes keys_a (a bin of
-// equal keys is copied there).
+// Oversize bins, as a cooperative grid with a barrier between the steps.  Such a
+// bin is a heavy tie as a rule (zeros, weights that are already shared) with a few
+// neighbours, sometimes a spike that the map does not resolve.  The splitters that
+// k_bin_sort took from a sample of it cut its keys into the classes "equal to
+// splitter i" and "between splitters".  The ties are written as runs (they need
+// neither moving nor sorting); what lies between goes to a class's region of a
+// scratch buffer, which one CTA sorts.  A class between splitters that is still
+// above WS_BIN_CAP takes LSD radix passes over the digits that vary.  The bin's
+// keys stay in keys_b and its classes in `tabs` (the way back finds a key's place
+// by its class).  Bound by latency (two barriers and two reads of the keys: 20 us)
+// up to about 2^22 keys, by the reads above.  Against LSD passes over whole bins
+// and a bisection of every element in its bin by 64 CTAs, FP32 ws_prox, lambda
+// 1e-2, us (the radix sort with a lookup by value before both):
+//   2^26   50 % zeros 10240 (18890; 10900), 99 % 3670 (21620; 4010), 7 values 3280
+//          (4700; 3720), 1000 values 3680 (6170; 3930), one value 1350 (2200; 2160)
+//   2^24   50 % zeros 5500 (7410; 5590), 99 % 1170 (5170; 1260), 7 values 900 (1230; 1030)
+//   2^20   1 % zeros 334 (394; 374), 50 % 300 (508; 369), 99 % 246 (596; 297)
+// (the rest of such a call is the tree of merges around the huge cluster).  Spikes
+// of a million different FP64 values that lie within 2^-30 of each other stay slower
+// than under the radix sort (2^24: 5600; 1620): their classes take its passes, and
+// a bisection for every element of the way back.
 // ---------------------------------------------------------------------------
+template <typename T>
 struct OverSmem {
-    uint32_t whist[(OVER_NT / 32) * 256];
-    uint32_t dcount[256], dstart[256], base[256];
+    typedef typename KeyOf<T>::K K;
+    union {
+        struct {                               // counting and placing: the table of the current bin
+            K spl[OVER_SPL + 1];
+            uint32_t start[2 * OVER_SPL + 2];  // start of every class in the bin
+            uint32_t cnt[2 * OVER_SPL + 1];
+            uint32_t place[OVER_SPL + 1];
+        } split;
+        struct {
+            K key[WS_BIN_CAP];
+            uint32_t whist[(OVER_NT / 32) * 256];
+            uint32_t dcount[256], dstart[256], base[256];
+        } sort;
+    } u;
+    int first[OVER_NT];   // first tile of every bin of a short list
     int wsum[OVER_NT / 32];
     int carry;
     int ent;
     unsigned long long diff;
 };
 
+// Sort of a class between splitters by the CTA, n <= WS_BIN_CAP keys: a bitonic
+// network in shared memory (1280 keys 3 us; LSD passes over their four digits took 15).
 template <typename T>
-__global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* ka,
+__device__ __noinline__ void over_sort_class(OverSmem<T>& s, const typename KeyOf<T>::K* src,
+                                             typename KeyOf<T>::K* dst, int n) {
+    typedef typename KeyOf<T>::K K;
+    constexpr int NT = OVER_NT;
+    const int t = threadIdx.x;
+    K* key = s.u.sort.key;
+    int m = 64;
+    while (m < n) m <<= 1;
+    __syncthreads();   // (the previous use of the shared memory is over)
+    for (int i = t; i < m; i += NT) key[i] = i < n ? __ldcg(src + i) : ~(K)0;
+    for (int k = 2; k <= m; k <<= 1)
+        for (int d = k >> 1; d > 0; d >>= 1) {
+            // (a warp's 32 pairs lie in one run of 64 keys while d < 64: only the steps across such runs, and the
+            // first one after them, need the CTA)
+            if (d >= 32 || k == 2) __syncthreads(); else __syncwarp();
+            for (int q = t; q < m / 2; q += NT) {
+                const int i = 2 * q - (q & (d - 1)), j = i + d;
+                const K a = key[i], b = key[j];
+                if ((a > b) == ((i & k) == 0)) { key[i] = b; key[j] = a; }
+            }
+        }
+    __syncthreads();
+    for (int i = t; i < n; i += NT) dst[i] = key[i];
+}
+
+template <typename T>
+__global__ void __launch_bounds__(OVER_NT, 2) k_oversize(typename KeyOf<T>::K* ka,
                                                          const typename KeyOf<T>::K* __restrict__ kb,
-                                                         typename KeyOf<T>::K* kt, SortCtl* ctl, OverBin* over, uint32_t* over_cnt,
+                                                         typename KeyOf<T>::K* kt, int64_t n_keys, SortCtl* ctl,
+                                                         OverBin* over, OverTab<typename KeyOf<T>::K>* tabs,
+                                                         OverClass* items, OverClass* big, uint32_t* over_cnt,
                                                          uint64_t spin_limit, uint32_t* status) {
     typedef KeyOf<T> KO;
     typedef typename KO::K K;
     constexpr int NT = OVER_NT, ITEMS = WS_SORT_ITEMS, TILE = WS_SORT_TILE, P = KO::BITS / 8;
-    __shared__ OverSmem s;
+    extern __shared__ __align__(16) unsigned char over_smem_raw[];
+    OverSmem<T>& s = *reinterpret_cast<OverSmem<T>*>(over_smem_raw);
     const int cnt = (int)ctl->over_count;
     if (cnt == 0 || ctl->abort) return;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     GridBarrier bar{&ctl->over_bar, &ctl->abort, status, spin_limit, 0u, false};
-    // tiles of the bins, in list order
-    if (blockIdx.x == 0) {
+    // tiles of the bins, in list order: a short list is numbered by every CTA for itself
+    // (the first one writes the numbers down), a long one by one CTA
+    auto number_tiles = [&](auto* list, int m) {
         if (t == 0) s.carry = 0;
         __syncthreads();
-        for (int e0 = 0; e0 < cnt; e0 += NT) {
+        for (int e0 = 0; e0 < m; e0 += NT) {
             const int e = e0 + t;
-            const int nt = e < cnt ? (over[e].n + TILE - 1) / TILE : 0;
+            const int nt = e < m ? (__ldcg(&list[e].n) + TILE - 1) / TILE : 0;
             int tot;
             const int ex = ws_block_excl_scan<NT, int>(nt, s.wsum, &tot);
-            if (e < cnt) __stcg(&over[e].first_tile, s.carry + ex);
+            if (m <= NT) s.first[t] = ex;
+            if (e < m && blockIdx.x == 0) __stcg(&list[e].first_tile, s.carry + ex);
             __syncthreads();
             if (t == 0) s.carry += tot;
             __syncthreads();
         }
+        return s.carry;
+    };
+    int n_tiles = 0;
+    const bool listed = cnt <= NT;
+    if (listed) n_tiles = number_tiles(over, cnt);
+    else {
+        if (blockIdx.x == 0) number_tiles(over, cnt);
+        if (!bar.sync()) return;
+        n_tiles = __ldcg(&over[cnt - 1].first_tile) + (__ldcg(&over[cnt - 1].n) + TILE - 1) / TILE;
+    }
+    auto first_of = [&](int e) -> int { return listed ? s.first[e] : __ldcg(&over[e].first_tile); };
+    // this CTA's tiles, contiguous: a table serves all tiles of its bin
+    const int t0 = (int)((int64_t)n_tiles * blockIdx.x / gridDim.x);
+    const int t1 = (int)((int64_t)n_tiles * (blockIdx.x + 1) / gridDim.x);
+    auto first_entry = [&]() -> int {   // bin of tile t0
+        int lo = 0, hi = cnt - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (first_of(mid) <= t0) lo = mid; else hi = mid - 1;
+        }
+        return lo;
+    };
+    const int e_first = t0 < t1 ? first_entry() : cnt;
+    // 1. keys per class.  The counts of a bin's tiles are added up in shared memory.
+    {
+        int tile = t0;
+        for (int e = e_first; tile < t1; ++e) {
+            const int64_t st = over[e].start;
+            const int ne = over[e].n, f = first_of(e), S = over[e].nspl;
+            const K spl = t < OVER_SPL ? __ldcg(&tabs[e].spl[t]) : (K)0;   // (beyond S: not used)
+            const int te = min(t1, f + (ne + TILE - 1) / TILE);
+            __syncthreads();
+            for (int j = t; j < 2 * OVER_SPL + 1; j += NT) s.u.split.cnt[j] = 0;
+            if (t <= OVER_SPL) s.u.split.spl[t] = t < S ? spl : ~(K)0;
+            __syncthreads();
+            for (; tile < te; ++tile) {
+                const int o0 = (tile - f) * TILE, n = min(TILE, ne - o0);
+                K key[ITEMS];
+#pragma unroll
+                for (int k = 0; k < ITEMS; ++k) key[k] = t + k * NT < n ? __ldg(kb + st + o0 + t + k * NT) : (K)0;
+                int cls[ITEMS];
+                ws_over_classes<K, ITEMS>(s.u.split.spl, S, key, cls);
+#pragma unroll
+                for (int k = 0; k < ITEMS; ++k) {
+                    if (k * NT >= n) break;   // (uniform)
+                    const bool in = t + k * NT < n;
+                    const unsigned crowd = ws_crowd(cls[k], in);
+                    if ((crowd >> lane) & 1u) {
+                        if (lane == __ffs((int)crowd) - 1) atomicAdd(&s.u.split.cnt[cls[k]], (uint32_t)__popc(crowd));
+                    } else if (in) {
+                        atomicAdd(&s.u.split.cnt[cls[k]], 1u);
+                    }
+                }
+            }
+            __syncthreads();
+            for (int j = t; j < 2 * S + 1; j += NT)
+                if (s.u.split.cnt[j]) atomicAdd(&tabs[e].cnt[j], s.u.split.cnt[j]);
+        }
     }
     if (!bar.sync()) return;
-    const int n_tiles = __ldcg(&over[cnt - 1].first_tile) + (over[cnt - 1].n + TILE - 1) / TILE;
+    // 2. the runs of ties, and the keys between splitters into the regions of their classes
+    {
+        int tile = t0;
+        for (int e = e_first; tile < t1; ++e) {
+            const int64_t st = over[e].start;
+            const int ne = over[e].n, f = first_of(e), S = over[e].nspl;
+            const K spl = t < OVER_SPL ? __ldcg(&tabs[e].spl[t]) : (K)0;   // (beyond S: not used)
+            const int te = min(t1, f + (ne + TILE - 1) / TILE);
+            __syncthreads();
+            if (t <= OVER_SPL) s.u.split.spl[t] = t < S ? spl : ~(K)0;
+            {
+                static_assert(2 * OVER_SPL + 2 <= OVER_NT && OVER_SPL < WS_BIN_CAP / 4, "a thread per class; the sample fits");
+                const int all = t < 2 * OVER_SPL + 1 ? (int)__ldcg(&tabs[e].cnt[t]) : 0, c = t < 2 * S + 1 ? all : 0;
+                const int ex = ws_block_excl_scan<NT, int>(c, s.wsum, nullptr);
+                if (t < 2 * S + 2) s.u.split.start[t] = (uint32_t)ex;
+                // (the bin's first tile lists the classes to sort)
+                if (tile == f && (t & 1) == 0 && c > 1) {
+                    OverClass oc = {};
+                    oc.start = st + ex;
+                    oc.n = c;
+                    if (c <= WS_BIN_CAP) items[atomicAdd(&ctl->over_items, 1u)] = oc;
+                    else big[atomicAdd(&ctl->over_big, 1u)] = oc;
+                }
+            }
+            __syncthreads();
+            for (; tile < te; ++tile) {
+                const int o0 = (tile - f) * TILE, n = min(TILE, ne - o0);
+                K key[ITEMS];
+                int cls[ITEMS];
+                uint32_t cr[ITEMS];   // class between splitters << 16 | rank among the tile's
+#pragma unroll
+                for (int k = 0; k < ITEMS; ++k) key[k] = t + k * NT < n ? __ldg(kb + st + o0 + t + k * NT) : (K)0;
+                if (t <= OVER_SPL) s.u.split.cnt[t] = 0;
+                __syncthreads();
+                ws_over_classes<K, ITEMS>(s.u.split.spl, S, key, cls);
+                bool any = false;
+#pragma unroll
+                for (int k = 0; k < ITEMS; ++k) {
+                    cr[k] = 0xffffffffu;
+                    if (t + k * NT < n && (cls[k] & 1) == 0) {
+                        cr[k] = ((uint32_t)cls[k] << 15) | atomicAdd(&s.u.split.cnt[cls[k] >> 1], 1u);
+                        any = true;
+                    }
+                }
+                if (__syncthreads_or(any)) {
+                    if (t <= S) {
+                        const uint32_t c = s.u.split.cnt[t];
+                        if (c) s.u.split.place[t] = s.u.split.start[2 * t] + atomicAdd(&tabs[e].cur[t], c);
+                    }
+                    __syncthreads();
+#pragma unroll
+                    for (int k = 0; k < ITEMS; ++k)
+                        if (cr[k] != 0xffffffffu) {
+                            const uint32_t c = cr[k] >> 16, p = s.u.split.place[c] + (cr[k] & 0xffffu);
+                            // (a class of one key needs no sorting)
+                            K* to = s.u.split.start[2 * c + 1] - s.u.split.start[2 * c] == 1u ? ka : kt;
+                            if (p < (uint32_t)ne) to[st + p] = key[k];
+                        }
+                }
+                for (int j = 0; j < S; ++j) {
+                    const int a = max((int)s.u.split.start[2 * j + 1], o0), b = min((int)s.u.split.start[2 * j + 2], o0 + n);
+                    const K v = s.u.split.spl[j];
+                    for (int i = a + t; i < b; i += NT) ka[st + i] = v;
+                }
+                __syncthreads();
+            }
+        }
+    }
+    if (!bar.sync()) return;
+    // 3. the classes between splitters
+    const int n_items = (int)__ldcg(&ctl->over_items);
+    for (int i = blockIdx.x; i < n_items; i += gridDim.x)
+        over_sort_class<T>(s, kt + __ldcg(&items[i].start), ka + __ldcg(&items[i].start), __ldcg(&items[i].n));
+    const int n_big = (int)__ldcg(&ctl->over_big);
+    if (n_big == 0) return;   // (uniform over the grid)
+    // 4. those above WS_BIN_CAP: LSD radix passes, which alternate between keys_a and a second
+    // scratch buffer so that the last one writes keys_a
+    K* kt2 = kt + n_keys;
+    if (blockIdx.x == 0) number_tiles(big, n_big);
+    if (!bar.sync()) return;
+    const int b_tiles = __ldcg(&big[n_big - 1].first_tile) + (__ldcg(&big[n_big - 1].n) + TILE - 1) / TILE;
     // entry of a tile (all threads; ends synchronised)
     auto entry = [&](int tile) -> int {
         __syncthreads();
         if (t == 0) {
-            int lo = 0, hi = cnt - 1;
+            int lo = 0, hi = n_big - 1;
             while (lo < hi) {
                 const int mid = (lo + hi + 1) >> 1;
-                if (__ldcg(&over[mid].first_tile) <= tile) lo = mid; else hi = mid - 1;
+                if (__ldcg(&big[mid].first_tile) <= tile) lo = mid; else hi = mid - 1;
             }
             s.ent = lo;
             s.diff = 0;
@@ -1118,22 +1427,22 @@ __global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* k
         return c;
     };
     // where pass i of m writes, and where it reads
-    auto out_of = [&](int i, int m) -> K* { return ((m - 1 - i) & 1) ? kt : ka; };
-    auto in_of = [&](int i, int m) -> const K* { return i == 0 ? kb : out_of(i - 1, m); };
+    auto out_of = [&](int i, int m) -> K* { return ((m - 1 - i) & 1) ? kt2 : ka; };
+    auto in_of = [&](int i, int m) -> const K* { return i == 0 ? kt : out_of(i - 1, m); };
     // bits that vary
-    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    for (int tile = blockIdx.x; tile < b_tiles; tile += gridDim.x) {
         const int e = entry(tile);
-        const int64_t st = over[e].start;
-        const int o0 = (tile - __ldcg(&over[e].first_tile)) * TILE, n = min(TILE, over[e].n - o0);
-        const K k0 = kb[st];
+        const int64_t st = __ldcg(&big[e].start);
+        const int o0 = (tile - __ldcg(&big[e].first_tile)) * TILE, n = min(TILE, __ldcg(&big[e].n) - o0);
+        const K k0 = __ldcg(kt + st);
         K d = 0;
-        for (int i = t; i < n; i += NT) d |= kb[st + o0 + i] ^ k0;
+        for (int i = t; i < n; i += NT) d |= __ldcg(kt + st + o0 + i) ^ k0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) d |= ws_shfl_xor_k(d, o);
         if (lane == 0 && d) atomicOr(&s.diff, (unsigned long long)d);
         __syncthreads();
         if (t == 0 && s.diff) {
-            atomicOr(&over[e].diff, s.diff);
+            atomicOr(&big[e].diff, s.diff);
             atomicOr(&ctl->over_diff, s.diff);
         }
     }
@@ -1142,25 +1451,26 @@ __global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* k
     for (int p = 0; p < P; ++p) {
         if (((all >> (8 * p)) & 0xffull) == 0) continue;   // (uniform over the grid)
         // digit counts of every tile
-        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        for (int tile = blockIdx.x; tile < b_tiles; tile += gridDim.x) {
             const int e = entry(tile);
-            const unsigned long long diff = __ldcg(&over[e].diff);
+            const unsigned long long diff = __ldcg(&big[e].diff);
             if (((diff >> (8 * p)) & 0xffull) == 0) continue;
-            const K* src = in_of(passes_before(diff, p), passes_before(diff, P)) + over[e].start;
-            const int o0 = (tile - __ldcg(&over[e].first_tile)) * TILE, n = min(TILE, over[e].n - o0);
-            if (t < 256) s.dcount[t] = 0;
+            const K* src = in_of(passes_before(diff, p), passes_before(diff, P)) + __ldcg(&big[e].start);
+            const int o0 = (tile - __ldcg(&big[e].first_tile)) * TILE, n = min(TILE, __ldcg(&big[e].n) - o0);
+            uint32_t* dcount = s.u.sort.dcount;
+            if (t < 256) dcount[t] = 0;
             __syncthreads();
-            for (int i = t; i < n; i += NT) atomicAdd(&s.dcount[(int)((__ldcg(src + o0 + i) >> (8 * p)) & 0xff)], 1u);
+            for (int i = t; i < n; i += NT) atomicAdd(&dcount[(int)((__ldcg(src + o0 + i) >> (8 * p)) & 0xff)], 1u);
             __syncthreads();
-            if (t < 256) __stcg(over_cnt + (size_t)tile * 256 + t, s.dcount[t]);
+            if (t < 256) __stcg(over_cnt + (size_t)tile * 256 + t, dcount[t]);
         }
         if (!bar.sync()) return;
-        // counts -> first position of every (tile, digit), one CTA per bin
-        for (int e = blockIdx.x; e < cnt; e += gridDim.x) {
-            const unsigned long long diff = __ldcg(&over[e].diff);
+        // counts -> first position of every (tile, digit), one CTA per class
+        for (int e = blockIdx.x; e < n_big; e += gridDim.x) {
+            const unsigned long long diff = __ldcg(&big[e].diff);
             if (((diff >> (8 * p)) & 0xffull) == 0) continue;
-            uint32_t* c = over_cnt + (size_t)__ldcg(&over[e].first_tile) * 256;
-            const int nt = (over[e].n + TILE - 1) / TILE;
+            uint32_t* c = over_cnt + (size_t)__ldcg(&big[e].first_tile) * 256;
+            const int nt = (__ldcg(&big[e].n) + TILE - 1) / TILE;
             __syncthreads();
             uint32_t run = 0;
             if (t < 256) {
@@ -1184,15 +1494,16 @@ __global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* k
         }
         if (!bar.sync()) return;
         // stable scatter
-        for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        for (int tile = blockIdx.x; tile < b_tiles; tile += gridDim.x) {
             const int e = entry(tile);
-            const unsigned long long diff = __ldcg(&over[e].diff);
+            const unsigned long long diff = __ldcg(&big[e].diff);
             if (((diff >> (8 * p)) & 0xffull) == 0) continue;
             const int i = passes_before(diff, p), m = passes_before(diff, P);
-            const K* src = in_of(i, m) + over[e].start;
-            K* dst = out_of(i, m) + over[e].start;
-            const int ne = over[e].n;
-            const int o0 = (tile - __ldcg(&over[e].first_tile)) * TILE, n = min(TILE, ne - o0);
+            const int64_t st = __ldcg(&big[e].start);
+            const K* src = in_of(i, m) + st;
+            K* dst = out_of(i, m) + st;
+            const int ne = __ldcg(&big[e].n);
+            const int o0 = (tile - __ldcg(&big[e].first_tile)) * TILE, n = min(TILE, ne - o0);
             K key[ITEMS];
             uint32_t dg[ITEMS];
             bool valid[ITEMS];
@@ -1204,24 +1515,25 @@ __global__ void __launch_bounds__(OVER_NT, 1) k_oversize(typename KeyOf<T>::K* k
                 key[k] = valid[k] ? __ldcg(src + o0 + q) : (K)0;
                 dg[k] = (uint32_t)((key[k] >> (8 * p)) & 0xff);
             }
-            if (t < 256) s.base[t] = __ldcg(over_cnt + (size_t)tile * 256 + t);
-            ws_rank_digits<NT, ITEMS, 1>(dg, valid, pos, s.whist, s.dcount, s.dstart);
+            uint32_t* base = s.u.sort.base;
+            if (t < 256) base[t] = __ldcg(over_cnt + (size_t)tile * 256 + t);
+            ws_rank_digits<NT, ITEMS, 1>(dg, valid, pos, s.u.sort.whist, s.u.sort.dcount, s.u.sort.dstart);
 #pragma unroll
             for (int k = 0; k < ITEMS; ++k)
                 if (valid[k]) {
-                    const uint32_t q = s.base[dg[k]] + (uint32_t)pos[k] - s.dstart[dg[k]];
+                    const uint32_t q = base[dg[k]] + (uint32_t)pos[k] - s.u.sort.dstart[dg[k]];
                     if (q < (uint32_t)ne) dst[q] = key[k];
                 }
         }
         if (!bar.sync()) return;
     }
-    // bins of equal keys
-    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    // classes of equal keys
+    for (int tile = blockIdx.x; tile < b_tiles; tile += gridDim.x) {
         const int e = entry(tile);
-        if (__ldcg(&over[e].diff) != 0) continue;
-        const int64_t st = over[e].start;
-        const int o0 = (tile - __ldcg(&over[e].first_tile)) * TILE, n = min(TILE, over[e].n - o0);
-        for (int i = t; i < n; i += NT) ka[st + o0 + i] = kb[st + o0 + i];
+        if (__ldcg(&big[e].diff) != 0) continue;
+        const int64_t st = __ldcg(&big[e].start);
+        const int o0 = (tile - __ldcg(&big[e].first_tile)) * TILE, n = min(TILE, __ldcg(&big[e].n) - o0);
+        for (int i = t; i < n; i += NT) ka[st + o0 + i] = __ldcg(kt + st + o0 + i);
     }
 }
 
@@ -1247,6 +1559,7 @@ static cudaError_t sort_prepare(int max_bins, int n_tiles, WsSortShape* sh) {
     auto *kb0 = k_bin_sort<T, false>, *kb1 = k_bin_sort<T, true>;
     if (!e) e = cudaFuncSetAttribute(kb0, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BinSmem<T>));
     if (!e) e = cudaFuncSetAttribute(kb1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BinSmem<T>));
+    if (!e) e = cudaFuncSetAttribute(ko, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(OverSmem<T>));
     if (e) return e;
     int dev = 0, sms = 0, np = 0, n1 = 0, no = 0;
     if ((e = cudaGetDevice(&dev))) return e;
@@ -1260,9 +1573,10 @@ static cudaError_t sort_prepare(int max_bins, int n_tiles, WsSortShape* sh) {
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&np, kp, PLAN_NT, plan_smem(sh->hist_cap)))) return e;
     if (np < 1) return cudaErrorInvalidConfiguration;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, k1, WS_SORT_NT, ksm))) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&no, ko, OVER_NT, 0))) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&no, ko, OVER_NT, sizeof(OverSmem<T>)))) return e;
     sh->part_grid = std::max(1, sms * n1);
     sh->over_grid = std::max(1, sms * no);
+    sh->out_extra = std::min(8 * sms, 2 * n_tiles);
     return cudaSuccess;
 }
 
@@ -1315,15 +1629,19 @@ static cudaError_t sort_run(const LargeWork<T>& W, const T* values, bool way_bac
     WS_LAUNCH(W.prof, WSK_BIN_SORT, st,
               ws_launch_chain(way_back ? k_bin_sort<T, true> : k_bin_sort<T, false>, W.n_bins, BIN_NT,
                               sizeof(BinSmem<T>), st, W.keys_b, W.keys_a, W.bin_seg, W.lsegs, W.bin_start, W.bin_cnt,
-                              W.bin_idx, W.ctl, W.over, W.n_keys));
+                              W.bin_idx, W.ctl, W.over, reinterpret_cast<OverTab<K>*>(W.over_tabs), W.n_keys));
     {
         K* ka = W.keys_a;
         K* kb = W.keys_b;
-        K* kt = reinterpret_cast<K*>(W.pairs_b);
-        void* args[] = {&ka, &kb, &kt, (void*)&W.ctl, (void*)&W.over, (void*)&W.over_cnt, &spin_limit, &status};
+        K* kt = reinterpret_cast<K*>(W.pairs_b);   // (two buffers of n_keys: a pair takes at least two keys)
+        static_assert(sizeof(OutPair<T>) >= 2 * sizeof(K), "the scratch fits");
+        OverTab<K>* tabs = reinterpret_cast<OverTab<K>*>(W.over_tabs);
+        void* args[] = {&ka, &kb, &kt, (void*)&W.n_keys, (void*)&W.ctl, (void*)&W.over, &tabs, (void*)&W.over_items,
+                        (void*)&W.over_big, (void*)&W.over_cnt, &spin_limit, &status};
         WS_LAUNCH(W.prof, WSK_OVERSIZE, st,
                   e = cudaLaunchCooperativeKernel((const void*)k_oversize<T>,
-                                                  dim3(std::min(sh.over_grid, W.n_sort_tiles)), dim3(OVER_NT), args, 0,
+                                                  dim3(std::min(sh.over_grid, W.n_sort_tiles)), dim3(OVER_NT), args,
+                                                  sizeof(OverSmem<T>),
                                                   st));
         if (e) return e;
     }

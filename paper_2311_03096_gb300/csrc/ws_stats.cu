@@ -30,6 +30,7 @@ __global__ void __launch_bounds__(256) k_R_tiles(const typename KeyOf<T>::K* __r
     typedef KeyOf<T> KO;
     typedef typename KO::K K;
     __shared__ i128 ws128[8];
+    ws_chain();
     const TileDesc td = tiles[blockIdx.x];
     const LargeSeg ls = lsegs[td.lseg];
     const K* seg = sorted + ls.kpos;
@@ -92,6 +93,7 @@ __global__ void __launch_bounds__(256) k_R_final(const LargeSeg* __restrict__ ls
                                                 double* R_out, double* metric_out, uint32_t* status) {
     typedef KeyOf<T> KO;
     __shared__ RPartial wp[8];
+    ws_chain();
     const LargeSeg ls = lsegs[blockIdx.x];
     i128 s = 0;
     long long dis = 0, nz = 0;
@@ -130,10 +132,10 @@ cudaError_t ws_large_R(const LargeWork<T>& W, const T* values, double* R_out, do
     if (e) return e;
     RPartial* part = reinterpret_cast<RPartial*>(partial);
     WS_LAUNCH(W.prof, WSK_MISC, st,
-              (k_R_tiles<T><<<W.n_sort_tiles, 256, 0, st>>>(sorted, W.sort_tiles, W.lsegs, W.seg_emin, part)));
+              ws_launch_chain(k_R_tiles<T>, W.n_sort_tiles, 256, 0, st, sorted, W.sort_tiles, W.lsegs, W.seg_emin, part));
     WS_LAUNCH(W.prof, WSK_MISC, st,
-              (k_R_final<T><<<W.n_lseg, 256, 0, st>>>(W.lsegs, W.sort_tiles, sorted, W.seg_emin, part, R_out,
-                                                     metric_out, status)));
+              ws_launch_chain(k_R_final<T>, W.n_lseg, 256, 0, st, W.lsegs, W.sort_tiles, sorted, W.seg_emin, part, R_out,
+                              metric_out, status));
     return cudaGetLastError();
 }
 
