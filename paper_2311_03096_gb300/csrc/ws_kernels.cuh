@@ -168,14 +168,14 @@ struct VertX {
     __device__ __forceinline__ i128 at(const TileX& t, int64_t tile, int v, int p) const {
         const i128* b = x + tile * (WS_HULL_TILE + 1);
         if (t.wide) return b[v];
-        return ws_mul_i64(p, t.q0) + ws_shl_i64(reinterpret_cast<const int64_t*>(b)[v], t.sh);
+        return (i128)p * (i128)t.q0 + ((i128)reinterpret_cast<const int64_t*>(b)[v] << t.sh);
     }
     // at(tile, v + 1, p + n) - at(tile, v, p), with the tile's TileX at hand
     __device__ __forceinline__ i128 step(const TileX& t, int64_t tile, int v, int n) const {
         const i128* b = x + tile * (WS_HULL_TILE + 1);
         if (t.wide) return b[v + 1] - b[v];
         const int64_t* q = reinterpret_cast<const int64_t*>(b) + v;
-        return ws_mul_i64(n, t.q0) + ws_shl_i64(q[1] - q[0], t.sh);
+        return (i128)t.q0 * (int64_t)n + ((i128)(q[1] - q[0]) << t.sh);
     }
 };
 

@@ -555,6 +555,7 @@ struct PartSmem {
     uint2 run[WS_FAN];        // start of the bucket's run inside the tile, and its destination
     uint32_t starts[WS_SORT_TILE / 32];   // a bit at the first place of every run
     int wsum[WS_SORT_NT / 32];
+    int tie;                              // bucket of a heavy tie in the tile before, or -1
 };
 
 // Ranks of a warp's keys (w: bin << 13 per key, the rank goes below) where many are in
@@ -618,6 +619,7 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
     int tile = next_tile(blockIdx.x);
     if (tile >= n_tiles) return;
     load(tiles[tile]);
+    if (t == 0) s.tie = -1;
     while (tile < n_tiles) {
         const int nxt = next_tile(tile + gridDim.x);
         const int len = tiles[tile].len;
@@ -643,18 +645,14 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
             __syncthreads();   // (the previous use of the shared memory is over)
             s.cnt[t] = 0;
             if (r0 == 0 && t < WS_SORT_TILE / 32) s.starts[t] = 0;
+            // A heavy tie's adds to its bucket would go one by one: where a bucket took a third of the tile
+            // before, a warp counts its keys for that bucket by votes and adds them once.  2^26 weights: 99 %
+            // zeros 835 -> 600 us for both passes, one value 779 -> 546.  With few buckets the adds are as
+            // fast: 8192 segments of 4097 183 us, by votes 207.
+            const int tie = nbk >= 8 ? s.tie : -1;
             __syncthreads();
-            // (a heavy tie's adds to its bucket would go one by one: in a warp whose first keys meet in a
-            // bucket its lanes are counted by votes, and added once.  2^26 weights: 99 % zeros 835 -> 600 us for
-            // both passes, one value 779 -> 546, N(0, 1) as before.  With few buckets every warp's keys meet, and
-            // the adds are as fast: 8192 segments of 4097 183 us, by votes 207)
-            uint32_t tie = 0xffffffffu;
-            if (nbk >= 8) {   // (uniform)
-                const uint32_t b = (br[0] >> bsh) - off;
-                const unsigned crowd = ws_crowd((int)b, t < len && b < WS_FAN);
-                if (crowd) tie = __shfl_sync(WS_FULL_MASK, b, __ffs((int)crowd) - 1);
-            }
-            if (tie == 0xffffffffu) {
+            if (t == 0) s.tie = -1;
+            if (tie < 0) {
 #pragma unroll
                 for (int k = 0; k < ITEMS; ++k) {
                     const uint32_t b = (br[k] >> bsh) - off;
@@ -664,13 +662,14 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
                 uint32_t* w = reinterpret_cast<uint32_t*>(s.key);
 #pragma unroll
                 for (int k = 0; k < ITEMS; ++k) w[t + k * NT] = br[k];
-                part_rank_tied(w, s.cnt, tie, bsh, off, len);
+                part_rank_tied(w, s.cnt, (uint32_t)tie, bsh, off, len);
 #pragma unroll
                 for (int k = 0; k < ITEMS; ++k) br[k] = w[t + k * NT];
             }
             __syncthreads();
             // start inside the tile, and the run's destination
             const uint32_t c = s.cnt[t];
+            if (c > WS_SORT_TILE / 3) atomicMax(&s.tie, t);
             const uint32_t g =
                 c ? atomicAdd(cursor + (FIRST ? sg.coarse_pos : sg.bin_pos + base) + r0 + t, c) : 0u;
             // (places in the low half, runs in the high one)
@@ -821,8 +820,8 @@ __device__ __noinline__ bool sort_warp(K* key, int n) {
     if (PLACE && n > 16) {
         const K k0 = key[0] >> 12;
         bool same = true;
-        for (int j = lane; j < n; j += 32) same &= (key[j] >> 12) == k0;
-        if (__all_sync(WS_FULL_MASK, same)) return true;
+        for (int j = lane; same && j - lane < n; j += 32) same = __all_sync(WS_FULL_MASK, j >= n || (key[j] >> 12) == k0);
+        if (same) return true;
         if (n > BIN_WARP_MAX) return false;
     }
     bool runs = false;
@@ -1576,7 +1575,7 @@ static cudaError_t sort_prepare(int max_bins, int n_tiles, WsSortShape* sh) {
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&no, ko, OVER_NT, sizeof(OverSmem<T>)))) return e;
     sh->part_grid = std::max(1, sms * n1);
     sh->over_grid = std::max(1, sms * no);
-    sh->out_extra = std::min(8 * sms, 2 * n_tiles);
+    sh->out_extra = std::min((sizeof(T) == 4 ? 6 : 3) * sms, n_tiles);   // (as many as are resident at once)
     return cudaSuccess;
 }
 
