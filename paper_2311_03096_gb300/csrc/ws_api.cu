@@ -266,7 +266,8 @@ ws_status build_plan(ws_plan* p) {
         }
         ls.hull_count = (int32_t)htiles.size() - ls.hull_first;
         // distribution sort: bins, buckets of the first pass, map
-        ls.nbins = len <= WS_BIN_CAP ? 1 : (int32_t)std::min<int64_t>((len + WS_BIN_MEAN - 1) / WS_BIN_MEAN, WS_BINS_MAX);
+        ls.nbins = len <= WS_BIN_CAP ? 1 : (int32_t)((len + WS_BIN_MEAN - 1) / WS_BIN_MEAN);   // (838861 at most)
+        if (len <= (int64_t)WS_BINS_RANK * WS_BIN_MEAN_BIG) ls.nbins = std::min(ls.nbins, WS_BINS_RANK);
         ls.fine_log2 = 0;
         if (ls.nbins > WS_ONE_LEVEL) {
             ls.fine_log2 = 7;

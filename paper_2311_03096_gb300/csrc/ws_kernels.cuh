@@ -87,7 +87,11 @@ constexpr int WS_BWD_PIECE = 16384; // pairs of a bin that one CTA adds
 constexpr int WS_BWD_FAN = 512;    // buckets of one move of the backward
 constexpr int WS_BIN_CAP = 4096;
 constexpr int WS_BIN_MEAN = 2560;
-constexpr int WS_BINS_MAX = 1 << 19;         // per segment (a partition's rank word holds 19 bits of bin)
+// Bins that leave a partition's rank word room for the rank.  More of them (a second
+// pass of four rounds per tile instead of two, and a word for the top bits) cost 1.4 as
+// much to partition, so bins grow to WS_BIN_MEAN_BIG keys first: 1.4e9 weights 74 ms, 81 with more bins.
+constexpr int WS_BINS_RANK = 1 << 19;
+constexpr int WS_BIN_MEAN_BIG = 3000;
 constexpr int WS_FAN = 512;                  // buckets a partition tile counts at a time
 constexpr int WS_ONE_LEVEL = 512;            // segments of at most this many bins take one partition pass
 constexpr int WS_CELLS = 2048;               // cells of the map (two-level segments; half as many otherwise)

@@ -580,7 +580,7 @@ __device__ __noinline__ void part_rank_tied(uint32_t* w, uint32_t* cnt, uint32_t
         if ((w[p] >> bsh) - off == tie) w[p] += at;
 }
 
-template <typename T, typename B, bool FIRST>
+template <typename T, typename B, bool FIRST, bool TOP>
 __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
     const T* __restrict__ values, const typename KeyOf<T>::K* __restrict__ keys_in, const B* __restrict__ bins_in,
     typename KeyOf<T>::K* __restrict__ out_a, typename KeyOf<T>::K* __restrict__ out_b, B* __restrict__ bins_out,
@@ -603,7 +603,8 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
         return tile;
     };
     K key[ITEMS];         // (loaded raw; made keys when the tile's turn comes, so that the loads stay in flight)
-    uint32_t br[ITEMS];   // bin << 13 | rank
+    // bin << 13 | rank.  TOP (more than 2^19 bins): the bin's top bit is in `top`, a bit per key
+    uint32_t br[ITEMS], top = 0;
     auto load = [&](const TileDesc& td) {
         const K* src = FIRST ? reinterpret_cast<const K*>(values) + td.vpos : keys_in + td.kpos;
         const B* bsrc = bins_in + td.kpos;
@@ -638,8 +639,13 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
 #pragma unroll
         for (int k = 0; k < ITEMS; ++k) {
             if (FIRST) key[k] = KO::key_of_bits(key[k]);
+            if (TOP) top = (k ? top : 0u) | ((br[k] >> 19) & 1u) << k;
             br[k] <<= 13;
         }
+        auto bin_of = [&](int k) -> uint32_t { return TOP ? (br[k] >> 13) | ((top >> k) & 1u) << 19 : br[k] >> 13; };
+        auto bucket_of = [&](int k, uint32_t off) -> uint32_t {   // (WS_FAN and above: not of this round)
+            return (TOP ? bin_of(k) >> (bsh - 13) : br[k] >> bsh) - off;
+        };
         for (int r0 = 0; r0 < nbk; r0 += WS_FAN) {
             const uint32_t off = (uint32_t)(base + r0);
             __syncthreads();   // (the previous use of the shared memory is over)
@@ -655,16 +661,16 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
             if (tie < 0) {
 #pragma unroll
                 for (int k = 0; k < ITEMS; ++k) {
-                    const uint32_t b = (br[k] >> bsh) - off;
+                    const uint32_t b = bucket_of(k, off);
                     if (t + k * NT < len && b < WS_FAN) br[k] = (br[k] & ~0x1fffu) | atomicAdd(&s.cnt[b], 1u);
                 }
             } else {   // (through the staging area: out of line, and the loop above keeps its registers)
                 uint32_t* w = reinterpret_cast<uint32_t*>(s.key);
 #pragma unroll
-                for (int k = 0; k < ITEMS; ++k) w[t + k * NT] = br[k];
-                part_rank_tied(w, s.cnt, (uint32_t)tie, bsh, off, len);
+                for (int k = 0; k < ITEMS; ++k) w[t + k * NT] = TOP ? min(bucket_of(k, off), (uint32_t)WS_FAN) << 13 : br[k];
+                part_rank_tied(w, s.cnt, (uint32_t)tie, TOP ? 13 : bsh, TOP ? 0u : off, len);
 #pragma unroll
-                for (int k = 0; k < ITEMS; ++k) br[k] = w[t + k * NT];
+                for (int k = 0; k < ITEMS; ++k) br[k] = TOP ? (br[k] & ~0x1fffu) | (w[t + k * NT] & 0x1fffu) : w[t + k * NT];
             }
             __syncthreads();
             // start inside the tile, and the run's destination
@@ -688,12 +694,12 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
             const int64_t kp = tiles[tile].kpos;
 #pragma unroll
             for (int k = 0; k < ITEMS; ++k) {
-                const uint32_t b = (br[k] >> bsh) - off;
+                const uint32_t b = bucket_of(k, off);
                 if (t + k * NT < len && b < WS_FAN) {
                     const uint2 run = s.run[b];
                     const uint32_t rk = br[k] & 0x1fffu, j = run.x + rk;
                     s.key[j] = key[k];
-                    s.bin[j] = (B)(br[k] >> 13);
+                    s.bin[j] = (B)bin_of(k);
                     if (map.loc) map.loc[kp + t + k * NT] = (uint16_t)(jb + j);
                 }
             }
@@ -1544,12 +1550,12 @@ size_t plan_smem(int hist_cap) { return sizeof(MapTab) + 4 * (size_t)hist_cap; }
 // Launch shapes of a plan's sort (and the kernels' shared-memory limits on
 // the plan's device).  max_bins: of its longest segment; samp_max: log2 of the
 // largest number of samples per tile.
-template <typename T, typename B>
+template <typename T, typename B, bool TOP>
 static cudaError_t sort_prepare(int max_bins, int n_tiles, WsSortShape* sh) {
     constexpr int HIST_MAX = 45056;
     auto* kp = k_sort_plan<T, B>;
-    auto* k1 = k_part<T, B, true>;
-    auto* k2 = k_part<T, B, false>;
+    auto* k1 = k_part<T, B, true, TOP>;
+    auto* k2 = k_part<T, B, false, TOP>;
     auto* ko = k_oversize<T>;
     const size_t ksm = sizeof(PartSmem<T, B>);
     cudaError_t e = cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan_smem(HIST_MAX));
@@ -1584,10 +1590,12 @@ cudaError_t ws_sort_prepare(int max_bins, int n_tiles, int samp_max, WsSortShape
     sh->wide = max_bins > 65536;
     sh->samp_max = samp_max;
     sh->max_bins = max_bins;
-    return sh->wide ? sort_prepare<T, uint32_t>(max_bins, n_tiles, sh) : sort_prepare<T, uint16_t>(max_bins, n_tiles, sh);
+    if (max_bins > WS_BINS_RANK) return sort_prepare<T, uint32_t, true>(max_bins, n_tiles, sh);
+    return sh->wide ? sort_prepare<T, uint32_t, false>(max_bins, n_tiles, sh)
+                    : sort_prepare<T, uint16_t, false>(max_bins, n_tiles, sh);
 }
 
-template <typename T, typename B>
+template <typename T, typename B, bool TOP>
 static cudaError_t sort_run(const LargeWork<T>& W, const T* values, bool way_back, uint32_t* status,
                             uint64_t spin_limit, cudaStream_t st) {
     typedef typename KeyOf<T>::K K;
@@ -1617,12 +1625,12 @@ static cudaError_t sort_run(const LargeWork<T>& W, const T* values, bool way_bac
     K* no_keys = nullptr;
     B* no_bins = nullptr;
     WS_LAUNCH(W.prof, WSK_PARTITION, st,
-              ws_launch_chain(k_part<T, B, true>, grid, WS_SORT_NT, ksm, st, values, no_keys, bins, W.keys_a,
+              ws_launch_chain(k_part<T, B, true, TOP>, grid, WS_SORT_NT, ksm, st, values, no_keys, bins, W.keys_a,
                               W.keys_b, bins2, way_back ? W.map1 : PassMap{}, W.sort_tiles, W.n_sort_tiles, W.lsegs,
                               W.cur1, W.ctl, status));
     if (W.two_level)
         WS_LAUNCH(W.prof, WSK_PARTITION, st,
-                  ws_launch_chain(k_part<T, B, false>, grid, WS_SORT_NT, ksm, st, no_values, W.keys_a, bins2, no_keys,
+                  ws_launch_chain(k_part<T, B, false, TOP>, grid, WS_SORT_NT, ksm, st, no_values, W.keys_a, bins2, no_keys,
                                   W.keys_b, no_bins, way_back ? W.map2 : PassMap{}, W.sort_tiles, W.n_sort_tiles,
                                   W.lsegs, W.cur2, W.ctl, status));
     WS_LAUNCH(W.prof, WSK_BIN_SORT, st,
@@ -1653,8 +1661,10 @@ cudaError_t ws_large_sort(const LargeWork<T>& W, const T* values, bool way_back,
     *sorted = nullptr;
     if (W.n_sort_tiles == 0) return cudaSuccess;
     *sorted = W.keys_a;
-    return W.sort_shape.wide ? sort_run<T, uint32_t>(W, values, way_back, status, spin_limit, st)
-                             : sort_run<T, uint16_t>(W, values, way_back, status, spin_limit, st);
+    if (W.sort_shape.max_bins > WS_BINS_RANK)
+        return sort_run<T, uint32_t, true>(W, values, way_back, status, spin_limit, st);
+    return W.sort_shape.wide ? sort_run<T, uint32_t, false>(W, values, way_back, status, spin_limit, st)
+                             : sort_run<T, uint16_t, false>(W, values, way_back, status, spin_limit, st);
 }
 
 template cudaError_t ws_sort_prepare<float>(int, int, int, WsSortShape*);

@@ -73,3 +73,29 @@ def check_lambda_zero(ws, w):
                                   "constant"])
 def test_distributions(ws, kind, d, dt):
     check_lambda_zero(ws, draw(kind, d, dt))
+
+
+@pytest.mark.parametrize("d", [(1 << 19) * 2560 + 12345, (1 << 19) * 3000 + 77])
+def test_bins_at_19_bits(ws, d):
+    """Segments of 2^19 bins and of more, with a tie of about a million copies: at lambda 0 the ids number the
+    values in their order."""
+    ctx = ws.Context.get()
+    ctx.set_small_max(-1)   # (drops the cached plans)
+    torch.cuda.empty_cache()
+    if torch.cuda.mem_get_info()[0] < 180e9:
+        pytest.skip("needs 180 GB")
+    w = torch.randn(d, generator=torch.Generator(device="cuda").manual_seed(12), device="cuda")
+    w[w.abs() < 2.0 ** -10] = 2.0 ** -10   # (no value loses bits in the fixed point)
+    plan = ws.Plan([0, d])
+    out, ids, nc = plan.forward(w, torch.zeros(1, dtype=torch.float64, device="cuda"))
+    ctx.check(what="prox")
+    c = int(nc.item())
+    assert int(ids.min()) == 0 and int(ids.max()) == c - 1
+    value = torch.full((c,), float("nan"), device="cuda")
+    for i in range(0, d, 1 << 28):
+        value[ids[i:i + (1 << 28)]] = w[i:i + (1 << 28)]
+    assert bool(torch.all(value[1:] > value[:-1]))
+    for i in range(0, d, 1 << 28):
+        x = w[i:i + (1 << 28)]
+        assert torch.equal(value[ids[i:i + (1 << 28)]], x)
+        assert bool(torch.all((out[i:i + (1 << 28)] - x).abs() <= 2.0 ** -22 * x.abs()))
