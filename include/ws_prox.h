@@ -197,8 +197,12 @@ ws_status ws_prox_backward(ws_ctx* ctx, const void* grad_out, const int32_t* clu
  * sorted positions a..b (1-based) moves with the mean velocity of its
  * particles (Sec. 3), so d out_i / d lambda_s = (d+1-a-b)/(d-1) for every i in
  * it (0 for segments of d <= 1).  grad_lambda[s] (DEVICE, n_seg doubles,
- * overwritten) receives sum_{i in s} grad_out[i] * d out_i / d lambda_s,
- * accumulated in FP64 with atomics (the order of the additions is not fixed).
+ * overwritten) receives sum_{i in s} grad_out[i] * d out_i / d lambda_s.
+ * Segments of up to 4096 elements: FP64 products and sums.  Longer ones: the
+ * products of a run of 6144 elements are added as integers (to 2^-98 of the
+ * largest product; runs with infinities or NaN in FP64), and the runs' sums in
+ * FP64 with atomics (the order of these additions is not fixed).  Either way
+ * the error stays below a few roundings of sum |grad_out[i] d out_i/d lambda|.
  * cluster_ids as written by the forward on the same plan layout (ranked by
  * value, which is what fixes each cluster's positions).  grad_out: n elements
  * of the plan's dtype.  Total of the plan's large-segment slots must be

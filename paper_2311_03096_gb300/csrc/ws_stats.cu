@@ -168,8 +168,8 @@ template cudaError_t ws_large_R<double>(const LargeWork<double>&, const double*,
 // a..b (1-based) has d out / d lambda = (d + 1 - a - b)/(d - 1); with 0-based
 // start s and size m that is (d - 2s - m)/(d - 1).  Starts follow from the
 // cluster sizes because cluster ids are ranked by value.  The result per
-// segment is sum_i grad_out[i] * d out_i / d lambda (FP64, atomics: the
-// summation order is not fixed).
+// segment is sum_i grad_out[i] * d out_i / d lambda (the sums of tiles are
+// added with FP64 atomics: their order is not fixed).
 // ---------------------------------------------------------------------------
 namespace {
 
@@ -393,30 +393,31 @@ __global__ void __launch_bounds__(1024) k_dlam_scan_totals(int32_t* csum, int nb
     }
 }
 
-// Sum of grad_out x (len - 2 start - size) over one sort tile, exactly: every
-// grad_out as a 63-bit integer at the tile's largest exponent (a value more
-// than 39 binades below it, 10 for double, loses the bits below 2^-63 of the
-// largest), the products and the sum in 128 bits, one rounding and one division
-// at the end.  FP64 multiplies and adds per element took 266 us at 2^24 (GB300
-// runs them at a small fraction of the FP32 rate; two gathers per element
-// beside them) and round more.
+// Sum of grad_out x (len - 2 start - size) over one sort tile: every product as
+// an integer of up to 84 bits, in units of 2^-113 of its warp's largest (a
+// product more than 28 binades below it, 58 for FP32, loses the bits below
+// that), the sums in 128 bits, one rounding and one division at the end.  The
+// scale comes from the products: the largest gradient may have weight 0 or 1,
+// and an integer of the gradient alone at its scale lost what others, with
+// weights up to the length, add (FP64 products did not).  FP64 multiplies and
+// adds per element took 266 us at 2^24 (GB300 runs them at a small fraction of
+// the FP32 rate; two gathers per element beside them) and round more.
 constexpr int DL_NT = 512;
 template <typename T>
-__global__ void __launch_bounds__(DL_NT) k_dlam_apply(const T* __restrict__ g, const int32_t* __restrict__ ids,
+__global__ void __launch_bounds__(DL_NT, sizeof(T) == 4 ? 1 : 2) k_dlam_apply(const T* __restrict__ g, const int32_t* __restrict__ ids,
                                                       const TileDesc* __restrict__ tiles,
                                                       const LargeSeg* __restrict__ lsegs,
                                                       const int32_t* __restrict__ cnt,
                                                       const uint32_t* __restrict__ key, double* out) {
     ws_chain();
     typedef KeyOf<T> KO;
-    constexpr int PER = WS_SORT_TILE / DL_NT, UP = 62 - KO::MANT;
+    constexpr int PER = WS_SORT_TILE / DL_NT;
     __shared__ long long wlo[DL_NT / 32], whi[DL_NT / 32];
-    __shared__ int s_emax;
+    __shared__ int we[DL_NT / 32];
     const TileDesc td = tiles[blockIdx.x];
     const LargeSeg& ls = lsegs[td.lseg];
     const int64_t slot0 = ls.kpos + td.lseg;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    if (t == 0) s_emax = 0;
     T gv[PER];
     int id[PER];
 #pragma unroll
@@ -434,24 +435,28 @@ __global__ void __launch_bounds__(DL_NT) k_dlam_apply(const T* __restrict__ g, c
     for (int k = 0; k < PER; ++k) {
         if (id[k] < 0 || (int64_t)id[k] >= ls.len) { id[k] = -1; gv[k] = (T)0; }
         kv[k] = id[k] >= 0 ? __ldg(key + slot0 + id[k]) : 0u;
-        if (gv[k] != (T)0) e = max(e, ws_eff_exp(gv[k]));
         odd |= !ws_isfinite(gv[k]);
     }
-    e = __reduce_max_sync(0xffffffffu, e);
-    const bool any_odd = __syncthreads_or(odd);
-    if (any_odd) {   // infinities and NaN: as FP64 arithmetic has it
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {   // (the weight; one bit above the product's binade)
+        const int32_t wt = id[k] >= 0 ? (int32_t)(top - kv[k]) : 0;
+        kv[k] = (uint32_t)wt;
+        if (gv[k] != (T)0 && wt != 0) e = max(e, ws_eff_exp(gv[k]) + 32 - __clz(abs(wt)));
+    }
+    // every warp at its own scale (no barrier while the weights arrive)
+    int emax = __reduce_max_sync(0xffffffffu, e);
+    if (__any_sync(0xffffffffu, odd)) {   // infinities and NaN: as FP64 arithmetic has it
         double acc = 0.0;
 #pragma unroll
         for (int k = 0; k < PER; ++k)
-            if (id[k] >= 0) acc += (double)gv[k] * ((double)(int32_t)(top - kv[k]) / (double)(ls.len - 1));
+            if (id[k] >= 0) acc += (double)gv[k] * ((double)(int32_t)kv[k] / (double)(ls.len - 1));
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if (lane == 0) atomicAdd(&out[ls.seg], acc);
-        return;
+#pragma unroll
+        for (int k = 0; k < PER; ++k) kv[k] = 0;   // (nothing left to add)
+        emax = 0;
     }
-    if (lane == 0) atomicMax(&s_emax, e);
-    __syncthreads();
-    const int emax = s_emax;
     i128 acc = 0;
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
@@ -459,21 +464,33 @@ __global__ void __launch_bounds__(DL_NT) k_dlam_apply(const T* __restrict__ g, c
         int ex = (int)((b >> KO::MANT) & KO::EXPMASK);
         uint64_t m = b & ((1ull << KO::MANT) - 1ull);
         if (ex == 0) ex = 1; else m |= 1ull << KO::MANT;
-        const int up = UP - (emax - ex);
-        const int64_t q = (int64_t)(up >= 0 ? m << up : (up > -64 ? m >> -up : 0ull));
-        const bool neg = (b >> (KO::BITS - 1)) & 1ull;
-        acc += (i128)(neg ? -q : q) * (int64_t)(int32_t)(top - kv[k]);
+        const int32_t wt = (int32_t)kv[k];
+        const uint64_t aw = (uint32_t)abs(wt);
+        const u128 p = sizeof(T) == 4 ? (u128)(m * aw) : (u128)m * aw;   // < 2^(MANT + 1 + bits of the weight)
+        const int up = ex - emax + 112 - KO::MANT;   // (then < 2^113: 6144 of them fit)
+        if (wt == 0) continue;
+        u128 q;
+        if (up < 0) q = up > -128 ? p >> -up : (u128)0;   // (rare)
+        else if (sizeof(T) == 4) q = p << up;
+        else {   // (up <= 59)
+            const uint64_t lo = (uint64_t)p, hi = (uint64_t)(p >> 64);
+            q = ((u128)((hi << up) | ((lo >> 1) >> (63 - up))) << 64) | (lo << up);
+        }
+        acc += ((b >> (KO::BITS - 1)) & 1ull) != (uint64_t)(wt < 0) ? -(i128)q : (i128)q;
     }
     acc = ws_warp_reduce_i128(acc);
-    if (lane == 0) { wlo[w] = (long long)(uint64_t)acc; whi[w] = (long long)(uint64_t)((u128)acc >> 64); }
+    if (lane == 0) { wlo[w] = (long long)(uint64_t)acc; whi[w] = (long long)(uint64_t)((u128)acc >> 64); we[w] = emax; }
     __syncthreads();
     if (t == 0) {
+        emax = 0;
+        for (int k = 0; k < DL_NT / 32; ++k) emax = max(emax, we[k]);
         i128 S = 0;
-        for (int k = 0; k < DL_NT / 32; ++k) S += (i128)(((u128)(uint64_t)whi[k] << 64) | (u128)(uint64_t)wlo[k]);
-        // grad_out = q 2^(emax - UP - bias - MANT)
+        for (int k = 0; k < DL_NT / 32; ++k)
+            S += (i128)(((u128)(uint64_t)whi[k] << 64) | (u128)(uint64_t)wlo[k]) >> min(emax - we[k], 127);
+        // product = q 2^(emax - bias - 112)
         const int bias = KO::EXPMASK >> 1;
         const double v = ws_i128_to_double(S) / (double)(ls.len - 1);
-        if (S != 0) atomicAdd(&out[ls.seg], ldexp(v, emax - UP - bias - KO::MANT));
+        if (S != 0) atomicAdd(&out[ls.seg], ldexp(v, emax - bias - 112));
     }
 }
 
