@@ -275,18 +275,18 @@ ws_status build_plan(ws_plan* p) {
             p->two_level = 1;
         }
         ls.n_coarse = ((ls.nbins - 1) >> ls.fine_log2) + 1;
-        ls.ncell = ls.fine_log2 ? WS_CELLS : WS_CELLS / 2;
+        ls.ncell = ls.nbins == 1 ? 0 : ls.fine_log2 ? WS_CELLS : WS_CELLS / 2;
         // samples per tile: 100 per bin for one-pass segments, 50 for longer ones (about 2^20 at most)
         ls.samp_log2 = ls.fine_log2 ? 7 : 8;
         while (ls.samp_log2 > 5 && ((int64_t)ls.sort_count << ls.samp_log2) > ((int64_t)1 << 20)) --ls.samp_log2;
         samp_max = std::max(samp_max, (int)ls.samp_log2);
         ls.bin_pos = (int32_t)bin_pos;
         ls.coarse_pos = (int32_t)coarse_pos;
-        ls.cell_pos = (int32_t)cell_pos;
+        ls.cell_pos = cell_pos;
         bin_pos += ls.nbins;
         coarse_pos += ls.n_coarse;
         cell_pos += 3 * ls.ncell;   // counts of the cells, then of their parts (at most two per cell on average)
-        if (cell_pos > INT32_MAX || bin_pos > INT32_MAX) return WS_ERR_NOMEM;
+        if (bin_pos > INT32_MAX) return WS_ERR_NOMEM;
         p->max_bins = std::max(p->max_bins, (int)ls.nbins);
         // backward: bins of cluster slots, moved into in one pass or two
         ls.bb_n = (int32_t)((len + WS_BWD_BIN - 1) >> WS_BWD_BIN_LOG2);

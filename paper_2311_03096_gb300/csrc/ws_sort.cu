@@ -168,7 +168,8 @@ __device__ __forceinline__ int sample_pos(int tile, int j, int len, int mlog) {
 // ---------------------------------------------------------------------------
 struct PlanSmem {
     unsigned long long hi, lo, mag;
-    int emin, parts;
+    int emin;
+    int map;   // the CTA has tiles of segments with more than one bin
     int wsum[PLAN_NT / 32];
 };
 
@@ -200,11 +201,34 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
 
     // 1. range of the sampled keys (one warp per tile; the CTA's first segment
     // is combined in shared memory)
-    if (t == 0) { S.hi = 0; S.lo = 0; S.mag = 0; }
+    if (t == 0) { S.hi = 0; S.lo = 0; S.mag = 0; S.map = 0; }
     __syncthreads();
+    bool bad = false;
     for (int tile = t0 + w; tile < t1; tile += PLAN_NT / 32) {
         const TileDesc td = tiles[tile];
-        const int ml = lsegs[td.lseg].samp_log2;
+        const LargeSeg& sg = lsegs[td.lseg];
+        if (sg.nbins == 1) {   // one tile and no map: the warp does all that the phases do for others
+            K amax = 0, amin = ~(K)0;   // (as in phase 4)
+#pragma unroll 4
+            for (int i = lane; i < td.len; i += 32) {
+                const K mag = (K)KO::bits(__ldg(values + td.vpos + i)) & (~(K)0 >> 1);
+                amax = max(amax, mag);
+                amin = min(amin, mag - 1);
+                bins[td.kpos + i] = 0;
+            }
+            bad |= (amax >> KO::MANT) >= (K)KO::EXPMASK;
+            int emin = amin != ~(K)0 ? max((int)((amin + 1) >> KO::MANT), 1) : 0x7fffffff;
+            emin = __reduce_min_sync(WS_FULL_MASK, emin);
+            if (lane == 0) {
+                seg_emin[td.lseg] = emin;
+                bin_cnt[sg.bin_pos] = (uint32_t)td.len;
+                bin_start[sg.bin_pos] = 0;
+                cur1[sg.coarse_pos] = 0;
+            }
+            continue;
+        }
+        if (lane == 0) S.map = 1;
+        const int ml = sg.samp_log2;
         const int m = min(td.len, 1 << ml);
         K hi = 0, lo = 0, mg = 0;   // (lo, mg: complements, so that 0 is neutral)
         K* keep = cache + ((size_t)(tile - t0) << samp_max);
@@ -238,11 +262,12 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
         }
     }
     __syncthreads();
-    if (t == 0 && seg0 >= 0) {
+    if (t == 0 && S.map) {   // (S.hi, S.lo: 0 if the first segment has one bin)
         atomicMax(seg_hi + seg0, S.hi);
         atomicMax(seg_lo + seg0, S.lo);
         if (sizeof(K) == 8) atomicMax(seg_lo + n_lseg + seg0, S.mag);
     }
+    const int tm = S.map ? t1 : t0;   // (uniform; the tile loops below are for segments with a map)
     bar.sync();
 
     // header of a segment from its sampled range
@@ -287,10 +312,11 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
 
     // 2. sampled keys per cell (counted in shared memory, added to the
     // segment's cells once per CTA)
-    for (int ta = t0; ta < t1;) {
+    for (int ta = t0; ta < tm;) {
         const int lseg = tiles[ta].lseg;
         const LargeSeg sg = lsegs[lseg];
         const int tb = min(t1, sg.sort_first + sg.sort_count);
+        if (sg.nbins == 1) { ta = tb; continue; }   // (uniform)
         const SortHdr h = header(lseg, sg);
         uint32_t* sc = tab.split;   // [ncell]
         for (int i = t; i < sg.ncell; i += PLAN_NT) sc[i] = 0;
@@ -312,15 +338,14 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
     // varies more inside a cell than the noise costs.  Returns the number.
     auto parts_of = [&](const LargeSeg& sg, const SortHdr& h) -> int {
         constexpr int PER = WS_CELLS / PLAN_NT;
-        int v[PER], bits[PER], sum = 0;
+        int v[PER], bits[PER], sum;
 #pragma unroll
         for (int i = 0; i < PER; ++i) {
             const int c = t * PER + i;
             v[i] = c < sg.ncell ? (int)__ldcg(cells + sg.cell_pos + c) : 0;
-            sum += v[i];
         }
-        int tot;
-        ws_block_excl_scan<PLAN_NT, int>(sum, S.wsum, &tot);
+        const int m = 1 << sg.samp_log2, tail = (int)(sg.len - (int64_t)(sg.sort_count - 1) * WS_SORT_TILE);
+        int tot = (sg.sort_count - 1) * m + min(tail, m);   // the segment's samples
         const int thr = max(96, tot / sg.ncell + 1);
         const int bmax = min(h.shift, 12);
         auto log2_of = [](int q) { return q > 0 ? 31 - __clz(q) : 0; };
@@ -351,10 +376,11 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
     };
 
     // 3. sampled keys per part
-    for (int ta = t0; ta < t1;) {
+    for (int ta = t0; ta < tm;) {
         const int lseg = tiles[ta].lseg;
         const LargeSeg sg = lsegs[lseg];
         const int tb = min(t1, sg.sort_first + sg.sort_count);
+        if (sg.nbins == 1) { ta = tb; continue; }   // (uniform)
         const SortHdr h = header(lseg, sg);
         const int parts = parts_of(sg, h);
         uint32_t* sc = reinterpret_cast<uint32_t*>(tab.knots);   // [parts]
@@ -378,11 +404,11 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
 
     // 4. knots of every segment (every CTA for the segments it needs), the bin
     // of every key, finiteness, smallest exponent
-    bool bad = false;
-    for (int ta = t0; ta < t1;) {
+    for (int ta = t0; ta < tm;) {
         const int lseg = tiles[ta].lseg;
         const LargeSeg sg = lsegs[lseg];
         const int tb = min(t1, sg.sort_first + sg.sort_count);
+        if (sg.nbins == 1) { ta = tb; continue; }   // (uniform)
         const bool local = sg.nbins <= hist_cap;
         const SortHdr h = header(lseg, sg);
         const int parts = parts_of(sg, h);
@@ -517,7 +543,7 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
         const int first = (int)(((int64_t)blockIdx.x + (int64_t)gridDim.x * (c0 / PLAN_NT) - c0 / PLAN_NT) % gridDim.x);
         for (int lseg = first; lseg < n_lseg; lseg += gridDim.x) {
             const LargeSeg sg = lsegs[lseg];
-            if (c0 >= sg.nbins) continue;   // (uniform)
+            if (c0 >= sg.nbins || sg.nbins == 1) continue;   // (uniform)
             const uint32_t* c = bin_cnt + sg.bin_pos;
             int before = 0;
 #pragma unroll 8
