@@ -17,7 +17,6 @@ only), on a bounded sample of the same workload.
 from __future__ import annotations
 
 import argparse
-import hashlib
 import json
 import os
 import statistics
@@ -43,8 +42,8 @@ ALGO_BYTES_PER_ELEM_F32 = {
     "sort_plan": 4,   # read the value
     "tile_hull": 4,   # read the sorted key (hull vertices are data dependent, not counted)
     "bin_out": 10,    # read the rank in the bin, write value and cluster id
-    "regroup": 20,    # read a place, read and write value and cluster id
-    "output": 20,     # read a place, value and cluster id, write out and cluster id
+    "regroup": 18,    # read a place (16 bits), read and write value and cluster id
+    "output": 18,     # read a place, value and cluster id, write out and cluster id
 }
 
 # Whole-step byte models per element (FP32 storage), fixed before tuning:
@@ -56,26 +55,6 @@ ALGO_BYTES_PER_ELEM_F32 = {
 IO_FLOOR_B = 12
 ONE_CTA_MAX_F32 = 4096   # FP32 segments up to this length run one CTA each
 MODEL_B = {"key_only_52B": 52, "index_payload_80B": 80}
-
-# DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one
-# ncu capture of the bench's own workload, and the hash of the source files the
-# kernel is built from when the counters were taken; reported as null once any
-# of them changes (see profiles/).
-NCU_SOURCES = {}
-NCU_TRAFFIC = {}
-NCU_SOURCE_HASH = {}
-
-
-def source_hash(files=None) -> str:
-    """Hash of the kernel sources (all of csrc/, or the listed files of it)."""
-    h = hashlib.sha256()
-    csrc = os.path.join(ROOT, "paper_2311_03096_gb300", "csrc")
-    for f in sorted(files if files is not None else os.listdir(csrc)):
-        with open(os.path.join(csrc, f), "rb") as fh:
-            h.update(f.encode())
-            h.update(fh.read())
-    return h.hexdigest()[:16]
-
 
 def load_peaks():
     p = os.path.join(ROOT, "MEASURED_PEAKS.json")
@@ -589,20 +568,17 @@ def main():
     if dom is not None:
         ms_avg = kern[dom][0] / kern[dom][1]
         per_launch = ALGO_BYTES_PER_ELEM_F32.get(dom)
-        traffic = None
-        if dom in NCU_TRAFFIC and NCU_SOURCE_HASH.get(dom) == source_hash(NCU_SOURCES.get(dom)):
-            traffic = NCU_TRAFFIC[dom]
         if per_launch is not None:
             achieved = per_launch * args.d / (ms_avg / 1e3) / 1e9
             roofline = {"bound": "hbm", "kernel": dom, "achieved": achieved, "peak": peak, "unit": "GB/s",
                         "frac": achieved / peak, "peak_source": f"{peak_kind} hbm_gbs",
-                        "bytes_per_launch": per_launch * args.d, "ms_per_launch": ms_avg, "traffic": traffic,
+                        "bytes_per_launch": per_launch * args.d, "ms_per_launch": ms_avg, "traffic": None,
                         "timing": "CUDA events around every launch on the launching stream, in a second run "
                                   "of the timed loop (same steps and inputs; the value comes from the first, "
                                   "unprofiled run)"}
         else:
             roofline = {"bound": "hbm", "kernel": dom, "achieved": None, "peak": peak, "unit": "GB/s", "frac": None,
-                        "ms_per_launch": ms_avg, "traffic": traffic}
+                        "ms_per_launch": ms_avg, "traffic": None}
 
     # ---- end to end through the public API with host buffers (pinned).  Every step
     # copies its input in and its result (values + ids) out; the copies of one step

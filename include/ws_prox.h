@@ -278,7 +278,7 @@ void ws_debug_set_ic_cap(ws_ctx* ctx, int cap);
  * All zero if no such call was made.  Benchmark hook. */
 ws_status ws_debug_hull_stats(ws_ctx* ctx, int64_t d, ws_dtype dtype, int64_t* counts, int n_counts);
 
-/* Runs only the radix sort of the device-wide path and writes, for every
+/* Runs only the sort of the device-wide path and writes, for every
  * segment that the plan sends down that path, its values sorted ascending in
  * IEEE total order (-0 before +0) at the segment's own position in
  * `sorted_out` (device, plan dtype); other positions are left untouched.

@@ -61,7 +61,6 @@ struct ws_plan {
     std::vector<void*> allocs;
     void* keys_a = nullptr;
     void* keys_b = nullptr;
-    uint32_t* hist = nullptr;
     SortCtl* ctl = nullptr;       // start of the words cleared before every sort
     size_t sort_zero_bytes = 0;
     unsigned long long* seg_hi = nullptr;
@@ -134,7 +133,6 @@ LargeWork<T> make_work(const ws_plan* p) {
     W.hull_tiles = p->d_hull_tiles;
     W.keys_a = (K*)p->keys_a;
     W.keys_b = (K*)p->keys_b;
-    W.hist = p->hist;
     W.ctl = p->ctl;
     W.sort_zero_bytes = p->sort_zero_bytes;
     W.seg_hi = p->seg_hi;
@@ -334,7 +332,6 @@ ws_status build_plan(ws_plan* p) {
     const size_t nk = (size_t)p->n_keys, nh = (size_t)p->n_hull_tiles, slots = nk + (size_t)p->n_lseg;
     if ((st = plan_alloc(p, &p->keys_a, ksize * nk))) return st;
     if ((st = plan_alloc(p, &p->keys_b, ksize * nk))) return st;
-    if ((st = plan_alloc(p, (void**)&p->hist, sizeof(uint64_t) * (3 * 256 + 2)))) return st;
     {
         // one block, cleared before every sort: control words, sampled ranges, cells, bin counts,
         // the merge tree's arrival counters

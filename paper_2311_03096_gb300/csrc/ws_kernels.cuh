@@ -98,7 +98,6 @@ constexpr int WS_CELLS = 2048;               // cells of the map (two-level segm
 constexpr int WS_HULL_NT = 256;              // threads per hull-tile CTA
 constexpr int WS_HULL_M = 16;                // points per thread chunk
 constexpr int WS_HULL_TILE = WS_HULL_NT * WS_HULL_M;       // 4096 elements per hull tile
-constexpr int WS_MAX_LEVELS = 32;           // merge-tree levels (segments < 2^31 elements)
 
 // One tile of a large segment (sort tiles and hull tiles use the same record).
 struct TileDesc {
@@ -359,7 +358,6 @@ struct LargeWork {
     OverClass* over_big;     // [n_keys / WS_BIN_CAP + 1] those above WS_BIN_CAP keys
     uint32_t* over_cnt;      // [n_keys / (WS_SORT_TILE / 2) + 1][256] digit counts of their tiles
     int32_t* seg_emin;       // [n_lseg] smallest effective exponent of a nonzero value
-    uint32_t* hist;          // counters of the backward's slot buckets: >= 3 * 256 + 2 64-bit words
     // hull
     uint16_t* vp;            // [n_hull_tiles][WS_HULL_TILE + 1] vertex points (tile-local)
     i128* vx;                // [n_hull_tiles][WS_HULL_TILE + 1] X at vertices (tile-local; see TileX)

@@ -722,7 +722,9 @@ __global__ void __launch_bounds__(256) k_root(const LargeSeg* __restrict__ lsegs
 // from the tile's keys (4 bytes per element, in shared memory) instead of the
 // prefix sums at its two vertices (16 bytes each): the same integer.  Bound by
 // issue (0.66; the values' 64-bit sums and one division per cluster); from the
-// prefix sums alone it took 460 us at 2^26, lambda 1e-2, instead of 311.
+// prefix sums alone it took 460 us at 2^26, lambda 1e-2, instead of 311.  SUM_MAX
+// 2, 4, 8, 16: 457, 357, 295, 295 us there, 95, 90, 84, 79 at 2^24, lambda 1, 60, 63,
+// 64, 65 for FP64 2^22, lambda 1 (eight sums of 2^58 are the most that 64 bits hold).
 // ---------------------------------------------------------------------------
 constexpr int HTW = HT / 32;   // rank words per hull tile
 constexpr int SUM_MAX = 8;

@@ -31,7 +31,7 @@
 // The partition is bound by shared-memory wavefronts (17 per 32 keys: the
 // counters, the staging and the copy out; 0.7 of the pipe), the bin sort by
 // issue (0.65) and the same pipe, the plan by the read of the values (0.104 of
-// its 0.150 ms) and five barriers.
+// its 0.150 ms) and four barriers.
 #include <algorithm>
 #include <type_traits>
 
@@ -612,7 +612,7 @@ __global__ void __launch_bounds__(WS_SORT_NT, sizeof(T) == 4 ? 3 : 2) k_part(
     typename KeyOf<T>::K* __restrict__ out_a, typename KeyOf<T>::K* __restrict__ out_b, B* __restrict__ bins_out,
     PassMap map,   // (map.loc nullable: how to undo the pass)
     const TileDesc* __restrict__ tiles, int n_tiles, const LargeSeg* __restrict__ lsegs, uint32_t* cursor,
-    const SortCtl* ctl, uint32_t* status) {
+    const SortCtl* ctl) {
     typedef KeyOf<T> KO;
     typedef typename KO::K K;
     constexpr int NT = WS_SORT_NT, ITEMS = WS_SORT_ITEMS;
@@ -1653,12 +1653,12 @@ static cudaError_t sort_run(const LargeWork<T>& W, const T* values, bool way_bac
     WS_LAUNCH(W.prof, WSK_PARTITION, st,
               ws_launch_chain(k_part<T, B, true, TOP>, grid, WS_SORT_NT, ksm, st, values, no_keys, bins, W.keys_a,
                               W.keys_b, bins2, way_back ? W.map1 : PassMap{}, W.sort_tiles, W.n_sort_tiles, W.lsegs,
-                              W.cur1, W.ctl, status));
+                              W.cur1, W.ctl));
     if (W.two_level)
         WS_LAUNCH(W.prof, WSK_PARTITION, st,
                   ws_launch_chain(k_part<T, B, false, TOP>, grid, WS_SORT_NT, ksm, st, no_values, W.keys_a, bins2, no_keys,
                                   W.keys_b, no_bins, way_back ? W.map2 : PassMap{}, W.sort_tiles, W.n_sort_tiles,
-                                  W.lsegs, W.cur2, W.ctl, status));
+                                  W.lsegs, W.cur2, W.ctl));
     WS_LAUNCH(W.prof, WSK_BIN_SORT, st,
               ws_launch_chain(way_back ? k_bin_sort<T, true> : k_bin_sort<T, false>, W.n_bins, BIN_NT,
                               sizeof(BinSmem<T>), st, W.keys_b, W.keys_a, W.bin_seg, W.lsegs, W.bin_start, W.bin_cnt,

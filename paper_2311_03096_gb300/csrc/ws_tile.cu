@@ -107,10 +107,9 @@ struct FastSmem {
 //            (t11 a lower bound; the next round tests what it leaves).
 //   Round r: every surviving block boundary b, with neighbouring boundaries
 //            a < b < c, stays iff the mean of y over [a, b) is strictly below
-//            the mean over [b, c) (the exact hull test at b); all boundaries
-//            are decided at once, as the paper's rounds do.  A boundary whose
-//            neighbours did not change keeps last round's answer, so only
-//            boundaries next to a removal are tested again.
+//            the mean over [b, c) (the exact hull test at b).  The lanes
+//            decide at once, each for its own 16 points, and follow a removal
+//            up inside them (ic_rounds in ws_hull.cuh).
 // When a round removes nothing every adjacent pair of blocks has increasing
 // means: the blocks are the tile's pool-adjacent-violators partition, and
 // their boundaries (with points 0 and n) its hull vertices.

@@ -82,3 +82,29 @@ def test_segments_with_and_without(ws, ctx, dt):  # noqa: F811
         for g, p, n in zip(got, parts, nc.cpu().numpy()):
             u, inv = np.unique(p, return_inverse=True)
             assert np.array_equal(g, inv) and n == len(u)
+
+
+@pytest.mark.parametrize("d", [70001, 1500001])
+def test_captured_call_with_and_without_ties(ws, ctx, d):  # noqa: F811
+    """One captured call replayed on values with heavy ties, without, and with other ones."""
+    import torch
+
+    g = torch.Generator(device="cuda").manual_seed(14)
+    base = torch.randn(d, generator=g, device="cuda")
+    r = torch.rand(d, generator=g, device="cuda")
+    inputs = [torch.where(r < p, torch.full_like(base, v), base) for p, v in ((0.5, 0.0), (0.0, 0.0), (0.9, 1.5), (0.3, -0.25))]
+    w = base.clone()
+    out, ids = torch.empty_like(w), torch.empty(d, dtype=torch.int32, device="cuda")
+    nc = torch.zeros(1, dtype=torch.int64, device="cuda")
+    ws.prox(w, 0.01, out=out, id_out=ids, n_clusters=nc)   # (the plan is made outside the capture)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ws.prox(w, 0.01, out=out, id_out=ids, n_clusters=nc)
+    for x in inputs + inputs[::-1]:
+        w.copy_(x)
+        graph.replay()
+        torch.cuda.synchronize()
+        ctx.check(what="replay")
+        want = ws.prox(x, 0.01)
+        assert torch.equal(out, want[0]) and torch.equal(ids, want[1]) and torch.equal(nc, want[2])
