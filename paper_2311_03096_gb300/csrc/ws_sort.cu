@@ -795,7 +795,7 @@ struct BinSmem {
     K lo, hi;
     uint32_t late[WS_BIN_CAP - BIN_REG * BIN_NT];    // group << 16 | rank of the keys not in registers
     int wsum[BIN_NT / 32];
-    int n_list, radix_needed;
+    int n_list, radix_needed, skew;
     uint32_t list[WS_BIN_CAP / (BIN_NET + 1) + 1];   // start << 16 | keys of the groups for the warps
 };
 
@@ -1049,7 +1049,7 @@ __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>:
     }
     const K* src = keys + start;
     reinterpret_cast<uint4*>(s.u.cnt)[t] = make_uint4(0, 0, 0, 0);
-    if (t == 0) { s.lo = ~(K)0; s.hi = 0; s.n_list = 0; s.radix_needed = 0; }
+    if (t == 0) { s.lo = ~(K)0; s.hi = 0; s.n_list = 0; s.radix_needed = 0; s.skew = 0; }
     // the first BIN_REG keys of a thread stay in registers; the few beyond (a
     // bin 1.2 times the mean or more) are read again, and their group kept in
     // shared memory
@@ -1074,16 +1074,31 @@ __global__ void __launch_bounds__(BIN_NT, 4) k_bin_sort(const typename KeyOf<T>:
     lo = s.lo;
     hi = s.hi;
     // group: linear in the key where sign and exponent are shared (the value is
-    // linear in the key there), else linear in the value
-    const bool same = ((lo ^ hi) >> KO::MANT) == 0;
+    // linear in the key there), else linear in the value; but linear in the key
+    // again where the bin spans several binades and most of it lies in a sixteenth of
+    // the span next to zero (heavy tails: a few groups held such a bin, which took
+    // radix passes: R of 4097 Cauchy weights 96 -> 69 us, of 20000 104 -> 61)
+    bool by_key = ((lo ^ hi) >> KO::MANT) == 0;
     const int range_bits = 64 - __clzll((long long)((uint64_t)(hi - lo) | 1ull));
     const int dsh = max(0, range_bits - 24);
     const int cut = PLACE ? max(0, range_bits - (KO::BITS - 12)) : 0;   // key bits that the words leave out
-    const float x0 = ws_trunc_f32(KO::from_key(lo));
-    const float span = same ? (float)(uint32_t)((hi - lo) >> dsh) + 1.0f : ws_trunc_f32(KO::from_key(hi)) - x0;
+    const float x0 = ws_trunc_f32(KO::from_key(lo)), x1 = ws_trunc_f32(KO::from_key(hi));
+    if ((hi >> KO::MANT) - (lo >> KO::MANT) >= 3) {   // (uniform)
+        const bool both = ((lo ^ hi) >> (KO::BITS - 1)) != 0;   // (signs)
+        const float near0 = (both ? 0.0f : fminf(fabsf(x0), fabsf(x1))) + (x1 - x0) * 0.0625f;
+        int c = 0;
+#pragma unroll
+        for (int k = 0; k < BIN_REG; ++k)
+            c += t + k * BIN_NT < n && fabsf(ws_trunc_f32(KO::from_key(key[k]))) < near0 ? 1 : 0;
+        c = __reduce_add_sync(WS_FULL_MASK, c);
+        if (lane == 0) atomicAdd(&s.skew, c);
+        __syncthreads();
+        by_key = 2 * s.skew > min(n, BIN_REG * BIN_NT);
+    }
+    const float span = by_key ? (float)(uint32_t)((hi - lo) >> dsh) + 1.0f : x1 - x0;
     const float scale = (span > 0.0f && span <= 3.0e38f) ? (float)BIN_GROUPS / span : 0.0f;
     auto group_of = [&](K k) -> uint32_t {   // group << 16 | rank
-        const float f = same ? (float)(uint32_t)((k - lo) >> dsh) : ws_trunc_f32(KO::from_key(k)) - x0;
+        const float f = by_key ? (float)(uint32_t)((k - lo) >> dsh) : ws_trunc_f32(KO::from_key(k)) - x0;
         const uint32_t b = min((uint32_t)(int)(f * scale), (uint32_t)BIN_GROUPS - 1u);
         return (b << 16) | atomicAdd(&s.u.cnt[b], 1u);
     };

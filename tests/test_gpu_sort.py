@@ -145,3 +145,21 @@ def test_hard_edges_and_the_gap_around_zero(ws, ctx, dt, kind, d):
     elif kind == "two spikes":
         x = np.where(x < 0, -1.0, 1.0) + 1e-6 * x
     check(ws, ctx, x.astype(dt))
+
+
+@pytest.mark.parametrize("dt", [np.float32, np.float64])
+@pytest.mark.parametrize("kind", ["cauchy", "lognormal", "negative lognormal", "one-sided cauchy", "tail and ties"])
+@pytest.mark.parametrize("d", [4097, 20000, 300001])
+def test_heavy_tails(ws, ctx, kind, d, dt):
+    """Bins over many binades with most of their keys at the end next to zero."""
+    rng = np.random.default_rng(d + 1)
+    x = rng.standard_cauchy(d)
+    if kind == "lognormal":
+        x = np.exp(4 * rng.standard_normal(d))
+    elif kind == "negative lognormal":
+        x = -np.exp(4 * rng.standard_normal(d))
+    elif kind == "one-sided cauchy":
+        x = np.abs(x)
+    elif kind == "tail and ties":
+        x = np.where(rng.random(d) < 0.3, 1e-3, np.exp(5 * rng.standard_normal(d)))
+    check(ws, ctx, x.astype(dt))
