@@ -418,12 +418,14 @@ ws_status build_plan(ws_plan* p) {
         B.n_bins = (int)bwd_map.size();
         bwd_map.resize((bwd_map.size() + 7) & ~(size_t)7, make_int2(0, -1));   // (k_bwd_scan reads eight bins at a time)
         const size_t nb = bwd_map.size(), nl4 = ((size_t)p->n_lseg + 3) & ~(size_t)3;
-        const size_t words = nl4 + 3 * nb + 1;
+        const size_t words = nl4 + 5 * nb + 1;
         B.zero_bytes = sizeof(int32_t) * words;
         if ((st = plan_alloc(p, (void**)&B.emax, B.zero_bytes))) return st;
         B.cnt = (uint32_t*)B.emax + nl4;
         B.extra = B.cnt + nb;
-        B.arrive = B.extra + nb;
+        B.xlo = B.extra + nb;
+        B.xhi = B.xlo + nb;
+        B.arrive = B.xhi + nb;
         B.n_items = (int32_t*)(B.arrive + nb);
         int2* map = nullptr;
         if ((st = plan_upload(p, &map, bwd_map))) return st;

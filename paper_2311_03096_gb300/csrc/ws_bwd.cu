@@ -42,6 +42,7 @@ constexpr int ANT = 256;              // k_bwd_bins
 constexpr int PIECE = WS_BWD_PIECE;
 constexpr int CHUNK = 8 * ANT;        // pairs of one step of k_bwd_bins
 constexpr int EXTRA = 4 * 152;        // CTAs of k_bwd_bins for the split bins
+constexpr int MAIN = 8192;            // and for the others at most (empty bins cost a CTA's launch: 24576 of them 50 us)
 constexpr int HIST_MAX = 16384;       // bins that k_bwd_prep counts in shared memory
 
 template <typename T> struct BwdFix;
@@ -178,7 +179,8 @@ template <typename T>
 __global__ void __launch_bounds__(PNT, 3) k_bwd_prep(const T* __restrict__ g, const int32_t* __restrict__ ids,
                                                      const TileDesc* __restrict__ tiles, int n_tiles,
                                                      const LargeSeg* __restrict__ lsegs, int n_hist, int32_t* seg_emax,
-                                                     uint32_t* cnt, uint32_t* extra, uint32_t* status) {
+                                                     uint32_t* cnt, uint32_t* extra, uint32_t* xlo, uint32_t* xhi,
+                                                     uint32_t* status) {
     extern __shared__ uint32_t hist[];   // [n_hist]
     const int t = threadIdx.x, lane = t & 31;
     for (int b = t; b < n_hist; b += PNT) hist[b] = 0;
@@ -208,7 +210,12 @@ __global__ void __launch_bounds__(PNT, 3) k_bwd_prep(const T* __restrict__ g, co
         if (lane == 0 && e > *(volatile int32_t*)(seg_emax + td.lseg)) atomicMax(seg_emax + td.lseg, e);
         if (__syncthreads_and(same)) {   // (also the barrier after the clearing of hist)
             if (id0 < 0 || (int64_t)id0 >= slen) bad = true;
-            else if (t == 0) atomicAdd(extra + bpos + (id0 >> WS_BWD_BIN_LOG2), 1u);
+            else if (t == 0 && td.len < slen) {   // (the only tile of its segment writes the mean itself)
+                const int b = bpos + (id0 >> WS_BWD_BIN_LOG2), r = id0 & (WS_BWD_BIN - 1);
+                atomicAdd(extra + b, 1u);
+                atomicMax(xlo + b, (uint32_t)(WS_BWD_BIN - r));
+                atomicMax(xhi + b, (uint32_t)(r + 1));
+            }
             continue;
         }
 #pragma unroll
@@ -303,12 +310,16 @@ __global__ void __launch_bounds__(SCAN_NT) k_bwd_scan(const uint32_t* __restrict
     if (t == 0) { start[n_bins] = (unsigned long long)run; *n_items = s_items; }
 }
 
-// The bins whose sums are formed in global memory start from zero: split ones,
-// and those that whole tiles add to (a warp per bin).
+// The slots whose sums are formed in global memory start from zero: those of split
+// bins, and from the first to the last one that whole tiles add to (a warp per bin).
+// (With whole bins there, segments of one cluster cleared and read 40 KB each: 2000 of
+// 10000 elements 248 us, now 211.)
 __global__ void __launch_bounds__(256) k_bwd_clear(const uint32_t* __restrict__ cnt,
-                                                   const uint32_t* __restrict__ extra, int n_bins,
-                                                   const int2* __restrict__ map, const LargeSeg* __restrict__ lsegs,
-                                                   unsigned long long* acc, int32_t* gcnt) {
+                                                   const uint32_t* __restrict__ extra,
+                                                   const uint32_t* __restrict__ xlo, const uint32_t* __restrict__ xhi,
+                                                   int n_bins, const int2* __restrict__ map,
+                                                   const LargeSeg* __restrict__ lsegs, unsigned long long* acc,
+                                                   int32_t* gcnt) {
     ws_chain();
     const int lane = threadIdx.x & 31;
     const int nw = (int)gridDim.x * 8;
@@ -318,7 +329,9 @@ __global__ void __launch_bounds__(256) k_bwd_clear(const uint32_t* __restrict__ 
         const LargeSeg& ls = lsegs[lseg];
         const int64_t r0 = (int64_t)(b - ls.bb_pos) << WS_BWD_BIN_LOG2;
         const int64_t r1 = min(r0 + WS_BWD_BIN, ls.len), slot0 = ls.kpos + lseg;
-        for (int64_t r = r0 + lane; r < r1; r += 32) {
+        const bool split = cnt[b] > PIECE;
+        const int64_t a = split ? r0 : r0 + WS_BWD_BIN - xlo[b], z = split ? r1 : r0 + xhi[b];
+        for (int64_t r = a + lane; r < z; r += 32) {
             acc[2 * (slot0 + r)] = 0ull;
             acc[2 * (slot0 + r) + 1] = 0ull;
             gcnt[slot0 + r] = 0;
@@ -350,7 +363,8 @@ __global__ void __launch_bounds__(PNT, 2) k_bwd_part(const typename KeyOf<T>::K*
                                                      const LargeSeg* __restrict__ lsegs,
                                                      const unsigned long long* __restrict__ start,
                                                      unsigned long long* cursor, const int32_t* __restrict__ seg_emax,
-                                                     unsigned long long* acc, int32_t* gcnt, int64_t n_pairs) {
+                                                     unsigned long long* acc, int32_t* gcnt, T* mean,
+                                                     int64_t n_pairs) {
     typedef KeyOf<T> KO;
     typedef typename KO::K K;
     static_assert(WS_BWD_FAN == PNT, "one bucket per thread");
@@ -412,8 +426,9 @@ __global__ void __launch_bounds__(PNT, 2) k_bwd_part(const typename KeyOf<T>::K*
                 if (id0 >= 0 && id0 < slen) {   // (uniform)
                     const int emax = seg_emax[lseg];
                     i128 sum = 0;
-#pragma unroll 1
-                    for (int i = t; i < len; i += PNT) sum += ws_bwd_fix<T>(ws_g_of_bits<T>(__ldg(g_in + cur.pos + i)), emax);
+#pragma unroll
+                    for (int k = 0; k < ITEMS; ++k)
+                        if (t + k * PNT < len) sum += ws_bwd_fix<T>(ws_g_of_bits<T>(gv[k]), emax);
                     sum = ws_warp_reduce_i128(sum);
                     if (lane == 0) { s.wlo[w] = (long long)(uint64_t)sum; s.whi[w] = (long long)(uint64_t)((u128)sum >> 64); }
                     __syncthreads();
@@ -422,8 +437,11 @@ __global__ void __launch_bounds__(PNT, 2) k_bwd_part(const typename KeyOf<T>::K*
                         for (int k = 0; k < PNT / 32; ++k)
                             tot += (i128)(((u128)(uint64_t)s.whi[k] << 64) | (u128)(uint64_t)s.wlo[k]);
                         const int64_t slot = sg.kpos + lseg + id0;
-                        ws_atomic_add_i128(acc + 2 * slot, tot);
-                        atomicAdd(gcnt + slot, len);
+                        if (len == slen) mean[slot] = ws_bwd_mean<T>(tot, len, emax);
+                        else {
+                            ws_atomic_add_i128(acc + 2 * slot, tot);
+                            atomicAdd(gcnt + slot, len);
+                        }
                     }
                 }
             }
@@ -495,7 +513,7 @@ __global__ void __launch_bounds__(PNT, 2) k_bwd_part(const typename KeyOf<T>::K*
 }
 
 // 4. the sums of a bin's slots in shared memory, and its means.  CTA b takes
-// bin b; the last EXTRA CTAs the pieces of the split ones.  Pairs are added in
+// bin b (and b + MAIN ..); the last EXTRA CTAs the pieces of the split ones.  Pairs are added in
 // steps of CHUNK; with more than 4096 of them the limbs are normalised after
 // every step (the top limb's carries go to the upper half of the counter, whose
 // lower half holds at most PIECE).
@@ -508,7 +526,9 @@ template <typename T>
 __global__ void __launch_bounds__(ANT, 4) k_bwd_bins(const typename KeyOf<T>::K* __restrict__ g_b,
                                                      const int32_t* __restrict__ id_b,
                                                      const uint32_t* __restrict__ cnt,
-                                                     const uint32_t* __restrict__ extra, int n_bins,
+                                                     const uint32_t* __restrict__ extra,
+                                                     const uint32_t* __restrict__ xlo,
+                                                     const uint32_t* __restrict__ xhi, int n_bins,
                                                      const int2* __restrict__ map, const LargeSeg* __restrict__ lsegs,
                                                      const unsigned long long* __restrict__ start,
                                                      const uint2* __restrict__ items,
@@ -533,6 +553,17 @@ __global__ void __launch_bounds__(ANT, 4) k_bwd_bins(const typename KeyOf<T>::K*
         const int nr = (int)min((int64_t)WS_BWD_BIN, ls.len - r0);
         const int64_t slot0 = ls.kpos + lseg + r0;
         const int emax = seg_emax[lseg];
+        // (what whole tiles added, and to which slots)
+        const int xa = more ? WS_BWD_BIN - (int)xlo[bin] : 0, xz = more ? (int)xhi[bin] : 0;
+        auto tiles_cnt = [&](int r) { return gcnt[slot0 + r]; };
+        auto tiles_sum = [&](int r) { return (i128)(((u128)acc[2 * (slot0 + r) + 1] << 64) | (u128)acc[2 * (slot0 + r)]); };
+        if (nbin == 0) {   // (no pairs: only these)
+            for (int r = xa + t; r < xz; r += ANT) {
+                const int c = tiles_cnt(r);
+                if (c) mean[slot0 + r] = ws_bwd_mean<T>(tiles_sum(r), c, emax);
+            }
+            return;
+        }
         const int64_t p0 = (int64_t)start[bin] + (piece > 0 ? (int64_t)piece * PIECE : 0);
         const int n = piece < 0 ? nbin : min(PIECE, nbin - piece * PIECE);
         __syncthreads();   // (the previous use of the shared memory is over)
@@ -596,9 +627,9 @@ __global__ void __launch_bounds__(ANT, 4) k_bwd_bins(const typename KeyOf<T>::K*
             for (int r = t; r < nr; r += ANT) {
                 int c = slot_cnt(r);
                 i128 S = slot_sum(r);
-                if (more) {   // (what whole tiles added)
-                    c += gcnt[slot0 + r];
-                    S += (i128)(((u128)acc[2 * (slot0 + r) + 1] << 64) | (u128)acc[2 * (slot0 + r)]);
+                if (r >= xa && r < xz) {
+                    c += tiles_cnt(r);
+                    S += tiles_sum(r);
                 }
                 if (c) mean[slot0 + r] = ws_bwd_mean<T>(S, c, emax);
             }
@@ -625,12 +656,14 @@ __global__ void __launch_bounds__(ANT, 4) k_bwd_bins(const typename KeyOf<T>::K*
             mean[slot0 + r] = ws_bwd_mean<T>(S, c, emax);
         }
     };
-    if ((int)blockIdx.x < n_bins) {
-        if (cnt[blockIdx.x] <= PIECE) run(blockIdx.x, -1);
+    const int n_main = (int)gridDim.x - EXTRA;
+    if ((int)blockIdx.x < n_main) {
+        for (int b = blockIdx.x; b < n_bins; b += n_main)
+            if (cnt[b] <= PIECE) run(b, -1);
         return;
     }
     const int ni = *n_items;
-    for (int i = (int)blockIdx.x - n_bins; i < ni; i += EXTRA) {
+    for (int i = (int)blockIdx.x - n_main; i < ni; i += EXTRA) {
         const uint2 it = items[i];
         run((int)it.x, (int)it.y);
     }
@@ -766,24 +799,25 @@ cudaError_t ws_large_backward(const LargeWork<T>& W, const T* g, const int32_t* 
     const int grid = std::min(nt, 2 * 152);
     WS_LAUNCH(W.prof, WSK_BWD, st,
               (k_bwd_prep<T><<<std::min(nt, 3 * 152), PNT, hsm, st>>>(g, ids, W.sort_tiles, nt, W.lsegs, n_hist, B.emax, B.cnt, B.extra,
-                                                     status)));
+                                                     B.xlo, B.xhi, status)));
     WS_LAUNCH(W.prof, WSK_BWD, st,
               ws_launch_chain(k_bwd_scan, 1, SCAN_NT, 0, st, B.cnt, B.n_bins, B.map, B.start, B.cur1, B.cur2, B.items,
                               B.n_items));
     WS_LAUNCH(W.prof, WSK_BWD, st,
-              ws_launch_chain(k_bwd_clear, std::min((B.n_bins + 7) / 8, 8 * 152), 256, 0, st, B.cnt, B.extra, B.n_bins,
-                              B.map, W.lsegs, W.bacc, W.bcnt));
+              ws_launch_chain(k_bwd_clear, std::min((B.n_bins + 7) / 8, 8 * 152), 256, 0, st, B.cnt, B.extra, B.xlo, B.xhi,
+                              B.n_bins, B.map, W.lsegs, W.bacc, W.bcnt));
     WS_LAUNCH(W.prof, WSK_BWD, st,
               ws_launch_chain(k_bwd_part<T, true>, grid, PNT, psm, st, reinterpret_cast<const K*>(g), ids, g_a, id_a,
                               g_b, id_b, W.sort_tiles, nt, W.lsegs, B.start, B.cur1, B.emax, W.bacc, W.bcnt,
-                              W.n_keys));
+                              W.bsum, W.n_keys));
     if (B.two_level)
         WS_LAUNCH(W.prof, WSK_BWD, st,
                   ws_launch_chain(k_bwd_part<T, false>, grid, PNT, psm, st, g_a, id_a, g_a, id_a, g_b, id_b,
-                                  W.sort_tiles, nt, W.lsegs, B.start, B.cur2, B.emax, W.bacc, W.bcnt, W.n_keys));
+                                  W.sort_tiles, nt, W.lsegs, B.start, B.cur2, B.emax, W.bacc, W.bcnt, W.bsum,
+                                  W.n_keys));
     WS_LAUNCH(W.prof, WSK_BWD, st,
-              ws_launch_chain(k_bwd_bins<T>, B.n_bins + EXTRA, ANT, bsm, st, g_b, id_b, B.cnt, B.extra, B.n_bins,
-                              B.map, W.lsegs, B.start, B.items, B.n_items, B.arrive, B.emax, W.bacc, W.bcnt, W.bsum));
+              ws_launch_chain(k_bwd_bins<T>, std::min(B.n_bins, MAIN) + EXTRA, ANT, bsm, st, g_b, id_b, B.cnt, B.extra, B.xlo, B.xhi,
+                              B.n_bins, B.map, W.lsegs, B.start, B.items, B.n_items, B.arrive, B.emax, W.bacc, W.bcnt, W.bsum));
     // (a gather that lives off the caches: a plain launch)
     WS_LAUNCH(W.prof, WSK_BWD, st,
               ws_launch_if(nt <= 2 * 152, k_bwd_apply<T>, nt, PNT, 0, st, ids, W.sort_tiles, W.lsegs, W.bsum, gin));

@@ -190,6 +190,8 @@ struct BwdWork {
     int32_t* emax;                 // [n_lseg] largest grad_out exponent
     uint32_t* cnt;                 // [n_bins] pairs
     uint32_t* extra;               // [n_bins] tiles of one cluster (they move no pairs)
+    uint32_t* xlo;                 // [n_bins] the slots these add to: WS_BWD_BIN - the first one (0: none)
+    uint32_t* xhi;                 // [n_bins] and the last one + 1
     uint32_t* arrive;              // [n_bins] finished pieces
     int32_t* n_items;              // pieces of the split bins
     const int2* map;               // [n_bins] (segment, bucket of the first move that starts here or -1)
