@@ -273,7 +273,7 @@ ws_status build_plan(ws_plan* p) {
             p->two_level = 1;
         }
         ls.n_coarse = ((ls.nbins - 1) >> ls.fine_log2) + 1;
-        ls.ncell = ls.nbins == 1 ? 0 : ls.fine_log2 ? WS_CELLS : WS_CELLS / 2;
+        ls.ncell = ls.sort_count == 1 ? 0 : ls.fine_log2 ? WS_CELLS : WS_CELLS / 2;
         // samples per tile: 100 per bin for one-pass segments, 50 for longer ones (about 2^20 at most)
         ls.samp_log2 = ls.fine_log2 ? 7 : 8;
         while (ls.samp_log2 > 5 && ((int64_t)ls.sort_count << ls.samp_log2) > ((int64_t)1 << 20)) --ls.samp_log2;

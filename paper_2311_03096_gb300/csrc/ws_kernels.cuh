@@ -121,7 +121,7 @@ struct LargeSeg {
     int32_t nbins;             // bins of the segment
     int32_t fine_log2;         // first pass: bucket = bin >> fine_log2 (0: one pass only)
     int32_t n_coarse;          // buckets of the first pass
-    int32_t ncell;             // cells of the segment's map (a power of two; 0 for one bin, which needs no map)
+    int32_t ncell;             // cells of the segment's map (a power of two; 0 for one tile, which needs no map)
     int32_t samp_log2;         // sampled elements per sort tile
     int32_t bin_pos, coarse_pos;   // slices of the per-bin / bucket arrays
     int64_t cell_pos;              // and of the cell array

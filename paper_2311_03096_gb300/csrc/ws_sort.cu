@@ -40,6 +40,8 @@
 namespace {
 
 constexpr int PLAN_NT = 1024;
+constexpr int PLAN_SMP = 8;   // samples per lane of a segment of one tile
+static_assert(WS_SORT_TILE <= 3 * WS_BIN_MEAN, "such a segment has at most three bins");
 constexpr int OVER_NT = WS_SORT_NT;
 
 __device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
@@ -169,7 +171,7 @@ __device__ __forceinline__ int sample_pos(int tile, int j, int len, int mlog) {
 struct PlanSmem {
     unsigned long long hi, lo, mag;
     int emin;
-    int map;   // the CTA has tiles of segments with more than one bin
+    int map;   // the CTA has tiles of segments with a map
     int wsum[PLAN_NT / 32];
 };
 
@@ -207,23 +209,61 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
     for (int tile = t0 + w; tile < t1; tile += PLAN_NT / 32) {
         const TileDesc td = tiles[tile];
         const LargeSeg& sg = lsegs[td.lseg];
-        if (sg.nbins == 1) {   // one tile and no map: the warp does all that the phases do for others
+        if (sg.sort_count == 1) {   // no map: the warp does all that the phases do for longer segments
+            const int nb = sg.nbins, len = td.len;
+            const T* src = values + td.vpos;
+            K s1 = ~(K)0, s2 = ~(K)0;   // the bins after the first start at these keys
+            if (nb > 1) {
+                const int m = 1 << sg.samp_log2;
+                K smp[PLAN_SMP];
+#pragma unroll
+                for (int q = 0; q < PLAN_SMP; ++q) {
+                    const int j = lane + 32 * q;
+                    smp[q] = j < m ? KO::to_key(__ldg(src + sample_pos(tile, j, len, sg.samp_log2))) : ~(K)0;
+                }
+                // the samples of rank m / nb and 2 m / nb, bit by bit
+                const int r1 = m / nb, r2 = nb > 2 ? 2 * m / nb : m;
+                s1 = s2 = 0;
+#pragma unroll 1
+                for (K bit = (K)1 << (KO::BITS - 1); bit != 0; bit >>= 1) {
+                    uint32_t c = 0;   // samples below s1 | bit, and below s2 | bit
+#pragma unroll
+                    for (int q = 0; q < PLAN_SMP; ++q) c += (smp[q] < (s1 | bit) ? 1u : 0u) + (smp[q] < (s2 | bit) ? 0x10000u : 0u);
+                    c = __reduce_add_sync(WS_FULL_MASK, c);
+                    if ((int)(c & 0xffffu) <= r1) s1 |= bit;
+                    if ((int)(c >> 16) <= r2) s2 |= bit;
+                }
+            }
             K amax = 0, amin = ~(K)0;   // (as in phase 4)
-#pragma unroll 4
-            for (int i = lane; i < td.len; i += 32) {
-                const K mag = (K)KO::bits(__ldg(values + td.vpos + i)) & (~(K)0 >> 1);
-                amax = max(amax, mag);
-                amin = min(amin, mag - 1);
-                bins[td.kpos + i] = 0;
+            int c1 = 0, c2 = 0;
+            B* bo = bins + td.kpos;
+            for (int i0 = lane; i0 - lane < len; i0 += 32 * 8) {
+                T v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] = __ldg(src + min(i0 + 32 * u, len - 1));
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const bool in = i0 + 32 * u < len;
+                    const K mag = (K)KO::bits(v[u]) & (~(K)0 >> 1), k = KO::to_key(v[u]);
+                    amax = max(amax, mag);
+                    amin = min(amin, mag - 1);
+                    const int b1 = nb > 1 && k >= s1, b2 = nb > 2 && k >= s2;
+                    c1 += in && b1;
+                    c2 += in && b2;
+                    if (in) bo[i0 + 32 * u] = (B)(b1 + b2);
+                }
             }
             bad |= (amax >> KO::MANT) >= (K)KO::EXPMASK;
             int emin = amin != ~(K)0 ? max((int)((amin + 1) >> KO::MANT), 1) : 0x7fffffff;
             emin = __reduce_min_sync(WS_FULL_MASK, emin);
-            if (lane == 0) {
-                seg_emin[td.lseg] = emin;
-                bin_cnt[sg.bin_pos] = (uint32_t)td.len;
-                bin_start[sg.bin_pos] = 0;
-                cur1[sg.coarse_pos] = 0;
+            c1 = __reduce_add_sync(WS_FULL_MASK, c1);
+            c2 = __reduce_add_sync(WS_FULL_MASK, c2);
+            if (lane == 0) seg_emin[td.lseg] = emin;
+            if (lane < nb) {
+                const int start = lane == 0 ? 0 : len - (lane == 1 ? c1 : c2), end = lane + 1 == nb ? len : len - (lane == 0 ? c1 : c2);
+                bin_cnt[sg.bin_pos + lane] = (uint32_t)(end - start);
+                bin_start[sg.bin_pos + lane] = (uint32_t)start;
+                cur1[sg.coarse_pos + lane] = (uint32_t)start;
             }
             continue;
         }
@@ -316,7 +356,7 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
         const int lseg = tiles[ta].lseg;
         const LargeSeg sg = lsegs[lseg];
         const int tb = min(t1, sg.sort_first + sg.sort_count);
-        if (sg.nbins == 1) { ta = tb; continue; }   // (uniform)
+        if (sg.sort_count == 1) { ta = tb; continue; }   // (uniform)
         const SortHdr h = header(lseg, sg);
         uint32_t* sc = tab.split;   // [ncell]
         for (int i = t; i < sg.ncell; i += PLAN_NT) sc[i] = 0;
@@ -380,7 +420,7 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
         const int lseg = tiles[ta].lseg;
         const LargeSeg sg = lsegs[lseg];
         const int tb = min(t1, sg.sort_first + sg.sort_count);
-        if (sg.nbins == 1) { ta = tb; continue; }   // (uniform)
+        if (sg.sort_count == 1) { ta = tb; continue; }   // (uniform)
         const SortHdr h = header(lseg, sg);
         const int parts = parts_of(sg, h);
         uint32_t* sc = reinterpret_cast<uint32_t*>(tab.knots);   // [parts]
@@ -408,7 +448,7 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
         const int lseg = tiles[ta].lseg;
         const LargeSeg sg = lsegs[lseg];
         const int tb = min(t1, sg.sort_first + sg.sort_count);
-        if (sg.nbins == 1) { ta = tb; continue; }   // (uniform)
+        if (sg.sort_count == 1) { ta = tb; continue; }   // (uniform)
         const bool local = sg.nbins <= hist_cap;
         const SortHdr h = header(lseg, sg);
         const int parts = parts_of(sg, h);
@@ -543,7 +583,7 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
         const int first = (int)(((int64_t)blockIdx.x + (int64_t)gridDim.x * (c0 / PLAN_NT) - c0 / PLAN_NT) % gridDim.x);
         for (int lseg = first; lseg < n_lseg; lseg += gridDim.x) {
             const LargeSeg sg = lsegs[lseg];
-            if (c0 >= sg.nbins || sg.nbins == 1) continue;   // (uniform)
+            if (c0 >= sg.nbins || sg.sort_count == 1) continue;   // (uniform)
             const uint32_t* c = bin_cnt + sg.bin_pos;
             int before = 0;
 #pragma unroll 8
