@@ -416,7 +416,7 @@ ws_status build_plan(ws_plan* p) {
     if (!p->sort_only) {
         BwdWork& B = p->bwd;
         B.n_bins = (int)bwd_map.size();
-        bwd_map.resize((bwd_map.size() + 7) & ~(size_t)7, make_int2(0, -1));   // (k_bwd_scan reads eight bins at a time)
+        bwd_map.resize((bwd_map.size() + 7) & ~(size_t)7, make_int2(0, -1));   // (k_bwd_scan reads two bins at a time)
         const size_t nb = bwd_map.size(), nl4 = ((size_t)p->n_lseg + 3) & ~(size_t)3;
         const size_t words = nl4 + 5 * nb + 1;
         B.zero_bytes = sizeof(int32_t) * words;
