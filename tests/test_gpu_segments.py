@@ -46,6 +46,19 @@ def test_short_segments(ctx, dt):
     same(ctx, w, offsets, lams, dt)
 
 
+@pytest.mark.parametrize("dt", [torch.float32, torch.float64])
+@pytest.mark.parametrize("n", [1, 2, 150, 700, 1350])   # one to nine segments of one tile per CTA
+def test_few_segments(ctx, n, dt):
+    rng = np.random.default_rng(n)
+    lens = rng.integers(1, 4097, n)
+    lens[: n // 5] = rng.integers(2049, 6145, n // 5)
+    lens[n // 2] = [1, 2049, 4097, 6144, 30000][n % 5]
+    offsets = np.concatenate([[0], np.cumsum(lens)])
+    w = torch.from_numpy(rng.standard_normal(int(offsets[-1]))).cuda().to(dt)
+    lams = torch.from_numpy(np.exp(rng.uniform(-7, 1, n))).cuda()
+    same(ctx, w, offsets, lams, dt)
+
+
 @pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
 def test_not_finite(ctx, bad):
     from paper_2311_03096_gb300 import ws
