@@ -482,7 +482,10 @@ struct TileHullSmem {
 // The general tile kernel: the exact hull of a tile whose prefix sums need
 // 128 bits (or whose bridge walks were too long for the lean kernel of
 // ws_tile.cu, which lists such tiles in gen_list).  A small grid walks the
-// list.  Four CTAs per SM (64 registers; only the rare merge paths spill).
+// list.  Four CTAs per SM (64 registers, 412/788 bytes of spills in FP64): many
+// tiles are what it takes long for.  8192 FP64 segments of 4097: 833 us; with
+// three CTAs and 76/76 bytes 990, with two and no spills 909.  A lone vector with
+// two such tiles would gain: 4194001 FP64 weights 460, 446 with two CTAs.
 template <typename T>
 __global__ void __launch_bounds__(HNT, 4) k_tile_hull(const typename KeyOf<T>::K* __restrict__ sorted,
                                                    const TileDesc* __restrict__ htiles,
