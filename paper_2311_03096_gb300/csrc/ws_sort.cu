@@ -41,11 +41,8 @@ namespace {
 
 constexpr int PLAN_NT = 1024;
 constexpr int PLAN_SMP = 8;   // samples per lane of a segment of one tile
-// Up to this many tiles the whole CTA counts each of its segments of one tile, beside the maps of its longer
-// ones; above, a warp counts one alone.  A warp takes 15 us for 6144 elements, and before the first grid barrier
-// every CTA waits for it: 28 segments of 16 to 1048576 weights 282 us so, 265 by the CTA in the map's place (262
-// to 264 with maps for all); one of 4694 weights 97 and 81 (87 to 95).  8192 rows of 4097, 54 tiles a CTA: 1704
-// by warps (2322 with maps).
+// Up to this many segments of one tile are counted by the whole CTA one after the
+// other, more by a warp each (15 us for 6144 elements).
 constexpr int PLAN_ONE = 8;
 static_assert(WS_SORT_TILE <= 3 * WS_BIN_MEAN, "such a segment has at most three bins");
 constexpr int OVER_NT = WS_SORT_NT;
@@ -183,6 +180,121 @@ struct PlanSmem {
     int wsum[PLAN_NT / 32];
 };
 
+// Segments of one tile (S.n_one of the CTA's tiles): their bins start at quantiles
+// of a sample, which a warp finds, and the elements are counted against these.  No
+// other CTA needs any of it in the plan, so that it stands where the CTA maps the
+// elements of its longer segments.  Out of line: inlined it cost the plans of longer
+// segments 2 us (instruction fetches).  true: a weight that is not finite.
+template <typename T, typename B>
+__device__ __noinline__ bool plan_one(PlanSmem& S, const T* __restrict__ values, const TileDesc* __restrict__ tiles, int t0,
+                                      int t1, const LargeSeg* __restrict__ lsegs, B* bins, uint32_t* bin_cnt,
+                                      uint32_t* bin_start, uint32_t* cur1, int32_t* seg_emin) {
+    typedef KeyOf<T> KO;
+    typedef typename KO::K K;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5, n_one = S.n_one;
+    const bool cta = n_one <= PLAN_ONE;   // (else a warp for each)
+    bool bad = false;
+    auto split = [&](const TileDesc& td, const LargeSeg& sg, int tile, K& s1, K& s2) {
+        const int nb = sg.nbins;
+        s1 = s2 = ~(K)0;   // the bins after the first start at these keys
+        if (nb == 1) return;
+        const int m = 1 << sg.samp_log2;
+        K smp[PLAN_SMP];
+#pragma unroll
+        for (int q = 0; q < PLAN_SMP; ++q) {
+            const int j = lane + 32 * q;
+            smp[q] = j < m ? KO::to_key(__ldg(values + td.vpos + sample_pos(tile, j, td.len, sg.samp_log2))) : ~(K)0;
+        }
+        // the samples of rank m / nb and 2 m / nb, bit by bit
+        const int r1 = m / nb, r2 = nb > 2 ? 2 * m / nb : m;
+        s1 = s2 = 0;
+#pragma unroll 1
+        for (K bit = (K)1 << (KO::BITS - 1); bit != 0; bit >>= 1) {
+            uint32_t c = 0;   // samples below s1 | bit, and below s2 | bit
+#pragma unroll
+            for (int q = 0; q < PLAN_SMP; ++q) c += (smp[q] < (s1 | bit) ? 1u : 0u) + (smp[q] < (s2 | bit) ? 0x10000u : 0u);
+            c = __reduce_add_sync(WS_FULL_MASK, c);
+            if ((int)(c & 0xffffu) <= r1) s1 |= bit;
+            if ((int)(c >> 16) <= r2) s2 |= bit;
+        }
+    };
+    auto done = [&](const TileDesc& td, const LargeSeg& sg, int c1, int c2, int emin) {   // (one thread)
+        seg_emin[td.lseg] = emin;
+        const int at[4] = {0, td.len - c1, td.len - c2, td.len}, nb = sg.nbins;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            if (q >= nb) break;
+            const int end = q + 1 == nb ? td.len : at[q + 1];
+            bin_cnt[sg.bin_pos + q] = (uint32_t)(end - at[q]);
+            bin_start[sg.bin_pos + q] = (uint32_t)at[q];
+            cur1[sg.coarse_pos + q] = (uint32_t)at[q];
+        }
+    };
+    if (cta) {
+        if (w < n_one) {
+            const int tile = S.one[w].tile;
+            const TileDesc td = tiles[tile];
+            K s1, s2;
+            split(td, lsegs[td.lseg], tile, s1, s2);
+            if (lane == 0) {
+                S.one[w].s1 = s1;
+                S.one[w].s2 = s2;
+                S.one[w].c1 = S.one[w].c2 = 0;
+                S.one[w].emin = 0x7fffffff;
+            }
+        }
+        __syncthreads();
+    }
+    const int i0 = cta ? t : lane, step = cta ? PLAN_NT : 32;
+    for (int q = cta ? 0 : w; q < (cta ? n_one : t1 - t0); q += cta ? 1 : PLAN_NT / 32) {
+        const int tile = cta ? S.one[q].tile : t0 + q;
+        const TileDesc td = tiles[tile];
+        const LargeSeg& sg = lsegs[td.lseg];
+        if (sg.sort_count != 1) continue;
+        const int nb = sg.nbins, len = td.len;
+        K s1, s2;
+        if (cta) { s1 = (K)S.one[q].s1; s2 = (K)S.one[q].s2; }
+        else split(td, sg, tile, s1, s2);
+        const T* src = values + td.vpos;
+        B* bo = bins + td.kpos;
+        K amax = 0, amin = ~(K)0;   // (as in phase 4)
+        int c1 = 0, c2 = 0;         // keys from s1 on, and from s2 on
+        for (int i = i0; i - lane < len; i += step * 8) {
+            T v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = __ldg(src + min(i + step * u, len - 1));
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const bool in = i + step * u < len;
+                const K mag = (K)KO::bits(v[u]) & (~(K)0 >> 1), k = KO::to_key(v[u]);
+                amax = max(amax, mag);
+                amin = min(amin, mag - 1);
+                const int b1 = nb > 1 && k >= s1, b2 = nb > 2 && k >= s2;
+                c1 += in && b1;
+                c2 += in && b2;
+                if (in) bo[i + step * u] = (B)(b1 + b2);
+            }
+        }
+        bad |= (amax >> KO::MANT) >= (K)KO::EXPMASK;
+        int emin = amin != ~(K)0 ? max((int)((amin + 1) >> KO::MANT), 1) : 0x7fffffff;
+        emin = __reduce_min_sync(WS_FULL_MASK, emin);
+        c1 = __reduce_add_sync(WS_FULL_MASK, c1);
+        c2 = __reduce_add_sync(WS_FULL_MASK, c2);
+        if (lane == 0) {
+            if (cta) { atomicAdd(&S.one[q].c1, c1); atomicAdd(&S.one[q].c2, c2); atomicMin(&S.one[q].emin, emin); }
+            else done(td, sg, c1, c2, emin);
+        }
+    }
+    if (cta) {
+        __syncthreads();
+        if (t < n_one) {
+            const TileDesc td = tiles[S.one[t].tile];
+            done(td, lsegs[td.lseg], S.one[t].c1, S.one[t].c2, S.one[t].emin);
+        }
+    }
+    return bad;
+}
+
 template <typename T, typename B>
 __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ values,
                                                           const TileDesc* __restrict__ tiles, int n_tiles,
@@ -214,85 +326,13 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
     if (t == 0) { S.hi = 0; S.lo = 0; S.mag = 0; S.map = 0; S.n_one = 0; }
     __syncthreads();
     bool bad = false;
-    // A segment of one tile has no map: its bins start at quantiles of its sample (one_split, a warp), and the
-    // elements are counted against these (one_tile, the threads i0 of `step`, whole warps).  No other CTA needs
-    // any of it here.
-    auto one_split = [&](const TileDesc& td, const LargeSeg& sg, int tile, K& s1, K& s2) {
-        const int nb = sg.nbins;
-        s1 = s2 = ~(K)0;   // the bins after the first start at these keys
-        if (nb == 1) return;
-        const int m = 1 << sg.samp_log2;
-        K smp[PLAN_SMP];
-#pragma unroll
-        for (int q = 0; q < PLAN_SMP; ++q) {
-            const int j = lane + 32 * q;
-            smp[q] = j < m ? KO::to_key(__ldg(values + td.vpos + sample_pos(tile, j, td.len, sg.samp_log2))) : ~(K)0;
-        }
-        // the samples of rank m / nb and 2 m / nb, bit by bit
-        const int r1 = m / nb, r2 = nb > 2 ? 2 * m / nb : m;
-        s1 = s2 = 0;
-#pragma unroll 1
-        for (K bit = (K)1 << (KO::BITS - 1); bit != 0; bit >>= 1) {
-            uint32_t c = 0;   // samples below s1 | bit, and below s2 | bit
-#pragma unroll
-            for (int q = 0; q < PLAN_SMP; ++q) c += (smp[q] < (s1 | bit) ? 1u : 0u) + (smp[q] < (s2 | bit) ? 0x10000u : 0u);
-            c = __reduce_add_sync(WS_FULL_MASK, c);
-            if ((int)(c & 0xffffu) <= r1) s1 |= bit;
-            if ((int)(c >> 16) <= r2) s2 |= bit;
-        }
-    };
-    auto one_tile = [&](const TileDesc& td, int nb, K s1, K s2, int i0, int step, int& c1, int& c2, int& emin) {
-        const T* src = values + td.vpos;
-        B* bo = bins + td.kpos;
-        const int len = td.len;
-        K amax = 0, amin = ~(K)0;   // (as in phase 4)
-        for (int i = i0; i - lane < len; i += step * 8) {
-            T v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = __ldg(src + min(i + step * u, len - 1));
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const bool in = i + step * u < len;
-                const K mag = (K)KO::bits(v[u]) & (~(K)0 >> 1), k = KO::to_key(v[u]);
-                amax = max(amax, mag);
-                amin = min(amin, mag - 1);
-                const int b1 = nb > 1 && k >= s1, b2 = nb > 2 && k >= s2;
-                c1 += in && b1;
-                c2 += in && b2;
-                if (in) bo[i + step * u] = (B)(b1 + b2);
-            }
-        }
-        bad |= (amax >> KO::MANT) >= (K)KO::EXPMASK;
-        emin = amin != ~(K)0 ? max((int)((amin + 1) >> KO::MANT), 1) : 0x7fffffff;
-        emin = __reduce_min_sync(WS_FULL_MASK, emin);
-        c1 = __reduce_add_sync(WS_FULL_MASK, c1);
-        c2 = __reduce_add_sync(WS_FULL_MASK, c2);
-    };
-    auto one_done = [&](const TileDesc& td, const LargeSeg& sg, int c1, int c2, int emin) {   // (one thread)
-        seg_emin[td.lseg] = emin;
-        const int at[4] = {0, td.len - c1, td.len - c2, td.len}, nb = sg.nbins;
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            if (q >= nb) break;
-            const int end = q + 1 == nb ? td.len : at[q + 1];
-            bin_cnt[sg.bin_pos + q] = (uint32_t)(end - at[q]);
-            bin_start[sg.bin_pos + q] = (uint32_t)at[q];
-            cur1[sg.coarse_pos + q] = (uint32_t)at[q];
-        }
-    };
-    const bool few = t1 - t0 <= PLAN_ONE;
     for (int tile = t0 + w; tile < t1; tile += PLAN_NT / 32) {
         const TileDesc td = tiles[tile];
         const LargeSeg& sg = lsegs[td.lseg];
-        if (sg.sort_count == 1) {   // no map
-            if (few) {   // (below, by the whole CTA)
-                if (lane == 0) S.one[atomicAdd(&S.n_one, 1)].tile = tile;
-            } else {
-                K s1, s2;
-                int c1 = 0, c2 = 0, emin = 0x7fffffff;
-                one_split(td, sg, tile, s1, s2);
-                one_tile(td, sg.nbins, s1, s2, lane, 32, c1, c2, emin);
-                if (lane == 0) one_done(td, sg, c1, c2, emin);
+        if (sg.sort_count == 1) {   // no map: plan_one below
+            if (lane == 0) {
+                const int q = atomicAdd(&S.n_one, 1);
+                if (q < PLAN_ONE) S.one[q].tile = tile;
             }
             continue;
         }
@@ -379,18 +419,6 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
         }
     };
 
-    if (w < S.n_one) {
-        const int tile = S.one[w].tile;
-        const TileDesc td = tiles[tile];
-        K s1, s2;
-        one_split(td, lsegs[td.lseg], tile, s1, s2);
-        if (lane == 0) {
-            S.one[w].s1 = s1;
-            S.one[w].s2 = s2;
-            S.one[w].c1 = S.one[w].c2 = 0;
-            S.one[w].emin = 0x7fffffff;
-        }
-    }
     // 2. sampled keys per cell (counted in shared memory, added to the
     // segment's cells once per CTA)
     for (int ta = t0; ta < tm;) {
@@ -483,19 +511,8 @@ __global__ void __launch_bounds__(PLAN_NT, 1) k_sort_plan(const T* __restrict__ 
     }
     bar.sync();
 
-    if (S.n_one > 0) {   // (uniform)
-        for (int q = 0; q < S.n_one; ++q) {
-            const TileDesc td = tiles[S.one[q].tile];
-            int c1 = 0, c2 = 0, emin = 0x7fffffff;
-            one_tile(td, lsegs[td.lseg].nbins, (K)S.one[q].s1, (K)S.one[q].s2, t, PLAN_NT, c1, c2, emin);
-            if (lane == 0) { atomicAdd(&S.one[q].c1, c1); atomicAdd(&S.one[q].c2, c2); atomicMin(&S.one[q].emin, emin); }
-        }
-        __syncthreads();
-        if (t < S.n_one) {
-            const TileDesc td = tiles[S.one[t].tile];
-            one_done(td, lsegs[td.lseg], S.one[t].c1, S.one[t].c2, S.one[t].emin);
-        }
-    }
+    if (S.n_one > 0) bad = plan_one<T, B>(S, values, tiles, t0, t1, lsegs, bins, bin_cnt, bin_start, cur1, seg_emin);
+
     // 4. knots of every segment (every CTA for the segments it needs), the bin
     // of every key, finiteness, smallest exponent
     for (int ta = t0; ta < tm;) {
