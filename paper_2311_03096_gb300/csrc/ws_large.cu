@@ -974,8 +974,9 @@ __device__ __noinline__ void bin_out_oversize(OverOutSmem<T>& s, int cta, int n_
     }
 }
 
+// (FP64: the staged pairs allow three CTAs; at six, 24/32 bytes of spills cost 5 of 64 us for 7.4M weights)
 template <typename T>
-__global__ void __launch_bounds__(256, 6) k_bin_out(const LargeSeg* __restrict__ lsegs, const SegRuntime* __restrict__ rt,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 6 : 3) k_bin_out(const LargeSeg* __restrict__ lsegs, const SegRuntime* __restrict__ rt,
                                                  const int32_t* __restrict__ bin_seg,
                                                  const uint32_t* __restrict__ bin_start,
                                                  const uint32_t* __restrict__ bin_cnt, int n_bins,
